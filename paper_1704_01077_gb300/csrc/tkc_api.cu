@@ -48,7 +48,7 @@ int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u3
     TKC_RC(dalloc(&w.sh, 1, st));
   }
   if (teams > w.teams_cap) {
-    TKC_RC(dalloc(&w.ctl, teams, st));
+    TKC_RC(dalloc(&w.ctl, 2 * (size_t)teams, st));
     TKC_RC(dalloc(&w.slots, (size_t)teams * 64 * kMaxWords, st));
     TKC_RC(dalloc(&w.cnt, (size_t)teams * 64 * kMaxWords, st));
     TKC_RC(dalloc(&w.wsum, (size_t)teams * 64 * kMaxWords, st));
@@ -79,6 +79,7 @@ int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u3
     TKC_RC(dalloc(&w.x_S, cap, st));
     TKC_RC(dalloc(&w.x_r, cap, st));
     TKC_RC(dalloc(&w.x_id, cap, st));
+    TKC_RC(dalloc(&w.f_end, cap, st));
     w.ng_cap = cap;
   }
   const u32 T = w.teams_cap;
@@ -117,11 +118,24 @@ int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u3
   return TKC_OK;
 }
 
+// Buffers of the filter between the opening and the main launch.
+static int ensure_filter(tkc_ctx *ctx, u32 count) {
+  Workspace &w = ctx->ws;
+  if (count <= w.f_cap) return TKC_OK;
+  w.f_cap = 0;
+  const u32 cap = std::max<u32>(count, 1024);
+  TKC_RC(dalloc(&w.f_order, cap, ctx->stream));
+  TKC_RC(dalloc(&w.f_mask, filter_mask_words(cap) + kFilterBlocks, ctx->stream));
+  w.f_cap = cap;
+  return TKC_OK;
+}
+
 static void free_workspace(tkc_ctx *ctx) {
   Workspace &w = ctx->ws;
   void *ptrs[] = {w.seen, w.F0, w.F1, w.N, w.FB0, w.FB1, w.L0, w.L1, w.Loff0, w.Loff1, w.VL, w.stamp, w.res_S, w.res_r,
                   w.slots, w.cnt, w.wsum, w.top_S, w.top_r, w.top_id, w.ctl, w.out_S, w.out_r, w.out_id,
-                  w.out_f, w.out_c, w.tied, w.g_ntop, w.g_stop, w.g_ctr, w.sh, w.x_seq, w.x_S, w.x_r, w.x_id};
+                  w.out_f, w.out_c, w.tied, w.g_ntop, w.g_stop, w.g_ctr, w.sh, w.x_seq, w.x_S, w.x_r, w.x_id,
+                  w.f_order, w.f_mask, w.f_end};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   w = Workspace();
@@ -314,15 +328,22 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     w.level_base = 0;
   }
   ctx->last_shard = nullptr;  // this run replaces the finished searches' (S, r)
-  if (!rs.keep_lists) {
-    TKC_TRY(cudaMemsetAsync(w.res_r, 0, (size_t)g->n * sizeof(u32), st));
-    TKC_TRY(cudaMemsetAsync(w.res_S, 0, (size_t)g->n * sizeof(u64), st));
-    TKC_TRY(cudaMemsetAsync(w.g_ntop, 0, (size_t)rs.ng * sizeof(unsigned), st));
-    TKC_TRY(cudaMemsetAsync(w.g_stop, 0, (size_t)rs.ng * sizeof(unsigned), st));
-    TKC_TRY(cudaMemsetAsync(w.g_ctr, 0, (size_t)rs.ng * 4 * sizeof(u64), st));
-    TKC_TRY(cudaMemsetAsync(w.x_seq, 0, (size_t)rs.ng * sizeof(unsigned), st));
-    TKC_TRY(cudaMemsetAsync(w.x_r, 0, (size_t)rs.ng * sizeof(u32), st));
-  }
+  // Opening: the first batch -- or as many as it takes for a full k-list --
+  // runs alone (one graph: on the whole grid; several: every graph's opening
+  // batch, on the teams), so that thresholds exist; then the filter drops the
+  // sources they abandon (k_filter_test) and the main launch searches the
+  // rest.  No host wait in between.  One-source searches and the deterministic
+  // schedule (both one team) take the order as it stands, since their counters
+  // are defined by it.
+  const bool exact_schedule = rs.B <= 1 || o.deterministic;
+  const u64 open_one = (u64)rs.B * std::max<u32>(1, (rs.kk + rs.B - 1) / rs.B);
+  const u32 nopen = rs.nocut ? 0u
+                    : rs.ng == 1 ? (u32)std::min<u64>(open_one, rs.norder)
+                                 : (rs.g_end ? rs.g_rest : 0u);
+  const bool opening = nopen > 0 && nopen < rs.norder && !exact_schedule;
+  const u32 open_teams = !opening ? 0u : rs.ng == 1 ? 1u : T;
+  if (opening) TKC_RC(ensure_filter(ctx, rs.norder - nopen));
+  TKC_RC(run_init(ctx, open_teams + T, g->n, rs.ng, !rs.keep_lists));
   if (rs.nseed) {
     const unsigned ns = rs.nseed;
     TKC_TRY(cudaMemcpyAsync(w.g_ntop, &ns, sizeof(unsigned), cudaMemcpyHostToDevice, st));
@@ -355,6 +376,10 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   p.n_bu_heavy = g->n_bu_heavy;
   p.heavy_in = g->heavy_in ? g->heavy_in : kHeavyIn;
   p.large_blocks = o.large_blocks;
+  // the bound after level 1 prunes only orders that do not know it already
+  // (NBCut's bounds hold level 2 and more)
+  if (opening && !rs.lb_key) TKC_RC(ensure_walks(const_cast<tkc_graph *>(g)));
+  p.walks = opening && !rs.lb_key ? g->walks : nullptr;
   p.alpha = g->alpha;
   p.omega = g->omega;
   p.order = rs.order;
@@ -423,98 +448,84 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     TKC_TRY(cudaMemsetAsync(p.trace, 0, (size_t)trace_cap * 16 * sizeof(u64), st));
     p.trace_cap = trace_cap;
   }
-  // Opening: with several teams on one graph, the first batch runs alone on
-  // the whole grid (one team), so that a threshold exists before the teams
-  // start and the batch that sets it gets every SM; the teams then take the
-  // rest of the order.  The k-lists and thresholds carry over.
-  const bool opening = T > 1 && rs.ng == 1 && !rs.nocut && rs.norder > rs.B;
-  struct Phase {
-    u32 teams, begin, count;
-  };
-  std::vector<Phase> phases;
-  if (opening) {
-    phases.push_back({1u, 0u, rs.B});
-    phases.push_back({T, rs.B, rs.norder - rs.B});
-  } else {
-    phases.push_back({T, 0u, rs.norder});
-  }
   memset(hctl, 0, sizeof(Ctl));
-  std::vector<Ctl> cs(T);
+  std::vector<Ctl> cs(open_teams + T);
+  Shared hsh;
   TKC_TRY(cudaEventRecord(ctx->ev[4], st));
-  for (const Phase &ph : phases) {
-    for (u32 t = 0; t < ph.teams; ++t) {
-      memset(&cs[t], 0, sizeof(Ctl));
-      cs[t].step = 1;  // start with an (empty) clear step whose epilogue seeds the first batch
-      cs[t].level_id = w.level_base;
-    }
-    TKC_TRY(cudaMemcpyAsync(w.ctl, cs.data(), ph.teams * sizeof(Ctl), cudaMemcpyHostToDevice, st));
-    TKC_TRY(cudaMemsetAsync(w.sh, 0, sizeof(Shared), st));
-    p.teams = ph.teams;
-    p.order = rs.order + ph.begin;
-    p.norder = ph.count;
-    p.nocut_prefix = rs.nocut_prefix > ph.begin ? rs.nocut_prefix - ph.begin : 0;
-    const int pblocks = std::max<int>((int)ph.teams, blocks / (int)ph.teams * (int)ph.teams);
-    TKC_RC(run_bfscut(ctx, p, rs.W, pblocks));
-    TKC_TRY(cudaMemcpyAsync(cs.data(), w.ctl, ph.teams * sizeof(Ctl), cudaMemcpyDeviceToHost, st));
-    Shared hsh;
-    TKC_TRY(cudaMemcpyAsync(&hsh, w.sh, sizeof(Shared), cudaMemcpyDeviceToHost, st));
-    TKC_TRY(cudaStreamSynchronize(st));
-    // the teams' counters add up; levels and batches too (they ran side by side)
-    for (u32 t = 0; t < ph.teams; ++t) {
-      const Ctl &x = cs[t];
-      hctl->edges_visited += x.edges_visited;
-      hctl->edges_scanned += x.edges_scanned;
-      hctl->bfs_started += x.bfs_started;
-      hctl->bfs_cut += x.bfs_cut;
-      hctl->bfs_finished += x.bfs_finished;
-      hctl->levels += x.levels;
-      hctl->batches += x.batches;
-      hctl->alg_bytes += x.alg_bytes;
-      hctl->st_td_levels += x.st_td_levels;
-      hctl->st_td_frontier += x.st_td_frontier;
-      hctl->st_td_arcs += x.st_td_arcs;
-      hctl->st_td_new += x.st_td_new;
-      hctl->st_bu_levels += x.st_bu_levels;
-      hctl->st_bu_scan_v += x.st_bu_scan_v;
-      hctl->st_bu_scan_a += x.st_bu_scan_a;
-      hctl->st_bu_new += x.st_bu_new;
-      hctl->st_bu_frontier += x.st_bu_frontier;
-      hctl->st_bu_rows += x.st_bu_rows;
-      hctl->st_seeded += x.st_seeded;
-      hctl->st_cleared += x.st_cleared;
-      hctl->st_compactions += x.st_compactions;
-      hctl->st_compact_dropped += x.st_compact_dropped;
-      hctl->trace_n += x.trace_n;
-      hctl->level_id = std::max(hctl->level_id, x.level_id);
-      if (!hctl->err) hctl->err = x.err;
-    }
-    if (!hctl->err) hctl->err = hsh.err;
-    w.level_base = hctl->level_id + 1;
-    if (p.trace) {
-      std::vector<u64> tr((size_t)trace_cap * 16);
-      TKC_TRY(cudaMemcpy(tr.data(), p.trace, tr.size() * sizeof(u64), cudaMemcpyDeviceToHost));
-      TKC_TRY(cudaMemset(p.trace, 0, tr.size() * sizeof(u64)));
-      FILE *f = fopen(trace_path, "a");
-      if (f) {
-        fprintf(f, "# n=%u arcs=%llu B=%u blocks=%d graphs=%u teams=%u\n", g->n, (unsigned long long)g->arcs, rs.B,
-                pblocks, rs.ng, ph.teams);
-        fprintf(f, "t_ns,kind,a,b,c,d,e,f,t_top,t_a_end,t_a_sync,t_b_end,t_flush,t_epi,team,y\n");
-        const u64 per = trace_cap / ph.teams;
-        for (u32 t = 0; t < ph.teams; ++t)
-          for (u64 i = 0; i < std::min<u64>(cs[t].trace_n, per); ++i) {
-            u64 *r = &tr[((size_t)t * per + i) * 16];
-            r[14] = t;
-            for (int j = 0; j < 16; ++j) fprintf(f, j ? ",%llu" : "%llu", r[j]);
-            fprintf(f, "\n");
-          }
-        fclose(f);
-      }
-      for (u32 t = 0; t < ph.teams; ++t) cs[t].trace_n = 0;
-    }
-    if (hctl->err) break;
+  p.trace_cap = p.trace ? trace_cap / 2 : 0;  // half for each launch
+  auto launch_phase = [&](u32 teams, Ctl *ctl) {
+    p.teams = teams;
+    p.ctl = ctl;
+    return run_bfscut(ctx, p, rs.W, std::max<int>((int)teams, blocks / (int)teams * (int)teams));
+  };
+  if (opening) {
+    p.norder = nopen;
+    TKC_RC(launch_phase(open_teams, w.ctl));
+    p.order = rs.order + nopen;
+    p.nocut_prefix = rs.nocut_prefix > nopen ? rs.nocut_prefix - nopen : 0;
+    TKC_RC(run_filter(ctx, p, open_teams, T, rs.norder - nopen));
+    p.order = w.f_order;
+    p.norder_dev = 1;
+    p.g_end = rs.g_end ? w.f_end : nullptr;
+    p.g_rest = 0;
+    if (p.trace) p.trace += (size_t)p.trace_cap * 16;
   }
+  TKC_RC(launch_phase(T, w.ctl + open_teams));
   TKC_TRY(cudaEventRecord(ctx->ev[5], st));
-  if (p.trace) TKC_TRY(cudaFree(p.trace));
+  TKC_TRY(cudaMemcpyAsync(cs.data(), w.ctl, cs.size() * sizeof(Ctl), cudaMemcpyDeviceToHost, st));
+  TKC_TRY(cudaMemcpyAsync(&hsh, w.sh, sizeof(Shared), cudaMemcpyDeviceToHost, st));
+  TKC_TRY(cudaStreamSynchronize(st));
+  // the teams' counters add up; levels and batches too (they ran side by side)
+  for (const Ctl &x : cs) {
+    hctl->edges_visited += x.edges_visited;
+    hctl->edges_scanned += x.edges_scanned;
+    hctl->bfs_started += x.bfs_started;
+    hctl->bfs_cut += x.bfs_cut;
+    hctl->bfs_finished += x.bfs_finished;
+    hctl->levels += x.levels;
+    hctl->batches += x.batches;
+    hctl->alg_bytes += x.alg_bytes;
+    hctl->st_td_levels += x.st_td_levels;
+    hctl->st_td_frontier += x.st_td_frontier;
+    hctl->st_td_arcs += x.st_td_arcs;
+    hctl->st_td_new += x.st_td_new;
+    hctl->st_bu_levels += x.st_bu_levels;
+    hctl->st_bu_scan_v += x.st_bu_scan_v;
+    hctl->st_bu_scan_a += x.st_bu_scan_a;
+    hctl->st_bu_new += x.st_bu_new;
+    hctl->st_bu_frontier += x.st_bu_frontier;
+    hctl->st_bu_rows += x.st_bu_rows;
+    hctl->st_seeded += x.st_seeded;
+    hctl->st_cleared += x.st_cleared;
+    hctl->st_compactions += x.st_compactions;
+    hctl->st_compact_dropped += x.st_compact_dropped;
+    hctl->level_id = std::max(hctl->level_id, x.level_id);
+    if (!hctl->err) hctl->err = x.err;
+  }
+  if (!hctl->err) hctl->err = hsh.err;
+  w.level_base = hctl->level_id + 1;
+  if (p.trace) {
+    u64 *tbase = opening ? p.trace - (size_t)p.trace_cap * 16 : p.trace;
+    std::vector<u64> tr((size_t)trace_cap * 16);
+    TKC_TRY(cudaMemcpy(tr.data(), tbase, tr.size() * sizeof(u64), cudaMemcpyDeviceToHost));
+    TKC_TRY(cudaFree(tbase));
+    FILE *f = fopen(trace_path, "a");
+    for (int ph = opening ? 0 : 1; f && ph < 2; ++ph) {
+      const u32 teams = ph == 0 ? open_teams : T, first = ph == 0 ? 0u : open_teams;
+      const u64 *half = tr.data() + (ph == 1 && opening ? (size_t)p.trace_cap * 16 : 0);
+      fprintf(f, "# n=%u arcs=%llu B=%u blocks=%d graphs=%u teams=%u\n", g->n, (unsigned long long)g->arcs, rs.B,
+              blocks, rs.ng, teams);
+      fprintf(f, "t_ns,kind,a,b,c,d,e,f,t_top,t_a_end,t_a_sync,t_b_end,t_flush,t_epi,team,y\n");
+      const u64 per = p.trace_cap / teams;
+      for (u32 t = 0; t < teams; ++t)
+        for (u64 i = 0; i < std::min<u64>(cs[first + t].trace_n, per); ++i) {
+          const u64 *r = half + ((size_t)t * per + i) * 16;
+          for (int j = 0; j < 16; ++j) fprintf(f, j ? ",%llu" : "%llu", j == 14 ? (u64)t : r[j]);
+          fprintf(f, "\n");
+        }
+    }
+    if (f) fclose(f);
+  }
   {
     tkc_run_stats &rs_out = ctx->last_stats;
     rs_out.n = g->n;
@@ -522,7 +533,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     rs_out.batch_bits = rs.B;
     rs_out.row_bytes = 8u * (u32)rs.W;
     rs_out.teams = T;
-    rs_out.launches = (u32)phases.size();
+    rs_out.launches = opening ? 2u : 1u;
     rs_out.td_levels = hctl->st_td_levels;
     rs_out.td_frontier = hctl->st_td_frontier;
     rs_out.td_frontier_arcs = hctl->st_td_arcs;
@@ -913,7 +924,7 @@ void tkc_free_graph(tkc_graph *g) {
   if (g->icol && g->icol != g->col) cudaFreeAsync(g->icol, st);
   void *ptrs[] = {g->off, g->col, g->deg_order, g->given_order, g->alpha, g->omega, g->scc_size, g->features,
                   g->learned_order, g->seeded_order, g->nb_order, g->nb_S, g->nb_r, g->nb_key, g->nb_hkey,
-                  g->nb_horder, g->comp, g->zero_ids};
+                  g->nb_horder, g->comp, g->zero_ids, g->walks};
   for (void *p : ptrs)
     if (p) cudaFreeAsync(p, st);
   g->ctx->graphs_alive--;
@@ -1667,7 +1678,7 @@ static int topk_many(tkc_ctx *ctx, tkc_graph *const *gs, uint32_t ng, uint32_t k
     free_search_csr(&U);
     void *ptrs[] = {U.off, U.col, U.ioff, U.icol, U.deg_order, U.alpha, U.omega, U.scc_size, U.comp, U.nb_S, U.nb_r,
                     U.nb_key, U.nb_hkey,
-                    U.nb_order, U.nb_horder, gid, d_vbase, d_abase, d_offptr, d_colptr, d_gdir, zflag, zlist,
+                    U.nb_order, U.nb_horder, U.walks, gid, d_vbase, d_abase, d_offptr, d_colptr, d_gdir, zflag, zlist,
                     zat, gorder, gkey, gend};
     for (void *q : ptrs)
       if (q) cudaFree(q);

@@ -21,6 +21,7 @@
 // Every grid-wide wait is bounded by a clock64 budget; on expiry the kernel
 // records TKC_ETIMEOUT and every block returns.
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include "tkc_internal.cuh"
@@ -867,6 +868,17 @@ __device__ void epilogue_compact(const RunParams &p, Smem<W> &sm) {
   __syncthreads();
 }
 
+// The bound after level 1 of source v (S_1 = its out-degree, n_1 = 1 more,
+// gamma_2 from the walks of length 2) exceeds the threshold: what the search
+// would find after running that level.
+__device__ __forceinline__ bool level1_exceeds(const RunParams &p, uint32_t v, uint32_t od, uint32_t alpha,
+                                               uint32_t omega, uint32_t g, u64 xS, uint32_t xr) {
+  const int directed = p.g_directed ? p.g_directed[g] : p.directed;
+  const u64 g2 = (u64)p.walks[v] - (directed ? 0u : od);
+  if (p.harmonic) return harmonic_below((double)od, 1, 1ull + od, g2, omega, xS);
+  return cut_exceeds(od, 1, 1ull + od, g2, alpha, omega, xS, xr);
+}
+
 // Epilogue after a clear step: seed the next batch of up to B sources.
 template <int W>
 __device__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
@@ -928,7 +940,8 @@ __device__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
     uint32_t a = valid ? p.alpha[v] : 0, o = valid ? p.omega[v] : 0;
     uint32_t gv = (valid && p.gid) ? p.gid[v] : 0;
     // level 0: S_0 = 0, n_0 = 1, gamma_1 = out-degree
-    bool cut = false, stop = false;
+    // (cut1: abandoned after level 1, whose arcs count as visited)
+    bool cut = false, cut1 = false, stop = false;
     // several graphs: a graph whose search stopped skips its later sources
     const bool stopped = valid && p.lb_key && p.gid && *(volatile unsigned *)&p.g_stop[gv];
     if (valid && !stopped && !p.nocut && idx >= p.nocut_prefix) {
@@ -938,10 +951,13 @@ __device__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
                __dmul_rn(__longlong_as_double((long long)~p.lb_key[v]), kHMargin) <
                    __longlong_as_double((long long)x.S);
         cut = !stop && x.have && harmonic_below(0.0, 0, 1, od, o, x.S);
+        cut1 = !stop && x.have && !cut && p.walks && level1_exceeds(p, v, od, a, o, gv, x.S, x.r);
       } else {
         stop = x.have && p.lb_key && nb_exceeds(p.lb_key[v], x.S, x.r);
         cut = !stop && x.have && cut_exceeds(0, 0, 1, od, a, o, x.S, x.r);
+        cut1 = !stop && x.have && !cut && p.walks && level1_exceeds(p, v, od, a, o, gv, x.S, x.r);
       }
+      cut |= cut1;
     }
     // nothing after a stopped position of its graph is searched, by any team
     if (stop) {
@@ -961,6 +977,10 @@ __device__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
     if (cut) {
       graph_count(p, gv, 1, 1);
       graph_count(p, gv, 2, 1);
+      if (cut1) {
+        graph_count(p, gv, 0, od);
+        atomicAdd(&c->edges_visited, (u64)od);
+      }
     }
     uint32_t s = assigned + pre;
     u64 myarcs = take ? od : 0;
@@ -1077,6 +1097,7 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
     p.Loff1 = p0.Loff1 + team * p0.vtx_stride;
     p.VL = p0.VL + team * p0.vtx_stride;
     p.stamp = p0.stamp + team * p0.vtx_stride;
+    if (p0.norder_dev) p.norder = p0.sh->norder;
     if (p0.trace) {
       p.trace_cap = p0.trace_cap / p0.teams;
       p.trace = p0.trace + (size_t)team * p.trace_cap * 16;
@@ -1500,7 +1521,192 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
   }
 }
 
+// ------------------------------------------------------------------ before the launches
+
+// Zeroes the control blocks (each starts with an empty clear step, whose
+// epilogue seeds the first batch), the shared block and, with nlist > 0, the
+// per-graph list state and res_r of n vertices.
+__global__ void k_run_init(Ctl *ctl, uint32_t nctl, unsigned level_base, Shared *sh, uint32_t nlist, unsigned *g_ntop,
+                           unsigned *g_stop, u64 *g_ctr, unsigned *x_seq, uint32_t *x_r, uint32_t *res_r,
+                           uint32_t n) {
+  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+  static_assert(sizeof(Ctl) % 8 == 0, "control blocks are zeroed by 64-bit words");
+  for (uint32_t i = t; i < nctl * (uint32_t)(sizeof(Ctl) / 8); i += nt) {
+    const uint32_t w = i % (uint32_t)(sizeof(Ctl) / 8);
+    if (w == offsetof(Ctl, step) / 8 || w == offsetof(Ctl, level_id) / 8) continue;
+    reinterpret_cast<u64 *>(ctl)[i] = 0;
+  }
+  for (uint32_t i = t; i < nctl; i += nt) {
+    // the two words skipped above
+    u64 *w = reinterpret_cast<u64 *>(ctl + i);
+    w[offsetof(Ctl, step) / 8] = 0;
+    w[offsetof(Ctl, level_id) / 8] = 0;
+    ctl[i].step = 1;
+    ctl[i].level_id = level_base;
+  }
+  if (t == 0) *sh = Shared{};
+  for (uint32_t i = t; i < nlist; i += nt) {
+    g_ntop[i] = g_stop[i] = x_seq[i] = 0;
+    x_r[i] = 0;
+    for (int j = 0; j < 4; ++j) g_ctr[4 * (size_t)i + j] = 0;
+  }
+  if (nlist)
+    for (uint32_t i = t; i < n; i += nt) res_r[i] = 0;
+}
+
+// Between the opening and the main launch: the sources of order[0, count)
+// that the thresholds so far abandon before they start -- by NBCut's stop
+// (not counted, as at seeding), by the level-0 bound or by the level-1 bound
+// -- are dropped in one grid-wide pass, so that the teams' batches hold only
+// sources that search.  Seeding takes B positions per step of about 10 us and
+// a batch abandoned after level 1 costs a level besides (R-MAT 20, DegCut:
+// 8 550 batches of 64 and 47.5 ms a call without it, 11.2 ms with it; BA with
+// 2 000 vertices, DegCut: 1.90 and 0.84 ms; NBCut unchanged within 0.5%).
+// Blocks take tiles of `tile` consecutive positions (a multiple of blockDim);
+// mask: one keep bit per position; blk: each block's kept count.
+constexpr int kFilterTPB = 256;  // a multiple of the warp; tiles are multiples of it
+__global__ void __launch_bounds__(kFilterTPB) k_filter_test(RunParams p, uint32_t count, uint32_t tile, Ctl *c,
+                                                            uint32_t *mask, uint32_t *blk) {
+  __shared__ u64 s_sum[3];
+  __shared__ unsigned s_keep;
+  if (threadIdx.x < 3) s_sum[threadIdx.x] = 0;
+  if (threadIdx.x == 0) s_keep = 0;
+  __syncthreads();
+  const u64 base = (u64)blockIdx.x * tile;
+  u64 started = 0, visited = 0;
+  unsigned kept = 0;
+  for (uint32_t o = threadIdx.x; o < tile; o += kFilterTPB) {
+    const u64 idx = base + o;
+    bool keep = idx < count;
+    if (keep && idx >= p.nocut_prefix) {
+      const uint32_t v = p.order[idx];
+      const uint32_t g = p.gid ? p.gid[v] : 0;
+      const uint32_t xr = p.x_r[g];
+      if (xr != 0) {
+        const u64 xS = p.x_S[g];
+        const bool stop = p.lb_key && (p.harmonic ? __dmul_rn(__longlong_as_double((long long)~p.lb_key[v]), kHMargin) <
+                                                        __longlong_as_double((long long)xS)
+                                                  : nb_exceeds(p.lb_key[v], xS, xr));
+        if (stop) {
+          keep = false;
+        } else {
+          const uint32_t sv = p.lab ? p.lab[v] : v;
+          const uint32_t od = p.off[sv + 1] - p.off[sv], a = p.alpha[v], om = p.omega[v];
+          const bool cut0 = p.harmonic ? harmonic_below(0.0, 0, 1, od, om, xS) : cut_exceeds(0, 0, 1, od, a, om, xS, xr);
+          const bool cut1 = !cut0 && p.walks && level1_exceeds(p, v, od, a, om, g, xS, xr);
+          if (cut0 || cut1) {
+            keep = false;
+            ++started;
+            graph_count(p, g, 1, 1);
+            graph_count(p, g, 2, 1);
+            if (cut1) {
+              visited += od;
+              graph_count(p, g, 0, od);
+            }
+          }
+        }
+      }
+    }
+    const unsigned m = __ballot_sync(FULL, keep);
+    if ((threadIdx.x & 31) == 0) mask[idx >> 5] = m;
+    kept += keep;
+  }
+  kept = __reduce_add_sync(FULL, kept);
+  if ((threadIdx.x & 31) == 0 && kept) atomicAdd(&s_keep, kept);
+  if (started) atomicAdd(&s_sum[0], started);
+  if (visited) atomicAdd(&s_sum[1], visited);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    blk[blockIdx.x] = s_keep;
+    if (s_sum[0]) {
+      atomicAdd(&c->bfs_started, s_sum[0]);
+      atomicAdd(&c->bfs_cut, s_sum[0]);
+    }
+    if (s_sum[1]) atomicAdd(&c->edges_visited, s_sum[1]);
+  }
+}
+
+// The kept sources in order; per graph one past its last kept position; the
+// main launch's control blocks continue the level stamps of the opening's and
+// the shared cursor starts over.
+__global__ void __launch_bounds__(kFilterTPB) k_filter_compact(RunParams p, uint32_t tile, const Ctl *open,
+                                                               uint32_t nopen, Ctl *ctl, uint32_t nctl,
+                                                               const uint32_t *mask, const uint32_t *blk,
+                                                               uint32_t *out, uint32_t *g_end) {
+  __shared__ uint32_t s_base;
+  __shared__ uint32_t s_warp[kFilterTPB / 32];
+  if (threadIdx.x == 0) s_base = 0;
+  __syncthreads();
+  uint32_t before = 0;
+  for (uint32_t i = threadIdx.x; i < blockIdx.x; i += kFilterTPB) before += blk[i];
+  before = __reduce_add_sync(FULL, before);
+  if ((threadIdx.x & 31) == 0 && before) atomicAdd(&s_base, before);
+  __syncthreads();
+  uint32_t at = s_base;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const u64 base = (u64)blockIdx.x * tile;
+  for (uint32_t o = 0; o < tile; o += kFilterTPB) {
+    const u64 idx = base + o + threadIdx.x;
+    const unsigned m = mask[idx >> 5];
+    if (lane == 0) s_warp[wid] = __popc(m);
+    __syncthreads();
+    uint32_t pos = at;
+    for (int w = 0; w < kFilterTPB / 32; ++w) {
+      if (w < wid) pos += s_warp[w];
+      at += s_warp[w];
+    }
+    if ((m >> lane) & 1u) {
+      pos += __popc(m & ((1u << lane) - 1u));
+      const uint32_t v = p.order[idx];
+      out[pos] = v;
+      if (g_end) atomicMax(&g_end[p.gid[v]], pos + 1);
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1) {
+    p.sh->norder = at;
+    p.sh->cursor = 0;
+    p.sh->first_done = 0;
+  }
+  if (threadIdx.x == 0 && blockIdx.x == 0) {
+    unsigned lvl = 0;
+    for (uint32_t i = 0; i < nopen; ++i) lvl = open[i].level_id > lvl ? open[i].level_id : lvl;
+    for (uint32_t i = 0; i < nctl; ++i) ctl[i].level_id = lvl + 1;
+  }
+}
+
 // ------------------------------------------------------------------ host side
+
+int run_init(tkc_ctx *ctx, uint32_t nctl, uint32_t n, uint32_t ng, bool reset_lists) {
+  Workspace &w = ctx->ws;
+  const uint32_t work = reset_lists ? (n > ng ? n : ng) : 1024;
+  const uint32_t blocks = work / 1024 + 1 < (uint32_t)ctx->num_sms * 8 ? work / 1024 + 1 : (uint32_t)ctx->num_sms * 8;
+  TKC_LAUNCH(k_run_init<<<blocks, 256, 0, ctx->stream>>>(w.ctl, nctl, w.level_base, w.sh, reset_lists ? ng : 0u,
+                                                         w.g_ntop, w.g_stop, w.g_ctr, w.x_seq, w.x_r, w.res_r, n));
+  TKC_TRY(cudaGetLastError());
+  return TKC_OK;
+}
+
+// Words of keep bits for `cap` positions, the last tile's overhang included.
+size_t filter_mask_words(uint32_t cap) { return ((size_t)cap + cap / kFilterBlocks + 2 * kFilterTPB) / 32 + 1; }
+
+int run_filter(tkc_ctx *ctx, const RunParams &p, uint32_t open_teams, uint32_t main_teams, uint32_t count) {
+  Workspace &w = ctx->ws;
+  cudaStream_t st = ctx->stream;
+  // at most kFilterBlocks blocks, so that a block sums the counts before it itself
+  uint32_t tile = (count + kFilterBlocks - 1) / kFilterBlocks;
+  tile = (tile + kFilterTPB - 1) / kFilterTPB * kFilterTPB;
+  if (tile == 0) tile = kFilterTPB;
+  const uint32_t nb = count ? (count + tile - 1) / tile : 1;
+  uint32_t *blk = w.f_mask + filter_mask_words(w.f_cap);
+  Ctl *main_ctl = w.ctl + open_teams;
+  if (p.gid) TKC_TRY(cudaMemsetAsync(w.f_end, 0, (size_t)p.ng * sizeof(uint32_t), st));
+  TKC_LAUNCH(k_filter_test<<<nb, kFilterTPB, 0, st>>>(p, count, tile, main_ctl, w.f_mask, blk));
+  TKC_LAUNCH(k_filter_compact<<<nb, kFilterTPB, 0, st>>>(p, tile, w.ctl, open_teams, main_ctl, main_teams, w.f_mask,
+                                                         blk, w.f_order, p.gid ? w.f_end : nullptr));
+  TKC_TRY(cudaGetLastError());
+  return TKC_OK;
+}
 
 // The larger blocks pay off on batched searches of large graphs (R-MAT 20 and
 // 22); one-source searches and graphs below 2^20 vertices (BA 10^6: 1.75 ms of

@@ -481,6 +481,43 @@ int ensure_zero_list(const tkc_graph *g) {
   return TKC_OK;
 }
 
+// ------------------------------------------------------------------ walks of length 2
+
+// walks[u] += sum of out-degrees over u's out-neighbours: 32 consecutive arcs
+// per warp step (a hub's row spread over many warps), the lanes of one source
+// added up first.
+__global__ void k_walks(const u32 *__restrict__ off, const u32 *__restrict__ col, u32 n, u64 arcs,
+                        u32 *__restrict__ walks) {
+  const int lane = threadIdx.x & 31;
+  grid_walk_arcs(off, n, arcs, [&](u32 u, u64 i, bool valid, u32) {
+    u32 d = 0;
+    if (valid) {
+      const u32 w = col[i];
+      d = off[w + 1] - off[w];
+    }
+    const unsigned peers = __match_any_sync(FULL, valid ? u : 0xffffffffu);
+    d = __reduce_add_sync(peers, d);
+    if (valid && d && __ffs(peers) - 1 == lane) atomicAdd(&walks[u], d);
+  });
+}
+
+// The sum over each vertex's out-neighbours of their out-degrees (below 2^32:
+// at most the graph's arcs): the Section 6 lemma's gamma after level 1, so
+// the bound after level 1 is known before a search starts.
+int ensure_walks(tkc_graph *g) {
+  if (g->walks || g->n == 0) return TKC_OK;
+  cudaStream_t st = g->ctx->stream;
+  u32 *w = nullptr;
+  TKC_TRY(cudaMallocAsync(&w, (size_t)g->n * sizeof(u32), st));
+  TKC_TRY(cudaMemsetAsync(w, 0, (size_t)g->n * sizeof(u32), st));
+  if (g->arcs)
+    TKC_LAUNCH(k_walks<<<grid_for((g->arcs + kArcChunk - 1) / kArcChunk * 32, 256), 256, 0, st>>>(
+        g->off, g->col, g->n, g->arcs, w));
+  TKC_TRY(cudaGetLastError());
+  g->walks = w;
+  return TKC_OK;
+}
+
 // ------------------------------------------------------------------ bottom-up work order
 
 __global__ void k_bu_keys(const u32 *ioff, u32 n, u32 heavy_in, u32 *key, u32 *val, u32 *count) {
