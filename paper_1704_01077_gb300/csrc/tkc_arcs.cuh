@@ -71,12 +71,23 @@ __device__ __forceinline__ void warp_walk_arcs(const uint32_t *off, uint32_t n, 
   }
 }
 
-// Arcs per warp task of the walks above: a few window and search rounds per
-// task against 64 groups of 32 arcs.
-constexpr uint32_t kArcChunk = 2048;
+// Arcs per warp task of the walks above.  A task is a chain of dependent loads
+// (the search, a window of row ends per 32 rows, 32 arcs a step), so a small
+// graph is cut into shorter tasks that fill the chip -- about 8 192 warps, the
+// least a task's search is worth being 128 arcs -- and a large one into tasks
+// of 2 048 arcs.  (With 2 048 at every size, the graphs of 1 000 to 200 000
+// vertices that a multi-graph call loads took 50 us of validation and 114 us
+// of symmetry check each on average, nearly all of it one warp's chain.)
+__host__ __device__ inline uint32_t arc_chunk(uint64_t arcs) {
+  const uint64_t c = (arcs / 8192 + 31) / 32 * 32;
+  return c < 128 ? 128u : c > 2048 ? 2048u : (uint32_t)c;
+}
+
+// Threads that give every task its own warp.
+inline uint64_t arc_threads(uint64_t arcs) { return (arcs + arc_chunk(arcs) - 1) / arc_chunk(arcs) * 32; }
 
 // Calls f(u, i, valid, rs) for every arc of the graph, the arcs dealt to the
-// grid's warps in tasks of kArcChunk consecutive indices (task c to warp
+// grid's warps in tasks of arc_chunk(arcs) consecutive indices (task c to warp
 // c mod warps: a kernel launched twice with the same grid gives each block
 // the same arcs).
 template <bool kRowStart = false, typename F>
@@ -84,8 +95,9 @@ __device__ __forceinline__ void grid_walk_arcs(const uint32_t *off, uint32_t n, 
   const int lane = threadIdx.x & 31;
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  for (uint64_t a0 = warp * kArcChunk; a0 < arcs; a0 += nwarps * kArcChunk) {
-    const uint64_t a1 = a0 + kArcChunk < arcs ? a0 + kArcChunk : arcs;
+  const uint32_t chunk = arc_chunk(arcs);
+  for (uint64_t a0 = warp * chunk; a0 < arcs; a0 += nwarps * chunk) {
+    const uint64_t a1 = a0 + chunk < arcs ? a0 + chunk : arcs;
     warp_walk_arcs<kRowStart>(off, n, a0, a1, lane, f);
   }
 }

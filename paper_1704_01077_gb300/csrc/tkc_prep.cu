@@ -204,7 +204,7 @@ static unsigned grid_for(u64 work, unsigned tpb, unsigned cap = 152 * 16) {
 int enqueue_validate(const tkc_graph *g, u32 *flag) {
   if (g->n == 0) return TKC_OK;
   cudaStream_t st = g->ctx->stream;
-  TKC_LAUNCH(k_validate<<<grid_for(std::max<u64>(g->n, (g->arcs + kArcChunk - 1) / kArcChunk * 32), 256), 256, 0,
+  TKC_LAUNCH(k_validate<<<grid_for(std::max<u64>(g->n, arc_threads(g->arcs)), 256), 256, 0,
                           st>>>(g->off, g->col, g->n, g->arcs, flag));
   TKC_TRY(cudaGetLastError());
   return TKC_OK;
@@ -215,7 +215,7 @@ int enqueue_validate(const tkc_graph *g, u32 *flag) {
 int enqueue_symmetric(const tkc_graph *g, u32 *flag) {
   if (g->n == 0 || g->directed) return TKC_OK;
   cudaStream_t st = g->ctx->stream;
-  TKC_LAUNCH(k_symmetric<<<grid_for((g->arcs + kArcChunk - 1) / kArcChunk * 32, 256), 256, 0, st>>>(
+  TKC_LAUNCH(k_symmetric<<<grid_for(arc_threads(g->arcs), 256), 256, 0, st>>>(
       g->off, g->col, g->n, g->arcs, flag));
   TKC_TRY(cudaGetLastError());
   return TKC_OK;
@@ -254,7 +254,7 @@ static int fill_in_arcs(const u32 *off, const u32 *col, u32 n, u64 arcs, const u
   u32 *cursor = nullptr;
   TKC_TRY(cudaMallocAsync(&cursor, (size_t)n * sizeof(u32), st));
   TKC_TRY(cudaMemcpyAsync(cursor, ioff, (size_t)n * sizeof(u32), cudaMemcpyDeviceToDevice, st));
-  TKC_LAUNCH(k_in_fill<<<grid_for((arcs + kArcChunk - 1) / kArcChunk * 32, 256), 256, 0, st>>>(
+  TKC_LAUNCH(k_in_fill<<<grid_for(arc_threads(arcs), 256), 256, 0, st>>>(
       off, col, n, arcs, cursor, icol));
   TKC_TRY(cudaGetLastError());
   TKC_TRY(cudaFreeAsync(cursor, st));
@@ -511,7 +511,7 @@ int ensure_walks(tkc_graph *g) {
   TKC_TRY(cudaMallocAsync(&w, (size_t)g->n * sizeof(u32), st));
   TKC_TRY(cudaMemsetAsync(w, 0, (size_t)g->n * sizeof(u32), st));
   if (g->arcs)
-    TKC_LAUNCH(k_walks<<<grid_for((g->arcs + kArcChunk - 1) / kArcChunk * 32, 256), 256, 0, st>>>(
+    TKC_LAUNCH(k_walks<<<grid_for(arc_threads(g->arcs), 256), 256, 0, st>>>(
         g->off, g->col, g->n, g->arcs, w));
   TKC_TRY(cudaGetLastError());
   g->walks = w;
@@ -653,7 +653,7 @@ static int build_labelled_copy(const tkc_graph *g, cudaStream_t st) {
   TKC_RC(scan_exclusive(g->s_off, g->s_off, (u64)n + 1, tmp, st));
   TKC_RC(scan_exclusive(g->s_ioff, g->s_ioff, (u64)n + 1, tmp, st));
   if (g->arcs) {
-    TKC_LAUNCH(k_relabel_cols<<<grid_for((g->arcs + kArcChunk - 1) / kArcChunk * 32, 256), 256, 0, st>>>(
+    TKC_LAUNCH(k_relabel_cols<<<grid_for(arc_threads(g->arcs), 256), 256, 0, st>>>(
         g->s_off, g->s_unlab, g->off, g->col, g->s_lab, n, g->arcs, gcol));
     TKC_TRY(cudaGetLastError());
   }

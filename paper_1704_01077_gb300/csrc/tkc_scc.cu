@@ -912,7 +912,7 @@ int reach_directed_gpu(tkc_graph *g, const u32 *gid, u32 ng) {
   const u64 reach_big = read_u32(flag, st, &rc);
   TKC_RC(rc);
   // condensation arcs, sorted by (cu, cv) and deduplicated
-  const unsigned cross_grid = grid_of((g->arcs + kArcChunk - 1) / kArcChunk * 32);
+  const unsigned cross_grid = grid_of(arc_threads(g->arcs));
   u32 *blk = nullptr, *blk_tmp = nullptr;
   TKC_TRY(b.get(&blk, (size_t)cross_grid + 1));
   TKC_TRY(b.get(&blk_tmp, ((size_t)cross_grid + 1) / 4096 + 2));
