@@ -94,6 +94,7 @@ int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u3
     TKC_RC(dalloc(&w.stamp, tv, st));
     TKC_RC(dalloc(&w.res_S, cap, st));
     TKC_RC(dalloc(&w.res_r, cap, st));
+    TKC_RC(dalloc(&w.lvl2, cap, st));
     TKC_RC(dalloc(&w.FB0, tfb, st));
     TKC_RC(dalloc(&w.FB1, tfb, st));
     TKC_TRY(cudaMemsetAsync(w.FB0, 0, tfb * sizeof(u32), st));
@@ -125,7 +126,8 @@ static int ensure_filter(tkc_ctx *ctx, u32 count) {
   w.f_cap = 0;
   const u32 cap = std::max<u32>(count, 1024);
   TKC_RC(dalloc(&w.f_order, cap, ctx->stream));
-  TKC_RC(dalloc(&w.f_mask, filter_mask_words(cap) + kFilterBlocks, ctx->stream));
+  TKC_RC(dalloc(&w.f_keep, cap, ctx->stream));
+  if (!w.f_count) TKC_RC(dalloc(&w.f_count, kFilterTiles, ctx->stream));
   w.f_cap = cap;
   return TKC_OK;
 }
@@ -135,7 +137,7 @@ static void free_workspace(tkc_ctx *ctx) {
   void *ptrs[] = {w.seen, w.F0, w.F1, w.N, w.FB0, w.FB1, w.L0, w.L1, w.Loff0, w.Loff1, w.VL, w.stamp, w.res_S, w.res_r,
                   w.slots, w.cnt, w.wsum, w.top_S, w.top_r, w.top_id, w.ctl, w.out_S, w.out_r, w.out_id,
                   w.out_f, w.out_c, w.tied, w.g_ntop, w.g_stop, w.g_ctr, w.sh, w.x_seq, w.x_S, w.x_r, w.x_id,
-                  w.f_order, w.f_mask, w.f_end};
+                  w.f_order, w.f_keep, w.f_count, w.f_end, w.lvl2};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   w = Workspace();
@@ -300,13 +302,18 @@ static u32 default_teams(u32 n, u32 B, u32 maxb, bool nb) {
   return std::max<u32>(1, maxb / 8);  // eight blocks (SMs) per team, every SM used
 }
 
-// Whether the search walks the in-degree labelling: batched searches of
+// Whether a search may walk the in-degree labelling: batched searches of
 // large graphs (its hot rows stay in L2); one-source searches and small
 // graphs (of a union: when no graph is large, each one's rows fit L2 anyway)
-// the graph itself.
-static bool labelled_search(const tkc_options &o, u32 B, u32 size_n) {
-  return o.relabel == 1 || (o.relabel == 0 && B > 1 && size_n >= (1u << 20));
+// the graph itself.  options.relabel = 1 always does.
+static bool labelled_by_size(const tkc_options &o, u32 B, u32 size_n) {
+  return o.relabel == 0 && B > 1 && size_n >= (1u << 20);
 }
+
+// With an opening the copy is built only when the filter leaves at least this
+// many batches: on R-MAT 22 it costs 3.4 to 5 ms of device work and saved 0.2 ms
+// per 128-source batch (51 -> 35 ms over 81 batches); the filter leaves one.
+constexpr u32 kLabelBatches = 24;
 
 static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   const tkc_graph *g = rs.g;
@@ -362,24 +369,24 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   p.n = g->n;
   p.directed = g->directed;
   p.arcs = g->arcs;
-  const bool relabel = labelled_search(o, rs.B, rs.size_n ? rs.size_n : g->n);
-  TKC_RC(ensure_search_csr(g, relabel));
-  const bool lab = g->s_mode == 1;
-  p.off = lab ? g->s_off : g->off;
-  p.col = lab ? g->s_col : g->col;
-  p.ioff = lab ? g->s_ioff : g->ioff;
-  p.icol = lab ? g->s_icol : g->icol;
-  p.lab = lab ? g->s_lab : nullptr;
-  p.unlab = lab ? g->s_unlab : nullptr;
-  p.bu_list = g->bu_list;
-  p.n_bu = g->n_bu;
-  p.n_bu_heavy = g->n_bu_heavy;
-  p.heavy_in = g->heavy_in ? g->heavy_in : kHeavyIn;
+  const bool by_size = labelled_by_size(o, rs.B, rs.size_n ? rs.size_n : g->n);
+  TKC_RC(ensure_search_csr(g, o.relabel == 1 || (by_size && (!opening || g->s_mode == 1))));
+  auto walk_search_csr = [&] {
+    const bool lab = g->s_mode == 1;
+    p.off = lab ? g->s_off : g->off;
+    p.col = lab ? g->s_col : g->col;
+    p.ioff = lab ? g->s_ioff : g->ioff;
+    p.icol = lab ? g->s_icol : g->icol;
+    p.lab = lab ? g->s_lab : nullptr;
+    p.unlab = lab ? g->s_unlab : nullptr;
+    p.bu_list = g->bu_list;
+    p.n_bu = g->n_bu;
+    p.n_bu_heavy = g->n_bu_heavy;
+    p.heavy_in = g->heavy_in ? g->heavy_in : kHeavyIn;
+  };
+  walk_search_csr();
   p.large_blocks = o.large_blocks;
-  // the bound after level 1 prunes only orders that do not know it already
-  // (NBCut's bounds hold level 2 and more)
-  if (opening && !rs.lb_key) TKC_RC(ensure_walks(const_cast<tkc_graph *>(g)));
-  p.walks = opening && !rs.lb_key ? g->walks : nullptr;
+  if (opening) TKC_RC(ensure_classes(g, rs.gid, rs.ng));
   p.alpha = g->alpha;
   p.omega = g->omega;
   p.order = rs.order;
@@ -463,7 +470,16 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     TKC_RC(launch_phase(open_teams, w.ctl));
     p.order = rs.order + nopen;
     p.nocut_prefix = rs.nocut_prefix > nopen ? rs.nocut_prefix - nopen : 0;
-    TKC_RC(run_filter(ctx, p, open_teams, T, rs.norder - nopen));
+    TKC_RC(run_filter(ctx, p, g, open_teams, T, rs.norder - nopen, w.lvl2));
+    p.lvl2 = w.lvl2;
+    if (by_size && g->s_mode != 1) {
+      TKC_TRY(cudaMemcpyAsync(&hsh, w.sh, sizeof(Shared), cudaMemcpyDeviceToHost, st));
+      TKC_TRY(cudaStreamSynchronize(st));
+      if (hsh.norder >= kLabelBatches * rs.B) {
+        TKC_RC(ensure_search_csr(g, true));
+        walk_search_csr();
+      }
+    }
     p.order = w.f_order;
     p.norder_dev = 1;
     p.g_end = rs.g_end ? w.f_end : nullptr;
@@ -924,7 +940,7 @@ void tkc_free_graph(tkc_graph *g) {
   if (g->icol && g->icol != g->col) cudaFreeAsync(g->icol, st);
   void *ptrs[] = {g->off, g->col, g->deg_order, g->given_order, g->alpha, g->omega, g->scc_size, g->features,
                   g->learned_order, g->seeded_order, g->nb_order, g->nb_S, g->nb_r, g->nb_key, g->nb_hkey,
-                  g->nb_horder, g->comp, g->zero_ids, g->walks};
+                  g->nb_horder, g->comp, g->zero_ids, g->cls, g->n_cls};
   for (void *p : ptrs)
     if (p) cudaFreeAsync(p, st);
   g->ctx->graphs_alive--;
@@ -1116,8 +1132,9 @@ static int topk_one(tkc_graph *g, uint32_t k, tkc_result *out, int harmonic) {
   cudaStream_t st = ctx->stream;
   TKC_TRY(cudaEventRecord(ctx->ev[0], st));
   const tkc_options &o = ctx->opt;
-  // a labelled search's copy of the graph is built alongside the preprocessing
-  if (labelled_search(o, o.batch_bits ? o.batch_bits : 64u, g->n)) TKC_RC(start_search_csr(g));
+  // a copy that the search is sure to walk is built alongside the preprocessing
+  if (o.relabel == 1 || (o.deterministic && labelled_by_size(o, o.batch_bits ? o.batch_bits : 64u, g->n)))
+    TKC_RC(start_search_csr(g));
   // the degree order only where it orders the sources (the NB order has its own)
   if (o.order == TKC_ORDER_DEG || o.order == TKC_ORDER_LEARNED) TKC_RC(ensure_degree_order(g));
   TKC_RC(ensure_zero_list(g));
@@ -1678,7 +1695,7 @@ static int topk_many(tkc_ctx *ctx, tkc_graph *const *gs, uint32_t ng, uint32_t k
     free_search_csr(&U);
     void *ptrs[] = {U.off, U.col, U.ioff, U.icol, U.deg_order, U.alpha, U.omega, U.scc_size, U.comp, U.nb_S, U.nb_r,
                     U.nb_key, U.nb_hkey,
-                    U.nb_order, U.nb_horder, U.walks, gid, d_vbase, d_abase, d_offptr, d_colptr, d_gdir, zflag, zlist,
+                    U.nb_order, U.nb_horder, U.cls, U.n_cls, gid, d_vbase, d_abase, d_offptr, d_colptr, d_gdir, zflag, zlist,
                     zat, gorder, gkey, gend};
     for (void *q : ptrs)
       if (q) cudaFree(q);

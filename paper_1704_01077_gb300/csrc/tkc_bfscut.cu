@@ -868,13 +868,10 @@ __device__ void epilogue_compact(const RunParams &p, Smem<W> &sm) {
   __syncthreads();
 }
 
-// The bound after level 1 of source v (S_1 = its out-degree, n_1 = 1 more,
-// gamma_2 from the walks of length 2) exceeds the threshold: what the search
-// would find after running that level.
-__device__ __forceinline__ bool level1_exceeds(const RunParams &p, uint32_t v, uint32_t od, uint32_t alpha,
-                                               uint32_t omega, uint32_t g, u64 xS, uint32_t xr) {
-  const int directed = p.g_directed ? p.g_directed[g] : p.directed;
-  const u64 g2 = (u64)p.walks[v] - (directed ? 0u : od);
+// The bound after level 1 of source v (S_1 = its out-degree, n_1 = 1 more, at
+// most g2 vertices at distance 2) exceeds the threshold.
+__device__ __forceinline__ bool level1_exceeds(const RunParams &p, uint32_t od, uint32_t alpha, uint32_t omega,
+                                               u64 g2, u64 xS, uint32_t xr) {
   if (p.harmonic) return harmonic_below((double)od, 1, 1ull + od, g2, omega, xS);
   return cut_exceeds(od, 1, 1ull + od, g2, alpha, omega, xS, xr);
 }
@@ -951,11 +948,11 @@ __device__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
                __dmul_rn(__longlong_as_double((long long)~p.lb_key[v]), kHMargin) <
                    __longlong_as_double((long long)x.S);
         cut = !stop && x.have && harmonic_below(0.0, 0, 1, od, o, x.S);
-        cut1 = !stop && x.have && !cut && p.walks && level1_exceeds(p, v, od, a, o, gv, x.S, x.r);
+        cut1 = !stop && x.have && !cut && p.lvl2 && level1_exceeds(p, od, a, o, p.lvl2[v], x.S, x.r);
       } else {
         stop = x.have && p.lb_key && nb_exceeds(p.lb_key[v], x.S, x.r);
         cut = !stop && x.have && cut_exceeds(0, 0, 1, od, a, o, x.S, x.r);
-        cut1 = !stop && x.have && !cut && p.walks && level1_exceeds(p, v, od, a, o, gv, x.S, x.r);
+        cut1 = !stop && x.have && !cut && p.lvl2 && level1_exceeds(p, od, a, o, p.lvl2[v], x.S, x.r);
       }
       cut |= cut1;
     }
@@ -1556,112 +1553,176 @@ __global__ void k_run_init(Ctl *ctl, uint32_t nctl, unsigned level_base, Shared 
 
 // Between the opening and the main launch: the sources of order[0, count)
 // that the thresholds so far abandon before they start -- by NBCut's stop
-// (not counted, as at seeding), by the level-0 bound or by the level-1 bound
-// -- are dropped in one grid-wide pass, so that the teams' batches hold only
-// sources that search.  Seeding takes B positions per step of about 10 us and
-// a batch abandoned after level 1 costs a level besides (R-MAT 20, DegCut:
-// 8 550 batches of 64 and 47.5 ms a call without it, 11.2 ms with it; BA with
-// 2 000 vertices, DegCut: 1.90 and 0.84 ms; NBCut unchanged within 0.5%).
-// Blocks take tiles of `tile` consecutive positions (a multiple of blockDim);
-// mask: one keep bit per position; blk: each block's kept count.
-constexpr int kFilterTPB = 256;  // a multiple of the warp; tiles are multiples of it
-__global__ void __launch_bounds__(kFilterTPB) k_filter_test(RunParams p, uint32_t count, uint32_t tile, Ctl *c,
-                                                            uint32_t *mask, uint32_t *blk) {
-  __shared__ u64 s_sum[3];
-  __shared__ unsigned s_keep;
-  if (threadIdx.x < 3) s_sum[threadIdx.x] = 0;
-  if (threadIdx.x == 0) s_keep = 0;
-  __syncthreads();
-  const u64 base = (u64)blockIdx.x * tile;
+// (not counted, as at seeding), by the level-0 bound, or by the bound after
+// level 1 with a level-2 size from in-degree classes -- are dropped in one
+// grid-wide pass, so that the teams' batches hold only sources that search.
+//
+// Level 2 of a source holds, of the n_c vertices of class c, at most
+// min(n_c, walks of length 2 ending in class c): vertices of small in-degree
+// are counted almost exactly, and the many walks that end in the few vertices
+// of large in-degree count each of those once.  (The plain sum of walks, which
+// gamma and the NB bounds use, exceeds the graph for any hub.)  A source left
+// over is searched with that bound in lvl2, tested again when it is seeded.
+//
+// Positions are dealt to the warps with a stride, since sources of long rows
+// are neighbours in the order; a lane sums a row of at most kFilterLane arcs,
+// the warp longer ones, four loads in flight each.  keep: a flag per position;
+// tile_cnt: kept positions per tile of `tile`.
+constexpr int kFilterTPB = 256;
+constexpr uint32_t kFilterLane = 16;
+
+__device__ __forceinline__ void add4(uint4 &a, const uint4 &b) {
+  a.x += b.x;
+  a.y += b.y;
+  a.z += b.z;
+  a.w += b.w;
+}
+
+// Sums of the class counts over the out-neighbours row[0, len), every
+// `step`-th from the first.  (Each sum is at most the graph's arcs, below 2^32.)
+__device__ __forceinline__ uint4 sum_classes(const uint32_t *__restrict__ row, const uint4 *__restrict__ cls,
+                                             uint32_t len, uint32_t step) {
+  uint4 s = make_uint4(0, 0, 0, 0);
+  uint32_t i = 0;  // len is below 2^26
+  for (; i + 3 * step < len; i += 4 * step) {
+    uint4 c[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) c[j] = cls[row[i + j * step]];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) add4(s, c[j]);
+  }
+  for (; i < len; i += step) add4(s, cls[row[i]]);
+  return s;
+}
+
+__global__ void __launch_bounds__(kFilterTPB) k_filter_test(RunParams p, uint32_t count, uint32_t tile,
+                                                            const uint32_t *__restrict__ off,
+                                                            const uint32_t *__restrict__ col,
+                                                            const uint4 *__restrict__ cls,
+                                                            const uint32_t *__restrict__ n_cls, Ctl *c, uint8_t *keep,
+                                                            uint32_t *tile_cnt, uint32_t *lvl2) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t warp = (blockIdx.x * kFilterTPB + threadIdx.x) >> 5, nwarps = (gridDim.x * kFilterTPB) >> 5;
   u64 started = 0, visited = 0;
-  unsigned kept = 0;
-  for (uint32_t o = threadIdx.x; o < tile; o += kFilterTPB) {
-    const u64 idx = base + o;
-    bool keep = idx < count;
-    if (keep && idx >= p.nocut_prefix) {
-      const uint32_t v = p.order[idx];
-      const uint32_t g = p.gid ? p.gid[v] : 0;
-      const uint32_t xr = p.x_r[g];
-      if (xr != 0) {
-        const u64 xS = p.x_S[g];
-        const bool stop = p.lb_key && (p.harmonic ? __dmul_rn(__longlong_as_double((long long)~p.lb_key[v]), kHMargin) <
-                                                        __longlong_as_double((long long)xS)
-                                                  : nb_exceeds(p.lb_key[v], xS, xr));
-        if (stop) {
-          keep = false;
-        } else {
-          const uint32_t sv = p.lab ? p.lab[v] : v;
-          const uint32_t od = p.off[sv + 1] - p.off[sv], a = p.alpha[v], om = p.omega[v];
-          const bool cut0 = p.harmonic ? harmonic_below(0.0, 0, 1, od, om, xS) : cut_exceeds(0, 0, 1, od, a, om, xS, xr);
-          const bool cut1 = !cut0 && p.walks && level1_exceeds(p, v, od, a, om, g, xS, xr);
-          if (cut0 || cut1) {
-            keep = false;
-            ++started;
-            graph_count(p, g, 1, 1);
-            graph_count(p, g, 2, 1);
-            if (cut1) {
-              visited += od;
-              graph_count(p, g, 0, od);
-            }
-          }
+  for (u64 first = warp; first < count; first += 32ull * nwarps) {
+    const u64 idx = first + (u64)lane * nwarps;
+    const bool valid = idx < count;
+    bool kept = valid, test1 = false;
+    uint32_t v = 0, g = 0, od = 0, a = 0, om = 0, b = 0, xr = 0;
+    u64 xS = 0;
+    if (valid) {
+      v = p.order[idx];
+      if (p.gid) g = p.gid[v];
+      b = off[v];
+      od = off[v + 1] - b;
+      if (idx >= p.nocut_prefix) xr = p.x_r[g];
+    }
+    if (xr != 0) {
+      xS = p.x_S[g];
+      const bool stop = p.lb_key && (p.harmonic ? __dmul_rn(__longlong_as_double((long long)~p.lb_key[v]), kHMargin) <
+                                                      __longlong_as_double((long long)xS)
+                                                : nb_exceeds(p.lb_key[v], xS, xr));
+      if (stop) {
+        kept = false;
+      } else {
+        a = p.alpha[v];
+        om = p.omega[v];
+        test1 = !(p.harmonic ? harmonic_below(0.0, 0, 1, od, om, xS) : cut_exceeds(0, 0, 1, od, a, om, xS, xr));
+        if (!test1) {
+          kept = false;
+          ++started;
+          graph_count(p, g, 1, 1);
+          graph_count(p, g, 2, 1);
         }
       }
     }
-    const unsigned m = __ballot_sync(FULL, keep);
-    if ((threadIdx.x & 31) == 0) mask[idx >> 5] = m;
-    kept += keep;
-  }
-  kept = __reduce_add_sync(FULL, kept);
-  if ((threadIdx.x & 31) == 0 && kept) atomicAdd(&s_keep, kept);
-  if (started) atomicAdd(&s_sum[0], started);
-  if (visited) atomicAdd(&s_sum[1], visited);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    blk[blockIdx.x] = s_keep;
-    if (s_sum[0]) {
-      atomicAdd(&c->bfs_started, s_sum[0]);
-      atomicAdd(&c->bfs_cut, s_sum[0]);
+    // level 1 (uncut sources and those without a threshold keep what gamma gives)
+    const bool walk = kept;
+    uint4 s = make_uint4(0, 0, 0, 0);
+    if (walk && od <= kFilterLane) s = sum_classes(col + b, cls, od, 1);
+    for (unsigned m = __ballot_sync(FULL, walk && od > kFilterLane); m; m &= m - 1) {
+      const int src = __ffs(m) - 1;
+      const uint32_t rb = __shfl_sync(FULL, b, src), len = __shfl_sync(FULL, od, src);  // len > kFilterLane
+      uint4 t = make_uint4(0, 0, 0, 0);
+      if (lane < len) t = sum_classes(col + rb + lane, cls, len - lane, 32);
+      t.x = __reduce_add_sync(FULL, t.x);
+      t.y = __reduce_add_sync(FULL, t.y);
+      t.z = __reduce_add_sync(FULL, t.z);
+      t.w = __reduce_add_sync(FULL, t.w);
+      if ((int)lane == src) s = t;
     }
-    if (s_sum[1]) atomicAdd(&c->edges_visited, s_sum[1]);
+    if (walk) {
+      const int directed = p.g_directed ? p.g_directed[g] : p.directed;
+      const u64 gamma = (u64)s.x + s.y + s.z + s.w - (directed ? 0u : od);
+      const uint32_t *nc = n_cls + 4 * (size_t)g;
+      const u64 by_class = (u64)min(s.x, nc[0]) + min(s.y, nc[1]) + min(s.z, nc[2]) + min(s.w, nc[3]);
+      const u64 g2 = gamma < by_class ? gamma : by_class;
+      lvl2[v] = (uint32_t)g2;  // by_class <= n
+      if (test1 && level1_exceeds(p, od, a, om, g2, xS, xr)) {
+        kept = false;
+        ++started;
+        visited += od;
+        graph_count(p, g, 1, 1);
+        graph_count(p, g, 2, 1);
+        graph_count(p, g, 0, od);
+      }
+    }
+    if (valid) {
+      keep[idx] = kept;
+      if (kept) atomicAdd(&tile_cnt[idx / tile], 1u);
+    }
   }
+  for (int o = 16; o > 0; o >>= 1) {
+    started += __shfl_down_sync(FULL, started, o);
+    visited += __shfl_down_sync(FULL, visited, o);
+  }
+  if (lane == 0 && started) {
+    atomicAdd(&c->bfs_started, started);
+    atomicAdd(&c->bfs_cut, started);
+  }
+  if (lane == 0 && visited) atomicAdd(&c->edges_visited, visited);
 }
 
-// The kept sources in order; per graph one past its last kept position; the
-// main launch's control blocks continue the level stamps of the opening's and
-// the shared cursor starts over.
-__global__ void __launch_bounds__(kFilterTPB) k_filter_compact(RunParams p, uint32_t tile, const Ctl *open,
-                                                               uint32_t nopen, Ctl *ctl, uint32_t nctl,
-                                                               const uint32_t *mask, const uint32_t *blk,
-                                                               uint32_t *out, uint32_t *g_end) {
+// The kept sources in order (a block per tile); per graph one past its last
+// kept position; the main launch's control blocks continue the level stamps
+// of the opening's and the shared cursor starts over.
+__global__ void __launch_bounds__(kFilterTPB) k_filter_compact(RunParams p, uint32_t count, uint32_t tile,
+                                                               const Ctl *open, uint32_t nopen, Ctl *ctl,
+                                                               uint32_t nctl, const uint8_t *keep,
+                                                               const uint32_t *tile_cnt, uint32_t *out,
+                                                               uint32_t *g_end) {
   __shared__ uint32_t s_base;
   __shared__ uint32_t s_warp[kFilterTPB / 32];
   if (threadIdx.x == 0) s_base = 0;
   __syncthreads();
   uint32_t before = 0;
-  for (uint32_t i = threadIdx.x; i < blockIdx.x; i += kFilterTPB) before += blk[i];
+  for (uint32_t i = threadIdx.x; i < blockIdx.x; i += kFilterTPB) before += tile_cnt[i];
   before = __reduce_add_sync(FULL, before);
   if ((threadIdx.x & 31) == 0 && before) atomicAdd(&s_base, before);
   __syncthreads();
   uint32_t at = s_base;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const u64 base = (u64)blockIdx.x * tile;
-  for (uint32_t o = 0; o < tile; o += kFilterTPB) {
-    const u64 idx = base + o + threadIdx.x;
-    const unsigned m = mask[idx >> 5];
-    if (lane == 0) s_warp[wid] = __popc(m);
-    __syncthreads();
-    uint32_t pos = at;
-    for (int w = 0; w < kFilterTPB / 32; ++w) {
-      if (w < wid) pos += s_warp[w];
-      at += s_warp[w];
+  if (tile_cnt[blockIdx.x] != 0) {
+    for (uint32_t o = 0; o < tile; o += kFilterTPB) {
+      const u64 idx = base + o + threadIdx.x;
+      const bool k = idx < count && keep[idx];
+      const unsigned m = __ballot_sync(FULL, k);
+      if (lane == 0) s_warp[wid] = __popc(m);
+      __syncthreads();
+      uint32_t pos = at;
+      for (int w = 0; w < kFilterTPB / 32; ++w) {
+        if (w < wid) pos += s_warp[w];
+        at += s_warp[w];
+      }
+      if (k) {
+        pos += __popc(m & ((1u << lane) - 1u));
+        const uint32_t v = p.order[idx];
+        out[pos] = v;
+        if (g_end) atomicMax(&g_end[p.gid[v]], pos + 1);
+      }
+      __syncthreads();
     }
-    if ((m >> lane) & 1u) {
-      pos += __popc(m & ((1u << lane) - 1u));
-      const uint32_t v = p.order[idx];
-      out[pos] = v;
-      if (g_end) atomicMax(&g_end[p.gid[v]], pos + 1);
-    }
-    __syncthreads();
   }
   if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1) {
     p.sh->norder = at;
@@ -1687,23 +1748,28 @@ int run_init(tkc_ctx *ctx, uint32_t nctl, uint32_t n, uint32_t ng, bool reset_li
   return TKC_OK;
 }
 
-// Words of keep bits for `cap` positions, the last tile's overhang included.
-size_t filter_mask_words(uint32_t cap) { return ((size_t)cap + cap / kFilterBlocks + 2 * kFilterTPB) / 32 + 1; }
-
-int run_filter(tkc_ctx *ctx, const RunParams &p, uint32_t open_teams, uint32_t main_teams, uint32_t count) {
+int run_filter(tkc_ctx *ctx, const RunParams &p, const tkc_graph *g, uint32_t open_teams, uint32_t main_teams,
+               uint32_t count, uint32_t *lvl2) {
   Workspace &w = ctx->ws;
   cudaStream_t st = ctx->stream;
-  // at most kFilterBlocks blocks, so that a block sums the counts before it itself
-  uint32_t tile = (count + kFilterBlocks - 1) / kFilterBlocks;
+  // at most kFilterTiles tiles, so that a compacting block sums the counts before it itself
+  uint32_t tile = (count + kFilterTiles - 1) / kFilterTiles;
   tile = (tile + kFilterTPB - 1) / kFilterTPB * kFilterTPB;
   if (tile == 0) tile = kFilterTPB;
-  const uint32_t nb = count ? (count + tile - 1) / tile : 1;
-  uint32_t *blk = w.f_mask + filter_mask_words(w.f_cap);
+  const uint32_t ntiles = count ? (count + tile - 1) / tile : 1;
   Ctl *main_ctl = w.ctl + open_teams;
+  // a warp per 32 positions, but all SMs' warps before a warp takes more than
+  // one: the few sources of NBCut's order past its stop are long rows
+  uint32_t nb = (count + kFilterTPB / 32 - 1) / (kFilterTPB / 32);
+  if (nb > (uint32_t)ctx->num_sms * 8) nb = (uint32_t)ctx->num_sms * 8;
+  if (nb == 0) nb = 1;
+  TKC_TRY(cudaMemsetAsync(w.f_count, 0, ntiles * sizeof(uint32_t), st));
   if (p.gid) TKC_TRY(cudaMemsetAsync(w.f_end, 0, (size_t)p.ng * sizeof(uint32_t), st));
-  TKC_LAUNCH(k_filter_test<<<nb, kFilterTPB, 0, st>>>(p, count, tile, main_ctl, w.f_mask, blk));
-  TKC_LAUNCH(k_filter_compact<<<nb, kFilterTPB, 0, st>>>(p, tile, w.ctl, open_teams, main_ctl, main_teams, w.f_mask,
-                                                         blk, w.f_order, p.gid ? w.f_end : nullptr));
+  TKC_LAUNCH(k_filter_test<<<nb, kFilterTPB, 0, st>>>(p, count, tile, g->off, g->col, g->cls, g->n_cls, main_ctl,
+                                                      w.f_keep, w.f_count, lvl2));
+  TKC_LAUNCH(k_filter_compact<<<ntiles, kFilterTPB, 0, st>>>(p, count, tile, w.ctl, open_teams, main_ctl, main_teams,
+                                                             w.f_keep, w.f_count, w.f_order,
+                                                             p.gid ? w.f_end : nullptr));
   TKC_TRY(cudaGetLastError());
   return TKC_OK;
 }

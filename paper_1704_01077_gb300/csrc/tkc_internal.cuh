@@ -148,10 +148,9 @@ struct RunParams {
   const uint32_t *order;
   uint32_t norder;  // sources in `order` to examine (all have out-degree >= 1)
   int norder_dev;   // 1: the length is sh->norder (the order is what the filter kept)
-  // per vertex: the sum of its out-neighbours' out-degrees, so that a source
-  // may be abandoned by the bound after level 1 without running that level
-  // (nullptr: level 0's bound only)
-  const uint32_t *walks;
+  // sources' level-2 bounds, known before they search (the filter's; nullptr:
+  // none): at most lvl2[v] vertices lie at distance 2 from v, gamma included
+  const uint32_t *lvl2;
   // search configuration
   // teams: independent groups of `gridDim.x / teams` blocks, each running its
   // own batches; per-team buffers sit at team * stride from the base pointers
@@ -234,8 +233,10 @@ struct Workspace {
   uint32_t *top_r = nullptr, *top_id = nullptr;
   Ctl *ctl = nullptr;               // two per team: the opening's and the main launch's
   uint32_t *f_order = nullptr;      // source order kept by the filter
-  uint32_t *f_mask = nullptr;       // its keep bits, then its blocks' counts
+  uint8_t *f_keep = nullptr;        // its keep flags
+  uint32_t *f_count = nullptr;      // kept positions per tile
   uint32_t *f_end = nullptr;        // per graph: one past its last kept position
+  uint32_t *lvl2 = nullptr;         // per vertex: level-2 bounds of the kept sources
   uint32_t f_cap = 0;               // positions f_order holds
   unsigned long long *out_S = nullptr;
   uint32_t *out_r = nullptr, *out_id = nullptr;
@@ -311,7 +312,10 @@ struct tkc_graph {
   uint32_t *scc_size = nullptr;               // size of the SCC (component, if undirected) of each vertex
   uint32_t *comp = nullptr;                   // SCC (component, if undirected) id of each vertex
   bool have_order = false, have_reach = false;
-  uint32_t *walks = nullptr;                  // sum of the out-neighbours' out-degrees (ensure_walks)
+  // out-neighbours of each vertex by in-degree class, and the graph's (or each
+  // graph's of a union) vertices per class (ensure_classes)
+  mutable uint4 *cls = nullptr;
+  mutable uint32_t *n_cls = nullptr;
   float *features = nullptr;                  // standardized vertex features, n x TKC_MLP_FEATURES
   uint32_t *learned_order = nullptr;          // filtered order by predicted farness
   uint32_t n_src_learned = 0;
@@ -352,7 +356,7 @@ int build_in_csr(const tkc_graph *g);
 int ensure_in_csr(const tkc_graph *g);
 int ensure_degree_order(tkc_graph *g);
 int ensure_zero_list(const tkc_graph *g);
-int ensure_walks(tkc_graph *g);
+int ensure_classes(const tkc_graph *g, const uint32_t *gid, uint32_t ng);
 // gid/ng (several graphs as one union, graphs in contiguous vertex ranges):
 // one pivot per graph in the first forward-backward round
 int ensure_reach_bounds(tkc_graph *g, const uint32_t *gid = nullptr, uint32_t ng = 0);
@@ -391,8 +395,8 @@ int run_bfscut(tkc_ctx *ctx, const RunParams &p, int words, int blocks);  // blo
 // shared block and (reset_lists) the k-lists, thresholds and finished searches
 int run_init(tkc_ctx *ctx, uint32_t nctl, uint32_t n, uint32_t ng, bool reset_lists);
 // drops the sources order[0, count) that the current thresholds abandon
-constexpr uint32_t kFilterBlocks = 2048;    // most blocks of the filter
-size_t filter_mask_words(uint32_t cap);
-int run_filter(tkc_ctx *ctx, const RunParams &p, uint32_t open_teams, uint32_t main_teams, uint32_t count);
+constexpr uint32_t kFilterTiles = 2048;  // most tiles of the filter's compaction
+int run_filter(tkc_ctx *ctx, const RunParams &p, const tkc_graph *g, uint32_t open_teams, uint32_t main_teams,
+               uint32_t count, uint32_t *lvl2);
 int max_coresident_blocks(tkc_ctx *ctx, int words);
 }  // namespace tkc

@@ -44,6 +44,25 @@ def test_source_counts_around_the_tiles(gpu_lib, ctx, n, order, directed):
         t.tkc_free_graph(h)
 
 
+# skewed in-degrees: the level-2 bound by in-degree class does the pruning;
+# harmonic and closeness, one graph in its own ids and in the labelled copy
+@pytest.mark.parametrize("scale", [8, 11, 13])
+@pytest.mark.parametrize("order", ["DEG", "NB"])
+@pytest.mark.parametrize("relabel", [0, 1])
+def test_level_2_by_in_degree_class(gpu_lib, ctx, scale, order, relabel):
+    t = gpu_lib
+    g = gg.rmat(scale, 8, seed=scale)
+    t.tkc_set_options(ctx, t.Options(order=getattr(t, "TKC_ORDER_" + order), batch_bits=64, relabel=relabel))
+    h = t.tkc_load_csr(ctx, g.n, g.offsets, g.cols, g.directed)
+    try:
+        for k in (1, 10, 100):
+            _same(t.tkc_topk_closeness(h, k), oracle.textbook_topk(g, k))
+        hr, want = t.tkc_topk_harmonic(h, 10), oracle.textbook_harmonic_topk(g, 10)
+        assert list(hr.ids) == list(want.ids) and hr.n_tied_at_kth == want.n_tied
+    finally:
+        t.tkc_free_graph(h)
+
+
 @pytest.mark.parametrize("seed_factor", [1, 6, 30])  # prefixes of 10, 60 and 300 sources, the opening is 64
 @pytest.mark.parametrize("order", ["LEARNED", "LEARNED_NB"])
 def test_uncut_prefix_past_the_opening(gpu_lib, ctx, order, seed_factor):
