@@ -119,9 +119,18 @@ int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u3
   return TKC_OK;
 }
 
-// Buffers of the filter between the opening and the main launch.
-static int ensure_filter(tkc_ctx *ctx, u32 count) {
+// Buffers of the opening's choice (nopen sources of one graph; 0: none) and of
+// the filter between the opening and the main launch.
+static int ensure_filter(tkc_ctx *ctx, u32 count, u32 nopen) {
   Workspace &w = ctx->ws;
+  if (nopen > w.o_cap) {
+    w.o_cap = 0;
+    const u32 cap = std::max<u32>(nopen, TKC_MAX_K);
+    TKC_RC(dalloc(&w.o_order, cap, ctx->stream));
+    if (!w.o_key) TKC_RC(dalloc(&w.o_key, kOpenPool, ctx->stream));
+    if (!w.o_taken) TKC_RC(dalloc(&w.o_taken, kOpenPool, ctx->stream));
+    w.o_cap = cap;
+  }
   if (count <= w.f_cap) return TKC_OK;
   w.f_cap = 0;
   const u32 cap = std::max<u32>(count, 1024);
@@ -137,7 +146,8 @@ static void free_workspace(tkc_ctx *ctx) {
   void *ptrs[] = {w.seen, w.F0, w.F1, w.N, w.FB0, w.FB1, w.L0, w.L1, w.Loff0, w.Loff1, w.VL, w.stamp, w.res_S, w.res_r,
                   w.slots, w.cnt, w.wsum, w.top_S, w.top_r, w.top_id, w.ctl, w.out_S, w.out_r, w.out_id,
                   w.out_f, w.out_c, w.tied, w.g_ntop, w.g_stop, w.g_ctr, w.sh, w.x_seq, w.x_S, w.x_r, w.x_id,
-                  w.f_order, w.f_keep, w.f_count, w.f_end, w.lvl2};
+                  w.f_order, w.f_keep, w.f_count, w.f_end, w.lvl2,
+                  w.o_order, w.o_key, w.o_taken};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   w = Workspace();
@@ -335,11 +345,11 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     w.level_base = 0;
   }
   ctx->last_shard = nullptr;  // this run replaces the finished searches' (S, r)
-  // Opening: the first batch -- or as many as it takes for a full k-list --
-  // runs alone (one graph: on the whole grid; several: every graph's opening
-  // batch, on the teams), so that thresholds exist; then the filter drops the
-  // sources they abandon (k_filter_test) and the main launch searches the
-  // rest.  No host wait in between.  One-source searches and the deterministic
+  // Opening: a batch of promising sources (k_open_keys) -- or as many batches
+  // as it takes for a full k-list -- runs alone (one graph: on the whole grid;
+  // several: every graph's opening batch, on the teams), so that thresholds
+  // exist; then the filter drops the sources they abandon (k_filter_test) and
+  // the main launch searches the rest.  No host wait in between.  One-source searches and the deterministic
   // schedule (both one team) take the order as it stands, since their counters
   // are defined by it.
   const bool exact_schedule = rs.B <= 1 || o.deterministic;
@@ -349,7 +359,8 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
                                  : (rs.g_end ? rs.g_rest : 0u);
   const bool opening = nopen > 0 && nopen < rs.norder && !exact_schedule;
   const u32 open_teams = !opening ? 0u : rs.ng == 1 ? 1u : T;
-  if (opening) TKC_RC(ensure_filter(ctx, rs.norder - nopen));
+  const bool pick = opening && rs.ng == 1;
+  if (opening) TKC_RC(ensure_filter(ctx, pick ? rs.norder : rs.norder - nopen, pick ? nopen : 0));
   TKC_RC(run_init(ctx, open_teams + T, g->n, rs.ng, !rs.keep_lists));
   if (rs.nseed) {
     const unsigned ns = rs.nseed;
@@ -387,6 +398,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   walk_search_csr();
   p.large_blocks = o.large_blocks;
   if (opening) TKC_RC(ensure_classes(g, rs.gid, rs.ng));
+  p.n_cls = opening ? g->n_cls : nullptr;
   p.alpha = g->alpha;
   p.omega = g->omega;
   p.order = rs.order;
@@ -466,11 +478,19 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     return run_bfscut(ctx, p, rs.W, std::max<int>((int)teams, blocks / (int)teams * (int)teams));
   };
   if (opening) {
+    if (pick) {
+      // the opening's sources keep their order, the uncut prefix first
+      TKC_RC(run_pick_opening(ctx, p, g, rs.norder, nopen));
+      p.order = w.o_order;
+    }
     p.norder = nopen;
     TKC_RC(launch_phase(open_teams, w.ctl));
-    p.order = rs.order + nopen;
+    // the whole order but the picked ones, or what follows the opening
+    const u32 first = pick ? 0u : nopen;
+    p.order = rs.order + first;
+    p.nocut_prefix = rs.nocut_prefix > first ? rs.nocut_prefix - first : 0;
+    TKC_RC(run_filter(ctx, p, g, open_teams, T, rs.norder - first, pick));
     p.nocut_prefix = rs.nocut_prefix > nopen ? rs.nocut_prefix - nopen : 0;
-    TKC_RC(run_filter(ctx, p, g, open_teams, T, rs.norder - nopen, w.lvl2));
     p.lvl2 = w.lvl2;
     if (by_size && g->s_mode != 1) {
       TKC_TRY(cudaMemcpyAsync(&hsh, w.sh, sizeof(Shared), cudaMemcpyDeviceToHost, st));

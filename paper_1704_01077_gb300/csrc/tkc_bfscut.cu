@@ -876,6 +876,15 @@ __device__ __forceinline__ bool level1_exceeds(const RunParams &p, uint32_t od, 
   return cut_exceeds(od, 1, 1ull + od, g2, alpha, omega, xS, xr);
 }
 
+// omega of v, capped by what its graph can reach at all.
+__device__ __forceinline__ uint32_t omega_of(const RunParams &p, uint32_t v, uint32_t g) {
+  const uint32_t o = p.omega[v];
+  if (!p.n_cls) return o;
+  const uint32_t *nc = p.n_cls + 4 * (size_t)g;
+  const uint32_t cap = nc[0] + nc[1] + nc[2] + nc[3] + 1;
+  return o < cap ? o : cap;
+}
+
 // Epilogue after a clear step: seed the next batch of up to B sources.
 template <int W>
 __device__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
@@ -934,8 +943,8 @@ __device__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
     uint32_t v = valid ? p.order[idx] : 0;
     const uint32_t sv = valid && p.lab ? p.lab[v] : v;  // its row's label
     uint32_t od = valid ? p.off[sv + 1] - p.off[sv] : 0;
-    uint32_t a = valid ? p.alpha[v] : 0, o = valid ? p.omega[v] : 0;
     uint32_t gv = (valid && p.gid) ? p.gid[v] : 0;
+    uint32_t a = valid ? p.alpha[v] : 0, o = valid ? omega_of(p, v, gv) : 0;
     // level 0: S_0 = 0, n_0 = 1, gamma_1 = out-degree
     // (cut1: abandoned after level 1, whose arcs count as visited)
     bool cut = false, cut1 = false, stop = false;
@@ -1564,12 +1573,14 @@ __global__ void k_run_init(Ctl *ctl, uint32_t nctl, unsigned level_base, Shared 
 // gamma and the NB bounds use, exceeds the graph for any hub.)  A source left
 // over is searched with that bound in lvl2, tested again when it is seeded.
 //
-// Positions are dealt to the warps with a stride, since sources of long rows
-// are neighbours in the order; a lane sums a row of at most kFilterLane arcs,
-// the warp longer ones, four loads in flight each.  keep: a flag per position;
-// tile_cnt: kept positions per tile of `tile`.
+// Positions are dealt to the blocks with a stride, since sources of long rows
+// are neighbours in the order; a lane sums a row of at most kRowLane arcs, a
+// warp one of at most kRowWarp, the block longer ones, four loads in flight
+// per thread.  keep: a flag per position; tile_cnt: kept positions per tile of
+// `tile`; taken: positions already searched by the opening (nullable, the
+// first ntaken).
 constexpr int kFilterTPB = 256;
-constexpr uint32_t kFilterLane = 16;
+constexpr uint32_t kRowLane = 16, kRowWarp = 512;
 
 __device__ __forceinline__ void add4(uint4 &a, const uint4 &b) {
   a.x += b.x;
@@ -1595,22 +1606,87 @@ __device__ __forceinline__ uint4 sum_classes(const uint32_t *__restrict__ row, c
   return s;
 }
 
+__device__ __forceinline__ uint4 warp_sum4(uint4 t) {
+  t.x = __reduce_add_sync(FULL, t.x);
+  t.y = __reduce_add_sync(FULL, t.y);
+  t.z = __reduce_add_sync(FULL, t.z);
+  t.w = __reduce_add_sync(FULL, t.w);
+  return t;
+}
+
+struct RowScratch {
+  unsigned n;
+  uint32_t b[kFilterTPB], len[kFilterTPB];
+  uint4 sum[kFilterTPB];
+};
+
+// Every thread's sum over its own row col[b, b + len) (len 0: none); called by
+// the whole block.
+__device__ __forceinline__ uint4 block_sum_rows(RowScratch &rs, const uint32_t *__restrict__ col,
+                                                const uint4 *__restrict__ cls, uint32_t b, uint32_t len) {
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) rs.n = 0;
+  __syncthreads();
+  uint4 s = make_uint4(0, 0, 0, 0);
+  unsigned slot = 0;
+  if (len > kRowWarp) {
+    slot = atomicAdd(&rs.n, 1u);
+    rs.b[slot] = b;
+    rs.len[slot] = len;
+    rs.sum[slot] = s;
+  }
+  if (len <= kRowLane) s = sum_classes(col + b, cls, len, 1);
+  for (unsigned m = __ballot_sync(FULL, len > kRowLane && len <= kRowWarp); m; m &= m - 1) {
+    const int src = __ffs(m) - 1;
+    const uint32_t rb = __shfl_sync(FULL, b, src), rl = __shfl_sync(FULL, len, src);  // rl >= 17
+    uint4 t = make_uint4(0, 0, 0, 0);
+    if ((uint32_t)lane < rl) t = sum_classes(col + rb + lane, cls, rl - lane, 32);
+    t = warp_sum4(t);
+    if (lane == src) s = t;
+  }
+  __syncthreads();
+  for (unsigned i = 0; i < rs.n; ++i) {
+    // rows longer than kRowWarp hold at least one arc per thread of the block
+    const uint4 t = warp_sum4(sum_classes(col + rs.b[i] + threadIdx.x, cls, rs.len[i] - threadIdx.x, kFilterTPB));
+    if (lane == 0) {
+      atomicAdd(&rs.sum[i].x, t.x);
+      atomicAdd(&rs.sum[i].y, t.y);
+      atomicAdd(&rs.sum[i].z, t.z);
+      atomicAdd(&rs.sum[i].w, t.w);
+    }
+  }
+  __syncthreads();
+  if (len > kRowWarp) s = rs.sum[slot];
+  return s;
+}
+static_assert(kRowWarp >= (uint32_t)kFilterTPB, "a block's row has an arc for every thread");
+
+// Bound on the size of level 2 from the class sums s of a source's out-neighbours.
+__device__ __forceinline__ uint32_t level2_bound(const RunParams &p, const uint4 &s, uint32_t od, uint32_t g) {
+  const int directed = p.g_directed ? p.g_directed[g] : p.directed;
+  const u64 gamma = (u64)s.x + s.y + s.z + s.w - (directed ? 0u : od);
+  const uint32_t *nc = p.n_cls + 4 * (size_t)g;
+  const u64 by_class = (u64)min(s.x, nc[0]) + min(s.y, nc[1]) + min(s.z, nc[2]) + min(s.w, nc[3]);
+  return (uint32_t)(gamma < by_class ? gamma : by_class);  // by_class <= n
+}
+
 __global__ void __launch_bounds__(kFilterTPB) k_filter_test(RunParams p, uint32_t count, uint32_t tile,
                                                             const uint32_t *__restrict__ off,
                                                             const uint32_t *__restrict__ col,
-                                                            const uint4 *__restrict__ cls,
-                                                            const uint32_t *__restrict__ n_cls, Ctl *c, uint8_t *keep,
+                                                            const uint4 *__restrict__ cls, const uint8_t *taken,
+                                                            uint32_t ntaken, Ctl *c, uint8_t *keep,
                                                             uint32_t *tile_cnt, uint32_t *lvl2) {
-  const uint32_t lane = threadIdx.x & 31;
-  const uint32_t warp = (blockIdx.x * kFilterTPB + threadIdx.x) >> 5, nwarps = (gridDim.x * kFilterTPB) >> 5;
+  __shared__ RowScratch rs;
+  const int lane = threadIdx.x & 31;
   u64 started = 0, visited = 0;
-  for (u64 first = warp; first < count; first += 32ull * nwarps) {
-    const u64 idx = first + (u64)lane * nwarps;
+  for (u64 first = blockIdx.x; first < count; first += (u64)kFilterTPB * gridDim.x) {
+    const u64 idx = first + (u64)threadIdx.x * gridDim.x;
     const bool valid = idx < count;
-    bool kept = valid, test1 = false;
+    bool kept = valid && !(taken && idx < ntaken && taken[idx]);
+    bool test1 = false;
     uint32_t v = 0, g = 0, od = 0, a = 0, om = 0, b = 0, xr = 0;
     u64 xS = 0;
-    if (valid) {
+    if (kept) {
       v = p.order[idx];
       if (p.gid) g = p.gid[v];
       b = off[v];
@@ -1626,7 +1702,7 @@ __global__ void __launch_bounds__(kFilterTPB) k_filter_test(RunParams p, uint32_
         kept = false;
       } else {
         a = p.alpha[v];
-        om = p.omega[v];
+        om = omega_of(p, v, g);
         test1 = !(p.harmonic ? harmonic_below(0.0, 0, 1, od, om, xS) : cut_exceeds(0, 0, 1, od, a, om, xS, xr));
         if (!test1) {
           kept = false;
@@ -1636,28 +1712,11 @@ __global__ void __launch_bounds__(kFilterTPB) k_filter_test(RunParams p, uint32_
         }
       }
     }
-    // level 1 (uncut sources and those without a threshold keep what gamma gives)
-    const bool walk = kept;
-    uint4 s = make_uint4(0, 0, 0, 0);
-    if (walk && od <= kFilterLane) s = sum_classes(col + b, cls, od, 1);
-    for (unsigned m = __ballot_sync(FULL, walk && od > kFilterLane); m; m &= m - 1) {
-      const int src = __ffs(m) - 1;
-      const uint32_t rb = __shfl_sync(FULL, b, src), len = __shfl_sync(FULL, od, src);  // len > kFilterLane
-      uint4 t = make_uint4(0, 0, 0, 0);
-      if (lane < len) t = sum_classes(col + rb + lane, cls, len - lane, 32);
-      t.x = __reduce_add_sync(FULL, t.x);
-      t.y = __reduce_add_sync(FULL, t.y);
-      t.z = __reduce_add_sync(FULL, t.z);
-      t.w = __reduce_add_sync(FULL, t.w);
-      if ((int)lane == src) s = t;
-    }
-    if (walk) {
-      const int directed = p.g_directed ? p.g_directed[g] : p.directed;
-      const u64 gamma = (u64)s.x + s.y + s.z + s.w - (directed ? 0u : od);
-      const uint32_t *nc = n_cls + 4 * (size_t)g;
-      const u64 by_class = (u64)min(s.x, nc[0]) + min(s.y, nc[1]) + min(s.z, nc[2]) + min(s.w, nc[3]);
-      const u64 g2 = gamma < by_class ? gamma : by_class;
-      lvl2[v] = (uint32_t)g2;  // by_class <= n
+    // level 1 (uncut sources and those without a threshold keep the bound)
+    const uint4 s = block_sum_rows(rs, col, cls, b, kept ? od : 0u);
+    if (kept) {
+      const uint32_t g2 = level2_bound(p, s, od, g);
+      lvl2[v] = g2;
       if (test1 && level1_exceeds(p, od, a, om, g2, xS, xr)) {
         kept = false;
         ++started;
@@ -1671,6 +1730,7 @@ __global__ void __launch_bounds__(kFilterTPB) k_filter_test(RunParams p, uint32_
       keep[idx] = kept;
       if (kept) atomicAdd(&tile_cnt[idx / tile], 1u);
     }
+    __syncthreads();
   }
   for (int o = 16; o > 0; o >>= 1) {
     started += __shfl_down_sync(FULL, started, o);
@@ -1681,6 +1741,143 @@ __global__ void __launch_bounds__(kFilterTPB) k_filter_test(RunParams p, uint32_
     atomicAdd(&c->bfs_cut, started);
   }
   if (lane == 0 && visited) atomicAdd(&c->edges_visited, visited);
+}
+
+// The opening's sources, one graph.  Which sources open is free (every one is
+// searched or abandoned once), and the threshold they leave decides how many
+// the filter keeps.  The order's head is not the best choice: in NBCut's order
+// the sources whose omega is far above their reach come first (R-MAT 22: the
+// first 128 sources left 3 000 and more for the main launch).  So the pool --
+// the first kOpenPool positions -- is ranked by the bound after level 1 with
+// level 2 by class and omega capped, which the threshold test itself uses.
+// key: high word of the bound's FP64 bits (only an order: exactness is not
+// needed), smallest first; sources never cut come first of all.
+__global__ void __launch_bounds__(kFilterTPB) k_open_keys(RunParams p, uint32_t pool,
+                                                          const uint32_t *__restrict__ off,
+                                                          const uint32_t *__restrict__ col,
+                                                          const uint4 *__restrict__ cls, uint32_t *key) {
+  __shared__ RowScratch rs;
+  for (u64 first = blockIdx.x; first < pool; first += (u64)kFilterTPB * gridDim.x) {
+    const u64 idx = first + (u64)threadIdx.x * gridDim.x;
+    const bool valid = idx < pool;
+    uint32_t v = 0, b = 0, od = 0;
+    if (valid) {
+      v = p.order[idx];
+      b = off[v];
+      od = off[v + 1] - b;
+    }
+    const uint4 s = block_sum_rows(rs, col, cls, b, od);
+    if (valid) {
+      const u64 g2 = level2_bound(p, s, od, 0), n1 = 1ull + od;
+      const uint32_t om = omega_of(p, v, 0);
+      uint32_t k = 0;
+      if (idx >= p.nocut_prefix) {
+        if (p.harmonic) {
+          const u64 w = om > n1 ? om - n1 : 0, near_ = g2 < w ? g2 : w;
+          const double U = (double)od + 0.5 * (double)near_ + (double)(w - near_) / 3.0;
+          k = ~(uint32_t)((u64)__double_as_longlong(U) >> 32);
+        } else {
+          u64 lo = p.alpha[v];
+          lo = lo < n1 ? n1 : lo;
+          const u64 hi = om < lo ? lo : om, kink = n1 + g2;
+          double best = __longlong_as_double(0x7ff0000000000000ll);
+          const u64 cand[3] = {lo, hi, kink > lo && kink < hi ? kink : hi};
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            const double r1 = (double)(cand[i] - 1);
+            const double f = (double)cut_sum(od, 1, n1, g2, cand[i]) / (r1 * r1);  // r >= 2: od >= 1
+            best = f < best ? f : best;
+          }
+          k = (uint32_t)((u64)__double_as_longlong(best) >> 32);
+        }
+      }
+      key[idx] = k;
+    }
+    __syncthreads();
+  }
+}
+
+// The nopen <= pool positions of smallest key (the first of equal ones), in
+// the order's order: one block, the keys in registers, four passes of 8 bits
+// for the nopen-th key and one scan.
+constexpr int kPickTPB = 1024, kPickPer = kOpenPool / kPickTPB;
+__global__ void __launch_bounds__(kPickTPB) k_open_pick(const uint32_t *order, const uint32_t *key, uint32_t pool,
+                                                        uint32_t nopen, uint32_t *out, uint8_t *taken) {
+  __shared__ uint32_t hist[256];
+  __shared__ uint32_t s_prefix, s_need, s_warp[2][kPickTPB / 32 + 1];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const uint32_t base = threadIdx.x * kPickPer;
+  uint32_t k[kPickPer];
+#pragma unroll
+  for (int i = 0; i < kPickPer; ++i) k[i] = base + i < pool ? key[base + i] : 0xffffffffu;
+  if (threadIdx.x == 0) {
+    s_prefix = 0;
+    s_need = nopen;
+  }
+  for (int shift = 24; shift >= 0; shift -= 8) {
+    if (threadIdx.x < 256) hist[threadIdx.x] = 0;
+    __syncthreads();
+    const uint32_t prefix = s_prefix, need = s_need, mask = shift == 24 ? 0u : 0xffffffffu << (shift + 8);
+#pragma unroll
+    for (int i = 0; i < kPickPer; ++i)
+      if (base + i < pool && (k[i] & mask) == prefix) atomicAdd(&hist[(k[i] >> shift) & 255u], 1u);
+    __syncthreads();
+    if (wid == 0) {
+      // lane l: bins 8l .. 8l + 7; the bin holding the need-th key
+      uint32_t sum = 0;
+      for (int j = 0; j < 8; ++j) sum += hist[8 * lane + j];
+      uint32_t incl = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += t;
+      }
+      uint32_t before = incl - sum;
+      if (before < need && incl >= need) {
+        int j = 0;
+        while (before + hist[8 * lane + j] < need) before += hist[8 * lane + j++];
+        s_prefix = prefix | (uint32_t)(8 * lane + j) << shift;
+        s_need = need - before;
+      }
+    }
+    __syncthreads();
+  }
+  // all keys below the nopen-th, and the first s_need equal to it
+  const uint32_t T = s_prefix, need = s_need;
+  uint32_t below = 0, equal = 0;
+#pragma unroll
+  for (int i = 0; i < kPickPer; ++i) {
+    below += base + i < pool && k[i] < T;
+    equal += base + i < pool && k[i] == T;
+  }
+  uint32_t bi = below, ei = equal;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t tb = __shfl_up_sync(FULL, bi, o), te = __shfl_up_sync(FULL, ei, o);
+    if (lane >= o) {
+      bi += tb;
+      ei += te;
+    }
+  }
+  if (lane == 31) {
+    s_warp[0][wid] = bi;
+    s_warp[1][wid] = ei;
+  }
+  __syncthreads();
+  uint32_t nb = bi - below, ne = ei - equal;  // below / equal ones before this thread's
+  for (int w = 0; w < wid; ++w) {
+    nb += s_warp[0][w];
+    ne += s_warp[1][w];
+  }
+#pragma unroll
+  for (int i = 0; i < kPickPer; ++i) {
+    if (base + i >= pool) break;
+    const bool eq = k[i] == T, take = k[i] < T || (eq && ne < need);
+    taken[base + i] = take;
+    if (take) out[nb + (ne < need ? ne : need)] = order[base + i];
+    nb += k[i] < T;
+    ne += eq;
+  }
 }
 
 // The kept sources in order (a block per tile); per graph one past its last
@@ -1748,8 +1945,25 @@ int run_init(tkc_ctx *ctx, uint32_t nctl, uint32_t n, uint32_t ng, bool reset_li
   return TKC_OK;
 }
 
+// Blocks for `count` positions: several per SM before a block takes more than
+// one position per thread, since a few positions may be long rows.
+static uint32_t filter_blocks(tkc_ctx *ctx, uint32_t count) {
+  const uint32_t nb = (count + 7) / 8, most = (uint32_t)ctx->num_sms * 8;
+  return nb < 1 ? 1 : nb < most ? nb : most;
+}
+
+int run_pick_opening(tkc_ctx *ctx, const RunParams &p, const tkc_graph *g, uint32_t count, uint32_t nopen) {
+  Workspace &w = ctx->ws;
+  cudaStream_t st = ctx->stream;
+  const uint32_t pool = count < kOpenPool ? count : kOpenPool;
+  TKC_LAUNCH(k_open_keys<<<filter_blocks(ctx, pool), kFilterTPB, 0, st>>>(p, pool, g->off, g->col, g->cls, w.o_key));
+  TKC_LAUNCH(k_open_pick<<<1, kPickTPB, 0, st>>>(p.order, w.o_key, pool, nopen, w.o_order, w.o_taken));
+  TKC_TRY(cudaGetLastError());
+  return TKC_OK;
+}
+
 int run_filter(tkc_ctx *ctx, const RunParams &p, const tkc_graph *g, uint32_t open_teams, uint32_t main_teams,
-               uint32_t count, uint32_t *lvl2) {
+               uint32_t count, bool picked) {
   Workspace &w = ctx->ws;
   cudaStream_t st = ctx->stream;
   // at most kFilterTiles tiles, so that a compacting block sums the counts before it itself
@@ -1758,15 +1972,11 @@ int run_filter(tkc_ctx *ctx, const RunParams &p, const tkc_graph *g, uint32_t op
   if (tile == 0) tile = kFilterTPB;
   const uint32_t ntiles = count ? (count + tile - 1) / tile : 1;
   Ctl *main_ctl = w.ctl + open_teams;
-  // a warp per 32 positions, but all SMs' warps before a warp takes more than
-  // one: the few sources of NBCut's order past its stop are long rows
-  uint32_t nb = (count + kFilterTPB / 32 - 1) / (kFilterTPB / 32);
-  if (nb > (uint32_t)ctx->num_sms * 8) nb = (uint32_t)ctx->num_sms * 8;
-  if (nb == 0) nb = 1;
   TKC_TRY(cudaMemsetAsync(w.f_count, 0, ntiles * sizeof(uint32_t), st));
   if (p.gid) TKC_TRY(cudaMemsetAsync(w.f_end, 0, (size_t)p.ng * sizeof(uint32_t), st));
-  TKC_LAUNCH(k_filter_test<<<nb, kFilterTPB, 0, st>>>(p, count, tile, g->off, g->col, g->cls, g->n_cls, main_ctl,
-                                                      w.f_keep, w.f_count, lvl2));
+  TKC_LAUNCH(k_filter_test<<<filter_blocks(ctx, count), kFilterTPB, 0, st>>>(
+      p, count, tile, g->off, g->col, g->cls, picked ? w.o_taken : nullptr, kOpenPool < count ? kOpenPool : count,
+      main_ctl, w.f_keep, w.f_count, w.lvl2));
   TKC_LAUNCH(k_filter_compact<<<ntiles, kFilterTPB, 0, st>>>(p, count, tile, w.ctl, open_teams, main_ctl, main_teams,
                                                              w.f_keep, w.f_count, w.f_order,
                                                              p.gid ? w.f_end : nullptr));

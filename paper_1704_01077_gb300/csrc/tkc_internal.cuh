@@ -151,6 +151,11 @@ struct RunParams {
   // sources' level-2 bounds, known before they search (the filter's; nullptr:
   // none): at most lvl2[v] vertices lie at distance 2 from v, gamma included
   const uint32_t *lvl2;
+  // per graph: vertices with an in-arc, by class (4 words; nullptr: omega as it
+  // stands).  A vertex reaches itself and vertices with an in-arc, so their
+  // number plus one caps omega: Algorithm 6 adds the biggest SCC's reach again
+  // along every way to it, which puts sources of small reach first.
+  const uint32_t *n_cls;
   // search configuration
   // teams: independent groups of `gridDim.x / teams` blocks, each running its
   // own batches; per-team buffers sit at team * stride from the base pointers
@@ -235,6 +240,10 @@ struct Workspace {
   uint32_t *f_order = nullptr;      // source order kept by the filter
   uint8_t *f_keep = nullptr;        // its keep flags
   uint32_t *f_count = nullptr;      // kept positions per tile
+  uint32_t *o_order = nullptr;      // the opening's sources
+  uint32_t *o_key = nullptr;        // the pool's keys
+  uint8_t *o_taken = nullptr;       // pool positions in the opening
+  uint32_t o_cap = 0;               // sources o_order holds
   uint32_t *f_end = nullptr;        // per graph: one past its last kept position
   uint32_t *lvl2 = nullptr;         // per vertex: level-2 bounds of the kept sources
   uint32_t f_cap = 0;               // positions f_order holds
@@ -396,7 +405,10 @@ int run_bfscut(tkc_ctx *ctx, const RunParams &p, int words, int blocks);  // blo
 int run_init(tkc_ctx *ctx, uint32_t nctl, uint32_t n, uint32_t ng, bool reset_lists);
 // drops the sources order[0, count) that the current thresholds abandon
 constexpr uint32_t kFilterTiles = 2048;  // most tiles of the filter's compaction
+constexpr uint32_t kOpenPool = 16384;    // sources at the head of the order the opening is picked from
+// the nopen sources for the opening, picked from the head of order[0, count)
+int run_pick_opening(tkc_ctx *ctx, const RunParams &p, const tkc_graph *g, uint32_t count, uint32_t nopen);
 int run_filter(tkc_ctx *ctx, const RunParams &p, const tkc_graph *g, uint32_t open_teams, uint32_t main_teams,
-               uint32_t count, uint32_t *lvl2);
+               uint32_t count, bool picked);
 int max_coresident_blocks(tkc_ctx *ctx, int words);
 }  // namespace tkc

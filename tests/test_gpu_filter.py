@@ -63,6 +63,23 @@ def test_level_2_by_in_degree_class(gpu_lib, ctx, scale, order, relabel):
         t.tkc_free_graph(h)
 
 
+# more sources than the pool the opening is picked from (16 384), and a GIVEN
+# order that puts the most central vertices last, outside the pool
+@pytest.mark.parametrize("n", [16384, 16385, 17001])
+def test_order_longer_than_the_pool(gpu_lib, ctx, n):
+    t = gpu_lib
+    g = gg.barabasi_albert(n, 3, n)
+    ref = oracle.textbook_topk(g, 10)
+    h = t.tkc_load_csr(ctx, g.n, g.offsets, g.cols, g.directed)
+    try:
+        t.tkc_set_source_order(h, np.argsort(g.outdeg(), kind="stable").astype(np.uint32))
+        for order in ("DEG", "NB", "GIVEN"):
+            t.tkc_set_options(ctx, t.Options(order=getattr(t, "TKC_ORDER_" + order)))
+            _same(t.tkc_topk_closeness(h, 10), ref)
+    finally:
+        t.tkc_free_graph(h)
+
+
 @pytest.mark.parametrize("seed_factor", [1, 6, 30])  # prefixes of 10, 60 and 300 sources, the opening is 64
 @pytest.mark.parametrize("order", ["LEARNED", "LEARNED_NB"])
 def test_uncut_prefix_past_the_opening(gpu_lib, ctx, order, seed_factor):
