@@ -1025,6 +1025,7 @@ static int source_order_of(tkc_graph *g, const tkc_options &o, u32 kk, int harmo
   *lb_key = nullptr;
   if (o.order == TKC_ORDER_NB) {
     TKC_RC(ensure_nb_bounds(g, nb_levels_of(o)));
+    TKC_RC(ensure_nb_order(g, harmonic != 0));
     *order = harmonic ? g->nb_horder : g->nb_order;
     *norder = g->n_src_nb;
     *lb_key = harmonic ? g->nb_hkey : g->nb_key;
@@ -1049,6 +1050,7 @@ static int source_order_of(tkc_graph *g, const tkc_options &o, u32 kk, int harmo
     // (still sorted by key, so the stop stays valid past the prefix)
     if (harmonic) return TKC_EINVAL;
     TKC_RC(ensure_nb_bounds(g, nb_levels_of(o)));
+    TKC_RC(ensure_nb_order(g, false));
     TKC_RC(ensure_seeded_order(g, (u32)std::min<u64>((u64)o.seed_factor * kk, 0xffffffffull), true));
     *order = g->seeded_order;
     *norder = g->n_src_nb;
@@ -1488,7 +1490,10 @@ static int topk_bound(tkc_graph *g, uint32_t k, tkc_result *out) {
   TKC_RC(ensure_degree_order(g));
   TKC_RC(ensure_reach_bounds(g));
   const bool nb = o.order == TKC_ORDER_NB;
-  if (nb) TKC_RC(ensure_nb_bounds(g, nb_levels_of(o)));
+  if (nb) {
+    TKC_RC(ensure_nb_bounds(g, nb_levels_of(o)));
+    TKC_RC(ensure_nb_order(g, false));
+  }
   const u32 *order0 = nb ? g->nb_order : g->deg_order;
   const u32 n0 = nb ? g->n_src_nb : g->n_src_deg;
   // defaults measured with NBBound on a 1000 x 1000 grid: 256 sources x 1 team 4.55 s, 256 x 2 4.16 s,
@@ -1785,6 +1790,7 @@ static int topk_many(tkc_ctx *ctx, tkc_graph *const *gs, uint32_t ng, uint32_t k
     // own graph, so they equal the per-graph values); all sources of all graphs
     // are then ordered by (key, union id)
     MULTI_RC(ensure_nb_bounds(&U, nb_levels_of(o), gid, d_gdir));
+    MULTI_RC(ensure_nb_order(&U, harmonic != 0));
   } else {
     MULTI_RC(ensure_degree_order(&U));
   }

@@ -343,6 +343,7 @@ struct tkc_graph {
   unsigned long long *nb_key = nullptr;       //   floor(S~ * 2^46 / (r-1)^2)
   unsigned long long *nb_hkey = nullptr;      // harmonic: ~(FP64 bits of the upper bound on h)
   uint32_t *nb_horder = nullptr;              // harmonic NBCut order: by (nb_hkey, id)
+  uint32_t nb_order_cap = 0, nb_horder_cap = 0;  // level caps those orders were sorted for (0 = not yet)
   // the graph as the search kernel walks it (ensure_search_csr): s_mode 0 =
   // the graph itself, 1 = a copy whose vertex i is vertex s_unlab[i] (s_lab is
   // the inverse), vertices by in-degree, largest first; -1 = not built yet
@@ -378,6 +379,9 @@ int filter_order(tkc_graph *g, const uint32_t *d_order_all, uint32_t *d_out, uin
 // gid/g_directed (several graphs as one union): per-vertex directedness
 int ensure_nb_bounds(tkc_graph *g, uint32_t max_levels, const uint32_t *gid = nullptr,
                      const uint8_t *g_directed = nullptr);
+// the NBCut order (harmonic: the harmonic one) of those bounds, in nb_order or
+// nb_horder; ensure_nb_bounds has run
+int ensure_nb_order(tkc_graph *g, bool harmonic);
 int nb_sort_sources(tkc_graph *g, const unsigned long long *key, uint32_t *order, uint32_t *count);
 // tkc_lb.cu
 int lb_init(tkc_graph *g, const unsigned long long *S0, const uint32_t *r0, const unsigned long long *key0,

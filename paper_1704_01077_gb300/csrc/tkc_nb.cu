@@ -344,23 +344,34 @@ int nb_sort_sources(tkc_graph *g, const u64 *key, u32 *order, u32 *count) {
   return TKC_OK;
 }
 
-// Computes the bound, the order keys and the NBCut order of g (cached until the
-// level cap changes).
+// The order a call needs is sorted when it is first needed: closeness and
+// harmonic searches use one each.
+int ensure_nb_order(tkc_graph *g, bool harmonic) {
+  u32 **order = harmonic ? &g->nb_horder : &g->nb_order;
+  u32 *cap = harmonic ? &g->nb_horder_cap : &g->nb_order_cap;
+  if (*cap == g->nb_cap && *order) return TKC_OK;
+  if (!*order) TKC_TRY(cudaMallocAsync(order, std::max<size_t>(g->n, 1) * sizeof(u32), g->ctx->stream));
+  TKC_RC(nb_sort_sources(g, harmonic ? g->nb_hkey : g->nb_key, *order, &g->n_src_nb));
+  *cap = g->nb_cap;
+  return TKC_OK;
+}
+
+// Computes the bound and the order keys of g (cached until the level cap
+// changes; ensure_nb_order sorts by them).
 int ensure_nb_bounds(tkc_graph *g, u32 K, const u32 *gid, const uint8_t *gdir) {
   if (K == 0 || K > 65535) return TKC_EINVAL;
-  if (g->nb_order && g->nb_cap == K) return TKC_OK;
+  if (g->nb_key && g->nb_cap == K) return TKC_OK;
+  g->nb_cap = g->nb_order_cap = g->nb_horder_cap = 0;
   TKC_RC(ensure_reach_bounds(g));
   tkc_ctx *ctx = g->ctx;
   cudaStream_t st = ctx->stream;
   const u32 n = g->n;
   const size_t n1 = std::max<size_t>(n, 1);
-  if (!g->nb_order) {
-    TKC_TRY(cudaMallocAsync(&g->nb_order, n1 * sizeof(u32), st));
+  if (!g->nb_hkey) {
     TKC_TRY(cudaMallocAsync(&g->nb_S, n1 * sizeof(u64), st));
     TKC_TRY(cudaMallocAsync(&g->nb_r, n1 * sizeof(u32), st));
     TKC_TRY(cudaMallocAsync(&g->nb_key, n1 * sizeof(u64), st));
     TKC_TRY(cudaMallocAsync(&g->nb_hkey, n1 * sizeof(u64), st));
-    TKC_TRY(cudaMallocAsync(&g->nb_horder, n1 * sizeof(u32), st));
   }
   if (n == 0) {
     g->n_src_nb = 0;
@@ -421,9 +432,6 @@ int ensure_nb_bounds(tkc_graph *g, u32 K, const u32 *gid, const uint8_t *gdir) {
   TKC_LAUNCH(k_nb_keys<<<grid_of(n), 256, 0, st>>>(n, s, g->nb_S, g->nb_r, g->nb_key, g->nb_hkey, err));
   int h_err = 0;
   TKC_TRY(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, st));
-  TKC_RC(nb_sort_sources(g, g->nb_key, g->nb_order, &g->n_src_nb));
-  u32 nh = 0;
-  TKC_RC(nb_sort_sources(g, g->nb_hkey, g->nb_horder, &nh));
   TKC_TRY(cudaStreamSynchronize(st));
   for (int i = 0; i < 3; ++i) TKC_TRY(cudaFreeAsync(N[i], st));
   void *frees[] = {s.c, s.P, s.bS, s.bR, s.flag, s.hU, segpos, seg_row, seg_begin, tmp, left, err};
@@ -446,6 +454,7 @@ int tkc_nb_bounds(tkc_graph *g, uint32_t max_levels, uint64_t *S_lb, uint32_t *r
   if (!g || max_levels > 65535) return TKC_EINVAL;
   TKC_TRY(cudaSetDevice(g->ctx->device));
   TKC_RC(ensure_nb_bounds(g, max_levels ? max_levels : 256u));
+  if (order || n_order) TKC_RC(ensure_nb_order(g, false));
   cudaStream_t st = g->ctx->stream;
   const size_t n = g->n;
   if (n) {
@@ -465,6 +474,7 @@ int tkc_nb_harmonic_bounds(tkc_graph *g, uint32_t max_levels, double *h_ub, uint
   if (!g || max_levels > 65535) return TKC_EINVAL;
   TKC_TRY(cudaSetDevice(g->ctx->device));
   TKC_RC(ensure_nb_bounds(g, max_levels ? max_levels : 256u));
+  if (order || n_order) TKC_RC(ensure_nb_order(g, true));
   cudaStream_t st = g->ctx->stream;
   const size_t n = g->n;
   if (n && h_ub) {

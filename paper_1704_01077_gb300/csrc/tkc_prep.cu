@@ -76,8 +76,26 @@ __global__ void k_scan_small(u32 *a, u32 len) {
   }
 }
 
+// Second pass: every block scans its tile from the sum of the tiles before it,
+// which bsum[block] holds (kSummed, after k_scan_small) or which the block adds
+// up itself.
+template <bool kSummed>
 __global__ void k_scan_apply(const u32 *in, u32 *out, u64 len, const u32 *bsum) {
   __shared__ u32 s_warp[33];
+  __shared__ u32 s_base;
+  u32 before = 0;
+  if (kSummed) {
+    before = bsum[blockIdx.x];
+  } else {
+    u32 mine = 0;
+    for (u32 i = threadIdx.x; i < blockIdx.x; i += kScanTPB) mine += bsum[i];
+    mine = __reduce_add_sync(FULL, mine);
+    if (threadIdx.x == 0) s_base = 0;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&s_base, mine);
+    __syncthreads();
+    before = s_base;
+  }
   u64 base = (u64)blockIdx.x * kScanTile + (u64)threadIdx.x * kScanItems;
   u32 v[kScanItems];
   u32 s = 0;
@@ -86,21 +104,53 @@ __global__ void k_scan_apply(const u32 *in, u32 *out, u64 len, const u32 *bsum) 
     s += v[i];
   }
   u32 total;
-  u32 pre = block_exscan_1024(s, s_warp, &total) + bsum[blockIdx.x];
+  u32 pre = block_exscan_1024(s, s_warp, &total) + before;
   for (int i = 0; i < kScanItems; ++i) {
     if (base + i < len) out[base + i] = pre;
     pre += v[i];
   }
 }
 
+// The whole scan by one block, tile after tile.
+__global__ void k_scan_one(const u32 *in, u32 *out, u32 len) {
+  __shared__ u32 s_warp[33];
+  u32 before = 0;
+  for (u32 t = 0; t < len; t += kScanTile) {
+    const u32 base = t + threadIdx.x * kScanItems;
+    u32 v[kScanItems];
+    u32 s = 0;
+    for (int i = 0; i < kScanItems; ++i) {
+      v[i] = base + i < len ? in[base + i] : 0;
+      s += v[i];
+    }
+    u32 total;
+    u32 pre = block_exscan_1024(s, s_warp, &total) + before;
+    for (int i = 0; i < kScanItems; ++i) {
+      if (base + i < len) out[base + i] = pre;
+      pre += v[i];
+    }
+    before += total;
+  }
+}
+
 // out[i] = sum of in[0..i); in and out may alias.  tmp holds ceil(len/4096) words.
+// A launch costs more than a short scan's work, so up to 4 tiles are one
+// block's (2 us a tile), and up to 1 024 tiles take two launches, each block
+// adding up at most 1 024 tile sums; only longer ones scan the sums between.
 static int scan_exclusive(const u32 *in, u32 *out, u64 len, u32 *tmp, cudaStream_t st) {
   if (len == 0) return TKC_OK;
   u64 nb = (len + kScanTile - 1) / kScanTile;
   if (nb > (u64)kScanTPB * 4096) return TKC_EOVERFLOW;
-  TKC_LAUNCH(k_scan_bsum<<<(unsigned)nb, kScanTPB, 0, st>>>(in, len, tmp));
-  TKC_LAUNCH(k_scan_small<<<1, kScanTPB, 0, st>>>(tmp, (u32)nb));
-  TKC_LAUNCH(k_scan_apply<<<(unsigned)nb, kScanTPB, 0, st>>>(in, out, len, tmp));
+  if (nb <= 4) {
+    TKC_LAUNCH(k_scan_one<<<1, kScanTPB, 0, st>>>(in, out, (u32)len));
+  } else if (nb <= 1024) {
+    TKC_LAUNCH(k_scan_bsum<<<(unsigned)nb, kScanTPB, 0, st>>>(in, len, tmp));
+    TKC_LAUNCH(k_scan_apply<false><<<(unsigned)nb, kScanTPB, 0, st>>>(in, out, len, tmp));
+  } else {
+    TKC_LAUNCH(k_scan_bsum<<<(unsigned)nb, kScanTPB, 0, st>>>(in, len, tmp));
+    TKC_LAUNCH(k_scan_small<<<1, kScanTPB, 0, st>>>(tmp, (u32)nb));
+    TKC_LAUNCH(k_scan_apply<true><<<(unsigned)nb, kScanTPB, 0, st>>>(in, out, len, tmp));
+  }
   TKC_TRY(cudaGetLastError());
   return TKC_OK;
 }
@@ -293,76 +343,156 @@ int ensure_in_csr(const tkc_graph *g) {
   return build_in_csr(g);
 }
 
-// ------------------------------------------------------------------ stable LSD radix sort (4-bit digits)
+// ------------------------------------------------------------------ stable LSD radix sort (8-bit digits)
 
 static constexpr int kRsTPB = 256;
-static constexpr int kRsRounds = 4;
+static constexpr int kRsWarps = kRsTPB / 32;
+static constexpr int kRsRounds = 16;  // elements per lane
 static constexpr int kRsTile = kRsTPB * kRsRounds;
 
-__global__ void k_rs_count(const u32 *key, u32 n, int shift, u32 *hist, u32 ntiles) {
-  __shared__ u32 cnt[16];
-  if (threadIdx.x < 16) cnt[threadIdx.x] = 0;
+__global__ void k_rs_count(const u32 *__restrict__ key, u32 n, int shift, u32 *__restrict__ hist, u32 ntiles) {
+  __shared__ u32 cnt[256];
+  cnt[threadIdx.x] = 0;
   __syncthreads();
+#pragma unroll 4
   for (int r = 0; r < kRsRounds; ++r) {
-    u64 i = (u64)blockIdx.x * kRsTile + r * kRsTPB + threadIdx.x;
-    if (i < n) atomicAdd(&cnt[(key[i] >> shift) & 15u], 1u);
+    const u64 i = (u64)blockIdx.x * kRsTile + r * kRsTPB + threadIdx.x;
+    if (i < n) atomicAdd(&cnt[(key[i] >> shift) & 255u], 1u);
   }
   __syncthreads();
-  if (threadIdx.x < 16) hist[threadIdx.x * ntiles + blockIdx.x] = cnt[threadIdx.x];
+  hist[threadIdx.x * ntiles + blockIdx.x] = cnt[threadIdx.x];
 }
 
-// Stable scatter: element order inside a tile is kept by ranking each round's
-// 256 elements by (warp, lane) and carrying per-digit running counts.
-__global__ void k_rs_scatter(const u32 *key, const u32 *val, u32 *key_out, u32 *val_out, u32 n, int shift,
-                             const u32 *hist, u32 ntiles) {
-  __shared__ u32 running[16];
-  __shared__ u32 wcnt[kRsTPB / 32][16];
+// Rank of this lane's element among its warp's so far with the same digit d
+// (256: no element); counts: the warp's running counts per digit.
+__device__ __forceinline__ u32 warp_rank(u32 d, u32 *counts, int lane) {
+  const unsigned peers = __match_any_sync(FULL, d);
+  u32 r = 0;
+  if (d < 256u) r = counts[d] + __popc(peers & ((1u << lane) - 1u));
+  __syncwarp();
+  if (d < 256u && __ffs(peers) - 1 == lane) counts[d] += __popc(peers);
+  __syncwarp();
+  return r;
+}
+
+// Stable scatter: a warp ranks its 512 consecutive elements in order, the
+// warps' counts per digit are summed in warp order, and hist (scanned) holds
+// where each tile's elements of a digit start.  Eight bits a pass: half the
+// passes, and so half the traffic and launches, of four bits.
+__global__ void __launch_bounds__(kRsTPB) k_rs_scatter(const u32 *__restrict__ key, const u32 *__restrict__ val,
+                                                       u32 *__restrict__ key_out, u32 *__restrict__ val_out, u32 n,
+                                                       int shift, const u32 *__restrict__ hist, u32 ntiles) {
+  __shared__ u32 cnt[kRsWarps][256];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (threadIdx.x < 16) running[threadIdx.x] = 0;
+  for (int i = threadIdx.x; i < kRsWarps * 256; i += kRsTPB) (&cnt[0][0])[i] = 0;
+  __syncthreads();
+  const u64 base = (u64)blockIdx.x * kRsTile + wid * (32 * kRsRounds) + lane;
+  u32 k[kRsRounds], rank[kRsRounds];
+#pragma unroll
+  for (int r = 0; r < kRsRounds; ++r) k[r] = base + 32 * r < n ? key[base + 32 * r] : 0u;
+#pragma unroll
+  for (int r = 0; r < kRsRounds; ++r)
+    rank[r] = warp_rank(base + 32 * r < n ? (k[r] >> shift) & 255u : 256u, cnt[wid], lane);
+  __syncthreads();
+  u32 at = hist[threadIdx.x * ntiles + blockIdx.x];
+#pragma unroll
+  for (int w = 0; w < kRsWarps; ++w) {
+    const u32 t = cnt[w][threadIdx.x];
+    cnt[w][threadIdx.x] = at;
+    at += t;
+  }
+  __syncthreads();
+#pragma unroll
   for (int r = 0; r < kRsRounds; ++r) {
-    for (int i = threadIdx.x; i < (kRsTPB / 32) * 16; i += kRsTPB) (&wcnt[0][0])[i] = 0;
+    if (base + 32 * r >= n) break;
+    const u32 pos = cnt[wid][(k[r] >> shift) & 255u] + rank[r];
+    key_out[pos] = k[r];
+    val_out[pos] = val[base + 32 * r];
+  }
+}
+
+// All passes of a short sort in one block: keys and values stay in shared
+// memory (a launch and two more for its scan, per pass, cost more than the work).
+static constexpr int kRsOneTPB = 1024;
+static constexpr int kRsOneRounds = 8;
+static constexpr u32 kRsOneMax = kRsOneTPB * kRsOneRounds;
+static constexpr size_t kRsOneSmem = (2 * (size_t)kRsOneMax + 32 * 256 + 33) * sizeof(u32);
+__global__ void __launch_bounds__(kRsOneTPB) k_rs_one(u32 *key, u32 *val, u32 n, int passes) {
+  extern __shared__ u32 sm[];
+  u32 *sk = sm, *sv = sk + kRsOneMax, *cnt = sv + kRsOneMax, *s_warp = cnt + 32 * 256;  // cnt[warp][digit]
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (u32 i = threadIdx.x; i < n; i += kRsOneTPB) {
+    sk[i] = key[i];
+    sv[i] = val[i];
+  }
+  const u32 base = wid * (32 * kRsOneRounds) + lane;
+  for (int ps = 0; ps < passes; ++ps) {
+    const int shift = 8 * ps;
+    for (int i = threadIdx.x; i < 32 * 256; i += kRsOneTPB) cnt[i] = 0;
     __syncthreads();
-    u64 idx = (u64)blockIdx.x * kRsTile + r * kRsTPB + threadIdx.x;
-    bool valid = idx < n;
-    u32 k = valid ? key[idx] : 0u;
-    u32 d = valid ? ((k >> shift) & 15u) : 16u;
-    u32 peers = __match_any_sync(FULL, d);
-    u32 rank = __popc(peers & ((1u << lane) - 1u));
-    if (valid && rank == 0) wcnt[wid][d] = __popc(peers);
+    u32 k[kRsOneRounds], v[kRsOneRounds], rank[kRsOneRounds];
+#pragma unroll
+    for (int r = 0; r < kRsOneRounds; ++r) {
+      const bool valid = base + 32 * r < n;
+      k[r] = valid ? sk[base + 32 * r] : 0u;
+      v[r] = valid ? sv[base + 32 * r] : 0u;
+    }
+#pragma unroll
+    for (int r = 0; r < kRsOneRounds; ++r)
+      rank[r] = warp_rank(base + 32 * r < n ? (k[r] >> shift) & 255u : 256u, cnt + 256 * wid, lane);
     __syncthreads();
-    if (valid) {
-      u32 pos = hist[d * ntiles + blockIdx.x] + running[d] + rank;
-      for (int w = 0; w < wid; ++w) pos += wcnt[w][d];
-      key_out[pos] = k;
-      val_out[pos] = val[idx];
+    // starts: digits in order, each digit's warps in order; a thread takes 8
+    // warps of one digit
+    const u32 d = threadIdx.x >> 2, w0 = (threadIdx.x & 3) * 8;
+    u32 sum = 0;
+    for (int w = 0; w < 8; ++w) sum += cnt[256 * (w0 + w) + d];
+    u32 total;
+    u32 at = block_exscan_1024(sum, s_warp, &total);
+    for (int w = 0; w < 8; ++w) {
+      const u32 t = cnt[256 * (w0 + w) + d];
+      cnt[256 * (w0 + w) + d] = at;
+      at += t;
     }
     __syncthreads();
-    if (threadIdx.x < 16) {
-      u32 s = 0;
-      for (int w = 0; w < kRsTPB / 32; ++w) s += wcnt[w][threadIdx.x];
-      running[threadIdx.x] += s;
+#pragma unroll
+    for (int r = 0; r < kRsOneRounds; ++r) {
+      if (base + 32 * r >= n) break;
+      const u32 pos = cnt[256 * wid + ((k[r] >> shift) & 255u)] + rank[r];
+      sk[pos] = k[r];
+      sv[pos] = v[r];
     }
     __syncthreads();
+  }
+  for (u32 i = threadIdx.x; i < n; i += kRsOneTPB) {
+    key[i] = sk[i];
+    val[i] = sv[i];
   }
 }
 
 // Sorts (key, val) by key ascending, keeping the input order of equal keys.
-// Only the low `bits` bits of the keys are looked at.  Result lands in key/val.
+// Only the low `bits` bits of the keys are looked at (rounded up to whole
+// digits: keys have no bits above).  Result lands in key/val.
 static int radix_sort_pairs(u32 *key, u32 *val, u32 n, int bits, cudaStream_t st) {
   if (n <= 1 || bits <= 0) return TKC_OK;
+  const int passes = (bits + 7) / 8;
+  if (n <= kRsOneMax) {
+    TKC_TRY(cudaFuncSetAttribute(k_rs_one, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRsOneSmem));
+    TKC_LAUNCH(k_rs_one<<<1, kRsOneTPB, kRsOneSmem, st>>>(key, val, n, passes));
+    TKC_TRY(cudaGetLastError());
+    return TKC_OK;
+  }
   u32 ntiles = (n + kRsTile - 1) / kRsTile;
   u32 *k2 = nullptr, *v2 = nullptr, *hist = nullptr, *tmp = nullptr;
-  size_t hlen = (size_t)16 * ntiles;
+  size_t hlen = (size_t)256 * ntiles;
   TKC_TRY(cudaMallocAsync(&k2, (size_t)n * sizeof(u32), st));
   TKC_TRY(cudaMallocAsync(&v2, (size_t)n * sizeof(u32), st));
   TKC_TRY(cudaMallocAsync(&hist, hlen * sizeof(u32), st));
   TKC_TRY(cudaMallocAsync(&tmp, (hlen / kScanTile + 2) * sizeof(u32), st));
   u32 *ka = key, *va = val, *kb = k2, *vb = v2;
-  int passes = (bits + 3) / 4;
   for (int ps = 0; ps < passes; ++ps) {
-    TKC_LAUNCH(k_rs_count<<<ntiles, kRsTPB, 0, st>>>(ka, n, 4 * ps, hist, ntiles));
+    TKC_LAUNCH(k_rs_count<<<ntiles, kRsTPB, 0, st>>>(ka, n, 8 * ps, hist, ntiles));
     TKC_RC(scan_exclusive(hist, hist, hlen, tmp, st));
-    TKC_LAUNCH(k_rs_scatter<<<ntiles, kRsTPB, 0, st>>>(ka, va, kb, vb, n, 4 * ps, hist, ntiles));
+    TKC_LAUNCH(k_rs_scatter<<<ntiles, kRsTPB, 0, st>>>(ka, va, kb, vb, n, 8 * ps, hist, ntiles));
     TKC_TRY(cudaGetLastError());
     std::swap(ka, kb);
     std::swap(va, vb);
