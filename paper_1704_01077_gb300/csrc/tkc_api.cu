@@ -73,6 +73,7 @@ int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u3
     u32 cap = std::max<u32>(ng, 16);
     TKC_RC(dalloc(&w.tied, cap, st));
     TKC_RC(dalloc(&w.g_ntop, cap, st));
+    TKC_RC(dalloc(&w.g_lock, cap, st));
     TKC_RC(dalloc(&w.g_stop, cap, st));
     TKC_RC(dalloc(&w.g_ctr, 4 * (size_t)cap, st));
     TKC_RC(dalloc(&w.x_seq, cap, st));
@@ -145,7 +146,7 @@ static void free_workspace(tkc_ctx *ctx) {
   Workspace &w = ctx->ws;
   void *ptrs[] = {w.seen, w.F0, w.F1, w.N, w.FB0, w.FB1, w.L0, w.L1, w.Loff0, w.Loff1, w.VL, w.stamp, w.res_S, w.res_r,
                   w.slots, w.cnt, w.wsum, w.top_S, w.top_r, w.top_id, w.ctl, w.out_S, w.out_r, w.out_id,
-                  w.out_f, w.out_c, w.tied, w.g_ntop, w.g_stop, w.g_ctr, w.sh, w.x_seq, w.x_S, w.x_r, w.x_id,
+                  w.out_f, w.out_c, w.tied, w.g_ntop, w.g_lock, w.g_stop, w.g_ctr, w.sh, w.x_seq, w.x_S, w.x_r, w.x_id,
                   w.f_order, w.f_keep, w.f_count, w.f_end, w.lvl2,
                   w.o_order, w.o_key, w.o_taken};
   for (void *p : ptrs)
@@ -298,6 +299,7 @@ struct RunSetup {
   // interleaved), and the first position after the openings
   const u32 *g_end;
   u32 g_rest;
+  const u32 *g_base;        // first vertex of each graph (ng + 1 words)
 };
 
 // Teams used when the options leave it to the library: one team for small
@@ -305,8 +307,12 @@ struct RunSetup {
 // so that the latency of one team's level steps overlaps with the others.
 // NBCut on one graph examines few sources, each batch deeper: fewer, larger
 // teams (measured on R-MAT 22: 4 teams 357 ms, 9 teams 372 ms, 19 teams 411 ms).
-static u32 default_teams(u32 n, u32 B, u32 maxb, bool nb) {
+// Several graphs: four blocks per team, since a level of one of the graphs is
+// short (512 graphs of 1 000 to 200 000 vertices, 128-bit batches: 19 teams
+// 203 ms a call, 38 teams 184 ms).
+static u32 default_teams(u32 n, u32 B, u32 maxb, bool nb, u32 ng) {
   if (B <= 1 || n < (1u << 14)) return 1;
+  if (ng > 1 && n >= (1u << 16)) return std::max<u32>(1, maxb / 4);
   if (nb) return std::max<u32>(1, maxb / 32);
   if (n < (1u << 16)) return std::max<u32>(1, maxb / 16);
   return std::max<u32>(1, maxb / 8);  // eight blocks (SMs) per team, every SM used
@@ -333,7 +339,13 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   int maxb = max_coresident_blocks(ctx, rs.W);
   if (maxb <= 0) return TKC_ECUDA;
   const bool nb_one = rs.lb_key != nullptr && rs.ng == 1;
-  u32 T = rs.B <= 1 ? 1u : (o.teams ? o.teams : default_teams(g->n, rs.B, (u32)maxb, nb_one));
+  u32 T = rs.B <= 1 ? 1u : (o.teams ? o.teams : default_teams(g->n, rs.B, (u32)maxb, nb_one, rs.ng));
+  // several graphs: every team's rows and lists cover the union, so as many
+  // teams as a quarter of the device's memory holds
+  if (rs.ng > 1 && !o.teams) {
+    const u64 per_team = (u64)g->n * (32 * rs.W + 24) + 1;
+    T = (u32)std::max<u64>(1, std::min<u64>(T, ctx->total_mem / 4 / per_team));
+  }
   if (rs.force_teams) T = rs.force_teams;
   // deterministic schedule: one team, so x moves only at its level barriers
   // (updateBoundsLB rounds fix their own team count: no cuts, already exact)
@@ -381,7 +393,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   p.directed = g->directed;
   p.arcs = g->arcs;
   const bool by_size = labelled_by_size(o, rs.B, rs.size_n ? rs.size_n : g->n);
-  TKC_RC(ensure_search_csr(g, o.relabel == 1 || (by_size && (!opening || g->s_mode == 1))));
+  TKC_RC(ensure_search_csr(g, o.relabel == 1 || (by_size && (!opening || g->s_mode == 1)), rs.gid, rs.ng));
   auto walk_search_csr = [&] {
     const bool lab = g->s_mode == 1;
     p.off = lab ? g->s_off : g->off;
@@ -393,6 +405,8 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     p.bu_list = g->bu_list;
     p.n_bu = g->n_bu;
     p.n_bu_heavy = g->n_bu_heavy;
+    p.g_bu = lab ? nullptr : g->g_bu;
+    p.g_base = p.g_bu ? rs.g_base : nullptr;
     p.heavy_in = g->heavy_in ? g->heavy_in : kHeavyIn;
   };
   walk_search_csr();
@@ -409,6 +423,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   p.g_rest = rs.g_rest;
   p.g_directed = rs.g_directed;
   p.g_ntop = w.g_ntop;
+  p.g_lock = w.g_lock;
   p.g_ctr = rs.ng > 1 ? w.g_ctr : nullptr;
   p.kk = rs.kk;
   p.B = rs.B;
@@ -531,6 +546,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     hctl->st_bu_new += x.st_bu_new;
     hctl->st_bu_frontier += x.st_bu_frontier;
     hctl->st_bu_rows += x.st_bu_rows;
+    hctl->st_bu_swept += x.st_bu_swept;
     hctl->st_seeded += x.st_seeded;
     hctl->st_cleared += x.st_cleared;
     hctl->st_compactions += x.st_compactions;
@@ -580,7 +596,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     rs_out.bu_new = hctl->st_bu_new;
     rs_out.bu_frontier = hctl->st_bu_frontier;
     rs_out.bu_rows_read = hctl->st_bu_rows;
-    rs_out.bu_swept = (uint64_t)(g->bu_list ? g->n_bu : g->n) * hctl->st_bu_levels;
+    rs_out.bu_swept = hctl->st_bu_swept;
     rs_out.seeded = hctl->st_seeded;
     rs_out.cleared = hctl->st_cleared;
     rs_out.compactions = hctl->st_compactions;
@@ -782,6 +798,8 @@ int tkc_create(tkc_ctx **out, const tkc_options *opt) {
   int coop = 0;
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device);
   cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device);
+  size_t mem_free = 0;
+  cudaMemGetInfo(&mem_free, &ctx->total_mem);
   if (!coop || ctx->num_sms <= 0) {
     delete ctx;
     return TKC_ECUDA;
@@ -1797,7 +1815,7 @@ static int topk_many(tkc_ctx *ctx, tkc_graph *const *gs, uint32_t ng, uint32_t k
   TKC_TRY(cudaEventRecord(ctx->ev[1], st));
   RunSetup rs;
   memset(&rs, 0, sizeof(rs));
-  u32 bits = o.batch_bits ? o.batch_bits : default_batch_bits(nv);
+  u32 bits = o.batch_bits ? o.batch_bits : default_batch_bits(nv, nb);
   rs.g = &U;
   rs.order = nb ? (harmonic ? U.nb_horder : U.nb_order) : U.deg_order;
   rs.norder = nb ? U.n_src_nb : U.n_src_deg;
@@ -1810,6 +1828,7 @@ static int topk_many(tkc_ctx *ctx, tkc_graph *const *gs, uint32_t ng, uint32_t k
   rs.ng = ng;
   rs.gid = gid;
   rs.g_directed = d_gdir;
+  rs.g_base = d_vbase;
   rs.size_n = maxn;
   // The sources graph by graph, each graph's in its own order: first the
   // first B sources of every graph (one opening batch per graph, searched

@@ -344,16 +344,17 @@ __device__ __forceinline__ bool row_nonzero(const u64 (&r)[W]) {
 }
 
 // Zeroes the frontier rows of the listed vertices and their frontier bits.
-// A long list clears the whole bitmap instead of one bit per vertex.
+// A long list clears the whole bitmap (of vertices [v0, v1), where all listed
+// ones lie) instead of one bit per vertex.
 template <int W>
-__device__ __forceinline__ void clear_frontier(u64 *F, uint32_t *FB, const uint32_t *list, uint32_t count, uint32_t n,
-                                               uint64_t gthread, uint64_t nthreads) {
+__device__ __forceinline__ void clear_frontier(u64 *F, uint32_t *FB, const uint32_t *list, uint32_t count, uint32_t v0,
+                                               uint32_t v1, uint64_t gthread, uint64_t nthreads) {
   for (uint64_t i = gthread; i < (uint64_t)count * W; i += nthreads) {
     uint32_t v = list[i / W];
     F[(size_t)v * W + (i % W)] = 0;
   }
-  if (count > n / 32) {
-    for (uint64_t i = gthread; i < n / 32 + 1; i += nthreads) FB[i] = 0;
+  if (count > (v1 - v0) / 32) {
+    for (uint64_t i = v0 / 32 + gthread; i < v1 / 32 + 1; i += nthreads) FB[i] = 0;
   } else {
     for (uint64_t i = gthread; i < count; i += nthreads) {
       uint32_t v = list[i];
@@ -494,64 +495,57 @@ __device__ __forceinline__ Thresh thresh_of(const RunParams &p, uint32_t g) {
 
 // Publishes graph g's current k-th entry (caller holds the merge lock).
 __device__ __forceinline__ void publish_thresh(const RunParams &p, uint32_t g) {
-  if (p.g_ntop[g] != p.kk) return;
+  if (*(volatile unsigned *)&p.g_ntop[g] != p.kk) return;
   size_t i = (size_t)g * p.kk + p.kk - 1;
-  unsigned s = p.x_seq[g];
+  unsigned s = *(volatile unsigned *)&p.x_seq[g];
   *(volatile unsigned *)&p.x_seq[g] = s + 1u;
   __threadfence();
-  *(volatile u64 *)&p.x_S[g] = p.top_S[i];
-  *(volatile uint32_t *)&p.x_id[g] = p.top_id[i];
-  *(volatile uint32_t *)&p.x_r[g] = p.top_r[i];
+  *(volatile u64 *)&p.x_S[g] = *(volatile u64 *)&p.top_S[i];
+  *(volatile uint32_t *)&p.x_id[g] = *(volatile uint32_t *)&p.top_id[i];
+  *(volatile uint32_t *)&p.x_r[g] = *(volatile uint32_t *)&p.top_r[i];
   __threadfence();
   st_release_u32(&p.x_seq[g], s + 2u);
 }
 
-// Merge lock shared by the teams; a wait beyond the budget is an error.
-__device__ __forceinline__ bool lock_lists(const RunParams &p) {
-  __shared__ int s_ok;
-  if (threadIdx.x == 0) {
-    long long t0 = clock64();
-    unsigned ns = 32;
-    int ok = 1;
-    while (atomicCAS(&p.sh->lock, 0, 1) != 0) {
-      if (ld_volatile_i32(&p.sh->err) != 0 || (uint64_t)(clock64() - t0) > p.timeout) {
-        atomicCAS(&p.sh->err, 0, TKC_ETIMEOUT);
-        atomicCAS(&p.ctl->err, 0, TKC_ETIMEOUT);
-        ok = 0;
-        break;
-      }
-      __nanosleep(ns);
-      if (ns < 256) ns <<= 1;
+// Lock of graph g's list, taken by one thread; a wait beyond the budget is an
+// error.
+__device__ __forceinline__ bool lock_list(const RunParams &p, uint32_t g) {
+  long long t0 = clock64();
+  unsigned ns = 32;
+  while (atomicCAS(&p.g_lock[g], 0, 1) != 0) {
+    if (ld_volatile_i32(&p.sh->err) != 0 || (uint64_t)(clock64() - t0) > p.timeout) {
+      atomicCAS(&p.sh->err, 0, TKC_ETIMEOUT);
+      atomicCAS(&p.ctl->err, 0, TKC_ETIMEOUT);
+      return false;
     }
-    __threadfence();
-    s_ok = ok;
+    __nanosleep(ns);
+    if (ns < 256) ns <<= 1;
   }
-  __syncthreads();
-  return s_ok != 0;
+  __threadfence();
+  return true;
 }
 
-__device__ __forceinline__ void unlock_lists(const RunParams &p) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    atomicExch(&p.sh->lock, 0);
-  }
+__device__ __forceinline__ void unlock_list(const RunParams &p, uint32_t g) {
+  __threadfence();
+  atomicExch(&p.g_lock[g], 0);
 }
 
 // Merges the block's candidate list (sm.cS/cr/cid, sm.ncand entries) into the
-// global top list.  Every entry's new position is its rank among the old list
-// and the candidates (keys are unique: farness then id), so each position below
-// k gets exactly one writer and the old list is read from a shared copy.
+// list of graph g (all candidates are g's).  Every entry's new position is its
+// rank among the old list and the candidates (keys are unique: farness then
+// id), so each position below k gets exactly one writer and the old list is
+// read from a shared copy.
 template <int W>
-__device__ void merge_topk_one(const RunParams &p, Smem<W> &sm) {
+__device__ void merge_topk_one(const RunParams &p, Smem<W> &sm, uint32_t g) {
   const uint32_t kk = p.kk;
-  uint32_t ntop = p.g_ntop[0];
+  const size_t at = (size_t)g * kk;
+  uint32_t ntop = *(volatile unsigned *)&p.g_ntop[g];
   uint32_t nc = sm.ncand;
   if (nc == 0) return;
   for (uint32_t i = threadIdx.x; i < ntop; i += blockDim.x) {
-    sm.tS[i] = p.top_S[i];
-    sm.tr[i] = p.top_r[i];
-    sm.tid[i] = p.top_id[i];
+    sm.tS[i] = *(volatile u64 *)&p.top_S[at + i];
+    sm.tr[i] = *(volatile uint32_t *)&p.top_r[at + i];
+    sm.tid[i] = *(volatile uint32_t *)&p.top_id[at + i];
   }
   __syncthreads();
   // rank of each candidate among existing entries and other candidates
@@ -568,9 +562,9 @@ __device__ void merge_topk_one(const RunParams &p, Smem<W> &sm) {
     for (uint32_t j = 0; j < nc; ++j)
       if (j != i && entry_less(p.harmonic, sm.cS[j], sm.cr[j], sm.cid[j], S, r, id)) ++rank;
     if (rank < kk) {
-      p.top_S[rank] = S;
-      p.top_r[rank] = r;
-      p.top_id[rank] = id;
+      p.top_S[at + rank] = S;
+      p.top_r[at + rank] = r;
+      p.top_id[at + rank] = id;
     }
   }
   for (uint32_t i = threadIdx.x; i < ntop; i += blockDim.x) {
@@ -578,19 +572,19 @@ __device__ void merge_topk_one(const RunParams &p, Smem<W> &sm) {
     for (uint32_t j = 0; j < nc; ++j)
       if (entry_less(p.harmonic, sm.cS[j], sm.cr[j], sm.cid[j], sm.tS[i], sm.tr[i], sm.tid[i])) ++rank;
     if (rank < kk) {
-      p.top_S[rank] = sm.tS[i];
-      p.top_r[rank] = sm.tr[i];
-      p.top_id[rank] = sm.tid[i];
+      p.top_S[at + rank] = sm.tS[i];
+      p.top_r[at + rank] = sm.tr[i];
+      p.top_id[at + rank] = sm.tid[i];
     }
   }
   __syncthreads();
   uint32_t nnew = ntop + nc < kk ? ntop + nc : kk;
-  if (threadIdx.x == 0) p.g_ntop[0] = nnew;
+  if (threadIdx.x == 0) p.g_ntop[g] = nnew;
   __syncthreads();
 }
 
-// Several graphs: the thread holding a graph's first candidate inserts that
-// graph's candidates into its list one by one (each list has one writer).
+// A batch of several graphs: the thread holding a graph's first candidate
+// inserts that graph's candidates into its list one by one, under its lock.
 template <int W>
 __device__ void merge_topk_many(const RunParams &p, Smem<W> &sm) {
   const uint32_t kk = p.kk;
@@ -599,10 +593,10 @@ __device__ void merge_topk_many(const RunParams &p, Smem<W> &sm) {
     const uint32_t g = sm.cg[i];
     bool first = true;
     for (uint32_t j = 0; j < i && first; ++j) first = sm.cg[j] != g;
-    if (!first) continue;
-    u64 *tS = p.top_S + (size_t)g * kk;
-    uint32_t *tr = p.top_r + (size_t)g * kk, *ti = p.top_id + (size_t)g * kk;
-    uint32_t cnt = p.g_ntop[g];
+    if (!first || !lock_list(p, g)) continue;
+    volatile u64 *tS = p.top_S + (size_t)g * kk;
+    volatile uint32_t *tr = p.top_r + (size_t)g * kk, *ti = p.top_id + (size_t)g * kk;
+    uint32_t cnt = *(volatile unsigned *)&p.g_ntop[g];
     for (uint32_t j = i; j < nc; ++j) {
       if (sm.cg[j] != g) continue;
       u64 S = sm.cS[j];
@@ -619,24 +613,34 @@ __device__ void merge_topk_many(const RunParams &p, Smem<W> &sm) {
       tr[pos] = r;
       ti[pos] = id;
     }
-    p.g_ntop[g] = cnt;
+    *(volatile unsigned *)&p.g_ntop[g] = cnt;
     publish_thresh(p, g);
+    unlock_list(p, g);
   }
   __syncthreads();
 }
 
 template <int W>
 __device__ __forceinline__ void merge_topk(const RunParams &p, Smem<W> &sm) {
+  __shared__ int s_ok;
   if (sm.ncand == 0) return;
-  if (!lock_lists(p)) return;
-  __threadfence();
-  if (p.ng == 1) {
-    merge_topk_one(p, sm);
-    if (threadIdx.x == 0) publish_thresh(p, 0);
-  } else {
+  const int g = p.ng == 1 ? 0 : p.g_bu ? p.ctl->bgraph : -1;
+  if (g < 0) {
     merge_topk_many(p, sm);
+    return;
   }
-  unlock_lists(p);
+  if (threadIdx.x == 0) s_ok = lock_list(p, g);
+  __syncthreads();
+  if (!s_ok) return;
+  __threadfence();
+  merge_topk_one(p, sm, g);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    publish_thresh(p, g);
+    unlock_list(p, g);
+  }
+  __syncthreads();
 }
 
 __device__ __forceinline__ void graph_count(const RunParams &p, uint32_t g, int which, u64 v) {
@@ -670,9 +674,16 @@ __device__ __forceinline__ void trace_stamp(const RunParams &p, int slot) {
 }
 
 // Direction of the next level: bottom-up when the frontier's arcs are a large
-// share of all arcs.
+// share of all arcs; several graphs, and the batch's searches all in one:
+// of that graph's arcs (a batch of several graphs stays top-down).
 __device__ __forceinline__ int choose_dir(const RunParams &p, u64 fl_arcs) {
-  return ((u128)fl_arcs * p.bu_num > (u128)p.arcs * p.bu_den) ? 1 : 0;
+  u64 arcs = p.arcs;
+  if (p.g_bu) {
+    const int g = p.ctl->bgraph;
+    if (g < 0) return 0;
+    arcs = p.off[p.g_base[g + 1]] - p.off[p.g_base[g]];
+  }
+  return ((u128)fl_arcs * p.bu_num > (u128)arcs * p.bu_den) ? 1 : 0;
 }
 
 // Frontier lists at most this long are never compacted (the pass and its
@@ -789,10 +800,11 @@ __device__ void epilogue_level(const RunParams &p, Smem<W> &sm) {
         c->st_td_arcs += fa;
         c->st_td_new += nl;
       } else {
-        const u64 swept = p.bu_list ? p.n_bu : p.n;
+        const u64 swept = p.g_bu ? p.g_bu[2 * (size_t)c->bgraph] : p.bu_list ? p.n_bu : p.n;
         bytes = swept * (4 + rb) + c->lvl_scan_v * 8 + c->lvl_scan_a * 8 + c->lvl_scan_r * rb + nl * (8 + 2 * rb) +
                 fl * (4 + rb);
         c->st_bu_levels += 1;
+        c->st_bu_swept += swept;
         c->st_bu_rows += c->lvl_scan_r;
         c->st_bu_scan_v += c->lvl_scan_v;
         c->st_bu_scan_a += c->lvl_scan_a;
@@ -885,6 +897,33 @@ __device__ __forceinline__ uint32_t omega_of(const RunParams &p, uint32_t v, uin
   return o < cap ? o : cap;
 }
 
+// Several graphs after their openings, the order graph by graph: takes up to
+// `room` positions of one graph -- of graph `same` (0xffffffff: any) -- so that
+// a batch's searches share one graph's arcs and may run bottom-up over it.
+// Returns the first position (p.norder: none) and their number in *take.  (A
+// failed exchange means another team took positions.)
+__device__ __forceinline__ uint32_t take_of_graph(const RunParams &p, uint32_t room, uint32_t same, uint32_t *take) {
+  uint32_t cur = *(volatile unsigned *)&p.sh->cursor;
+  while (cur < p.norder) {
+    const uint32_t g = p.gid[p.order[cur]];
+    if (same != 0xffffffffu && g != same) break;
+    const uint32_t end = p.g_end[g];
+    const bool stopped = p.lb_key && *(volatile unsigned *)&p.g_stop[g];
+    const uint32_t next = stopped || end - cur < room ? end : cur + room;
+    const uint32_t old = atomicCAS(&p.sh->cursor, cur, next);
+    if (old != cur) {
+      cur = old;
+    } else if (stopped) {
+      cur = next;
+    } else {
+      *take = next - cur;
+      return cur;
+    }
+  }
+  *take = 0;
+  return p.norder;
+}
+
 // Epilogue after a clear step: seed the next batch of up to B sources.
 template <int W>
 __device__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
@@ -897,8 +936,12 @@ __device__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
   uint32_t *FLoff = c->lcur ? p.Loff1 : p.Loff0;
   uint32_t assigned = 0, last_base = 0;
   u64 arcs_total = 0, started = 0, cut0 = 0;
-  __shared__ uint32_t s_base;
+  __shared__ uint32_t s_base, s_take, s_gmin, s_gmax;
   __shared__ int s_gate;
+  if (threadIdx.x == 0) {
+    s_gmin = 0xffffffffu;
+    s_gmax = 0;
+  }
   if (threadIdx.x < W) sm.active[threadIdx.x] = 0;
   // One graph and several teams, no threshold yet: the other teams start only
   // after team 0's first batch.  Until then every source they took would be
@@ -931,13 +974,20 @@ __device__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
   const bool lb_done = p.lvl && c->batches >= 1;
   while (!lb_done && assigned < B) {
     const uint32_t room = B - assigned;
-    if (threadIdx.x == 0) s_base = atomicAdd(&p.sh->cursor, room);
+    if (threadIdx.x == 0) {
+      if (p.g_bu && p.g_end && p.g_rest == 0)
+        s_base = take_of_graph(p, room, assigned ? s_gmin : 0xffffffffu, &s_take);
+      else {
+        s_base = atomicAdd(&p.sh->cursor, room);
+        s_take = room;
+      }
+    }
     __syncthreads();
-    const uint32_t base = s_base;
+    const uint32_t base = s_base, most = s_take;
     __syncthreads();
     if (base >= p.norder) break;
     last_base = base;
-    const uint32_t cnt = room < p.norder - base ? room : p.norder - base;
+    const uint32_t cnt = most < p.norder - base ? most : p.norder - base;
     const uint32_t idx = base + threadIdx.x;
     const bool valid = threadIdx.x < cnt;
     uint32_t v = valid ? p.order[idx] : 0;
@@ -1007,6 +1057,10 @@ __device__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
       sl.nocut = idx < p.nocut_prefix;
       sl.pad = 0;
       sl.H = 0.0;
+      if (p.g_bu) {
+        atomicMin(&s_gmin, gv);
+        atomicMax(&s_gmax, gv);
+      }
       if (p.lvl_src) p.lvl_src[p.team * B + s] = v;
       p.slots[s] = sl;
       graph_count(p, gv, 1, 1);
@@ -1066,6 +1120,7 @@ __device__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
       if (p.team == 0) ((volatile Shared *)p.sh)->first_done = 1u;
     } else {
       c->step = 0;
+      c->bgraph = s_gmin == s_gmax ? (int)s_gmin : -1;
       c->dir = choose_dir(p, arcs_total);
     }
   }
@@ -1132,6 +1187,9 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
     uint32_t *NL = lcur ? p.L0 : p.L1;
     uint32_t *NLoff = lcur ? p.Loff0 : p.Loff1;
     const uint32_t fl_count = vc->fl_count;
+    // the vertices this batch's searches can touch
+    const int bg = p.g_bu ? vc->bgraph : -1;
+    const uint32_t v0 = bg >= 0 ? p.g_base[bg] : 0u, v1 = bg >= 0 ? p.g_base[bg + 1] : p.n;
     if (step == 1) {
       if (tb == 0) trace_stamp(p, 8);
       // ---- clear step: zero the rows touched by the finished batch
@@ -1140,7 +1198,7 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
         uint32_t v = p.VL[i / W];
         p.seen[(size_t)v * W + (i % W)] = 0;
       }
-      clear_frontier<W>(Fcur, FBcur, FL, fl_count, p.n, gthread, nthreads);
+      clear_frontier<W>(Fcur, FBcur, FL, fl_count, v0, v1, gthread, nthreads);
       if (tb == 0) trace_stamp(p, 12);
       if (!team_sync(c, p.sh, bpt, p.timeout, [&] { epilogue_seed<W>(p, sm); })) break;
       continue;
@@ -1290,7 +1348,7 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
         warp_count_slots<W>(nw, od, sm.cnt, sm.wsum, lane);
         warp_append_plain(valid && was_empty, w, &c->vl_count, p.VL, lane);
       }
-      clear_frontier<W>(Fcur, FBcur, FL, fl_count, p.n, gthread, nthreads);
+      clear_frontier<W>(Fcur, FBcur, FL, fl_count, v0, v1, gthread, nthreads);
     } else {
       // ---- phase A, bottom-up: each vertex ORs its in-neighbours' frontier rows
       u64 act[W];
@@ -1302,8 +1360,9 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
       // holding list entries j, j + hg, j + 2 hg, ... so that the longest rows
       // land in different warps; then chunks of kBuChunkVerts consecutive
       // entries of the shorter rows (labels ascending).
-      const uint32_t nheavy = p.bu_list ? p.n_bu_heavy : 0u;
-      const uint32_t nlight = p.bu_list ? p.n_bu - nheavy : p.n;
+      const uint32_t *list = bg >= 0 ? p.bu_list + v0 : p.bu_list;
+      const uint32_t nheavy = bg >= 0 ? p.g_bu[2 * bg + 1] : list ? p.n_bu_heavy : 0u;
+      const uint32_t nlight = bg >= 0 ? p.g_bu[2 * bg] - nheavy : list ? p.n_bu - nheavy : p.n;
       const uint32_t hg = (nheavy + 31) / 32;
       const uint32_t nitems = hg + (nlight + kBuChunkVerts - 1) / kBuChunkVerts;
       for (;;) {
@@ -1322,10 +1381,10 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
           if (hitem) {
             const uint32_t e = gi + hg * (uint32_t)lane;
             valid = e < nheavy;
-            w = valid ? p.bu_list[e] : 0;
+            w = valid ? list[e] : 0;
           } else {
             valid = base + lane < g1;
-            w = valid ? (p.bu_list ? p.bu_list[nheavy + base + lane] : base + lane) : 0;
+            w = valid ? (list ? list[nheavy + base + lane] : base + lane) : 0;
           }
           u64 nw[W], sr[W], miss[W];
           uint32_t od = 0, e0 = 0, ee = 0;
@@ -1496,7 +1555,7 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
       if (!team_sync(c, p.sh, bpt, p.timeout, [] {})) break;
       if (tb == 0) trace_stamp(p, 10);
       // ---- phase B: only the old frontier rows need clearing
-      clear_frontier<W>(Fcur, FBcur, FL, fl_count, p.n, gthread, nthreads);
+      clear_frontier<W>(Fcur, FBcur, FL, fl_count, v0, v1, gthread, nthreads);
     }
     if (tb == 0) trace_stamp(p, 11);
     // flush the block's per-slot counters
@@ -1533,8 +1592,8 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
 // epilogue seeds the first batch), the shared block and, with nlist > 0, the
 // per-graph list state and res_r of n vertices.
 __global__ void k_run_init(Ctl *ctl, uint32_t nctl, unsigned level_base, Shared *sh, uint32_t nlist, unsigned *g_ntop,
-                           unsigned *g_stop, u64 *g_ctr, unsigned *x_seq, uint32_t *x_r, uint32_t *res_r,
-                           uint32_t n) {
+                           unsigned *g_stop, int *g_lock, u64 *g_ctr, unsigned *x_seq, uint32_t *x_r,
+                           uint32_t *res_r, uint32_t n) {
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
   static_assert(sizeof(Ctl) % 8 == 0, "control blocks are zeroed by 64-bit words");
   for (uint32_t i = t; i < nctl * (uint32_t)(sizeof(Ctl) / 8); i += nt) {
@@ -1553,6 +1612,7 @@ __global__ void k_run_init(Ctl *ctl, uint32_t nctl, unsigned level_base, Shared 
   if (t == 0) *sh = Shared{};
   for (uint32_t i = t; i < nlist; i += nt) {
     g_ntop[i] = g_stop[i] = x_seq[i] = 0;
+    g_lock[i] = 0;
     x_r[i] = 0;
     for (int j = 0; j < 4; ++j) g_ctr[4 * (size_t)i + j] = 0;
   }
@@ -1940,7 +2000,8 @@ int run_init(tkc_ctx *ctx, uint32_t nctl, uint32_t n, uint32_t ng, bool reset_li
   const uint32_t work = reset_lists ? (n > ng ? n : ng) : 1024;
   const uint32_t blocks = work / 1024 + 1 < (uint32_t)ctx->num_sms * 8 ? work / 1024 + 1 : (uint32_t)ctx->num_sms * 8;
   TKC_LAUNCH(k_run_init<<<blocks, 256, 0, ctx->stream>>>(w.ctl, nctl, w.level_base, w.sh, reset_lists ? ng : 0u,
-                                                         w.g_ntop, w.g_stop, w.g_ctr, w.x_seq, w.x_r, w.res_r, n));
+                                                         w.g_ntop, w.g_stop, w.g_lock, w.g_ctr, w.x_seq, w.x_r, w.res_r,
+                                                         n));
   TKC_TRY(cudaGetLastError());
   return TKC_OK;
 }

@@ -97,14 +97,14 @@ struct Ctl {
   unsigned long long st_bu_levels, st_bu_scan_v, st_bu_scan_a, st_bu_new, st_bu_frontier, st_bu_rows;
   unsigned long long st_seeded, st_cleared;
   unsigned long long st_compactions, st_compact_dropped;
+  unsigned long long st_bu_swept;
   int lcur;          // which list buffer holds the current frontier list (compaction swaps it alone)
-  int pad2;
+  int bgraph;        // several graphs: the graph of every search of the batch, -1 when they differ
 };
 
 // State shared by all teams of one run.
 struct Shared {
   unsigned int cursor;   // next position in the source order (teams take chunks)
-  int lock;              // guards the k-lists while a team merges
   int err;               // first error of any team
   unsigned int first_done;  // team 0 has finished its first batch (other teams may start)
   unsigned int norder;   // sources the filter kept (the main launch's order length)
@@ -143,6 +143,11 @@ struct RunParams {
   // others by label (nullptr: every vertex, by label)
   const uint32_t *bu_list;
   uint32_t n_bu, n_bu_heavy;
+  // several graphs in their own ids: graph g's vertices with an in-arc are
+  // bu_list[g_base[g], g_base[g] + g_bu[2 g]), the g_bu[2 g + 1] long rows
+  // first; a batch of one graph's searches runs bottom-up over that part
+  // (nullptr: bottom-up by the union's arcs, over the whole list)
+  const uint32_t *g_base, *g_bu;
   uint32_t heavy_in;  // in-rows longer than this are walked by the whole warp
   uint32_t large_blocks;  // tkc_options.large_blocks: 0 = by size, 1 = larger blocks, 2 = 512 threads
   const uint32_t *order;
@@ -179,6 +184,7 @@ struct RunParams {
   uint32_t g_rest;
   const uint8_t *g_directed;  // per graph (nullptr: `directed` for all)
   unsigned int *g_ntop;       // entries in each graph's top list
+  int *g_lock;                // guards each graph's list while a team merges into it
   unsigned long long *g_ctr;  // per graph: edges_visited, bfs_started, bfs_cut, bfs_finished (nullable)
   uint32_t kk;        // min(k, n); 0 never reaches the kernel
   uint32_t B;         // active slots per batch (1..64*W)
@@ -252,6 +258,7 @@ struct Workspace {
   double *out_f = nullptr, *out_c = nullptr;
   unsigned int *tied = nullptr;     // per graph
   unsigned int *g_ntop = nullptr;   // per graph
+  int *g_lock = nullptr;            // per graph
   unsigned int *g_stop = nullptr;   // per graph: NBCut stop reached
   unsigned long long *g_ctr = nullptr;  // 4 per graph
   Shared *sh = nullptr;
@@ -295,6 +302,7 @@ struct tkc_ctx {
   cudaStream_t stream = nullptr;
   tkc_options opt{};
   int num_sms = 0;
+  size_t total_mem = 0;  // bytes of device memory
   tkc::Workspace ws;
   cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   cudaStream_t aux = nullptr;    // helper stream: the labelled copy, built while `stream` preprocesses
@@ -354,6 +362,7 @@ struct tkc_graph {
   mutable cudaEvent_t s_ready = nullptr;      // the copy is being built on the context's helper stream
   mutable uint32_t *bu_list = nullptr;        // bottom-up sweep order of that CSR: vertices with an in-arc, hubs first
   mutable uint32_t n_bu = 0, n_bu_heavy = 0;
+  mutable uint32_t *g_bu = nullptr;           // a union in its own ids: per graph n_bu and n_bu_heavy (device)
   mutable uint32_t heavy_in = 0;              // the list's long-row threshold (kHeavyIn or kHeavyInLabelled)
 };
 
@@ -371,7 +380,8 @@ int ensure_classes(const tkc_graph *g, const uint32_t *gid, uint32_t ng);
 // one pivot per graph in the first forward-backward round
 int ensure_reach_bounds(tkc_graph *g, const uint32_t *gid = nullptr, uint32_t ng = 0);
 // the search kernel's CSR and bottom-up list (relabel: the in-degree labelling)
-int ensure_search_csr(const tkc_graph *g, bool relabel);
+// (gid/ng: a union; in its own ids the list is then graph by graph)
+int ensure_search_csr(const tkc_graph *g, bool relabel, const uint32_t *gid = nullptr, uint32_t ng = 0);
 int start_search_csr(const tkc_graph *g);  // the labelled copy, on the helper stream
 void free_search_csr(const tkc_graph *g);
 int filter_order(tkc_graph *g, const uint32_t *d_order_all, uint32_t *d_out, uint32_t *count);

@@ -61,7 +61,8 @@ struct Layout {
   static constexpr size_t top_r = top_S + 256;
   static constexpr size_t top_id = top_r + 256;
   static constexpr size_t g_ntop = top_id + 256;
-  static constexpr size_t shared = g_ntop + 256;
+  static constexpr size_t g_lock = g_ntop + 256;
+  static constexpr size_t shared = g_lock + 256;
   static constexpr size_t x_seq = shared + 256;
   static constexpr size_t x_S = x_seq + 256;
   static constexpr size_t x_r = x_S + 256;
@@ -195,6 +196,7 @@ extern "C" int tkc_distance_sums_noalloc(const uint32_t *offsets, const uint32_t
   p.gid = nullptr;
   p.g_directed = nullptr;
   p.g_ntop = (unsigned *)(base + L::g_ntop);
+  p.g_lock = (int *)(base + L::g_lock);
   p.g_ctr = nullptr;
   p.kk = 1;
   p.B = kSlots;

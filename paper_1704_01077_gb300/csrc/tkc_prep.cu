@@ -702,6 +702,29 @@ __global__ void k_bu_keys(const u32 *ioff, u32 n, u32 heavy_in, u32 *key, u32 *v
   if ((threadIdx.x & 31) == 0 && heavy) atomicAdd(&count[1], heavy);
 }
 
+// The same for a union, graph by graph (keys (graph, class)); g_cnt receives
+// each graph's vertices with an in-arc and with a long row.
+__global__ void k_bu_keys_many(const u32 *ioff, u32 n, u32 heavy_in, const u32 *gid, u32 *key, u32 *val, u32 *g_cnt) {
+  const int lane = threadIdx.x & 31;
+  for (u32 base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; base < n; base += gridDim.x * blockDim.x) {
+    const u32 v = base + lane;
+    u32 indeg = 0, g = 0xffffffffu;
+    if (v < n) {
+      g = gid[v];
+      indeg = ioff[v + 1] - ioff[v];
+      key[v] = 64 * g + (indeg > heavy_in ? (u32)__clz(indeg) : indeg ? 32u : 33u);
+      val[v] = v;
+    }
+    // the warp's lanes of one graph add up first
+    const unsigned peers = __match_any_sync(FULL, g);
+    const unsigned any = __ballot_sync(FULL, indeg != 0) & peers, heavy = __ballot_sync(FULL, indeg > heavy_in) & peers;
+    if (v < n && __ffs(peers) - 1 == lane) {
+      if (any) atomicAdd(&g_cnt[2 * (size_t)g], (u32)__popc(any));
+      if (heavy) atomicAdd(&g_cnt[2 * (size_t)g + 1], (u32)__popc(heavy));
+    }
+  }
+}
+
 // The vertices that bottom-up levels sweep, for the in-arc CSR `ioff`: those
 // with an in-arc (no other vertex can be discovered bottom-up; a source is
 // seeded directly).  First the n_heavy vertices of more than heavy_in in-arcs,
@@ -710,14 +733,25 @@ __global__ void k_bu_keys(const u32 *ioff, u32 n, u32 heavy_in, u32 *key, u32 *v
 // share a few frontier-bitmap words.  Only the order of work depends on it,
 // not any result.  *list is allocated here; cnt (device, 2 words) receives
 // the number of vertices with an in-arc and of long rows.
-static int build_bu_list(const u32 *ioff, u32 n, u32 heavy_in, cudaStream_t st, u32 **list, u32 *cnt) {
+// A union (gid, ng graphs): the list graph by graph, every graph's vertices
+// from its first id's position on; g_cnt (device, 2 words per graph) receives
+// the counts instead.
+static int build_bu_list(const u32 *ioff, u32 n, u32 heavy_in, cudaStream_t st, u32 **list, u32 *cnt,
+                         const u32 *gid = nullptr, u32 ng = 0, u32 *g_cnt = nullptr) {
   u32 *keys = nullptr, *ids = nullptr;
   TKC_TRY(cudaMallocAsync(&ids, (size_t)n * sizeof(u32), st));
   TKC_TRY(cudaMallocAsync(&keys, (size_t)n * sizeof(u32), st));
   TKC_TRY(cudaMemsetAsync(cnt, 0, 2 * sizeof(u32), st));
-  TKC_LAUNCH(k_bu_keys<<<grid_for(n, 256), 256, 0, st>>>(ioff, n, heavy_in, keys, ids, cnt));
+  int bits = 6;
+  if (gid) {
+    TKC_TRY(cudaMemsetAsync(g_cnt, 0, 2 * (size_t)ng * sizeof(u32), st));
+    TKC_LAUNCH(k_bu_keys_many<<<grid_for(n, 256), 256, 0, st>>>(ioff, n, heavy_in, gid, keys, ids, g_cnt));
+    while ((ng - 1) >> (bits - 6)) ++bits;
+  } else {
+    TKC_LAUNCH(k_bu_keys<<<grid_for(n, 256), 256, 0, st>>>(ioff, n, heavy_in, keys, ids, cnt));
+  }
   TKC_TRY(cudaGetLastError());
-  TKC_RC(radix_sort_pairs(keys, ids, n, 6, st));
+  TKC_RC(radix_sort_pairs(keys, ids, n, bits, st));
   TKC_TRY(cudaFreeAsync(keys, st));
   *list = ids;
   return TKC_OK;
@@ -765,9 +799,10 @@ void free_search_csr(const tkc_graph *g) {
   }
   if (g->s_ioff && g->s_ioff != g->s_off) cudaFreeAsync(g->s_ioff, st);
   if (g->s_icol && g->s_icol != g->s_col) cudaFreeAsync(g->s_icol, st);
-  void *ptrs[] = {g->s_off, g->s_col, g->s_lab, g->s_unlab, g->bu_list, g->s_cnt};
+  void *ptrs[] = {g->s_off, g->s_col, g->s_lab, g->s_unlab, g->bu_list, g->s_cnt, g->g_bu};
   for (void *q : ptrs)
     if (q) cudaFreeAsync(q, st);
+  g->g_bu = nullptr;
   g->s_off = g->s_col = g->s_ioff = g->s_icol = g->s_lab = g->s_unlab = g->s_cnt = nullptr;
   g->bu_list = nullptr;
   g->n_bu = g->n_bu_heavy = 0;
@@ -856,7 +891,7 @@ static int finish_started_copy(const tkc_graph *g) {
   return read_bu_counts(g);
 }
 
-int ensure_search_csr(const tkc_graph *g, bool relabel) {
+int ensure_search_csr(const tkc_graph *g, bool relabel, const u32 *gid, u32 ng) {
   TKC_RC(finish_started_copy(g));
   const int want = relabel ? 1 : 0;
   if (g->s_mode == want || g->n == 0) return TKC_OK;
@@ -866,7 +901,10 @@ int ensure_search_csr(const tkc_graph *g, bool relabel) {
   if (!relabel) {
     g->heavy_in = kHeavyIn;
     TKC_TRY(cudaMallocAsync(&g->s_cnt, 2 * sizeof(u32), st));
-    TKC_RC(build_bu_list(g->ioff, g->n, g->heavy_in, st, &g->bu_list, g->s_cnt));
+    // (a graph number takes 26 bits of a key beside the class's 6)
+    const bool many = gid && ng > 1 && ng <= (1u << 26);
+    if (many) TKC_TRY(cudaMallocAsync(&g->g_bu, 2 * (size_t)ng * sizeof(u32), st));
+    TKC_RC(build_bu_list(g->ioff, g->n, g->heavy_in, st, &g->bu_list, g->s_cnt, many ? gid : nullptr, ng, g->g_bu));
   } else {
     TKC_RC(build_labelled_copy(g, st));
   }
