@@ -18,6 +18,50 @@
 static thread_local char g_last_err[512] = {0};
 static std::atomic<unsigned long long> g_launches{0};
 
+static thread_local tkc_ctx *t_ctx = nullptr;  // the context this thread entered last
+
+int tkc::enter(tkc_ctx *ctx) {
+  TKC_TRY(cudaSetDevice(ctx->device));
+  t_ctx = ctx;
+  return TKC_OK;
+}
+
+cudaError_t tkc::dev_malloc_bytes(void **p, size_t bytes, cudaStream_t st) {
+  tkc_ctx *ctx = t_ctx;
+  if (!ctx->pool) {
+    cudaMemPoolProps props;
+    memset(&props, 0, sizeof(props));
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = ctx->device;
+    cudaError_t e = cudaMemPoolCreate(&ctx->pool, &props);
+    if (e != cudaSuccess) {
+      ctx->pool = nullptr;
+      return e;
+    }
+    uint64_t keep = ctx->total_mem / kPoolKeepShare;
+    cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  }
+  return cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
+}
+
+cudaError_t tkc::read_back(void *dst, const void *src, size_t bytes, cudaStream_t st) {
+  tkc_ctx *ctx = t_ctx;
+  if (bytes > ctx->stage_bytes && bytes <= kStageMost) {
+    if (ctx->stage) cudaFreeHost(ctx->stage);
+    ctx->stage = nullptr;
+    ctx->stage_bytes = 0;
+    const size_t want = std::max<size_t>(bytes, 16384);
+    if (cudaMallocHost(&ctx->stage, want) == cudaSuccess) ctx->stage_bytes = want;
+    else cudaGetLastError();  // no page-locked memory left: straight into the caller's
+  }
+  const bool staged = bytes <= ctx->stage_bytes;
+  cudaError_t e = cudaMemcpyAsync(staged ? ctx->stage : dst, src, bytes, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e == cudaSuccess && staged) memcpy(dst, ctx->stage, bytes);
+  return e;
+}
+
 void tkc::note_launches(unsigned count) { g_launches.fetch_add(count, std::memory_order_relaxed); }
 
 void tkc_set_last_cuda_error(cudaError_t e, const char *what, const char *file, int line) {
@@ -37,7 +81,7 @@ static int dalloc(T **p, size_t count, cudaStream_t st) {
     TKC_TRY(cudaFreeAsync(*p, st));
     *p = nullptr;
   }
-  TKC_TRY(cudaMallocAsync((void **)p, std::max<size_t>(count, 1) * sizeof(T), st));
+  TKC_TRY(dev_malloc(p, std::max<size_t>(count, 1) * sizeof(T), st));
   return TKC_OK;
 }
 
@@ -62,11 +106,6 @@ int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u3
     TKC_RC(dalloc(&w.top_S, cap, st));
     TKC_RC(dalloc(&w.top_r, cap, st));
     TKC_RC(dalloc(&w.top_id, cap, st));
-    TKC_RC(dalloc(&w.out_S, cap, st));
-    TKC_RC(dalloc(&w.out_r, cap, st));
-    TKC_RC(dalloc(&w.out_id, cap, st));
-    TKC_RC(dalloc(&w.out_f, cap, st));
-    TKC_RC(dalloc(&w.out_c, cap, st));
     w.top_cap = cap;
   }
   if (ng > w.ng_cap) {
@@ -145,8 +184,7 @@ static int ensure_filter(tkc_ctx *ctx, u32 count, u32 nopen) {
 static void free_workspace(tkc_ctx *ctx) {
   Workspace &w = ctx->ws;
   void *ptrs[] = {w.seen, w.F0, w.F1, w.N, w.FB0, w.FB1, w.L0, w.L1, w.Loff0, w.Loff1, w.VL, w.stamp, w.res_S, w.res_r,
-                  w.slots, w.cnt, w.wsum, w.top_S, w.top_r, w.top_id, w.ctl, w.out_S, w.out_r, w.out_id,
-                  w.out_f, w.out_c, w.tied, w.g_ntop, w.g_lock, w.g_stop, w.g_ctr, w.sh, w.x_seq, w.x_S, w.x_r, w.x_id,
+                  w.slots, w.cnt, w.wsum, w.top_S, w.top_r, w.top_id, w.ctl, w.out, w.tied, w.g_ntop, w.g_lock, w.g_stop, w.g_ctr, w.sh, w.x_seq, w.x_S, w.x_r, w.x_id,
                   w.f_order, w.f_keep, w.f_count, w.f_end, w.lvl2,
                   w.o_order, w.o_key, w.o_taken};
   for (void *p : ptrs)
@@ -208,15 +246,39 @@ __global__ void k_count_ties(const u64 *res_S, const u32 *res_r, const u32 *gid,
   }
 }
 
+// A run's results in one block of memory, so that one copy brings them to the
+// host: lists of m = ng * kk entries, then per-graph words.
+struct OutPack {
+  u32 m, ng;
+  __host__ __device__ size_t S() const { return 0; }
+  __host__ __device__ size_t f() const { return 8 * (size_t)m; }
+  __host__ __device__ size_t c() const { return 16 * (size_t)m; }
+  __host__ __device__ size_t ctr() const { return 24 * (size_t)m; }
+  __host__ __device__ size_t r() const { return ctr() + 32 * (size_t)ng; }
+  __host__ __device__ size_t id() const { return r() + 4 * (size_t)m; }
+  __host__ __device__ size_t tied() const { return id() + 4 * (size_t)m; }
+  __host__ __device__ size_t ntop() const { return tied() + 4 * (size_t)ng; }
+  __host__ __device__ size_t bytes() const { return ntop() + 4 * (size_t)ng; }
+};
+
 // Final list of graph blockIdx.x: its top entries, then (if fewer than k of
 // its vertices reach another vertex) closeness-0 vertices in id order.  f and
 // c are one IEEE product and one quotient of exact integers.  Harmonic runs:
 // c = h (the list key's FP64 value), f = 1/h, S not kept (0).
 __global__ void k_output(const u64 *top_S, const u32 *top_r, const u32 *top_id, const unsigned *g_ntop, u32 kk,
-                         const GraphOut *go, int harmonic, u64 *oS, u32 *or_, u32 *oid, double *of, double *oc) {
+                         const GraphOut *go, int harmonic, const unsigned *tied, const u64 *g_ctr, OutPack pk,
+                         unsigned char *out) {
+  u64 *oS = (u64 *)(out + pk.S()), *octr = (u64 *)(out + pk.ctr());
+  double *of = (double *)(out + pk.f()), *oc = (double *)(out + pk.c());
+  u32 *or_ = (u32 *)(out + pk.r()), *oid = (u32 *)(out + pk.id());
   const u32 g = blockIdx.x;
   const GraphOut G = go[g];
   const u32 ntop = g_ntop[g];
+  if (threadIdx.x < 4) octr[4 * (size_t)g + threadIdx.x] = g_ctr[4 * (size_t)g + threadIdx.x];
+  if (threadIdx.x == 0) {
+    ((u32 *)(out + pk.tied()))[g] = tied[g];
+    ((u32 *)(out + pk.ntop()))[g] = ntop;
+  }
   for (u32 i = threadIdx.x; i < G.kk; i += blockDim.x) {
     size_t src = (size_t)g * kk + i;
     u64 S;
@@ -478,7 +540,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   const char *trace_path = getenv("TKC_TRACE");
   const uint32_t trace_cap = 1u << 20;
   if (trace_path) {
-    TKC_TRY(cudaMallocAsync(&p.trace, (size_t)trace_cap * 16 * sizeof(u64), st));
+    TKC_TRY(dev_malloc(&p.trace, (size_t)trace_cap * 16 * sizeof(u64), st));
     TKC_TRY(cudaMemsetAsync(p.trace, 0, (size_t)trace_cap * 16 * sizeof(u64), st));
     p.trace_cap = trace_cap;
   }
@@ -508,8 +570,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     p.nocut_prefix = rs.nocut_prefix > nopen ? rs.nocut_prefix - nopen : 0;
     p.lvl2 = w.lvl2;
     if (by_size && g->s_mode != 1) {
-      TKC_TRY(cudaMemcpyAsync(&hsh, w.sh, sizeof(Shared), cudaMemcpyDeviceToHost, st));
-      TKC_TRY(cudaStreamSynchronize(st));
+      TKC_TRY(read_back(&hsh, w.sh, sizeof(Shared), st));
       if (hsh.norder >= kLabelBatches * rs.B) {
         TKC_RC(ensure_search_csr(g, true));
         walk_search_csr();
@@ -523,9 +584,8 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   }
   TKC_RC(launch_phase(T, w.ctl + open_teams));
   TKC_TRY(cudaEventRecord(ctx->ev[5], st));
-  TKC_TRY(cudaMemcpyAsync(cs.data(), w.ctl, cs.size() * sizeof(Ctl), cudaMemcpyDeviceToHost, st));
-  TKC_TRY(cudaMemcpyAsync(&hsh, w.sh, sizeof(Shared), cudaMemcpyDeviceToHost, st));
-  TKC_TRY(cudaStreamSynchronize(st));
+  TKC_TRY(read_back(cs.data(), w.ctl, cs.size() * sizeof(Ctl), st));
+  TKC_TRY(read_back(&hsh, w.sh, sizeof(Shared), st));
   // the teams' counters add up; levels and batches too (they ran side by side)
   for (const Ctl &x : cs) {
     hctl->edges_visited += x.edges_visited;
@@ -624,38 +684,40 @@ static int finish_run(tkc_ctx *ctx, const RunSetup &rs, const std::vector<GraphO
   cudaStream_t st = ctx->stream;
   const u32 ng = rs.ng;
   GraphOut *go = nullptr;
-  TKC_TRY(cudaMallocAsync(&go, ng * sizeof(GraphOut), st));
+  TKC_TRY(dev_malloc(&go, ng * sizeof(GraphOut), st));
   TKC_TRY(cudaMemcpyAsync(go, go_h.data(), ng * sizeof(GraphOut), cudaMemcpyHostToDevice, st));
   TKC_TRY(cudaMemsetAsync(w.tied, 0, ng * sizeof(unsigned), st));
   unsigned blocks = (unsigned)std::max<u64>(1, std::min<u64>((rs.g->n + 255) / 256, (u64)ctx->num_sms * 8));
   TKC_LAUNCH(k_count_ties<<<blocks, 256, 0, st>>>(w.res_S, w.res_r, rs.gid, rs.g->n, w.top_S, w.top_r, w.g_ntop,
                                                   rs.kk, go, rs.harmonic, w.tied));
-  TKC_LAUNCH(k_output<<<ng, 256, 0, st>>>(w.top_S, w.top_r, w.top_id, w.g_ntop, rs.kk, go, rs.harmonic, w.out_S,
-                                          w.out_r, w.out_id, w.out_f, w.out_c));
+  const OutPack pk{rs.kk * ng, ng};
+  if (pk.bytes() > w.out_cap) {
+    w.out_cap = 0;
+    TKC_RC(dalloc(&w.out, std::max<size_t>(pk.bytes(), 65536), st));
+    w.out_cap = std::max<size_t>(pk.bytes(), 65536);
+  }
+  TKC_LAUNCH(k_output<<<ng, 256, 0, st>>>(w.top_S, w.top_r, w.top_id, w.g_ntop, rs.kk, go, rs.harmonic, w.tied,
+                                          w.g_ctr, pk, w.out));
   TKC_TRY(cudaGetLastError());
-  ntop.resize(ng);
-  tied.resize(ng);
-  gctr.resize(4 * (size_t)ng);
-  TKC_TRY(cudaMemcpyAsync(ntop.data(), w.g_ntop, ng * sizeof(unsigned), cudaMemcpyDeviceToHost, st));
-  TKC_TRY(cudaMemcpyAsync(tied.data(), w.tied, ng * sizeof(unsigned), cudaMemcpyDeviceToHost, st));
-  if (ng > 1)
-    TKC_TRY(cudaMemcpyAsync(gctr.data(), w.g_ctr, 4 * (size_t)ng * sizeof(u64), cudaMemcpyDeviceToHost, st));
+  TKC_TRY(cudaFreeAsync(go, st));
+  std::vector<unsigned char> h(pk.bytes());
+  TKC_TRY(read_back(h.data(), w.out, pk.bytes(), st));
+  const u32 *h_tied = (const u32 *)(h.data() + pk.tied()), *h_ntop = (const u32 *)(h.data() + pk.ntop());
+  const u64 *h_ctr = (const u64 *)(h.data() + pk.ctr());
+  ntop.assign(h_ntop, h_ntop + ng);
+  tied.assign(h_tied, h_tied + ng);
+  gctr.assign(h_ctr, h_ctr + 4 * (size_t)ng);
   for (u32 i = 0; i < ng; ++i) {
     tkc_result *out = &outs[i];
     const u32 kg = go_h[i].kk;
     const size_t src = (size_t)i * rs.kk;
     if (!kg) continue;
-    if (out->ids) TKC_TRY(cudaMemcpyAsync(out->ids, w.out_id + src, kg * sizeof(u32), cudaMemcpyDeviceToHost, st));
-    if (out->dist_sum)
-      TKC_TRY(cudaMemcpyAsync(out->dist_sum, w.out_S + src, kg * sizeof(u64), cudaMemcpyDeviceToHost, st));
-    if (out->reach) TKC_TRY(cudaMemcpyAsync(out->reach, w.out_r + src, kg * sizeof(u32), cudaMemcpyDeviceToHost, st));
-    if (out->farness)
-      TKC_TRY(cudaMemcpyAsync(out->farness, w.out_f + src, kg * sizeof(double), cudaMemcpyDeviceToHost, st));
-    if (out->closeness)
-      TKC_TRY(cudaMemcpyAsync(out->closeness, w.out_c + src, kg * sizeof(double), cudaMemcpyDeviceToHost, st));
+    if (out->ids) memcpy(out->ids, h.data() + pk.id() + 4 * src, kg * sizeof(u32));
+    if (out->dist_sum) memcpy(out->dist_sum, h.data() + pk.S() + 8 * src, kg * sizeof(u64));
+    if (out->reach) memcpy(out->reach, h.data() + pk.r() + 4 * src, kg * sizeof(u32));
+    if (out->farness) memcpy(out->farness, h.data() + pk.f() + 8 * src, kg * sizeof(double));
+    if (out->closeness) memcpy(out->closeness, h.data() + pk.c() + 8 * src, kg * sizeof(double));
   }
-  TKC_TRY(cudaFreeAsync(go, st));
-  TKC_TRY(cudaStreamSynchronize(st));
   for (u32 i = 0; i < ng; ++i)
     if (ntop[i] < go_h[i].kk) tied[i] = go_h[i].nzero;  // the k-th is a closeness-0 vertex
   return TKC_OK;
@@ -839,6 +901,8 @@ void tkc_destroy(tkc_ctx *ctx) {
     cudaStreamDestroy(ctx->aux);
   }
   if (ctx->aux_in) cudaEventDestroy(ctx->aux_in);
+  if (ctx->stage) cudaFreeHost(ctx->stage);
+  if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
   delete ctx;
 }
 
@@ -865,8 +929,8 @@ static int upload_graph(tkc_ctx *ctx, uint32_t n, uint64_t arcs, const uint32_t 
   g->directed = directed ? 1 : 0;
   ctx->graphs_alive++;
   cudaMemcpyKind kind = ptr_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  cudaError_t e = cudaMallocAsync(&g->off, ((size_t)n + 1) * sizeof(u32), st);
-  if (e == cudaSuccess) e = cudaMallocAsync(&g->col, std::max<size_t>(arcs, 1) * sizeof(u32), st);
+  cudaError_t e = dev_malloc(&g->off, ((size_t)n + 1) * sizeof(u32), st);
+  if (e == cudaSuccess) e = dev_malloc(&g->col, std::max<size_t>(arcs, 1) * sizeof(u32), st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(g->off, offsets, ((size_t)n + 1) * sizeof(u32), kind, st);
   if (e == cudaSuccess && arcs) e = cudaMemcpyAsync(g->col, cols, arcs * sizeof(u32), kind, st);
   if (e != cudaSuccess) {
@@ -882,7 +946,7 @@ int tkc_load_csr(tkc_ctx *ctx, uint32_t n, uint64_t arcs, const uint32_t *offset
                  int directed, int ptr_on_device, tkc_graph **out) {
   if (!ctx || !out) return TKC_EINVAL;
   *out = nullptr;
-  TKC_TRY(cudaSetDevice(ctx->device));
+  TKC_RC(enter(ctx));
   tkc_graph *g = nullptr;
   TKC_RC(upload_graph(ctx, n, arcs, offsets, cols, directed, ptr_on_device, &g));
   int rc = validate_graph(g);
@@ -907,7 +971,7 @@ int tkc_load_csr_many(tkc_ctx *ctx, uint32_t ng, const uint32_t *n, const uint64
   if (!ctx || (ng && (!n || !arcs || !offsets || !cols || !directed || !out))) return TKC_EINVAL;
   if (first_bad) *first_bad = ng;
   if (ng == 0) return TKC_OK;
-  TKC_TRY(cudaSetDevice(ctx->device));
+  TKC_RC(enter(ctx));
   cudaStream_t st = ctx->stream;
   for (u32 i = 0; i < ng; ++i) out[i] = nullptr;
   auto fail = [&](int rc, u32 bad) {
@@ -926,7 +990,7 @@ int tkc_load_csr_many(tkc_ctx *ctx, uint32_t ng, const uint32_t *n, const uint64
   // checks of the undirected ones follow (they need checked rows)
   u32 *flags = nullptr;
   std::vector<u32> hf(ng, 0);
-  cudaError_t e = cudaMallocAsync(&flags, (size_t)ng * sizeof(u32), st);
+  cudaError_t e = dev_malloc(&flags, (size_t)ng * sizeof(u32), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, (size_t)ng * sizeof(u32), st);
   if (e != cudaSuccess) {
     tkc_set_last_cuda_error(e, "tkc_load_csr_many", __FILE__, __LINE__);
@@ -968,7 +1032,7 @@ int tkc_load_csr_many(tkc_ctx *ctx, uint32_t ng, const uint32_t *n, const uint64
 void tkc_free_graph(tkc_graph *g) {
   if (!g) return;
   if (g->ctx->last_shard == g) g->ctx->last_shard = nullptr;
-  cudaSetDevice(g->ctx->device);
+  enter(g->ctx);
   // every buffer came from the stream-ordered allocator on the context's
   // stream: freed in stream order, after the work that used it, without
   // waiting for it here
@@ -987,7 +1051,7 @@ void tkc_free_graph(tkc_graph *g) {
 
 int tkc_source_order(tkc_graph *g, uint32_t *order) {
   if (!g || (!order && g->n)) return TKC_EINVAL;
-  TKC_TRY(cudaSetDevice(g->ctx->device));
+  TKC_RC(enter(g->ctx));
   TKC_RC(ensure_degree_order(g));
   if (g->n) TKC_TRY(cudaMemcpyAsync(order, g->deg_order, g->n * sizeof(u32), cudaMemcpyDeviceToHost, g->ctx->stream));
   TKC_TRY(cudaStreamSynchronize(g->ctx->stream));
@@ -1001,12 +1065,12 @@ int tkc_set_source_order(tkc_graph *g, const uint32_t *order) {
     if (order[i] >= g->n || seen[order[i]]) return TKC_EINVAL;
     seen[order[i]] = 1;
   }
-  TKC_TRY(cudaSetDevice(g->ctx->device));
+  TKC_RC(enter(g->ctx));
   cudaStream_t st = g->ctx->stream;
   if (g->n == 0) return TKC_OK;
   u32 *tmp = nullptr;
-  if (!g->given_order) TKC_TRY(cudaMallocAsync(&g->given_order, (size_t)g->n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&tmp, (size_t)g->n * sizeof(u32), st));
+  if (!g->given_order) TKC_TRY(dev_malloc(&g->given_order, (size_t)g->n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&tmp, (size_t)g->n * sizeof(u32), st));
   TKC_TRY(cudaMemcpyAsync(tmp, order, g->n * sizeof(u32), cudaMemcpyHostToDevice, st));
   TKC_RC(filter_order(g, tmp, g->given_order, &g->n_src_given));
   TKC_TRY(cudaFreeAsync(tmp, st));
@@ -1016,7 +1080,7 @@ int tkc_set_source_order(tkc_graph *g, const uint32_t *order) {
 
 int tkc_reach_bounds(tkc_graph *g, uint32_t *alpha, uint32_t *omega) {
   if (!g || ((!alpha || !omega) && g->n)) return TKC_EINVAL;
-  TKC_TRY(cudaSetDevice(g->ctx->device));
+  TKC_RC(enter(g->ctx));
   TKC_RC(ensure_reach_bounds(g));
   cudaStream_t st = g->ctx->stream;
   if (g->n) {
@@ -1162,7 +1226,7 @@ static int topk_one(tkc_graph *g, uint32_t k, tkc_result *out, int harmonic) {
   tkc_ctx *ctx = g->ctx;
   u32 kk = std::min<u32>(k, g->n);
   if (kk > 0 && out->capacity < kk) return TKC_EINVAL;
-  TKC_TRY(cudaSetDevice(ctx->device));
+  TKC_RC(enter(ctx));
   tkc_result r = *out;
   reset_result(&r, kk);
   if (kk == 0) {
@@ -1283,7 +1347,7 @@ static int topk_shard(tkc_graph *g, uint32_t k, uint32_t first, uint32_t shard, 
     if (i && !entry_before(seed_S[i - 1], seed_r[i - 1], seed_id[i - 1], seed_S[i], seed_r[i], seed_id[i]))
       return TKC_EINVAL;  // best first, no repeats
   }
-  TKC_TRY(cudaSetDevice(ctx->device));
+  TKC_RC(enter(ctx));
   tkc_result r = *out;
   reset_result(&r, kk);
   if (kk == 0) {
@@ -1303,7 +1367,7 @@ static int topk_shard(tkc_graph *g, uint32_t k, uint32_t first, uint32_t shard, 
   u32 count = nfull > start ? (u32)((nfull - start + nshards - 1) / nshards) : 0;
   if (limit && count > limit) count = limit;
   u32 *sorder = nullptr;
-  TKC_TRY(cudaMallocAsync(&sorder, std::max<size_t>(count, 1) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&sorder, std::max<size_t>(count, 1) * sizeof(u32), st));
   if (count)
     TKC_LAUNCH(k_shard_order<<<(count + 255) / 256 < 4096 ? (count + 255) / 256 : 4096, 256, 0, st>>>(
         full, (u32)start, nshards, count, sorder));
@@ -1362,7 +1426,7 @@ int tkc_autotune(tkc_graph *g, uint32_t k, tkc_options *best) {
   if (!g || !best) return TKC_EINVAL;
   if (k > TKC_MAX_K) return TKC_EINVAL;
   tkc_ctx *ctx = g->ctx;
-  TKC_TRY(cudaSetDevice(ctx->device));
+  TKC_RC(enter(ctx));
   *best = ctx->opt;
   u32 kk = std::min<u32>(k, g->n);
   if (kk == 0) return TKC_OK;
@@ -1375,7 +1439,7 @@ int tkc_autotune(tkc_graph *g, uint32_t k, tkc_options *best) {
   const u32 stride = std::max<u32>(1, (ns - head) / std::max<u32>(1, want - head));
   const u32 count = head + (ns > head ? (ns - head + stride - 1) / stride : 0);
   u32 *order = nullptr;
-  TKC_TRY(cudaMallocAsync(&order, std::max<u32>(count, 1) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&order, std::max<u32>(count, 1) * sizeof(u32), st));
   TKC_LAUNCH(k_sample_order<<<(count + 255) / 256 > 0 ? std::min<u32>((count + 255) / 256, 4096) : 1, 256, 0, st>>>(
       g->deg_order, ns, head, stride, count, order));
   TKC_TRY(cudaGetLastError());
@@ -1435,7 +1499,7 @@ int tkc_distance_sums(tkc_graph *g, uint32_t nsrc, const uint32_t *srcs, uint64_
   if (!g || (nsrc && (!srcs || !S || !r))) return TKC_EINVAL;
   if (nsrc == 0) return TKC_OK;
   tkc_ctx *ctx = g->ctx;
-  TKC_TRY(cudaSetDevice(ctx->device));
+  TKC_RC(enter(ctx));
   for (u32 i = 0; i < nsrc; ++i)
     if (srcs[i] >= g->n) return TKC_EINVAL;
   std::vector<u32> uniq(srcs, srcs + nsrc);
@@ -1445,7 +1509,7 @@ int tkc_distance_sums(tkc_graph *g, uint32_t nsrc, const uint32_t *srcs, uint64_
   TKC_RC(ensure_reach_bounds(g));
   cudaStream_t st = ctx->stream;
   u32 *dsrc = nullptr;
-  TKC_TRY(cudaMallocAsync(&dsrc, uniq.size() * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&dsrc, uniq.size() * sizeof(u32), st));
   TKC_TRY(cudaMemcpyAsync(dsrc, uniq.data(), uniq.size() * sizeof(u32), cudaMemcpyHostToDevice, st));
   RunSetup rs;
   memset(&rs, 0, sizeof(rs));
@@ -1495,7 +1559,7 @@ static int topk_bound(tkc_graph *g, uint32_t k, tkc_result *out) {
   if (o.order != TKC_ORDER_DEG && o.order != TKC_ORDER_NB) return TKC_EINVAL;
   u32 kk = std::min<u32>(k, g->n);
   if (kk > 0 && out->capacity < kk) return TKC_EINVAL;
-  TKC_TRY(cudaSetDevice(ctx->device));
+  TKC_RC(enter(ctx));
   tkc_result r = *out;
   reset_result(&r, kk);
   if (kk == 0) {
@@ -1555,21 +1619,21 @@ static int topk_bound(tkc_graph *g, uint32_t k, tkc_result *out) {
     }                   \
   } while (0)
   const size_t n1 = std::max<size_t>(n, 1);
-  LB_TRY(cudaMallocAsync(&bS, n1 * sizeof(u64), st));
-  LB_TRY(cudaMallocAsync(&key, n1 * sizeof(u64), st));
-  LB_TRY(cudaMallocAsync(&bR, n1 * sizeof(u32), st));
-  LB_TRY(cudaMallocAsync(&done, n1, st));
-  LB_TRY(cudaMallocAsync(&cand, n1 * sizeof(u32), st));
-  LB_TRY(cudaMallocAsync(&pos, (n1 + 1) * sizeof(u32), st));
-  LB_TRY(cudaMallocAsync(&tmp, ((n1 + 1) / 4096 + 16) * sizeof(u32), st));
-  LB_TRY(cudaMallocAsync(&lo, n1 * sizeof(u32), st));
-  LB_TRY(cudaMallocAsync(&smax, sizeof(u64), st));
-  LB_TRY(cudaMallocAsync(&hist, (size_t)TB * cap * sizeof(u32), st));
-  LB_TRY(cudaMallocAsync(&Ltab, (size_t)TB * cap * sizeof(u64), st));
-  LB_TRY(cudaMallocAsync(&depth, (size_t)TB * sizeof(u32), st));
-  LB_TRY(cudaMallocAsync(&bkeys, (size_t)TB * sizeof(u64), st));
-  LB_TRY(cudaMallocAsync(&srcs, (size_t)TB * sizeof(u32), st));
-  LB_TRY(cudaMallocAsync(&lvl, n1 * TB * sizeof(uint16_t), st));
+  LB_TRY(dev_malloc(&bS, n1 * sizeof(u64), st));
+  LB_TRY(dev_malloc(&key, n1 * sizeof(u64), st));
+  LB_TRY(dev_malloc(&bR, n1 * sizeof(u32), st));
+  LB_TRY(dev_malloc(&done, n1, st));
+  LB_TRY(dev_malloc(&cand, n1 * sizeof(u32), st));
+  LB_TRY(dev_malloc(&pos, (n1 + 1) * sizeof(u32), st));
+  LB_TRY(dev_malloc(&tmp, ((n1 + 1) / 4096 + 16) * sizeof(u32), st));
+  LB_TRY(dev_malloc(&lo, n1 * sizeof(u32), st));
+  LB_TRY(dev_malloc(&smax, sizeof(u64), st));
+  LB_TRY(dev_malloc(&hist, (size_t)TB * cap * sizeof(u32), st));
+  LB_TRY(dev_malloc(&Ltab, (size_t)TB * cap * sizeof(u64), st));
+  LB_TRY(dev_malloc(&depth, (size_t)TB * sizeof(u32), st));
+  LB_TRY(dev_malloc(&bkeys, (size_t)TB * sizeof(u64), st));
+  LB_TRY(dev_malloc(&srcs, (size_t)TB * sizeof(u32), st));
+  LB_TRY(dev_malloc(&lvl, n1 * TB * sizeof(uint16_t), st));
   LB_TRY(cudaMemsetAsync(lvl, 0xff, n1 * TB * sizeof(uint16_t), st));
   LB_RC(lb_init(g, nb ? g->nb_S : nullptr, nb ? g->nb_r : nullptr, nb ? g->nb_key : nullptr, bS, bR, key, done));
   TKC_TRY(cudaEventRecord(ctx->ev[1], st));
@@ -1689,7 +1753,7 @@ static int topk_many(tkc_ctx *ctx, tkc_graph *const *gs, uint32_t ng, uint32_t k
   if (!ctx || (ng && (!gs || !outs))) return TKC_EINVAL;
   if (k > TKC_MAX_K) return TKC_EINVAL;
   if (ng == 0) return TKC_OK;
-  TKC_TRY(cudaSetDevice(ctx->device));
+  TKC_RC(enter(ctx));
   cudaStream_t st = ctx->stream;
   const tkc_options &o = ctx->opt;
   // the union is searched in degree order, or in NBCut order (each graph stops on its own)
@@ -1741,7 +1805,7 @@ static int topk_many(tkc_ctx *ctx, tkc_graph *const *gs, uint32_t ng, uint32_t k
                     U.nb_order, U.nb_horder, U.cls, U.n_cls, gid, d_vbase, d_abase, d_offptr, d_colptr, d_gdir, zflag, zlist,
                     zat, gorder, gkey, gend};
     for (void *q : ptrs)
-      if (q) cudaFree(q);
+      if (q) cudaFreeAsync(q, st);
   };
 #define MULTI_TRY(expr)                                              \
   do {                                                               \
@@ -1760,14 +1824,14 @@ static int topk_many(tkc_ctx *ctx, tkc_graph *const *gs, uint32_t ng, uint32_t k
       return rc;        \
     }                   \
   } while (0)
-  MULTI_TRY(cudaMallocAsync(&U.off, ((size_t)nv + 1) * sizeof(u32), st));
-  MULTI_TRY(cudaMallocAsync(&U.col, std::max<size_t>(na, 1) * sizeof(u32), st));
-  MULTI_TRY(cudaMallocAsync(&gid, std::max<size_t>(nv, 1) * sizeof(u32), st));
-  MULTI_TRY(cudaMallocAsync(&d_vbase, (ng + 1) * sizeof(u32), st));
-  MULTI_TRY(cudaMallocAsync(&d_abase, (ng + 1) * sizeof(u64), st));
-  MULTI_TRY(cudaMallocAsync(&d_offptr, ng * sizeof(u64), st));
-  MULTI_TRY(cudaMallocAsync(&d_colptr, ng * sizeof(u64), st));
-  MULTI_TRY(cudaMallocAsync(&d_gdir, ng, st));
+  MULTI_TRY(dev_malloc(&U.off, ((size_t)nv + 1) * sizeof(u32), st));
+  MULTI_TRY(dev_malloc(&U.col, std::max<size_t>(na, 1) * sizeof(u32), st));
+  MULTI_TRY(dev_malloc(&gid, std::max<size_t>(nv, 1) * sizeof(u32), st));
+  MULTI_TRY(dev_malloc(&d_vbase, (ng + 1) * sizeof(u32), st));
+  MULTI_TRY(dev_malloc(&d_abase, (ng + 1) * sizeof(u64), st));
+  MULTI_TRY(dev_malloc(&d_offptr, ng * sizeof(u64), st));
+  MULTI_TRY(dev_malloc(&d_colptr, ng * sizeof(u64), st));
+  MULTI_TRY(dev_malloc(&d_gdir, ng, st));
   MULTI_TRY(cudaMemcpyAsync(d_vbase, vbase.data(), (ng + 1) * sizeof(u32), cudaMemcpyHostToDevice, st));
   MULTI_TRY(cudaMemcpyAsync(d_abase, abase.data(), (ng + 1) * sizeof(u64), cudaMemcpyHostToDevice, st));
   MULTI_TRY(cudaMemcpyAsync(d_offptr, offptr.data(), ng * sizeof(u64), cudaMemcpyHostToDevice, st));
@@ -1784,10 +1848,10 @@ static int topk_many(tkc_ctx *ctx, tkc_graph *const *gs, uint32_t ng, uint32_t k
   std::vector<u32> zpos(ng + 1);
   {
     u32 *ztmp = nullptr;
-    MULTI_TRY(cudaMallocAsync(&zflag, ((size_t)nv + 1) * sizeof(u32), st));
-    MULTI_TRY(cudaMallocAsync(&zlist, std::max<size_t>(nv, 1) * sizeof(u32), st));
-    MULTI_TRY(cudaMallocAsync(&zat, ((size_t)ng + 1) * sizeof(u32), st));
-    MULTI_TRY(cudaMallocAsync(&ztmp, (((size_t)nv + 1) / 4096 + 2) * sizeof(u32), st));
+    MULTI_TRY(dev_malloc(&zflag, ((size_t)nv + 1) * sizeof(u32), st));
+    MULTI_TRY(dev_malloc(&zlist, std::max<size_t>(nv, 1) * sizeof(u32), st));
+    MULTI_TRY(dev_malloc(&zat, ((size_t)ng + 1) * sizeof(u32), st));
+    MULTI_TRY(dev_malloc(&ztmp, (((size_t)nv + 1) / 4096 + 2) * sizeof(u32), st));
     TKC_LAUNCH(k_zero_flags<<<gb, 256, 0, st>>>(U.off, nv, zflag));
     MULTI_RC(scan_exclusive_u32(zflag, zflag, (u64)nv + 1, ztmp, st));
     TKC_LAUNCH(k_zero_compact<<<gb, 256, 0, st>>>(U.off, zflag, gid, d_vbase, nv, zlist));
@@ -1841,11 +1905,11 @@ static int topk_many(tkc_ctx *ctx, tkc_graph *const *gs, uint32_t ng, uint32_t k
   // own searches.
   if (rs.norder > 0 && ng > 1) {
     u32 *gbeg = nullptr, *p1 = nullptr;
-    MULTI_TRY(cudaMallocAsync(&gorder, (size_t)rs.norder * sizeof(u32), st));
-    MULTI_TRY(cudaMallocAsync(&gkey, (size_t)rs.norder * sizeof(u32), st));
-    MULTI_TRY(cudaMallocAsync(&gend, (size_t)2 * ng * sizeof(u32), st));
-    MULTI_TRY(cudaMallocAsync(&gbeg, (size_t)ng * sizeof(u32), st));
-    MULTI_TRY(cudaMallocAsync(&p1, sizeof(u32), st));
+    MULTI_TRY(dev_malloc(&gorder, (size_t)rs.norder * sizeof(u32), st));
+    MULTI_TRY(dev_malloc(&gkey, (size_t)rs.norder * sizeof(u32), st));
+    MULTI_TRY(dev_malloc(&gend, (size_t)2 * ng * sizeof(u32), st));
+    MULTI_TRY(dev_malloc(&gbeg, (size_t)ng * sizeof(u32), st));
+    MULTI_TRY(dev_malloc(&p1, sizeof(u32), st));
     MULTI_TRY(cudaMemsetAsync(gend, 0, (size_t)2 * ng * sizeof(u32), st));
     MULTI_TRY(cudaMemcpyAsync(gorder, rs.order, (size_t)rs.norder * sizeof(u32), cudaMemcpyDeviceToDevice, st));
     MULTI_TRY(cudaMemcpyAsync(p1, &rs.norder, sizeof(u32), cudaMemcpyHostToDevice, st));
@@ -1919,10 +1983,10 @@ int tkc_count_tied(tkc_graph *g, uint64_t S, uint32_t r, uint32_t *count) {
   if (!g || !count || r < 2) return TKC_EINVAL;
   if (g->ctx->last_shard != g) return TKC_EINVAL;
   tkc_ctx *ctx = g->ctx;
-  TKC_TRY(cudaSetDevice(ctx->device));
+  TKC_RC(enter(ctx));
   cudaStream_t st = ctx->stream;
   unsigned *d = nullptr;
-  TKC_TRY(cudaMallocAsync(&d, sizeof(unsigned), st));
+  TKC_TRY(dev_malloc(&d, sizeof(unsigned), st));
   TKC_TRY(cudaMemsetAsync(d, 0, sizeof(unsigned), st));
   const u32 n = g->n;
   const unsigned blocks = (unsigned)std::max<u64>(1, std::min<u64>(((u64)n + 255) / 256, (u64)ctx->num_sms * 8));

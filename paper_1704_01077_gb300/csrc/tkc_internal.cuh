@@ -253,9 +253,7 @@ struct Workspace {
   uint32_t *f_end = nullptr;        // per graph: one past its last kept position
   uint32_t *lvl2 = nullptr;         // per vertex: level-2 bounds of the kept sources
   uint32_t f_cap = 0;               // positions f_order holds
-  unsigned long long *out_S = nullptr;
-  uint32_t *out_r = nullptr, *out_id = nullptr;
-  double *out_f = nullptr, *out_c = nullptr;
+  unsigned char *out = nullptr;     // packed results of a run (OutPack)
   unsigned int *tied = nullptr;     // per graph
   unsigned int *g_ntop = nullptr;   // per graph
   int *g_lock = nullptr;            // per graph
@@ -265,12 +263,37 @@ struct Workspace {
   unsigned int *x_seq = nullptr;
   unsigned long long *x_S = nullptr;
   uint32_t *x_r = nullptr, *x_id = nullptr;
-  uint32_t top_cap = 0;   // entries of top_* / out_* (graphs x k)
+  uint32_t top_cap = 0;   // entries of top_* (graphs x k)
+  size_t out_cap = 0;     // bytes of out
   uint32_t ng_cap = 0;    // graphs of tied / g_ntop / g_ctr / x_*
   uint32_t teams_cap = 0; // teams the per-team buffers are sized for
   unsigned int level_base = 0;  // stamp epoch carried across runs
 };
 
+}  // namespace tkc
+
+struct tkc_ctx;
+
+namespace tkc {
+// Every entry point starts with enter(ctx): it selects the context's device
+// and, for this thread, the context's memory pool and host staging buffer.
+int enter(tkc_ctx *ctx);
+// Device memory from the entered context's pool, in stream order.  The pool
+// belongs to the context and keeps at most 1 / kPoolKeepShare of the device's
+// memory that nothing uses (the device's default pool returns free memory to the driver at every
+// synchronisation, so that each call mapped its scratch anew: 2 ms of a
+// 13 ms call on R-MAT 22, 6 ms with 512 graphs); tkc_destroy gives it back.
+cudaError_t dev_malloc_bytes(void **p, size_t bytes, cudaStream_t st);
+template <typename T>
+cudaError_t dev_malloc(T **p, size_t bytes, cudaStream_t st) {
+  return dev_malloc_bytes(reinterpret_cast<void **>(p), bytes, st);
+}
+// Copies device memory to the host after `st`'s work so far and waits for it.
+// Short reads go through the context's page-locked buffer: a copy into
+// pageable memory is staged by the driver and costs about 4 us more.
+cudaError_t read_back(void *dst, const void *src, size_t bytes, cudaStream_t st);
+constexpr size_t kPoolKeepShare = 32;
+constexpr size_t kStageMost = 1u << 20;
 }  // namespace tkc
 
 // Source-order model: 5 -> 64 -> 64 -> 1 MLP, fp32 master weights with a
@@ -303,6 +326,9 @@ struct tkc_ctx {
   tkc_options opt{};
   int num_sms = 0;
   size_t total_mem = 0;  // bytes of device memory
+  cudaMemPool_t pool = nullptr;  // device memory of the context and its graphs
+  void *stage = nullptr;         // page-locked host buffer of short reads (read_back)
+  size_t stage_bytes = 0;
   tkc::Workspace ws;
   cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   cudaStream_t aux = nullptr;    // helper stream: the labelled copy, built while `stream` preprocesses

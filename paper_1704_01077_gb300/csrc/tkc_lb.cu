@@ -214,8 +214,7 @@ int lb_sorted_candidates(tkc_graph *g, const u32 *order0, u32 n0, const uint8_t 
   if (m) {
     TKC_LAUNCH(k_lb_key_lo<<<grid_of(m), 256, 0, st>>>(m, cand, key, scratch_lo, scratch_max));
     u64 mk = 0;
-    TKC_TRY(cudaMemcpyAsync(&mk, scratch_max, sizeof(u64), cudaMemcpyDeviceToHost, st));
-    TKC_TRY(cudaStreamSynchronize(st));
+    TKC_TRY(read_back(&mk, scratch_max, sizeof(u64), st));
     int bits = 0;
     while (bits < 64 && (mk >> bits) != 0) ++bits;
     if (bits <= 32) {

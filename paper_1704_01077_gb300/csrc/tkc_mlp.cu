@@ -428,18 +428,18 @@ int ensure_features(tkc_graph *g) {
   float *w2 = nullptr;
   u32 *c0 = nullptr, *c1 = nullptr;
   double *sums = nullptr;
-  TKC_TRY(cudaMallocAsync(&g->features, (size_t)n * F * sizeof(float), st));
-  TKC_TRY(cudaMallocAsync(&w2, (size_t)n * sizeof(float), st));
-  TKC_TRY(cudaMallocAsync(&c0, (size_t)n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&c1, (size_t)n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&sums, 2 * F * sizeof(double), st));
+  TKC_TRY(dev_malloc(&g->features, (size_t)n * F * sizeof(float), st));
+  TKC_TRY(dev_malloc(&w2, (size_t)n * sizeof(float), st));
+  TKC_TRY(dev_malloc(&c0, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&c1, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&sums, 2 * F * sizeof(double), st));
   TKC_LAUNCH(k_two_walks<<<grid_of((u64)n * 32), 256, 0, st>>>(g->off, g->col, n, w2));
   TKC_LAUNCH(k_core_init<<<grid_of(n), 256, 0, st>>>(g->off, g->ioff, n, g->directed, c0));
   u32 *flag = nullptr;
   uint8_t *d0 = nullptr, *d1 = nullptr;
-  TKC_TRY(cudaMallocAsync(&flag, sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&d0, n, st));
-  TKC_TRY(cudaMallocAsync(&d1, n, st));
+  TKC_TRY(dev_malloc(&flag, sizeof(u32), st));
+  TKC_TRY(dev_malloc(&d0, n, st));
+  TKC_TRY(dev_malloc(&d1, n, st));
   TKC_TRY(cudaMemsetAsync(d0, 1, n, st));  // every vertex is computed in the first step
   for (u64 it = 0;; ++it) {
     // a step that changes something lowers at least one value, and the values
@@ -452,8 +452,7 @@ int ensure_features(tkc_graph *g) {
     std::swap(c0, c1);
     std::swap(d0, d1);
     u32 h = 0;
-    TKC_TRY(cudaMemcpyAsync(&h, flag, sizeof(u32), cudaMemcpyDeviceToHost, st));
-    TKC_TRY(cudaStreamSynchronize(st));
+    TKC_TRY(read_back(&h, flag, sizeof(u32), st));
     if (!h) break;
   }
   TKC_TRY(cudaFreeAsync(flag, st));
@@ -484,7 +483,7 @@ int ensure_learned_order(tkc_graph *g) {
   TKC_RC(ensure_features(g));
   cudaStream_t st = ctx->stream;
   const u32 n = g->n;
-  if (!g->learned_order) TKC_TRY(cudaMallocAsync(&g->learned_order, std::max<size_t>(n, 1) * sizeof(u32), st));
+  if (!g->learned_order) TKC_TRY(dev_malloc(&g->learned_order, std::max<size_t>(n, 1) * sizeof(u32), st));
   if (n == 0) {
     g->n_src_learned = 0;
     g->learned_version = ctx->mlp.version;
@@ -492,9 +491,9 @@ int ensure_learned_order(tkc_graph *g) {
   }
   float *y = nullptr;
   u32 *key = nullptr, *val = nullptr;
-  TKC_TRY(cudaMallocAsync(&y, (size_t)n * sizeof(float), st));
-  TKC_TRY(cudaMallocAsync(&key, (size_t)n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&val, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&y, (size_t)n * sizeof(float), st));
+  TKC_TRY(dev_malloc(&key, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&val, (size_t)n * sizeof(u32), st));
   TKC_RC(forward(ctx, g->features, n, y));
   TKC_LAUNCH(k_score_keys<<<grid_of(n), 256, 0, st>>>(y, n, key, val));
   TKC_RC(radix_sort_u32_pairs(key, val, n, 32, st));  // stable: equal predictions keep id order
@@ -540,12 +539,12 @@ int ensure_seeded_order(tkc_graph *g, u32 prefix, bool nb) {
   cudaStream_t st = ctx->stream;
   const u32 *base = nb ? g->nb_order : g->deg_order;
   const u32 ns = nb ? g->n_src_nb : g->n_src_deg;
-  if (!g->seeded_order) TKC_TRY(cudaMallocAsync(&g->seeded_order, std::max<size_t>(g->n, 1) * sizeof(u32), st));
+  if (!g->seeded_order) TKC_TRY(dev_malloc(&g->seeded_order, std::max<size_t>(g->n, 1) * sizeof(u32), st));
   uint8_t *mark = nullptr;
   u32 *pos = nullptr, *tmp = nullptr;
-  TKC_TRY(cudaMallocAsync(&mark, std::max<size_t>(g->n, 1), st));
-  TKC_TRY(cudaMallocAsync(&pos, ((size_t)ns + 1) * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&tmp, ((size_t)ns + 1) / 4096 * sizeof(u32) + 16, st));
+  TKC_TRY(dev_malloc(&mark, std::max<size_t>(g->n, 1), st));
+  TKC_TRY(dev_malloc(&pos, ((size_t)ns + 1) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&tmp, ((size_t)ns + 1) / 4096 * sizeof(u32) + 16, st));
   TKC_TRY(cudaMemsetAsync(mark, 0, std::max<size_t>(g->n, 1), st));
   if (prefix) {
     TKC_LAUNCH(k_mark_prefix<<<grid_of(prefix), 256, 0, st>>>(g->learned_order, prefix, mark));
@@ -574,7 +573,7 @@ extern "C" {
 
 int tkc_mlp_init(tkc_ctx *ctx, uint64_t seed) {
   if (!ctx) return TKC_EINVAL;
-  TKC_TRY(cudaSetDevice(ctx->device));
+  TKC_RC(enter(ctx));
   TKC_RC(ensure_mlp(ctx));
   TKC_LAUNCH(k_mlp_init<<<grid_of(P), 256, 0, ctx->stream>>>(ctx->mlp.w, seed));
   TKC_LAUNCH(k_to_bf16<<<grid_of(P), 256, 0, ctx->stream>>>(ctx->mlp.w, ctx->mlp.wb));
@@ -585,7 +584,7 @@ int tkc_mlp_init(tkc_ctx *ctx, uint64_t seed) {
 
 int tkc_set_source_model(tkc_ctx *ctx, const float *params, uint32_t nparams) {
   if (!ctx || !params || nparams != (uint32_t)P) return TKC_EINVAL;
-  TKC_TRY(cudaSetDevice(ctx->device));
+  TKC_RC(enter(ctx));
   TKC_RC(ensure_mlp(ctx));
   TKC_TRY(cudaMemcpyAsync(ctx->mlp.w, params, P * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
   TKC_LAUNCH(k_to_bf16<<<grid_of(P), 256, 0, ctx->stream>>>(ctx->mlp.w, ctx->mlp.wb));
@@ -596,7 +595,7 @@ int tkc_set_source_model(tkc_ctx *ctx, const float *params, uint32_t nparams) {
 
 int tkc_get_source_model(tkc_ctx *ctx, float *params, uint32_t nparams) {
   if (!ctx || !params || nparams != (uint32_t)P || !ctx->mlp.ready) return TKC_EINVAL;
-  TKC_TRY(cudaSetDevice(ctx->device));
+  TKC_RC(enter(ctx));
   TKC_TRY(cudaMemcpyAsync(params, ctx->mlp.w, P * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
   TKC_TRY(cudaStreamSynchronize(ctx->stream));
   return TKC_OK;
@@ -604,7 +603,7 @@ int tkc_get_source_model(tkc_ctx *ctx, float *params, uint32_t nparams) {
 
 int tkc_vertex_features(tkc_graph *g, float *x) {
   if (!g || (!x && g->n)) return TKC_EINVAL;
-  TKC_TRY(cudaSetDevice(g->ctx->device));
+  TKC_RC(enter(g->ctx));
   TKC_RC(ensure_features(g));
   if (g->n)
     TKC_TRY(cudaMemcpyAsync(x, g->features, (size_t)g->n * F * sizeof(float), cudaMemcpyDeviceToDevice,
@@ -615,7 +614,7 @@ int tkc_vertex_features(tkc_graph *g, float *x) {
 
 int tkc_mlp_forward(tkc_ctx *ctx, const float *x, uint32_t m, float *y) {
   if (!ctx || (m && (!x || !y)) || !ctx->mlp.ready) return TKC_EINVAL;
-  TKC_TRY(cudaSetDevice(ctx->device));
+  TKC_RC(enter(ctx));
   TKC_RC(forward(ctx, x, m, y));
   TKC_TRY(cudaStreamSynchronize(ctx->stream));
   return TKC_OK;
@@ -636,7 +635,7 @@ static int gradient(tkc_ctx *ctx, const float *x, const float *t, u32 m, float *
 
 int tkc_mlp_gradient(tkc_ctx *ctx, const float *x, const float *t, uint32_t m, float *grad, float *loss) {
   if (!ctx || !x || !t || !grad || m == 0 || !ctx->mlp.ready) return TKC_EINVAL;
-  TKC_TRY(cudaSetDevice(ctx->device));
+  TKC_RC(enter(ctx));
   TKC_RC(gradient(ctx, x, t, m, loss));
   TKC_TRY(cudaMemcpyAsync(grad, ctx->mlp.grad, P * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
   TKC_TRY(cudaStreamSynchronize(ctx->stream));
@@ -645,7 +644,7 @@ int tkc_mlp_gradient(tkc_ctx *ctx, const float *x, const float *t, uint32_t m, f
 
 int tkc_mlp_train_step(tkc_ctx *ctx, const float *x, const float *t, uint32_t m, float lr, float *loss) {
   if (!ctx || !x || !t || m == 0 || !ctx->mlp.ready || !(lr > 0.f)) return TKC_EINVAL;
-  TKC_TRY(cudaSetDevice(ctx->device));
+  TKC_RC(enter(ctx));
   MlpState &s = ctx->mlp;
   TKC_RC(gradient(ctx, x, t, m, loss));
   s.step++;

@@ -315,9 +315,9 @@ int nb_sort_sources(tkc_graph *g, const u64 *key, u32 *order, u32 *count) {
   if (n == 0) return TKC_OK;
   u32 *ids = nullptr, *lo = nullptr;
   u64 *maxkey = nullptr;
-  TKC_TRY(cudaMallocAsync(&ids, (size_t)n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&lo, (size_t)n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&maxkey, sizeof(u64), st));
+  TKC_TRY(dev_malloc(&ids, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&lo, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&maxkey, sizeof(u64), st));
   TKC_TRY(cudaMemsetAsync(maxkey, 0, sizeof(u64), st));
   TKC_LAUNCH(k_iota<<<grid_of(n), 256, 0, st>>>(n, ids));
   TKC_RC(filter_order(g, ids, order, count));  // synchronises
@@ -325,8 +325,7 @@ int nb_sort_sources(tkc_graph *g, const u64 *key, u32 *order, u32 *count) {
   if (ns) {
     TKC_LAUNCH(k_key_parts<<<grid_of(ns), 256, 0, st>>>(ns, order, key, lo, maxkey));
     u64 mk = 0;
-    TKC_TRY(cudaMemcpyAsync(&mk, maxkey, sizeof(u64), cudaMemcpyDeviceToHost, st));
-    TKC_TRY(cudaStreamSynchronize(st));
+    TKC_TRY(read_back(&mk, maxkey, sizeof(u64), st));
     int bits = 0;
     while (bits < 64 && (mk >> bits) != 0) ++bits;
     if (bits <= 32) {
@@ -350,7 +349,7 @@ int ensure_nb_order(tkc_graph *g, bool harmonic) {
   u32 **order = harmonic ? &g->nb_horder : &g->nb_order;
   u32 *cap = harmonic ? &g->nb_horder_cap : &g->nb_order_cap;
   if (*cap == g->nb_cap && *order) return TKC_OK;
-  if (!*order) TKC_TRY(cudaMallocAsync(order, std::max<size_t>(g->n, 1) * sizeof(u32), g->ctx->stream));
+  if (!*order) TKC_TRY(dev_malloc(order, std::max<size_t>(g->n, 1) * sizeof(u32), g->ctx->stream));
   TKC_RC(nb_sort_sources(g, harmonic ? g->nb_hkey : g->nb_key, *order, &g->n_src_nb));
   *cap = g->nb_cap;
   return TKC_OK;
@@ -368,10 +367,10 @@ int ensure_nb_bounds(tkc_graph *g, u32 K, const u32 *gid, const uint8_t *gdir) {
   const u32 n = g->n;
   const size_t n1 = std::max<size_t>(n, 1);
   if (!g->nb_hkey) {
-    TKC_TRY(cudaMallocAsync(&g->nb_S, n1 * sizeof(u64), st));
-    TKC_TRY(cudaMallocAsync(&g->nb_r, n1 * sizeof(u32), st));
-    TKC_TRY(cudaMallocAsync(&g->nb_key, n1 * sizeof(u64), st));
-    TKC_TRY(cudaMallocAsync(&g->nb_hkey, n1 * sizeof(u64), st));
+    TKC_TRY(dev_malloc(&g->nb_S, n1 * sizeof(u64), st));
+    TKC_TRY(dev_malloc(&g->nb_r, n1 * sizeof(u32), st));
+    TKC_TRY(dev_malloc(&g->nb_key, n1 * sizeof(u64), st));
+    TKC_TRY(dev_malloc(&g->nb_hkey, n1 * sizeof(u64), st));
   }
   if (n == 0) {
     g->n_src_nb = 0;
@@ -385,27 +384,26 @@ int ensure_nb_bounds(tkc_graph *g, u32 K, const u32 *gid, const uint8_t *gdir) {
   u32 *segpos = nullptr, *seg_row = nullptr, *seg_begin = nullptr, *tmp = nullptr;
   u32 *left = nullptr;
   int *err = nullptr;
-  for (int i = 0; i < 3; ++i) TKC_TRY(cudaMallocAsync(&N[i], n1 * sizeof(u64), st));
-  TKC_TRY(cudaMallocAsync(&s.c, n1 * sizeof(u64), st));
-  TKC_TRY(cudaMallocAsync(&s.P, n1 * sizeof(u64), st));
-  TKC_TRY(cudaMallocAsync(&s.bS, n1 * sizeof(u64), st));
-  TKC_TRY(cudaMallocAsync(&s.bR, n1 * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&s.flag, n1, st));
-  TKC_TRY(cudaMallocAsync(&s.hU, n1 * sizeof(double), st));
-  TKC_TRY(cudaMallocAsync(&segpos, (n1 + 1) * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&tmp, ((n1 + 1) / 4096 + 16) * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&left, 2 * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&err, sizeof(int), st));
+  for (int i = 0; i < 3; ++i) TKC_TRY(dev_malloc(&N[i], n1 * sizeof(u64), st));
+  TKC_TRY(dev_malloc(&s.c, n1 * sizeof(u64), st));
+  TKC_TRY(dev_malloc(&s.P, n1 * sizeof(u64), st));
+  TKC_TRY(dev_malloc(&s.bS, n1 * sizeof(u64), st));
+  TKC_TRY(dev_malloc(&s.bR, n1 * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&s.flag, n1, st));
+  TKC_TRY(dev_malloc(&s.hU, n1 * sizeof(double), st));
+  TKC_TRY(dev_malloc(&segpos, (n1 + 1) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&tmp, ((n1 + 1) / 4096 + 16) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&left, 2 * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&err, sizeof(int), st));
   TKC_TRY(cudaMemsetAsync(err, 0, sizeof(int), st));
   // heavy-row segments
   TKC_LAUNCH(k_seg_count<<<grid_of(n), 256, 0, st>>>(n, g->off, segpos));
   TKC_RC(scan_exclusive_u32(segpos, segpos, (u64)n + 1, tmp, st));
   u32 nseg = 0;
-  TKC_TRY(cudaMemcpyAsync(&nseg, segpos + n, sizeof(u32), cudaMemcpyDeviceToHost, st));
-  TKC_TRY(cudaStreamSynchronize(st));
+  TKC_TRY(read_back(&nseg, segpos + n, sizeof(u32), st));
   if (nseg) {
-    TKC_TRY(cudaMallocAsync(&seg_row, (size_t)nseg * sizeof(u32), st));
-    TKC_TRY(cudaMallocAsync(&seg_begin, (size_t)nseg * sizeof(u32), st));
+    TKC_TRY(dev_malloc(&seg_row, (size_t)nseg * sizeof(u32), st));
+    TKC_TRY(dev_malloc(&seg_begin, (size_t)nseg * sizeof(u32), st));
     TKC_LAUNCH(k_seg_emit<<<grid_of(n), 256, 0, st>>>(n, g->off, segpos, seg_row, seg_begin));
   }
   // sweeps: N[i % 3] holds N~_i
@@ -424,15 +422,13 @@ int ensure_nb_bounds(tkc_graph *g, u32 K, const u32 *gid, const uint8_t *gdir) {
                                                       prev2, cur, s, left, err));
     TKC_TRY(cudaGetLastError());
     u32 h_left = 0;
-    TKC_TRY(cudaMemcpyAsync(&h_left, left, sizeof(u32), cudaMemcpyDeviceToHost, st));
-    TKC_TRY(cudaStreamSynchronize(st));
+    TKC_TRY(read_back(&h_left, left, sizeof(u32), st));
     levels = k;
     if (h_left == 0) break;
   }
   TKC_LAUNCH(k_nb_keys<<<grid_of(n), 256, 0, st>>>(n, s, g->nb_S, g->nb_r, g->nb_key, g->nb_hkey, err));
   int h_err = 0;
-  TKC_TRY(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, st));
-  TKC_TRY(cudaStreamSynchronize(st));
+  TKC_TRY(read_back(&h_err, err, sizeof(int), st));
   for (int i = 0; i < 3; ++i) TKC_TRY(cudaFreeAsync(N[i], st));
   void *frees[] = {s.c, s.P, s.bS, s.bR, s.flag, s.hU, segpos, seg_row, seg_begin, tmp, left, err};
   for (void *p : frees)
@@ -452,7 +448,7 @@ extern "C" {
 int tkc_nb_bounds(tkc_graph *g, uint32_t max_levels, uint64_t *S_lb, uint32_t *r_lb, uint64_t *key,
                   uint32_t *order, uint32_t *n_order, uint32_t *levels) {
   if (!g || max_levels > 65535) return TKC_EINVAL;
-  TKC_TRY(cudaSetDevice(g->ctx->device));
+  TKC_RC(enter(g->ctx));
   TKC_RC(ensure_nb_bounds(g, max_levels ? max_levels : 256u));
   if (order || n_order) TKC_RC(ensure_nb_order(g, false));
   cudaStream_t st = g->ctx->stream;
@@ -472,23 +468,21 @@ int tkc_nb_bounds(tkc_graph *g, uint32_t max_levels, uint64_t *S_lb, uint32_t *r
 
 int tkc_nb_harmonic_bounds(tkc_graph *g, uint32_t max_levels, double *h_ub, uint32_t *order, uint32_t *n_order) {
   if (!g || max_levels > 65535) return TKC_EINVAL;
-  TKC_TRY(cudaSetDevice(g->ctx->device));
+  TKC_RC(enter(g->ctx));
   TKC_RC(ensure_nb_bounds(g, max_levels ? max_levels : 256u));
   if (order || n_order) TKC_RC(ensure_nb_order(g, true));
   cudaStream_t st = g->ctx->stream;
   const size_t n = g->n;
   if (n && h_ub) {
     std::vector<u64> keys(n);
-    TKC_TRY(cudaMemcpyAsync(keys.data(), g->nb_hkey, n * sizeof(u64), cudaMemcpyDeviceToHost, st));
-    TKC_TRY(cudaStreamSynchronize(st));
+    TKC_TRY(read_back(keys.data(), g->nb_hkey, n * sizeof(u64), st));
     for (size_t i = 0; i < n; ++i) {
       const u64 b = ~keys[i];
       memcpy(&h_ub[i], &b, sizeof(double));
     }
   }
   if (n && order && g->n_src_nb)
-    TKC_TRY(cudaMemcpyAsync(order, g->nb_horder, (size_t)g->n_src_nb * sizeof(u32), cudaMemcpyDeviceToHost, st));
-  TKC_TRY(cudaStreamSynchronize(st));
+    TKC_TRY(read_back(order, g->nb_horder, (size_t)g->n_src_nb * sizeof(u32), st));
   if (n_order) *n_order = g->n_src_nb;
   return TKC_OK;
 }

@@ -275,16 +275,14 @@ int validate_graph(tkc_graph *g) {
   cudaStream_t st = g->ctx->stream;
   if (g->n == 0) return TKC_OK;
   u32 *flags = nullptr;
-  TKC_TRY(cudaMallocAsync(&flags, sizeof(u32), st));
+  TKC_TRY(dev_malloc(&flags, sizeof(u32), st));
   TKC_TRY(cudaMemsetAsync(flags, 0, sizeof(u32), st));
   TKC_RC(enqueue_validate(g, flags));
   u32 hf = 0;
-  TKC_TRY(cudaMemcpyAsync(&hf, flags, sizeof(u32), cudaMemcpyDeviceToHost, st));
-  TKC_TRY(cudaStreamSynchronize(st));
+  TKC_TRY(read_back(&hf, flags, sizeof(u32), st));
   if (hf == 0 && !g->directed) {
     TKC_RC(enqueue_symmetric(g, flags));
-    TKC_TRY(cudaMemcpyAsync(&hf, flags, sizeof(u32), cudaMemcpyDeviceToHost, st));
-    TKC_TRY(cudaStreamSynchronize(st));
+    TKC_TRY(read_back(&hf, flags, sizeof(u32), st));
   }
   TKC_TRY(cudaFreeAsync(flags, st));
   if (hf) return TKC_EGRAPH;
@@ -302,7 +300,7 @@ static int fill_in_arcs(const u32 *off, const u32 *col, u32 n, u64 arcs, const u
                         cudaStream_t st) {
   if (!arcs) return TKC_OK;
   u32 *cursor = nullptr;
-  TKC_TRY(cudaMallocAsync(&cursor, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&cursor, (size_t)n * sizeof(u32), st));
   TKC_TRY(cudaMemcpyAsync(cursor, ioff, (size_t)n * sizeof(u32), cudaMemcpyDeviceToDevice, st));
   TKC_LAUNCH(k_in_fill<<<grid_for(arc_threads(arcs), 256), 256, 0, st>>>(
       off, col, n, arcs, cursor, icol));
@@ -316,9 +314,9 @@ static int fill_in_arcs(const u32 *off, const u32 *col, u32 n, u64 arcs, const u
 static int transpose_csr(const u32 *off, const u32 *col, u32 n, u64 arcs, u32 **ioff, u32 **icol,
                          cudaStream_t st) {
   u32 *tmp = nullptr;
-  TKC_TRY(cudaMallocAsync(ioff, ((size_t)n + 1) * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(icol, std::max<size_t>(arcs, 1) * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&tmp, (((size_t)n + 1) / kScanTile + 2) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(ioff, ((size_t)n + 1) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(icol, std::max<size_t>(arcs, 1) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&tmp, (((size_t)n + 1) / kScanTile + 2) * sizeof(u32), st));
   TKC_TRY(cudaMemsetAsync(*ioff, 0, ((size_t)n + 1) * sizeof(u32), st));
   if (arcs) {
     TKC_LAUNCH(k_in_count<<<grid_for(arcs, 256), 256, 0, st>>>(col, arcs, *ioff));
@@ -484,10 +482,10 @@ static int radix_sort_pairs(u32 *key, u32 *val, u32 n, int bits, cudaStream_t st
   u32 ntiles = (n + kRsTile - 1) / kRsTile;
   u32 *k2 = nullptr, *v2 = nullptr, *hist = nullptr, *tmp = nullptr;
   size_t hlen = (size_t)256 * ntiles;
-  TKC_TRY(cudaMallocAsync(&k2, (size_t)n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&v2, (size_t)n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&hist, hlen * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&tmp, (hlen / kScanTile + 2) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&k2, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&v2, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&hist, hlen * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&tmp, (hlen / kScanTile + 2) * sizeof(u32), st));
   u32 *ka = key, *va = val, *kb = k2, *vb = v2;
   for (int ps = 0; ps < passes; ++ps) {
     TKC_LAUNCH(k_rs_count<<<ntiles, kRsTPB, 0, st>>>(ka, n, 8 * ps, hist, ntiles));
@@ -549,15 +547,14 @@ int ensure_degree_order(tkc_graph *g) {
     return TKC_OK;
   }
   u32 *keys = nullptr, *stats = nullptr;
-  if (!g->deg_order) TKC_TRY(cudaMallocAsync(&g->deg_order, (size_t)n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&keys, (size_t)n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&stats, 2 * sizeof(u32), st));
+  if (!g->deg_order) TKC_TRY(dev_malloc(&g->deg_order, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&keys, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&stats, 2 * sizeof(u32), st));
   TKC_TRY(cudaMemsetAsync(stats, 0, 2 * sizeof(u32), st));
   TKC_LAUNCH(k_maxdeg<<<grid_for(n, 256), 256, 0, st>>>(g->off, n, stats, stats + 1));
   TKC_TRY(cudaGetLastError());
   u32 hs[2];
-  TKC_TRY(cudaMemcpyAsync(hs, stats, sizeof(hs), cudaMemcpyDeviceToHost, st));
-  TKC_TRY(cudaStreamSynchronize(st));
+  TKC_TRY(read_back(hs, stats, sizeof(hs), st));
   TKC_LAUNCH(k_deg_keys<<<grid_for(n, 256), 256, 0, st>>>(g->off, n, hs[0], keys, g->deg_order));
   TKC_TRY(cudaGetLastError());
   int bits = 0;
@@ -594,9 +591,9 @@ int ensure_zero_list(const tkc_graph *g) {
     return TKC_OK;
   }
   u32 *flag = nullptr, *tmp = nullptr;
-  TKC_TRY(cudaMallocAsync(&flag, ((size_t)n + 1) * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&tmp, (((size_t)n + 1) / kScanTile + 2) * sizeof(u32), st));
-  if (!g->zero_ids) TKC_TRY(cudaMallocAsync(&g->zero_ids, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&flag, ((size_t)n + 1) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&tmp, (((size_t)n + 1) / kScanTile + 2) * sizeof(u32), st));
+  if (!g->zero_ids) TKC_TRY(dev_malloc(&g->zero_ids, (size_t)n * sizeof(u32), st));
   TKC_LAUNCH(k_zero_flag<<<grid_for((u64)n + 1, 256), 256, 0, st>>>(g->off, n, flag));
   TKC_RC(scan_exclusive(flag, flag, (u64)n + 1, tmp, st));
   TKC_LAUNCH(k_zero_out<<<grid_for(n, 256), 256, 0, st>>>(g->off, flag, n, g->zero_ids));
@@ -667,9 +664,9 @@ int ensure_classes(const tkc_graph *g, const u32 *gid, u32 ng) {
   cudaStream_t st = g->ctx->stream;
   const size_t n = g->n;
   uint8_t *cls = nullptr;
-  TKC_TRY(cudaMallocAsync(&cls, n, st));
-  if (!g->n_cls) TKC_TRY(cudaMallocAsync(&g->n_cls, (size_t)kClasses * ng * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&g->cls, n * sizeof(uint4), st));
+  TKC_TRY(dev_malloc(&cls, n, st));
+  if (!g->n_cls) TKC_TRY(dev_malloc(&g->n_cls, (size_t)kClasses * ng * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&g->cls, n * sizeof(uint4), st));
   TKC_TRY(cudaMemsetAsync(g->n_cls, 0, (size_t)kClasses * ng * sizeof(u32), st));
   TKC_TRY(cudaMemsetAsync(g->cls, 0, n * sizeof(uint4), st));
   TKC_LAUNCH(k_classes<<<grid_for(n, 256), 256, 0, st>>>(g->ioff, g->n, gid, cls, g->n_cls));
@@ -739,8 +736,8 @@ __global__ void k_bu_keys_many(const u32 *ioff, u32 n, u32 heavy_in, const u32 *
 static int build_bu_list(const u32 *ioff, u32 n, u32 heavy_in, cudaStream_t st, u32 **list, u32 *cnt,
                          const u32 *gid = nullptr, u32 ng = 0, u32 *g_cnt = nullptr) {
   u32 *keys = nullptr, *ids = nullptr;
-  TKC_TRY(cudaMallocAsync(&ids, (size_t)n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&keys, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&ids, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&keys, (size_t)n * sizeof(u32), st));
   TKC_TRY(cudaMemsetAsync(cnt, 0, 2 * sizeof(u32), st));
   int bits = 6;
   if (gid) {
@@ -826,15 +823,15 @@ void free_search_csr(const tkc_graph *g) {
 static int build_labelled_copy(const tkc_graph *g, cudaStream_t st) {
   const u32 n = g->n;
   u32 *keys = nullptr, *gcol = nullptr, *tmp = nullptr;
-  TKC_TRY(cudaMallocAsync(&g->s_cnt, 2 * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&g->s_unlab, (size_t)n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&g->s_lab, (size_t)n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&g->s_off, ((size_t)n + 1) * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&g->s_ioff, ((size_t)n + 1) * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&g->s_icol, std::max<size_t>(g->arcs, 1) * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&gcol, std::max<size_t>(g->arcs, 1) * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&keys, (size_t)n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&tmp, (((size_t)n + 1) / kScanTile + 2) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&g->s_cnt, 2 * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&g->s_unlab, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&g->s_lab, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&g->s_off, ((size_t)n + 1) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&g->s_ioff, ((size_t)n + 1) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&g->s_icol, std::max<size_t>(g->arcs, 1) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&gcol, std::max<size_t>(g->arcs, 1) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&keys, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&tmp, (((size_t)n + 1) / kScanTile + 2) * sizeof(u32), st));
   // key n - indegree (in [1, n]: no vertex has n in-arcs), ascending
   TKC_LAUNCH(k_relabel_keys<<<grid_for(n, 256), 256, 0, st>>>(g->ioff, n, n, keys, g->s_unlab));
   TKC_TRY(cudaGetLastError());
@@ -875,8 +872,7 @@ static int build_labelled_copy(const tkc_graph *g, cudaStream_t st) {
 static int read_bu_counts(const tkc_graph *g) {
   cudaStream_t st = g->ctx->stream;
   u32 c[2] = {0, 0};
-  TKC_TRY(cudaMemcpyAsync(c, g->s_cnt, sizeof(c), cudaMemcpyDeviceToHost, st));
-  TKC_TRY(cudaStreamSynchronize(st));
+  TKC_TRY(read_back(c, g->s_cnt, sizeof(c), st));
   g->n_bu = c[0];
   g->n_bu_heavy = c[1];
   return TKC_OK;
@@ -900,10 +896,10 @@ int ensure_search_csr(const tkc_graph *g, bool relabel, const u32 *gid, u32 ng) 
   cudaStream_t st = g->ctx->stream;
   if (!relabel) {
     g->heavy_in = kHeavyIn;
-    TKC_TRY(cudaMallocAsync(&g->s_cnt, 2 * sizeof(u32), st));
+    TKC_TRY(dev_malloc(&g->s_cnt, 2 * sizeof(u32), st));
     // (a graph number takes 26 bits of a key beside the class's 6)
     const bool many = gid && ng > 1 && ng <= (1u << 26);
-    if (many) TKC_TRY(cudaMallocAsync(&g->g_bu, 2 * (size_t)ng * sizeof(u32), st));
+    if (many) TKC_TRY(dev_malloc(&g->g_bu, 2 * (size_t)ng * sizeof(u32), st));
     TKC_RC(build_bu_list(g->ioff, g->n, g->heavy_in, st, &g->bu_list, g->s_cnt, many ? gid : nullptr, ng, g->g_bu));
   } else {
     TKC_RC(build_labelled_copy(g, st));
@@ -955,14 +951,13 @@ int filter_order(tkc_graph *g, const u32 *d_order_all, u32 *d_out, u32 *count) {
   cudaStream_t st = g->ctx->stream;
   const u32 n = g->n;
   u32 *pos = nullptr, *tmp = nullptr;
-  TKC_TRY(cudaMallocAsync(&pos, ((size_t)n + 1) * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&tmp, (((size_t)n + 1) / kScanTile + 2) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&pos, ((size_t)n + 1) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&tmp, (((size_t)n + 1) / kScanTile + 2) * sizeof(u32), st));
   TKC_LAUNCH(k_flag_src<<<grid_for(n, 256), 256, 0, st>>>(d_order_all, g->off, n, pos));
   TKC_RC(scan_exclusive(pos, pos, (u64)n + 1, tmp, st));
   TKC_LAUNCH(k_compact<<<grid_for(n, 256), 256, 0, st>>>(d_order_all, pos, n, d_out));
   TKC_TRY(cudaGetLastError());
-  TKC_TRY(cudaMemcpyAsync(count, pos + n, sizeof(u32), cudaMemcpyDeviceToHost, st));
-  TKC_TRY(cudaStreamSynchronize(st));
+  TKC_TRY(read_back(count, pos + n, sizeof(u32), st));
   TKC_TRY(cudaFreeAsync(pos, st));
   TKC_TRY(cudaFreeAsync(tmp, st));
   return TKC_OK;
@@ -1029,9 +1024,9 @@ static int reach_undirected(tkc_graph *g) {
   cudaStream_t st = g->ctx->stream;
   const u32 n = g->n;
   u32 *parent = nullptr, *size = nullptr, *changed = nullptr;
-  TKC_TRY(cudaMallocAsync(&parent, (size_t)n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&size, (size_t)n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&changed, sizeof(u32), st));
+  TKC_TRY(dev_malloc(&parent, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&size, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&changed, sizeof(u32), st));
   TKC_LAUNCH(k_cc_init<<<grid_for(n, 256), 256, 0, st>>>(parent, n));
   for (int it = 0;; ++it) {
     if (it > 4096) return TKC_ETIMEOUT;
@@ -1040,8 +1035,7 @@ static int reach_undirected(tkc_graph *g) {
     TKC_LAUNCH(k_cc_compress<<<grid_for(n, 256), 256, 0, st>>>(parent, n));
     TKC_TRY(cudaGetLastError());
     u32 hc = 0;
-    TKC_TRY(cudaMemcpyAsync(&hc, changed, sizeof(u32), cudaMemcpyDeviceToHost, st));
-    TKC_TRY(cudaStreamSynchronize(st));
+    TKC_TRY(read_back(&hc, changed, sizeof(u32), st));
     if (!hc) break;
   }
   TKC_TRY(cudaMemsetAsync(size, 0, (size_t)n * sizeof(u32), st));
@@ -1067,10 +1061,10 @@ int ensure_reach_bounds(tkc_graph *g, const u32 *gid, u32 ng) {
     g->have_reach = true;
     return TKC_OK;
   }
-  if (!g->alpha) TKC_TRY(cudaMallocAsync(&g->alpha, (size_t)g->n * sizeof(u32), st));
-  if (!g->omega) TKC_TRY(cudaMallocAsync(&g->omega, (size_t)g->n * sizeof(u32), st));
-  if (!g->scc_size) TKC_TRY(cudaMallocAsync(&g->scc_size, (size_t)g->n * sizeof(u32), st));
-  if (!g->comp) TKC_TRY(cudaMallocAsync(&g->comp, (size_t)g->n * sizeof(u32), st));
+  if (!g->alpha) TKC_TRY(dev_malloc(&g->alpha, (size_t)g->n * sizeof(u32), st));
+  if (!g->omega) TKC_TRY(dev_malloc(&g->omega, (size_t)g->n * sizeof(u32), st));
+  if (!g->scc_size) TKC_TRY(dev_malloc(&g->scc_size, (size_t)g->n * sizeof(u32), st));
+  if (!g->comp) TKC_TRY(dev_malloc(&g->comp, (size_t)g->n * sizeof(u32), st));
   TKC_RC(ensure_in_csr(g));
   TKC_RC(g->directed ? reach_directed_gpu(g, gid, ng) : reach_undirected(g));
   g->have_reach = true;

@@ -296,9 +296,9 @@ int bfs_reach(tkc_ctx *ctx, const u32 *off, const u32 *col, const u32 *roff, con
   u32 *q = nullptr;
   u64 *qo = nullptr;
   BfsCtl *c = nullptr;
-  TKC_TRY(cudaMallocAsync(&q, (size_t)2 * n * sizeof(u32), st));
-  TKC_TRY(cudaMallocAsync(&qo, (size_t)2 * n * sizeof(u64), st));
-  TKC_TRY(cudaMallocAsync(&c, sizeof(BfsCtl), st));
+  TKC_TRY(dev_malloc(&q, (size_t)2 * n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&qo, (size_t)2 * n * sizeof(u64), st));
+  TKC_TRY(dev_malloc(&c, sizeof(BfsCtl), st));
   TKC_TRY(cudaMemsetAsync(c, 0, sizeof(BfsCtl), st));
   TKC_TRY(cudaMemsetAsync(mark, 0xff, (size_t)n * sizeof(u32), st));
   u32 *q0 = q, *q1 = q + n;
@@ -316,8 +316,7 @@ int bfs_reach(tkc_ctx *ctx, const u32 *off, const u32 *col, const u32 *roff, con
   note_launches(1);
   TKC_TRY(cudaLaunchCooperativeKernel((const void *)k_bfs_reach, dim3(blocks), dim3(kBfsThreads), args, 0, st));
   int err = 0;
-  TKC_TRY(cudaMemcpyAsync(&err, &c->err, sizeof(int), cudaMemcpyDeviceToHost, st));
-  TKC_TRY(cudaStreamSynchronize(st));
+  TKC_TRY(read_back(&err, &c->err, sizeof(int), st));
   TKC_TRY(cudaFreeAsync(q, st));
   TKC_TRY(cudaFreeAsync(qo, st));
   TKC_TRY(cudaFreeAsync(c, st));
@@ -771,7 +770,7 @@ struct DevBufs {
   }
   template <typename T>
   cudaError_t get(T **p, size_t count) {
-    cudaError_t e = cudaMallocAsync((void **)p, std::max<size_t>(count, 1) * sizeof(T), st);
+    cudaError_t e = dev_malloc(p, std::max<size_t>(count, 1) * sizeof(T), st);
     if (e == cudaSuccess) ptrs.push_back(*p);
     return e;
   }
@@ -826,8 +825,7 @@ int reach_directed_gpu(tkc_graph *g, const u32 *gid, u32 ng) {
     TKC_TRY(cudaMemsetAsync(best, 0, sizeof(u64), st));
     TKC_LAUNCH(k_pivot<<<grid_of(n), 256, 0, st>>>(outd, ind, active, n, best));
     u64 hb = 0;
-    TKC_TRY(cudaMemcpyAsync(&hb, best, sizeof(u64), cudaMemcpyDeviceToHost, st));
-    TKC_TRY(cudaStreamSynchronize(st));
+    TKC_TRY(read_back(&hb, best, sizeof(u64), st));
     if (hb == 0) break;  // nothing left
     if (round == 0 && gid && ng > 1) {
       // Several graphs: one pivot per graph and one forward and one backward
@@ -894,12 +892,10 @@ int reach_directed_gpu(tkc_graph *g, const u32 *gid, u32 ng) {
   TKC_TRY(cudaMemsetAsync(best, 0, sizeof(u64), st));
   TKC_LAUNCH(k_biggest<<<grid_of(n), 256, 0, st>>>(wgt, minid, n, best));
   u64 hb = 0;
-  TKC_TRY(cudaMemcpyAsync(&hb, best, sizeof(u64), cudaMemcpyDeviceToHost, st));
-  TKC_TRY(cudaStreamSynchronize(st));
+  TKC_TRY(read_back(&hb, best, sizeof(u64), st));
   const u32 big_min = 0xffffffffu - (u32)(hb & 0xffffffffu);
   u32 big = 0;
-  TKC_TRY(cudaMemcpyAsync(&big, comp + big_min, sizeof(u32), cudaMemcpyDeviceToHost, st));
-  TKC_TRY(cudaStreamSynchronize(st));
+  TKC_TRY(read_back(&big, comp + big_min, sizeof(u32), st));
   // exact reach of the biggest SCC (forward), and the SCCs that reach it
   // (backward); only reachability is used, the same from every vertex of the
   // SCC, so the first pivot's sweeps serve when it lies in the biggest SCC
