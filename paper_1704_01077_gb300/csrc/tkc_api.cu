@@ -115,10 +115,7 @@ int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u3
     TKC_RC(dalloc(&w.g_lock, cap, st));
     TKC_RC(dalloc(&w.g_stop, cap, st));
     TKC_RC(dalloc(&w.g_ctr, 4 * (size_t)cap, st));
-    TKC_RC(dalloc(&w.x_seq, cap, st));
-    TKC_RC(dalloc(&w.x_S, cap, st));
-    TKC_RC(dalloc(&w.x_r, cap, st));
-    TKC_RC(dalloc(&w.x_id, cap, st));
+    TKC_RC(dalloc(&w.x, cap, st));
     TKC_RC(dalloc(&w.f_end, cap, st));
     w.ng_cap = cap;
   }
@@ -184,7 +181,7 @@ static int ensure_filter(tkc_ctx *ctx, u32 count, u32 nopen) {
 static void free_workspace(tkc_ctx *ctx) {
   Workspace &w = ctx->ws;
   void *ptrs[] = {w.seen, w.F0, w.F1, w.N, w.FB0, w.FB1, w.L0, w.L1, w.Loff0, w.Loff1, w.VL, w.stamp, w.res_S, w.res_r,
-                  w.slots, w.cnt, w.wsum, w.top_S, w.top_r, w.top_id, w.ctl, w.out, w.tied, w.g_ntop, w.g_lock, w.g_stop, w.g_ctr, w.sh, w.x_seq, w.x_S, w.x_r, w.x_id,
+                  w.slots, w.cnt, w.wsum, w.top_S, w.top_r, w.top_id, w.ctl, w.out, w.tied, w.g_ntop, w.g_lock, w.g_stop, w.g_ctr, w.sh, w.x,
                   w.f_order, w.f_keep, w.f_count, w.f_end, w.lvl2,
                   w.o_order, w.o_key, w.o_taken};
   for (void *p : ptrs)
@@ -443,9 +440,8 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     TKC_TRY(cudaMemcpyAsync(w.top_r, rs.seed_r, ns * sizeof(u32), cudaMemcpyHostToDevice, st));
     TKC_TRY(cudaMemcpyAsync(w.top_id, rs.seed_id, ns * sizeof(u32), cudaMemcpyHostToDevice, st));
     if (ns == rs.kk) {  // a full list: its k-th entry is the published threshold
-      TKC_TRY(cudaMemcpyAsync(w.x_S, rs.seed_S + ns - 1, sizeof(u64), cudaMemcpyHostToDevice, st));
-      TKC_TRY(cudaMemcpyAsync(w.x_r, rs.seed_r + ns - 1, sizeof(u32), cudaMemcpyHostToDevice, st));
-      TKC_TRY(cudaMemcpyAsync(w.x_id, rs.seed_id + ns - 1, sizeof(u32), cudaMemcpyHostToDevice, st));
+      const u64 x[2] = {rs.seed_S[ns - 1], (u64)rs.seed_r[ns - 1] << 32 | rs.seed_id[ns - 1]};
+      TKC_TRY(cudaMemcpyAsync(w.x, x, sizeof(x), cudaMemcpyHostToDevice, st));
     }
     TKC_TRY(cudaStreamSynchronize(st));  // the seed arrays are the caller's pageable memory
   }
@@ -504,10 +500,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   p.vtx_stride = w.n_cap;
   p.fb_stride = w.n_cap / 32 + 1;
   p.sh = w.sh;
-  p.x_seq = w.x_seq;
-  p.x_S = w.x_S;
-  p.x_r = w.x_r;
-  p.x_id = w.x_id;
+  p.x = w.x;
   // default: a level runs bottom-up when its frontier's arcs exceed 1/8 of all arcs
   p.bu_num = o.bu_num ? o.bu_num : 8;
   p.bu_den = o.bu_num ? std::max<u32>(o.bu_den, 1) : 1;

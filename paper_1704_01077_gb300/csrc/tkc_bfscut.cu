@@ -48,19 +48,39 @@ __device__ __forceinline__ void st_release_u32(unsigned *p, unsigned v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 __device__ __forceinline__ int ld_volatile_i32(const int *p) { return *(volatile const int *)p; }
+// One 128-bit word, read and written whole.
+__device__ __forceinline__ ulonglong2 ld_relaxed_128(const ulonglong2 *p) {
+  ulonglong2 v;
+  asm volatile("{ .reg .b128 t; ld.relaxed.gpu.global.b128 t, [%2]; mov.b128 {%0, %1}, t; }"
+               : "=l"(v.x), "=l"(v.y)
+               : "l"(p)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed_128(ulonglong2 *p, unsigned long long lo, unsigned long long hi) {
+  asm volatile("{ .reg .b128 t; mov.b128 t, {%1, %2}; st.relaxed.gpu.global.b128 [%0], t; }" ::"l"(p), "l"(lo), "l"(hi)
+               : "memory");
+}
 
 // Barrier over the `nblocks` blocks of one team (all co-resident: the launch
 // is cooperative).  The last block to arrive runs `epi` (whole block) before
-// releasing the others.  Returns false when the run must stop: an error
-// recorded by this team or any other, including a timed-out wait.
+// releasing the others.  Returns false when a wait ran out or met an error
+// recorded by this team or any other: a block that leaves never arrives again,
+// so the blocks of its team meet the error at their next wait.
+//
+// A level of a small graph is two of these and little else, so the wait polls
+// the generation alone, at full rate at first (an L2 round trip each), and
+// looks at the error words only every 16th time: with both words read on every
+// poll and a sleep between, a release took 2.7 us to be seen.
 template <typename Epi>
 __device__ __forceinline__ bool team_sync(Ctl *ctl, Shared *sh, unsigned nblocks, uint64_t timeout, Epi epi) {
-  __shared__ int s_last;
+  __shared__ int s_last, s_ok;
   __shared__ unsigned s_gen;
   __syncthreads();
   if (threadIdx.x == 0) {
     unsigned gen = ld_acquire_u32(&ctl->bar_gen);
     s_gen = gen;
+    s_ok = 1;
     __threadfence();
     unsigned arrived = atomicAdd(&ctl->bar_count, 1u) + 1u;
     s_last = (arrived == nblocks);
@@ -76,23 +96,26 @@ __device__ __forceinline__ bool team_sync(Ctl *ctl, Shared *sh, unsigned nblocks
       st_release_u32(&ctl->bar_gen, s_gen + 1u);
     }
   } else if (threadIdx.x == 0) {
-    long long t0 = clock64();
-    unsigned ns = 32;
-    while (ld_acquire_u32(&ctl->bar_gen) == s_gen) {
-      if (ld_volatile_i32(&ctl->err) != 0 || ld_volatile_i32(&sh->err) != 0) break;
-      if ((uint64_t)(clock64() - t0) > timeout) {
-        atomicCAS(&ctl->err, 0, TKC_ETIMEOUT);
-        atomicCAS(&sh->err, 0, TKC_ETIMEOUT);
-        atomicCAS(&ctl->err_where, 0, 1);
-        break;
+    const long long t0 = clock64();
+    for (unsigned poll = 1; ld_acquire_u32(&ctl->bar_gen) == s_gen; ++poll) {
+      const bool late = (uint64_t)(clock64() - t0) > timeout;
+      if ((poll & 15u) == 0 || late) {
+        if (late) {
+          atomicCAS(&ctl->err, 0, TKC_ETIMEOUT);
+          atomicCAS(&sh->err, 0, TKC_ETIMEOUT);
+          atomicCAS(&ctl->err_where, 0, 1);
+        }
+        if (ld_volatile_i32(&ctl->err) != 0 || ld_volatile_i32(&sh->err) != 0) {
+          s_ok = 0;
+          break;
+        }
       }
-      __nanosleep(ns);
-      if (ns < 256) ns <<= 1;
+      if (poll > 64) __nanosleep(128);
     }
     __threadfence();
   }
   __syncthreads();
-  return ld_volatile_i32(&ctl->err) == 0 && ld_volatile_i32(&sh->err) == 0;
+  return s_ok != 0;
 }
 
 // ------------------------------------------------------------------ exact arithmetic
@@ -398,7 +421,9 @@ struct Smem {
   u64 scan64[kMaxThreads / 32 + 1];
   u64 acc[4];
   unsigned bu_next;  // bottom-up level: next of this block's vertex chunks
+  alignas(8) uint32_t cmd[kCmdWords];  // the step's control words (Ctl from `step` on)
 };
+static_assert(offsetof(Ctl, step) % 8 == 0 && kCmdWords <= 64, "the control words are copied as they lie");
 
 // Block-wide exclusive scan of one uint32 per thread; returns the prefix and
 // writes the total to *total.
@@ -460,9 +485,7 @@ __device__ u64 block_exscan64(Smem<W> &sm, u64 x, u64 *total) {
 
 // ------------------------------------------------------------------ epilogues
 
-// The k-th entry of graph g's list as last published (seqlock: the writer
-// makes the sequence odd, writes, makes it even).  A read that keeps seeing
-// a write in progress reports no threshold, which only means no cut.
+// The k-th entry of graph g's list as last published.
 struct Thresh {
   bool have;
   u64 S;
@@ -470,41 +493,22 @@ struct Thresh {
 };
 
 __device__ __forceinline__ Thresh thresh_of(const RunParams &p, uint32_t g) {
+  const ulonglong2 v = ld_relaxed_128(p.x + g);
   Thresh t;
-  t.have = false;
-  t.S = 0;
-  t.r = t.id = 0;
-  for (int tries = 0; tries < 64; ++tries) {
-    unsigned s1 = ld_acquire_u32(&p.x_seq[g]);
-    if (s1 & 1u) continue;
-    u64 S = *(volatile const u64 *)&p.x_S[g];
-    uint32_t r = *(volatile const uint32_t *)&p.x_r[g];
-    uint32_t id = *(volatile const uint32_t *)&p.x_id[g];
-    __threadfence();
-    unsigned s2 = *(volatile const unsigned *)&p.x_seq[g];
-    if (s1 == s2) {
-      t.have = r != 0;
-      t.S = S;
-      t.r = r;
-      t.id = id;
-      return t;
-    }
-  }
+  t.S = v.x;
+  t.r = (uint32_t)(v.y >> 32);
+  t.id = (uint32_t)v.y;
+  t.have = t.r != 0;
   return t;
 }
 
-// Publishes graph g's current k-th entry (caller holds the merge lock).
+// Publishes graph g's current k-th entry (caller holds the list's lock).
 __device__ __forceinline__ void publish_thresh(const RunParams &p, uint32_t g) {
   if (*(volatile unsigned *)&p.g_ntop[g] != p.kk) return;
-  size_t i = (size_t)g * p.kk + p.kk - 1;
-  unsigned s = *(volatile unsigned *)&p.x_seq[g];
-  *(volatile unsigned *)&p.x_seq[g] = s + 1u;
-  __threadfence();
-  *(volatile u64 *)&p.x_S[g] = *(volatile u64 *)&p.top_S[i];
-  *(volatile uint32_t *)&p.x_id[g] = *(volatile uint32_t *)&p.top_id[i];
-  *(volatile uint32_t *)&p.x_r[g] = *(volatile uint32_t *)&p.top_r[i];
-  __threadfence();
-  st_release_u32(&p.x_seq[g], s + 2u);
+  const size_t i = (size_t)g * p.kk + p.kk - 1;
+  const u64 S = *(volatile u64 *)&p.top_S[i];
+  const u64 r = *(volatile uint32_t *)&p.top_r[i], id = *(volatile uint32_t *)&p.top_id[i];
+  st_relaxed_128(p.x + g, S, r << 32 | id);
 }
 
 // Lock of graph g's list, taken by one thread; a wait beyond the budget is an
@@ -650,8 +654,7 @@ __device__ __forceinline__ void graph_count(const RunParams &p, uint32_t g, int 
 // Adds a finished search to the candidate list if it can enter the top list.
 template <int W>
 __device__ __forceinline__ void offer_candidate(const RunParams &p, Smem<W> &sm, u64 S, uint32_t r, uint32_t v,
-                                                uint32_t g) {
-  Thresh x = thresh_of(p, g);
+                                                uint32_t g, const Thresh &x) {
   if (x.have && !entry_less(p.harmonic, S, r, v, x.S, x.r, x.id)) return;
   unsigned pos = atomicAdd(&sm.ncand, 1u);
   sm.cS[pos] = S;
@@ -690,30 +693,49 @@ __device__ __forceinline__ int choose_dir(const RunParams &p, u64 fl_arcs) {
 // barrier would cost more than the dead entries).
 constexpr uint32_t kCompactMin = 4096;
 
+// Runs in one block while the team waits, so it is written for few dependent
+// round trips to L2: slots, counters, the threshold and the control words are
+// loaded together, a thread keeps its slot in registers, statistics are added
+// without waiting, and the threshold is read again only after a merge.
 template <int W>
-__device__ void epilogue_level(const RunParams &p, Smem<W> &sm) {
+__device__ __noinline__ void epilogue_level(const RunParams &p, Smem<W> &sm) {
+  static_assert(64 * W <= kMinThreads, "a thread per slot");
   Ctl *c = p.ctl;
-  const uint32_t B = p.B;
   trace_stamp(p, 13);
+  const uint32_t s = threadIdx.x;
+  Slot sl;
+  unsigned cn = 0;
+  u64 ws = 0;
+  bool act = false;
+  if (s < p.B) {
+    sl = p.slots[s];
+    cn = p.cnt[s];
+    ws = p.wsum[s];
+    act = sl.state == 1;
+  }
+  Thresh x = thresh_of(p, p.ng == 1 || !act ? 0u : sl.graph);
+  // the level just run (thread 0)
+  u64 packed = 0, fa = 0, lsv = 0, lsa = 0, lsr = 0;
+  uint32_t fl = 0;
+  int dir = 0;
   if (threadIdx.x == 0) {
+    volatile Ctl *vc = c;
+    packed = vc->nl_packed;
+    fa = vc->fl_arcs;
+    lsv = vc->lvl_scan_v;
+    lsa = vc->lvl_scan_a;
+    lsr = vc->lvl_scan_r;
+    fl = vc->fl_count;
+    dir = vc->dir;
     sm.ncand = 0;
     sm.nactive = 0;
   }
   if (threadIdx.x < W) sm.active[threadIdx.x] = 0;
-  for (int i = threadIdx.x; i < 4; i += blockDim.x) sm.acc[i] = 0;
+  if (threadIdx.x < 4) sm.acc[threadIdx.x] = 0;
   __syncthreads();
   // 1. per-slot level update
-  int cont[(64 * W + kMinThreads - 1) / kMinThreads];
-  uint32_t finished = 0;
-#pragma unroll
-  for (int t = 0; t < (64 * W + kMinThreads - 1) / kMinThreads; ++t) {
-    uint32_t s = threadIdx.x + t * blockDim.x;
-    cont[t] = 0;
-    if (s >= B) continue;
-    Slot sl = p.slots[s];
-    if (sl.state != 1) continue;
-    unsigned cn = p.cnt[s];
-    u64 ws = p.wsum[s];
+  bool cont = false;
+  if (act) {
     p.cnt[s] = 0;
     p.wsum[s] = 0;
     if (cn == 0) {
@@ -722,9 +744,10 @@ __device__ void epilogue_level(const RunParams &p, Smem<W> &sm) {
       const u64 key = p.harmonic ? (u64)__double_as_longlong(sl.H) : sl.S;
       p.res_S[sl.v] = key;
       p.res_r[sl.v] = (uint32_t)sl.nd;
-      ++finished;
+      p.slots[s].state = 2;
+      atomicAdd(&sm.acc[0], 1ull);
       graph_count(p, sl.graph, 3, 1);
-      offer_candidate(p, sm, key, (uint32_t)sl.nd, sl.v, sl.graph);
+      offer_candidate(p, sm, key, (uint32_t)sl.nd, sl.v, sl.graph, x);
     } else {
       const int directed = p.g_directed ? p.g_directed[sl.graph] : p.directed;
       sl.d += 1;
@@ -735,114 +758,52 @@ __device__ void epilogue_level(const RunParams &p, Smem<W> &sm) {
           atomicCAS(&c->err, 0, TKC_EOVERFLOW);
       }
       sl.S += (u64)sl.d * cn;
-      sl.H = __dadd_rn(sl.H, __ddiv_rn((double)cn, (double)sl.d));
+      if (p.harmonic) sl.H = __dadd_rn(sl.H, __ddiv_rn((double)cn, (double)sl.d));
       sl.nd += cn;
       sl.g = ws - (directed ? 0ull : (u64)cn);
       sl.arcs = ws;
-      cont[t] = 1;
+      cont = true;
     }
-    p.slots[s] = sl;
   }
-  if (finished) atomicAdd(&sm.acc[0], (u64)finished);
   __syncthreads();
   // 2. top-k merge and the new threshold
-  merge_topk(p, sm);
+  if (sm.ncand) {
+    merge_topk(p, sm);
+    if (cont) x = thresh_of(p, p.ng == 1 ? 0u : sl.graph);
+  }
   // 3. BFSCut test for the slots that continue
-  uint32_t cuts = 0;
-  u64 visited = 0;
-#pragma unroll
-  for (int t = 0; t < (64 * W + kMinThreads - 1) / kMinThreads; ++t) {
-    uint32_t s = threadIdx.x + t * blockDim.x;
-    if (!cont[t]) continue;
-    Slot sl = p.slots[s];
-    Thresh x = thresh_of(p, sl.graph);
-    const bool below = x.have && (p.harmonic ? harmonic_below(sl.H, sl.d, sl.nd, sl.g, sl.omega, x.S)
-                                             : cut_exceeds(sl.S, sl.d, sl.nd, sl.g, sl.alpha, sl.omega, x.S, x.r));
-    if (!p.nocut && !sl.nocut && below) {
-      sl.state = 2;
-      ++cuts;
+  if (cont) {
+    const bool below = !p.nocut && !sl.nocut && x.have &&
+                       (p.harmonic ? harmonic_below(sl.H, sl.d, sl.nd, sl.g, sl.omega, x.S)
+                                   : cut_exceeds(sl.S, sl.d, sl.nd, sl.g, sl.alpha, sl.omega, x.S, x.r));
+    if (below) {
+      p.slots[s].state = 2;
+      atomicAdd(&sm.acc[1], 1ull);
       graph_count(p, sl.graph, 2, 1);
-      p.slots[s] = sl;
     } else {
-      visited += sl.arcs;
+      p.slots[s] = sl;
+      atomicAdd(&sm.acc[2], sl.arcs);
       graph_count(p, sl.graph, 0, sl.arcs);
       atomicOr(&sm.active[s >> 6], 1ull << (s & 63));
       atomicAdd(&sm.nactive, 1u);
     }
   }
-  if (cuts) atomicAdd(&sm.acc[1], (u64)cuts);
-  if (visited) atomicAdd(&sm.acc[2], visited);
   __syncthreads();
   if (threadIdx.x == 0) {
-    c->bfs_finished += sm.acc[0];
-    c->bfs_cut += sm.acc[1];
-    c->edges_visited += sm.acc[2];
-    c->levels += 1;
-    u64 packed = c->nl_packed;
-    {
-      // cost model of the level just run (bytes that must move):
-      //  top-down : per frontier vertex list+offsets (16) + F row read and clear;
-      //             per frontier arc column (4) + seen row read + N row update;
-      //             per new vertex list (8) + N read/clear, seen read/write, F write
-      //  bottom-up: per swept list entry (vertices with an in-arc) the entry (4)
-      //             and its seen row; per scanned vertex in-offsets (8); per
-      //             scanned in-arc its column (4) and frontier-bitmap word (4);
-      //             per frontier in-neighbour found its F row; per new vertex
-      //             seen/F writes + list (8); per old frontier vertex list (4) +
-      //             F row clear
-      const u64 rb = 8ull * W;
-      const u64 fl = c->fl_count, fa = c->fl_arcs, nl = packed >> kPackShift;
-      u64 bytes;
-      if (c->dir == 0) {
-        bytes = fl * (16 + 2 * rb) + fa * (4 + 2 * rb) + nl * (8 + 5 * rb);
-        c->st_td_levels += 1;
-        c->st_td_frontier += fl;
-        c->st_td_arcs += fa;
-        c->st_td_new += nl;
-      } else {
-        const u64 swept = p.g_bu ? p.g_bu[2 * (size_t)c->bgraph] : p.bu_list ? p.n_bu : p.n;
-        bytes = swept * (4 + rb) + c->lvl_scan_v * 8 + c->lvl_scan_a * 8 + c->lvl_scan_r * rb + nl * (8 + 2 * rb) +
-                fl * (4 + rb);
-        c->st_bu_levels += 1;
-        c->st_bu_swept += swept;
-        c->st_bu_rows += c->lvl_scan_r;
-        c->st_bu_scan_v += c->lvl_scan_v;
-        c->st_bu_scan_a += c->lvl_scan_a;
-        c->st_bu_new += nl;
-        c->st_bu_frontier += fl;
-      }
-      c->alg_bytes += bytes;
-      if (p.trace) {
-        u64 idx = c->trace_n++;
-        if (idx < p.trace_cap) {
-          u64 t;
-          asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-          u64 *rec = p.trace + idx * 16;
-          rec[0] = t;
-          rec[1] = (u64)c->dir;
-          rec[2] = fl;
-          rec[3] = fa;
-          rec[4] = nl;
-          rec[5] = c->lvl_scan_v;
-          rec[6] = c->lvl_scan_a;
-          rec[7] = sm.nactive;
-        }
-      }
-      c->lvl_scan_v = 0;
-      c->lvl_scan_a = 0;
-      c->lvl_scan_r = 0;
-    }
+    const u64 nl = packed >> kPackShift, nla = packed & kArcMask;
+    // next step first, then the statistics
     c->nl_packed = 0;
     c->cur ^= 1;
     c->lcur ^= 1;
     c->bdepth += 1;
-    c->fl_count = (uint32_t)(packed >> kPackShift);
-    c->fl_arcs = packed & kArcMask;
+    c->fl_count = (uint32_t)nl;
+    c->fl_arcs = nla;
     c->level_id += 1;
+#pragma unroll
     for (int j = 0; j < W; ++j) c->active[j] = sm.active[j];
     if (sm.nactive == 0) {
       c->step = 1;  // clear the batch's rows, then seed the next batch
-    } else if (c->fl_count > kCompactMin && sm.acc[2] * 2 < c->fl_arcs) {
+    } else if (nl > kCompactMin && sm.acc[2] * 2 < nla) {
       // the new frontier list was built before this level's cuts: when the
       // surviving searches' own frontier arcs (sm.acc[2], an upper bound on
       // the arcs of the list entries they still use) are less than half of
@@ -851,7 +812,60 @@ __device__ void epilogue_level(const RunParams &p, Smem<W> &sm) {
       c->step = 2;
     } else {
       c->step = 0;
-      c->dir = choose_dir(p, c->fl_arcs);
+      c->dir = choose_dir(p, nla);
+    }
+    // cost model of the level just run (bytes that must move):
+    //  top-down : per frontier vertex list+offsets (16) + F row read and clear;
+    //             per frontier arc column (4) + seen row read + N row update;
+    //             per new vertex list (8) + N read/clear, seen read/write, F write
+    //  bottom-up: per swept list entry (vertices with an in-arc) the entry (4)
+    //             and its seen row; per scanned vertex in-offsets (8); per
+    //             scanned in-arc its column (4) and frontier-bitmap word (4);
+    //             per frontier in-neighbour found its F row; per new vertex
+    //             seen/F writes + list (8); per old frontier vertex list (4) +
+    //             F row clear
+    const u64 rb = 8ull * W;
+    u64 bytes;
+    if (dir == 0) {
+      bytes = fl * (16 + 2 * rb) + fa * (4 + 2 * rb) + nl * (8 + 5 * rb);
+      atomicAdd(&c->st_td_levels, 1ull);
+      atomicAdd(&c->st_td_frontier, (u64)fl);
+      atomicAdd(&c->st_td_arcs, fa);
+      atomicAdd(&c->st_td_new, nl);
+    } else {
+      const u64 swept = p.g_bu ? p.g_bu[2 * (size_t)c->bgraph] : p.bu_list ? p.n_bu : p.n;
+      bytes = swept * (4 + rb) + lsv * 8 + lsa * 8 + lsr * rb + nl * (8 + 2 * rb) + fl * (4 + rb);
+      atomicAdd(&c->st_bu_levels, 1ull);
+      atomicAdd(&c->st_bu_swept, swept);
+      atomicAdd(&c->st_bu_rows, lsr);
+      atomicAdd(&c->st_bu_scan_v, lsv);
+      atomicAdd(&c->st_bu_scan_a, lsa);
+      atomicAdd(&c->st_bu_new, nl);
+      atomicAdd(&c->st_bu_frontier, (u64)fl);
+      c->lvl_scan_v = 0;
+      c->lvl_scan_a = 0;
+      c->lvl_scan_r = 0;
+    }
+    atomicAdd(&c->alg_bytes, bytes);
+    if (sm.acc[0]) atomicAdd(&c->bfs_finished, sm.acc[0]);
+    if (sm.acc[1]) atomicAdd(&c->bfs_cut, sm.acc[1]);
+    if (sm.acc[2]) atomicAdd(&c->edges_visited, sm.acc[2]);
+    atomicAdd(&c->levels, 1ull);
+    if (p.trace) {
+      u64 idx = c->trace_n++;
+      if (idx < p.trace_cap) {
+        u64 t;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+        u64 *rec = p.trace + idx * 16;
+        rec[0] = t;
+        rec[1] = (u64)dir;
+        rec[2] = fl;
+        rec[3] = fa;
+        rec[4] = nl;
+        rec[5] = lsv;
+        rec[6] = lsa;
+        rec[7] = sm.nactive;
+      }
     }
   }
   __syncthreads();
@@ -861,7 +875,7 @@ __device__ void epilogue_level(const RunParams &p, Smem<W> &sm) {
 // buffer) becomes the frontier list, and the level's direction is chosen from
 // its arcs.
 template <int W>
-__device__ void epilogue_compact(const RunParams &p, Smem<W> &sm) {
+__device__ __noinline__ void epilogue_compact(const RunParams &p, Smem<W> &sm) {
   Ctl *c = p.ctl;
   if (threadIdx.x == 0) {
     const u64 packed = c->nl_packed;
@@ -926,7 +940,7 @@ __device__ __forceinline__ uint32_t take_of_graph(const RunParams &p, uint32_t r
 
 // Epilogue after a clear step: seed the next batch of up to B sources.
 template <int W>
-__device__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
+__device__ __noinline__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
   Ctl *c = p.ctl;
   trace_stamp(p, 13);
   const uint32_t B = p.B;
@@ -1173,9 +1187,12 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
   const uint32_t nthreads = bpt * TPB;
 
   while (true) {
-    const int step = ld_volatile_i32(&c->step);
-    if (ld_volatile_i32(&c->done)) break;
-    volatile Ctl *vc = c;
+    // the control words of this step, one round trip for all of them
+    if (threadIdx.x < kCmdWords) sm.cmd[threadIdx.x] = ((volatile uint32_t *)&c->step)[threadIdx.x];
+    __syncthreads();
+    const Ctl *vc = reinterpret_cast<const Ctl *>(reinterpret_cast<const char *>(sm.cmd) - offsetof(Ctl, step));
+    const int step = vc->step;
+    if (vc->done) break;
     const int cur = vc->cur;
     u64 *Fcur = cur ? p.F1 : p.F0;
     u64 *Fnext = cur ? p.F0 : p.F1;
@@ -1261,18 +1278,26 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
       // dependent loads)
       constexpr int TU = W <= 2 ? 4 : 2;  // warp steps unrolled per iteration
       u64 CH = (fl_arcs + 2ull * nwarps - 1) / (2ull * nwarps);
-      CH = (CH + TU * APS - 1) / (TU * APS) * (TU * APS);
-      if (CH < TU * APS) CH = TU * APS;
+      // (a frontier too small for TU steps on every warp: one task per warp, of
+      // as few steps as that takes, since the level then lasts one task's chain)
+      if (fl_arcs <= (u64)nwarps * (TU * APS)) {
+        CH = (fl_arcs + nwarps - 1) / nwarps;
+        CH = (CH + APS - 1) / APS * APS;
+      } else {
+        CH = (CH + TU * APS - 1) / (TU * APS) * (TU * APS);
+      }
       const int grp = lane / W, j = lane % W;
       const u64 actj = sm.active[j];
       for (u64 base = (u64)gwarp * CH; base < fl_arcs; base += (u64)nwarps * CH) {
         u64 end = base + CH < fl_arcs ? base + CH : fl_arcs;
-        // entry holding arc `base`: last i with FLoff[i] <= base
+        // entry holding arc `base`: last i with FLoff[i] <= base, by a 32-way
+        // search (one round trip per factor of 32)
         uint32_t lo = 0, hi = fl_count;
         while (hi - lo > 1) {
-          uint32_t mid = (lo + hi) >> 1;
-          if (FLoff[mid] <= base) lo = mid;
-          else hi = mid;
+          const uint32_t stepw = (hi - lo + 31) / 32, at = lo + stepw * (uint32_t)lane;
+          const unsigned m = __ballot_sync(FULL, lane == 0 || (at < hi && FLoff[at] <= base));
+          lo += stepw * (31u - (uint32_t)__clz(m));
+          hi = lo + stepw < hi ? lo + stepw : hi;
         }
         uint32_t ent = lo;
         // TU warp steps per iteration: every arc's loads are issued before
@@ -1359,12 +1384,15 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
       // counter as they finish: first groups of 32 long in-rows, group j
       // holding list entries j, j + hg, j + 2 hg, ... so that the longest rows
       // land in different warps; then chunks of kBuChunkVerts consecutive
-      // entries of the shorter rows (labels ascending).
+      // entries of the shorter rows (labels ascending), or of 32.
       const uint32_t *list = bg >= 0 ? p.bu_list + v0 : p.bu_list;
       const uint32_t nheavy = bg >= 0 ? p.g_bu[2 * bg + 1] : list ? p.n_bu_heavy : 0u;
       const uint32_t nlight = bg >= 0 ? p.g_bu[2 * bg] - nheavy : list ? p.n_bu - nheavy : p.n;
       const uint32_t hg = (nheavy + 31) / 32;
-      const uint32_t nitems = hg + (nlight + kBuChunkVerts - 1) / kBuChunkVerts;
+      // chunks of kBuChunkVerts entries, of 32 when that leaves warps with fewer
+      // than four chunks: a level then waits for a warp's 32 entries, not 128
+      const uint32_t bch = nlight >= 4 * kBuChunkVerts * nwarps ? kBuChunkVerts : 32u;
+      const uint32_t nitems = hg + (nlight + bch - 1) / bch;
       for (;;) {
         uint32_t j = 0;
         if (lane == 0) j = atomicAdd(&sm.bu_next, 1u);
@@ -1373,8 +1401,8 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
         if (gi64 >= nitems) break;
         const uint32_t gi = (uint32_t)gi64;
         const bool hitem = gi < hg;
-        const uint32_t g0 = hitem ? 0u : (gi - hg) * kBuChunkVerts;
-        const uint32_t g1 = hitem ? 32u : (g0 + kBuChunkVerts < nlight ? g0 + kBuChunkVerts : nlight);
+        const uint32_t g0 = hitem ? 0u : (gi - hg) * bch;
+        const uint32_t g1 = hitem ? 32u : (g0 + bch < nlight ? g0 + bch : nlight);
         for (uint32_t base = g0; base < g1; base += 32) {
           bool valid;
           uint32_t w;
@@ -1592,8 +1620,8 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
 // epilogue seeds the first batch), the shared block and, with nlist > 0, the
 // per-graph list state and res_r of n vertices.
 __global__ void k_run_init(Ctl *ctl, uint32_t nctl, unsigned level_base, Shared *sh, uint32_t nlist, unsigned *g_ntop,
-                           unsigned *g_stop, int *g_lock, u64 *g_ctr, unsigned *x_seq, uint32_t *x_r,
-                           uint32_t *res_r, uint32_t n) {
+                           unsigned *g_stop, int *g_lock, u64 *g_ctr, ulonglong2 *x, uint32_t *res_r,
+                           uint32_t n) {
   const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
   static_assert(sizeof(Ctl) % 8 == 0, "control blocks are zeroed by 64-bit words");
   for (uint32_t i = t; i < nctl * (uint32_t)(sizeof(Ctl) / 8); i += nt) {
@@ -1611,9 +1639,9 @@ __global__ void k_run_init(Ctl *ctl, uint32_t nctl, unsigned level_base, Shared 
   }
   if (t == 0) *sh = Shared{};
   for (uint32_t i = t; i < nlist; i += nt) {
-    g_ntop[i] = g_stop[i] = x_seq[i] = 0;
+    g_ntop[i] = g_stop[i] = 0;
     g_lock[i] = 0;
-    x_r[i] = 0;
+    x[i] = make_ulonglong2(0, 0);
     for (int j = 0; j < 4; ++j) g_ctr[4 * (size_t)i + j] = 0;
   }
   if (nlist)
@@ -1751,10 +1779,13 @@ __global__ void __launch_bounds__(kFilterTPB) k_filter_test(RunParams p, uint32_
       if (p.gid) g = p.gid[v];
       b = off[v];
       od = off[v + 1] - b;
-      if (idx >= p.nocut_prefix) xr = p.x_r[g];
+      if (idx >= p.nocut_prefix) {
+        const ulonglong2 x = p.x[g];
+        xS = x.x;
+        xr = (uint32_t)(x.y >> 32);
+      }
     }
     if (xr != 0) {
-      xS = p.x_S[g];
       const bool stop = p.lb_key && (p.harmonic ? __dmul_rn(__longlong_as_double((long long)~p.lb_key[v]), kHMargin) <
                                                       __longlong_as_double((long long)xS)
                                                 : nb_exceeds(p.lb_key[v], xS, xr));
@@ -2000,8 +2031,7 @@ int run_init(tkc_ctx *ctx, uint32_t nctl, uint32_t n, uint32_t ng, bool reset_li
   const uint32_t work = reset_lists ? (n > ng ? n : ng) : 1024;
   const uint32_t blocks = work / 1024 + 1 < (uint32_t)ctx->num_sms * 8 ? work / 1024 + 1 : (uint32_t)ctx->num_sms * 8;
   TKC_LAUNCH(k_run_init<<<blocks, 256, 0, ctx->stream>>>(w.ctl, nctl, w.level_base, w.sh, reset_lists ? ng : 0u,
-                                                         w.g_ntop, w.g_stop, w.g_lock, w.g_ctr, w.x_seq, w.x_r, w.res_r,
-                                                         n));
+                                                         w.g_ntop, w.g_stop, w.g_lock, w.g_ctr, w.x, w.res_r, n));
   TKC_TRY(cudaGetLastError());
   return TKC_OK;
 }

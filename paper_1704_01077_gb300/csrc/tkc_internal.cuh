@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include <map>
@@ -63,19 +64,23 @@ struct Ctl {
   unsigned int bar_pad[30];
   int err;
   int err_where;
-  // loop state
+  // loop state, written by the epilogues and read by every block at the head of
+  // a step in one go (kCmdWords words from `step` on)
   int step;          // 0 = level, 1 = clear + seed, 2 = compact the frontier list to the active slots
   int done;
   int dir;           // 0 = top-down, 1 = bottom-up
   int cur;           // which frontier buffer / list is current
+  int lcur;          // which list buffer holds the current frontier list (compaction swaps it alone)
+  int bgraph;        // several graphs: the graph of every search of the batch, -1 when they differ
+  unsigned int bdepth;    // depth reached by the current batch (0 after seeding)
   unsigned int level_id;  // global level stamp
-  unsigned int cursor;    // next position in the source order
   unsigned int fl_count;  // current frontier list size
   unsigned int vl_count;  // visited-list size (vertices with a non-zero seen row)
-  unsigned int pad0;
   unsigned long long fl_arcs;    // arcs out of the current frontier list
-  unsigned long long nl_packed;  // next list: count << 38 | arcs
   unsigned long long active[kMaxWords];
+  unsigned long long nl_packed;  // next list: count << 38 | arcs
+  unsigned int cursor;    // next position in the source order
+  unsigned int pad0;
   // counters
   unsigned long long edges_visited;
   unsigned long long edges_scanned;
@@ -90,17 +95,14 @@ struct Ctl {
   unsigned long long lvl_scan_a;
   unsigned long long lvl_scan_r;  // this level's frontier rows loaded by the bottom-up walks
   unsigned long long trace_n;  // records written to the optional trace
-  unsigned int bdepth;         // depth reached by the current batch (0 after seeding)
-  unsigned int pad1;
   // per-level totals of the run (tkc_last_run_stats)
   unsigned long long st_td_levels, st_td_frontier, st_td_arcs, st_td_new;
   unsigned long long st_bu_levels, st_bu_scan_v, st_bu_scan_a, st_bu_new, st_bu_frontier, st_bu_rows;
   unsigned long long st_seeded, st_cleared;
   unsigned long long st_compactions, st_compact_dropped;
   unsigned long long st_bu_swept;
-  int lcur;          // which list buffer holds the current frontier list (compaction swaps it alone)
-  int bgraph;        // several graphs: the graph of every search of the batch, -1 when they differ
 };
+constexpr int kCmdWords = (offsetof(Ctl, nl_packed) - offsetof(Ctl, step)) / 4;
 
 // State shared by all teams of one run.
 struct Shared {
@@ -170,10 +172,9 @@ struct RunParams {
   uint64_t vtx_stride;   // 32-bit words between the teams' lists and stamps
   uint64_t fb_stride;    // 32-bit words between the teams' frontier bitmaps
   Shared *sh;
-  // published k-th entry of each graph's list (seqlock: odd = being written)
-  unsigned int *x_seq;
-  unsigned long long *x_S;
-  uint32_t *x_r, *x_id;
+  // published k-th entry of each graph's list: {S, r << 32 | id}, r = 0 while
+  // the list is not full; read and written as one 128-bit word
+  ulonglong2 *x;
   // several graphs in one run, as their disjoint union (ng = 1: one graph)
   uint32_t ng;
   const uint32_t *gid;        // graph of each vertex (nullptr: every vertex in graph 0)
@@ -260,9 +261,7 @@ struct Workspace {
   unsigned int *g_stop = nullptr;   // per graph: NBCut stop reached
   unsigned long long *g_ctr = nullptr;  // 4 per graph
   Shared *sh = nullptr;
-  unsigned int *x_seq = nullptr;
-  unsigned long long *x_S = nullptr;
-  uint32_t *x_r = nullptr, *x_id = nullptr;
+  ulonglong2 *x = nullptr;          // per graph: the published k-th entry
   uint32_t top_cap = 0;   // entries of top_* (graphs x k)
   size_t out_cap = 0;     // bytes of out
   uint32_t ng_cap = 0;    // graphs of tied / g_ntop / g_ctr / x_*
