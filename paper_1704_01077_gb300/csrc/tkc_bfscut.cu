@@ -237,10 +237,12 @@ __device__ __forceinline__ u64 warp_or(u64 x) {
 }
 
 // Adds, for every slot bit of the 32 lanes' rows, the number of lanes with
-// the bit set and the sum of those lanes' `od` into the block counters.
+// the bit set and the sum of those lanes' `od` into the block counters.  (A
+// search finds a vertex once, so its sums stay below the graph's arcs and so
+// below 2^32; 64-bit shared-memory additions would be compare-and-swap loops.)
 template <int W>
 __device__ __forceinline__ void warp_count_slots(const u64 (&nw)[W], uint32_t od, unsigned *s_cnt,
-                                                 u64 *s_wsum, int lane) {
+                                                 unsigned *s_wsum, int lane) {
   uint32_t anyw = 0;
 #pragma unroll
   for (int j = 0; j < W; ++j) anyw |= (nw[j] != 0);
@@ -260,7 +262,7 @@ __device__ __forceinline__ void warp_count_slots(const u64 (&nw)[W], uint32_t od
     cmax = cv[jh] > cmax ? cv[jh] : cmax;
   }
   const uint32_t maxc = __reduce_max_sync(FULL, cmax);
-  u64 ws[2 * W];
+  uint32_t ws[2 * W];
 #pragma unroll
   for (int jh = 0; jh < 2 * W; ++jh) ws[jh] = 0;
   // about 6 instructions per half for a walk step or a plane, 1 more per plane
@@ -282,7 +284,7 @@ __device__ __forceinline__ void warp_count_slots(const u64 (&nw)[W], uint32_t od
     for (int p = 0; p < planes; ++p) {
       const uint32_t plane = __ballot_sync(FULL, (odm >> p) & 1u);
 #pragma unroll
-      for (int jh = 0; jh < 2 * W; ++jh) ws[jh] += (u64)__popc(colv[jh] & plane) << p;
+      for (int jh = 0; jh < 2 * W; ++jh) ws[jh] += (uint32_t)__popc(colv[jh] & plane) << p;
     }
   }
 #pragma unroll
@@ -408,7 +410,7 @@ __device__ __forceinline__ void record_levels(const RunParams &p, uint32_t w, co
 template <int W>
 struct Smem {
   unsigned cnt[64 * W];
-  u64 wsum[64 * W];
+  unsigned wsum[64 * W];
   u64 active[W];
   // epilogue scratch
   u64 tS[kTopMax];
@@ -730,7 +732,6 @@ __device__ __noinline__ void epilogue_level(const RunParams &p, Smem<W> &sm) {
     sm.ncand = 0;
     sm.nactive = 0;
   }
-  if (threadIdx.x < W) sm.active[threadIdx.x] = 0;
   if (threadIdx.x < 4) sm.acc[threadIdx.x] = 0;
   __syncthreads();
   // 1. per-slot level update
@@ -745,7 +746,6 @@ __device__ __noinline__ void epilogue_level(const RunParams &p, Smem<W> &sm) {
       p.res_S[sl.v] = key;
       p.res_r[sl.v] = (uint32_t)sl.nd;
       p.slots[s].state = 2;
-      atomicAdd(&sm.acc[0], 1ull);
       graph_count(p, sl.graph, 3, 1);
       offer_candidate(p, sm, key, (uint32_t)sl.nd, sl.v, sl.graph, x);
     } else {
@@ -772,20 +772,34 @@ __device__ __noinline__ void epilogue_level(const RunParams &p, Smem<W> &sm) {
     if (cont) x = thresh_of(p, p.ng == 1 ? 0u : sl.graph);
   }
   // 3. BFSCut test for the slots that continue
+  bool below = false;
   if (cont) {
-    const bool below = !p.nocut && !sl.nocut && x.have &&
+    below = !p.nocut && !sl.nocut && x.have &&
                        (p.harmonic ? harmonic_below(sl.H, sl.d, sl.nd, sl.g, sl.omega, x.S)
                                    : cut_exceeds(sl.S, sl.d, sl.nd, sl.g, sl.alpha, sl.omega, x.S, x.r));
     if (below) {
       p.slots[s].state = 2;
-      atomicAdd(&sm.acc[1], 1ull);
       graph_count(p, sl.graph, 2, 1);
     } else {
       p.slots[s] = sl;
-      atomicAdd(&sm.acc[2], sl.arcs);
       graph_count(p, sl.graph, 0, sl.arcs);
-      atomicOr(&sm.active[s >> 6], 1ull << (s & 63));
-      atomicAdd(&sm.nactive, 1u);
+    }
+  }
+  // the warp's slots together: a thread per slot, so a warp's continuing slots
+  // are half a word of the active mask (arcs are below 2^32: two 16-bit sums)
+  if (threadIdx.x < 64 * W) {
+    const bool stay = cont && !below;
+    const unsigned m = __ballot_sync(FULL, stay), mf = __ballot_sync(FULL, act && !cont), mc = __ballot_sync(FULL, below);
+    const uint32_t arcs = stay ? (uint32_t)sl.arcs : 0u;
+    const uint32_t lo = __reduce_add_sync(FULL, arcs & 0xffffu), hi = __reduce_add_sync(FULL, arcs >> 16);
+    if ((threadIdx.x & 31) == 0) {
+      reinterpret_cast<uint32_t *>(sm.active)[threadIdx.x >> 5] = m;
+      if (m) {
+        atomicAdd(&sm.nactive, (unsigned)__popc(m));
+        atomicAdd(&sm.acc[2], lo + ((u64)hi << 16));
+      }
+      if (mf) atomicAdd(&sm.acc[0], (u64)__popc(mf));
+      if (mc) atomicAdd(&sm.acc[1], (u64)__popc(mc));
     }
   }
   __syncthreads();
@@ -1086,7 +1100,7 @@ __device__ __noinline__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
       FL[s] = sv;
       FLoff[s] = (uint32_t)(arcs_total + arcs_pre);
       p.VL[s] = sv;
-      atomicOr(&sm.active[s >> 6], bit);
+      atomicOr(reinterpret_cast<uint32_t *>(sm.active) + (s >> 5), 1u << (s & 31));
     }
     uint32_t ncut;
     block_exscan(sm, cut ? 1u : 0u, &ncut);
@@ -1601,7 +1615,7 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
     for (int i = threadIdx.x; i < 64 * W; i += TPB) {
       if (sm.cnt[i]) {
         atomicAdd(&p.cnt[i], sm.cnt[i]);
-        atomicAdd(&p.wsum[i], sm.wsum[i]);
+        atomicAdd(&p.wsum[i], (u64)sm.wsum[i]);
       }
     }
     if (threadIdx.x == 0 && sm.acc[3]) {
