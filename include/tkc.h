@@ -80,11 +80,14 @@ typedef struct {
                               without cutting, so x starts from exact farness values (0 = none) */
   uint64_t timeout_cycles; /* budget of every device-side wait, in SM clock cycles (0 = default 2^34) */
   uint32_t teams;          /* independent groups of SMs, each running its own source batches and sharing
-                              the threshold and the k-lists (0 = library default: 1 in plain mode and below
-                              2^14 vertices; NBCut on one graph one team per 32 SMs; otherwise one per 16 SMs
-                              below 2^16 vertices and one per 8 SMs from 2^16 up).  With several teams on one
-                              graph the first batch runs alone on the whole grid, so that a threshold exists
-                              before the teams start. */
+                              the threshold and the k-lists (0 = library default: 1 in plain mode; below 2^14
+                              vertices up to 8; NBCut on one graph one team per 32 SMs; several graphs in one
+                              launch one per 4 SMs from 2^16 vertices up, as memory allows; complete searches up
+                              to one per batch; otherwise one per 16 SMs below 2^16 vertices and one per 8 SMs
+                              from 2^16 up).  Unless the schedule is deterministic or one source at a time, a
+                              batch of promising sources (as many as it takes for a full list) runs alone
+                              first, so that a threshold exists, and sources it abandons are dropped before
+                              the teams start. */
   uint32_t nb_levels;      /* TKC_ORDER_NB: most level sweeps of computeBoundsNB, 1..65535 (0 = 256) */
   uint32_t large_blocks;   /* threads per block of the search kernel: 0 = library choice (the larger blocks -- 1024
                               threads for 64- and 128-bit batches -- for batched searches on graphs of
@@ -264,7 +267,7 @@ int tkc_topk_harmonic_multi(tkc_ctx *ctx, tkc_graph *const *gs, uint32_t ng, uin
  * directed) gets the bound S(w) >= L(d(s,w)) - outdeg(w), L(i) = 2 x (vertices
  * within one level of i; directed: at most one level deeper) + the level
  * distance of all other vertices - 2, over R(s) including s.  The search runs
- * in rounds of options.teams batches of options.batch_bits sources (defaults: 8 x 64 from 2^16 vertices up,
+ * in rounds of options.teams batches of options.batch_bits sources (defaults: 4 x 128 from 2^16 vertices up,
  * else 1 x 256; batch_bits 1 = one source per round):
  * the unsearched vertices of smallest bound key floor(2^46 S_lb/(r-1)^2), ties
  * by their position in the initial order, and stops when that key exceeds the

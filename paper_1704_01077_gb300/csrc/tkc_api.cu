@@ -361,20 +361,31 @@ struct RunSetup {
   const u32 *g_base;        // first vertex of each graph (ng + 1 words)
 };
 
-// Teams used when the options leave it to the library: one team for small
-// graphs (a level is short and the whole GPU serves it), more for large ones
-// so that the latency of one team's level steps overlaps with the others.
-// NBCut on one graph examines few sources, each batch deeper: fewer, larger
-// teams (measured on R-MAT 22: 4 teams 357 ms, 9 teams 372 ms, 19 teams 411 ms).
-// Several graphs: four blocks per team, since a level of one of the graphs is
-// short (512 graphs of 1 000 to 200 000 vertices, 128-bit batches: 19 teams
-// 203 ms a call, 38 teams 184 ms).
+// Teams used when the options leave it to the library, so that the latency of
+// one team's level steps overlaps with the others'.  NBCut on one graph
+// examines few sources, each batch deeper: fewer, larger teams (measured on
+// R-MAT 22: 4 teams 357 ms, 9 teams 372 ms, 19 teams 411 ms).  Several graphs:
+// four blocks per team, since a level of one of the graphs is short (512
+// graphs of 1 000 to 200 000 vertices, 128-bit batches: 19 teams 203 ms a
+// call, 38 teams 184 ms).  Small graphs: teams of as many blocks as give every
+// warp of a sweep one group of 32 vertices, at most eight, since batches of
+// side-by-side teams cut against an older threshold.
 static u32 default_teams(u32 n, u32 B, u32 maxb, bool nb, u32 ng) {
-  if (B <= 1 || n < (1u << 14)) return 1;
+  if (B <= 1) return 1;
+  if (n < (1u << 14)) return std::max<u32>(1, std::min<u32>(8, maxb / std::max<u32>(8, (n + 511) / 512)));
   if (ng > 1 && n >= (1u << 16)) return std::max<u32>(1, maxb / 4);
   if (nb) return std::max<u32>(1, maxb / 32);
   if (n < (1u << 16)) return std::max<u32>(1, maxb / 16);
   return std::max<u32>(1, maxb / 8);  // eight blocks (SMs) per team, every SM used
+}
+
+// Complete searches (no cuts): the batches do not depend on one another, so
+// there are as many teams as batches -- down to one block each, which then has
+// no barrier to wait at -- while their rows and lists together fit L2.
+static u32 nocut_teams(u32 n, u32 B, u32 W, u32 maxb, u32 norder) {
+  const u64 fit = (96ull << 20) / ((u64)n * (32 * W + 24) + 1);
+  const u32 teams = std::max<u32>((u32)std::min<u64>(fit, maxb), default_teams(n, B, maxb, false, 1));
+  return std::max<u32>(1, std::min<u32>(teams, (norder + B - 1) / B));
 }
 
 // Whether a search may walk the in-degree labelling: batched searches of
@@ -398,7 +409,10 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   int maxb = max_coresident_blocks(ctx, rs.W);
   if (maxb <= 0) return TKC_ECUDA;
   const bool nb_one = rs.lb_key != nullptr && rs.ng == 1;
-  u32 T = rs.B <= 1 ? 1u : (o.teams ? o.teams : default_teams(g->n, rs.B, (u32)maxb, nb_one, rs.ng));
+  u32 T = rs.B <= 1 ? 1u
+          : o.teams ? o.teams
+          : rs.nocut && rs.ng == 1 ? nocut_teams(g->n, rs.B, (u32)rs.W, (u32)maxb, rs.norder)
+                                   : default_teams(g->n, rs.B, (u32)maxb, nb_one, rs.ng);
   // several graphs: every team's rows and lists cover the union, so as many
   // teams as a quarter of the device's memory holds
   if (rs.ng > 1 && !o.teams) {
@@ -526,7 +540,8 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   p.res_S = w.res_S;
   p.res_r = w.res_r;
   p.ctl = w.ctl;
-  int blocks = o.blocks ? (int)o.blocks : (int)std::max<u64>(8, ((u64)g->n + 511) / 512);
+  // each team: a warp of a sweep per 32 vertices, at least eight blocks
+  int blocks = o.blocks ? (int)o.blocks : (int)std::min<u64>(maxb, (u64)T * std::max<u64>(8, ((u64)g->n + 511) / 512));
   blocks = std::min(blocks, maxb);
   blocks = std::max<int>(T, blocks / (int)T * (int)T);  // a multiple of the team count
   // optional per-step trace for profiling: TKC_TRACE=<csv path>
@@ -545,7 +560,9 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   auto launch_phase = [&](u32 teams, Ctl *ctl) {
     p.teams = teams;
     p.ctl = ctl;
-    return run_bfscut(ctx, p, rs.W, std::max<int>((int)teams, blocks / (int)teams * (int)teams));
+    // (one team: no more blocks than it would have alone)
+    const int most = teams > 1 || o.blocks ? blocks : std::min<int>(blocks, std::max<int>(8, (int)((g->n + 511) / 512)));
+    return run_bfscut(ctx, p, rs.W, std::max<int>((int)teams, most / (int)teams * (int)teams));
   };
   if (opening) {
     if (pick) {
@@ -1571,15 +1588,15 @@ static int topk_bound(tkc_graph *g, uint32_t k, tkc_result *out) {
   }
   const u32 *order0 = nb ? g->nb_order : g->deg_order;
   const u32 n0 = nb ? g->n_src_nb : g->n_src_deg;
-  // defaults measured with NBBound on a 1000 x 1000 grid: 256 sources x 1 team 4.55 s, 256 x 2 4.16 s,
-  // 128 x 4 4.03 s, 64 x 8 3.48 s, 64 x 16 3.99 s (more sources per round refresh the bounds less often)
+  // defaults measured with NBBound on a 301 x 299 grid: 64 sources x 8 teams 122 ms, 128 x 4 111 ms,
+  // 256 x 2 110 ms, 64 x 16 131 ms (more sources per round refresh the bounds less often)
   const bool large = n >= (1u << 16);
-  const u32 B = o.batch_bits ? o.batch_bits : (large ? 64u : 256u);
+  const u32 B = o.batch_bits ? o.batch_bits : (large ? 128u : 256u);
   const u32 cap = std::min<u32>(n + 1, 65535u);  // levels per search (depth < n)
-  // teams run one batch each per round (0: one team below 2^16 vertices, else 8)
+  // teams run one batch each per round (0: one team below 2^16 vertices, else as many as make 512 sources)
   int maxb = max_coresident_blocks(ctx, words_for(B));
   if (maxb <= 0) return TKC_ECUDA;
-  const u32 T = std::max<u32>(1, std::min<u32>(B <= 1 ? 1u : (o.teams ? o.teams : (large ? 8u : 1u)), (u32)maxb));
+  const u32 T = std::max<u32>(1, std::min<u32>(B <= 1 ? 1u : (o.teams ? o.teams : (large ? 512u / B : 1u)), (u32)maxb));
   const u32 TB = T * B;  // sources per round
   TKC_RC(ensure_workspace(ctx, n, words_for(B), kk, 1, T));
   u64 *bS = nullptr, *key = nullptr, *Ltab = nullptr, *smax = nullptr, *bkeys = nullptr;
