@@ -30,6 +30,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "tkc_grid.cuh"
 #include "tkc_internal.cuh"
 
 namespace tkc {
@@ -57,6 +58,11 @@ unsigned grid_of(u64 work, unsigned tpb = 256, unsigned cap = 152 * 16) {
 
 enum : uint8_t { kFinished = 1, kHave = 2 };
 
+// Graphs up to this size run their sweeps in one launch (k_nb_sweeps); larger
+// ones fill the chip better with the gather and the level pass apart (they
+// need 32 and 64 registers).
+constexpr u32 kNbLoop = 1u << 17;
+
 // ---------------------------------------------------------------- gather
 
 __device__ __forceinline__ u64 warp_sum(u64 x) {
@@ -66,9 +72,10 @@ __device__ __forceinline__ u64 warp_sum(u64 x) {
 }
 
 // sum[v] = sum of prev[w] over out-neighbours w, capped at kCap; heavy rows
-// get 0 here and their segments are added by k_nb_gather_heavy.
-__global__ void k_nb_gather(u32 n, const u32 *__restrict__ off, const u32 *__restrict__ col,
-                            const u64 *__restrict__ prev, u64 *__restrict__ sum) {
+// are left alone when kSkipHeavy, else get 0 here; their segments are added by
+// nb_gather_heavy.
+template <bool kSkipHeavy>
+__device__ __forceinline__ void nb_gather(u32 n, const u32 *off, const u32 *col, const u64 *prev, u64 *sum) {
   const int lane = threadIdx.x & 31;
   const u64 nwarps = (u64)gridDim.x * (blockDim.x >> 5);
   for (u64 w = (u64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w * 32 < n; w += nwarps) {
@@ -99,13 +106,17 @@ __global__ void k_nb_gather(u32 n, const u32 *__restrict__ off, const u32 *__res
       part = warp_sum(part);
       if (lane == src) s = part;
     }
-    if (v < n) sum[v] = deg > kHeavy ? 0 : (s < kCap ? s : kCap);
+    if (v < n && !(kSkipHeavy && deg > kHeavy)) sum[v] = deg > kHeavy ? 0 : (s < kCap ? s : kCap);
   }
 }
 
-__global__ void k_nb_gather_heavy(u32 nseg, const u32 *__restrict__ seg_row, const u32 *__restrict__ seg_begin,
-                                  const u32 *__restrict__ off, const u32 *__restrict__ col,
-                                  const u64 *__restrict__ prev, u64 *__restrict__ sum) {
+__global__ void k_nb_gather(u32 n, const u32 *__restrict__ off, const u32 *__restrict__ col,
+                            const u64 *__restrict__ prev, u64 *__restrict__ sum) {
+  nb_gather<false>(n, off, col, prev, sum);
+}
+
+__device__ __forceinline__ void nb_gather_heavy(u32 nseg, const u32 *seg_row, const u32 *seg_begin, const u32 *off,
+                                                const u32 *col, const u64 *prev, u64 *sum) {
   const int lane = threadIdx.x & 31;
   const u64 nwarps = (u64)gridDim.x * (blockDim.x >> 5);
   for (u64 w = (u64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); w < nseg; w += nwarps) {
@@ -121,6 +132,12 @@ __global__ void k_nb_gather_heavy(u32 nseg, const u32 *__restrict__ seg_row, con
     part = warp_sum(part);
     if (lane == 0) atomicAdd(&sum[row], part < kCap ? part : kCap);
   }
+}
+
+__global__ void k_nb_gather_heavy(u32 nseg, const u32 *__restrict__ seg_row, const u32 *__restrict__ seg_begin,
+                                  const u32 *__restrict__ off, const u32 *__restrict__ col,
+                                  const u64 *__restrict__ prev, u64 *__restrict__ sum) {
+  nb_gather_heavy(nseg, seg_row, seg_begin, off, col, prev, sum);
 }
 
 // segment list of the heavy rows
@@ -171,11 +188,12 @@ __device__ __forceinline__ void candidate(u64 S, u64 r, bool &have, u64 &bS, u64
 // Level k: cur holds the gathered sums (k >= 2) and receives N~_k; prev2 holds
 // N~_{k-2}.  Unfinished vertices are counted into *left; an impossible
 // subtraction or an empty candidate set raises *err.
-__global__ void k_nb_level(u32 n, u32 k, u32 K, int directed, const u32 *__restrict__ gid,
-                           const uint8_t *__restrict__ gdir, const u32 *__restrict__ off,
-                           const u32 *__restrict__ alpha, const u32 *__restrict__ omega,
-                           const u64 *__restrict__ prev2, u64 *__restrict__ cur, NbState st, u32 *left,
-                           int *err) {
+// kZeroHeavy: prev2 of the heavy rows is zeroed once read (it receives the next
+// level's gathered sums, which start at 0).
+template <bool kZeroHeavy>
+__device__ __forceinline__ void nb_level(u32 n, u32 k, u32 K, int directed, const u32 *gid, const uint8_t *gdir,
+                                         const u32 *off, const u32 *alpha, const u32 *omega, u64 *prev2, u64 *cur,
+                                         const NbState &st, u32 *left, int *err) {
   u32 mine = 0;
   for (u32 v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
     const u64 deg = off[v + 1] - off[v];
@@ -202,6 +220,7 @@ __global__ void k_nb_level(u32 n, u32 k, u32 K, int directed, const u32 *__restr
       }
     }
     cur[v] = x;
+    if (kZeroHeavy && deg > kHeavy) prev2[v] = 0;
     uint8_t f = st.flag[v];
     if (f & kFinished) continue;
     bool have = f & kHave;
@@ -250,6 +269,44 @@ __global__ void k_nb_level(u32 n, u32 k, u32 K, int directed, const u32 *__restr
   }
   mine = __reduce_add_sync(FULL, mine);
   if ((threadIdx.x & 31) == 0 && mine) atomicAdd(left, mine);
+}
+
+__global__ void k_nb_level(u32 n, u32 k, u32 K, int directed, const u32 *__restrict__ gid,
+                           const uint8_t *__restrict__ gdir, const u32 *__restrict__ off,
+                           const u32 *__restrict__ alpha, const u32 *__restrict__ omega, u64 *__restrict__ prev2,
+                           u64 *__restrict__ cur, NbState st, u32 *left, int *err) {
+  nb_level<false>(n, k, K, directed, gid, gdir, off, alpha, omega, prev2, cur, st, left, err);
+}
+
+// All sweeps of a small graph in one cooperative launch: two barriers a sweep
+// instead of three launches, a copy and a host wait (about 20 us, and up to
+// 256 sweeps on a street network).  N0, N1, N2: the count arrays, N~_i in
+// N[i % 3]; left[2]: unfinished vertices, two zero words used in turn; *levels
+// = sweeps run.
+constexpr int kNbTPB = 256;
+__global__ void __launch_bounds__(kNbTPB) k_nb_sweeps(u32 n, u32 K, int directed, const u32 *gid, const uint8_t *gdir,
+                                                      const u32 *off, const u32 *col, const u32 *alpha,
+                                                      const u32 *omega, u64 *N0, u64 *N1, u64 *N2, NbState st,
+                                                      u32 nseg, const u32 *seg_row, const u32 *seg_begin, u32 *left,
+                                                      u32 *levels, int *err, GridBar *bar, u64 timeout) {
+  for (u32 k = 1; k <= K; ++k) {
+    u64 *cur = k % 3 == 0 ? N0 : k % 3 == 1 ? N1 : N2;
+    u64 *prev1 = k % 3 == 0 ? N2 : k % 3 == 1 ? N0 : N1;
+    u64 *prev2 = k % 3 == 0 ? N1 : k % 3 == 1 ? N2 : N0;
+    if (k >= 2) {
+      nb_gather<true>(n, off, col, prev1, cur);
+      if (nseg) nb_gather_heavy(nseg, seg_row, seg_begin, off, col, prev1, cur);
+      if (!grid_sync(bar, timeout, [] {})) return;
+    }
+    u32 *l = left + (k & 1);
+    nb_level<true>(n, k, K, directed, gid, gdir, off, alpha, omega, prev2, cur, st, l, err);
+    if (!grid_sync(bar, timeout, [&] {
+          left[(k & 1) ^ 1] = 0;
+          *levels = k;
+        }))
+      return;
+    if (*(volatile u32 *)l == 0) return;
+  }
 }
 
 __global__ void k_nb_init(u32 n, NbState st, u64 *prev1, u64 *prev2) {
@@ -409,22 +466,49 @@ int ensure_nb_bounds(tkc_graph *g, u32 K, const u32 *gid, const uint8_t *gdir) {
   // sweeps: N[i % 3] holds N~_i
   TKC_LAUNCH(k_nb_init<<<grid_of(n), 256, 0, st>>>(n, s, N[0], N[2]));
   u32 levels = 0;
-  const unsigned gwarps = grid_of((u64)((n + 31) / 32) * 32, 256);
-  for (u32 k = 1; k <= K; ++k) {
-    u64 *cur = N[k % 3], *prev1 = N[(k + 2) % 3], *prev2 = N[(k + 1) % 3];
-    if (k >= 2) {
-      TKC_LAUNCH(k_nb_gather<<<gwarps, 256, 0, st>>>(n, g->off, g->col, prev1, cur));
-      if (nseg) TKC_LAUNCH(k_nb_gather_heavy<<<grid_of((u64)nseg * 32, 256), 256, 0, st>>>(
-                    nseg, seg_row, seg_begin, g->off, g->col, prev1, cur));
+  int loop_err = 0;
+  if (n <= kNbLoop) {
+    // (the sums of heavy rows at level 2 start from N[2], zeroed by k_nb_init)
+    GridBar *bar = nullptr;
+    TKC_TRY(dev_malloc(&bar, sizeof(GridBar) + 4 * sizeof(u32), st));
+    TKC_TRY(cudaMemsetAsync(bar, 0, sizeof(GridBar) + 4 * sizeof(u32), st));
+    u32 *words = reinterpret_cast<u32 *>(bar + 1), *d_levels = words + 2;
+    u64 timeout = grid_timeout(ctx);
+    void *args[] = {(void *)&n,       (void *)&K,    (void *)&g->directed, (void *)&gid,     (void *)&gdir,
+                    (void *)&g->off,  (void *)&g->col, (void *)&g->alpha,  (void *)&g->omega, (void *)&N[0],
+                    (void *)&N[1],    (void *)&N[2], (void *)&s,           (void *)&nseg,    (void *)&seg_row,
+                    (void *)&seg_begin, (void *)&words, (void *)&d_levels, (void *)&err,     (void *)&bar,
+                    (void *)&timeout};
+    const int blocks = grid_blocks(ctx, k_nb_sweeps, kNbTPB, n);
+    if (blocks <= 0) return TKC_ECUDA;
+    note_launches(1);
+    TKC_TRY(cudaLaunchCooperativeKernel((const void *)k_nb_sweeps, dim3(blocks), dim3(kNbTPB), args, 0, st));
+    struct {
+      GridBar bar;
+      u32 left[2], levels;
+    } h;
+    TKC_TRY(read_back(&h, bar, sizeof(GridBar) + 3 * sizeof(u32), st));
+    TKC_TRY(cudaFreeAsync(bar, st));
+    loop_err = h.bar.err;
+    levels = h.levels;
+  } else {
+    const unsigned gwarps = grid_of((u64)((n + 31) / 32) * 32, 256);
+    for (u32 k = 1; k <= K; ++k) {
+      u64 *cur = N[k % 3], *prev1 = N[(k + 2) % 3], *prev2 = N[(k + 1) % 3];
+      if (k >= 2) {
+        TKC_LAUNCH(k_nb_gather<<<gwarps, 256, 0, st>>>(n, g->off, g->col, prev1, cur));
+        if (nseg) TKC_LAUNCH(k_nb_gather_heavy<<<grid_of((u64)nseg * 32, 256), 256, 0, st>>>(
+                      nseg, seg_row, seg_begin, g->off, g->col, prev1, cur));
+      }
+      TKC_TRY(cudaMemsetAsync(left, 0, sizeof(u32), st));
+      TKC_LAUNCH(k_nb_level<<<grid_of(n), 256, 0, st>>>(n, k, K, g->directed, gid, gdir, g->off, g->alpha, g->omega,
+                                                        prev2, cur, s, left, err));
+      TKC_TRY(cudaGetLastError());
+      u32 h_left = 0;
+      TKC_TRY(read_back(&h_left, left, sizeof(u32), st));
+      levels = k;
+      if (h_left == 0) break;
     }
-    TKC_TRY(cudaMemsetAsync(left, 0, sizeof(u32), st));
-    TKC_LAUNCH(k_nb_level<<<grid_of(n), 256, 0, st>>>(n, k, K, g->directed, gid, gdir, g->off, g->alpha, g->omega,
-                                                      prev2, cur, s, left, err));
-    TKC_TRY(cudaGetLastError());
-    u32 h_left = 0;
-    TKC_TRY(read_back(&h_left, left, sizeof(u32), st));
-    levels = k;
-    if (h_left == 0) break;
   }
   TKC_LAUNCH(k_nb_keys<<<grid_of(n), 256, 0, st>>>(n, s, g->nb_S, g->nb_r, g->nb_key, g->nb_hkey, err));
   int h_err = 0;
@@ -433,6 +517,7 @@ int ensure_nb_bounds(tkc_graph *g, u32 K, const u32 *gid, const uint8_t *gdir) {
   void *frees[] = {s.c, s.P, s.bS, s.bR, s.flag, s.hU, segpos, seg_row, seg_begin, tmp, left, err};
   for (void *p : frees)
     if (p) TKC_TRY(cudaFreeAsync(p, st));
+  if (loop_err) return loop_err;
   if (h_err) return TKC_EGRAPH;
   g->nb_levels = levels;
   g->nb_cap = K;

@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "tkc_arcs.cuh"
+#include "tkc_grid.cuh"
 #include "tkc_internal.cuh"
 
 namespace tkc {
@@ -57,37 +58,46 @@ __global__ void k_trim_init(const u32 *off, const u32 *ioff, u32 n, u32 *outd, u
 }
 
 // Removes vertices without an active in-arc or out-arc (each is its own SCC)
-// and lowers the counters of their neighbours.  One warp per removed vertex
-// walks its arcs.
-__global__ void k_trim_round(const u32 *off, const u32 *col, const u32 *ioff, const u32 *icol, u32 n, u32 *outd,
-                             u32 *ind, uint8_t *active, u32 *comp, u32 *changed) {
+// and lowers the counters of their neighbours, round after round until none is
+// left (one cooperative launch).  One warp per removed vertex walks its arcs.
+// changed: two zero words, used in turn.
+constexpr int kLoopTPB = 256;  // threads per block of the launches that loop over rounds
+
+__global__ void __launch_bounds__(kLoopTPB) k_trim(const u32 *off, const u32 *col, const u32 *ioff, const u32 *icol,
+                                                   u32 n, u32 *outd, u32 *ind, uint8_t *active, u32 *comp,
+                                                   u32 *changed, GridBar *bar, u64 timeout) {
   const int lane = threadIdx.x & 31;
-  for (u32 base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; base < n; base += gridDim.x * blockDim.x) {
-    u32 v = base + lane;
-    bool rm = v < n && active[v] && (outd[v] == 0 || ind[v] == 0);
-    if (rm) {
-      active[v] = 0;
-      comp[v] = v;
+  for (u32 round = 0;; ++round) {
+    u32 *ch = changed + (round & 1);
+    for (u32 base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; base < n; base += gridDim.x * blockDim.x) {
+      u32 v = base + lane;
+      bool rm = v < n && active[v] && (outd[v] == 0 || ind[v] == 0);
+      if (rm) {
+        active[v] = 0;
+        comp[v] = v;
+      }
+      u32 mask = __ballot_sync(FULL, rm);
+      if (mask && lane == 0) *ch = 1;
+      while (mask) {
+        int src = __ffs(mask) - 1;
+        mask &= mask - 1;
+        u32 x = base + src;
+        for (u32 i = off[x] + lane; i < off[x + 1]; i += 32) atomicSub(&ind[col[i]], 1u);
+        for (u32 i = ioff[x] + lane; i < ioff[x + 1]; i += 32) atomicSub(&outd[icol[i]], 1u);
+      }
     }
-    u32 mask = __ballot_sync(FULL, rm);
-    if (mask && lane == 0) *changed = 1;
-    while (mask) {
-      int src = __ffs(mask) - 1;
-      mask &= mask - 1;
-      u32 x = base + src;
-      for (u32 i = off[x] + lane; i < off[x + 1]; i += 32) atomicSub(&ind[col[i]], 1u);
-      for (u32 i = ioff[x] + lane; i < ioff[x + 1]; i += 32) atomicSub(&outd[icol[i]], 1u);
-    }
+    // the other word was read by every block before it arrived here
+    if (!grid_sync(bar, timeout, [&] { changed[(round & 1) ^ 1] = 0; })) return;
+    if (*(volatile u32 *)ch == 0) return;
   }
 }
 
 // ---------------------------------------------------------------- reach BFS, one cooperative launch
 
-// Control block of the reach BFS: grid barrier alone in its cache line, then
-// the frontier queues' packed counters (count << 38 | out-arcs).
+// Control block of the reach BFS: grid barrier, then the frontier queues'
+// packed counters (count << 38 | out-arcs).
 struct BfsCtl {
-  unsigned bar_count, bar_gen, bar_pad[30];
-  int err;
+  GridBar bar;
   unsigned level;
   unsigned long long q[2];
 };
@@ -95,55 +105,6 @@ struct BfsCtl {
 constexpr int kBfsThreads = 512;
 constexpr int kQShift = 38;
 constexpr u64 kQArcs = (1ull << kQShift) - 1;
-
-__device__ __forceinline__ unsigned ld_acq(const unsigned *p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_rel(unsigned *p, unsigned v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// Grid barrier of the cooperative launch; the last block to arrive runs
-// `epi` (thread 0) first.  Every wait is bounded: on expiry the kernel
-// records TKC_ETIMEOUT and returns false, as do all blocks once it is set.
-template <typename Epi>
-__device__ bool bfs_sync(BfsCtl *c, u64 timeout, Epi epi) {
-  __shared__ int s_last;
-  __shared__ unsigned s_gen;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    s_gen = ld_acq(&c->bar_gen);
-    __threadfence();
-    s_last = atomicAdd(&c->bar_count, 1u) + 1u == gridDim.x;
-  }
-  __syncthreads();
-  if (s_last) {
-    if (threadIdx.x == 0) {
-      __threadfence();
-      epi();
-      c->bar_count = 0;
-      __threadfence();
-      st_rel(&c->bar_gen, s_gen + 1u);
-    }
-  } else if (threadIdx.x == 0) {
-    const long long t0 = clock64();
-    unsigned ns = 32;
-    while (ld_acq(&c->bar_gen) == s_gen) {
-      if (*(volatile int *)&c->err) break;
-      if ((u64)(clock64() - t0) > timeout) {
-        atomicCAS(&c->err, 0, TKC_ETIMEOUT);
-        break;
-      }
-      __nanosleep(ns);
-      if (ns < 256) ns <<= 1;
-    }
-    __threadfence();
-  }
-  __syncthreads();
-  return *(volatile int *)&c->err == 0;
-}
 
 // Appends the lanes with `pred` to a queue whose counter packs count << 38 |
 // out-arcs (one atomic per warp); qo[pos] = the arcs of the entries before.
@@ -254,7 +215,7 @@ __global__ void __launch_bounds__(kBfsThreads) k_bfs_reach(const u32 *off, const
         q_append(got, v, got ? off[v + 1] - off[v] : 0u, npk, NQ, NQO, lane);
       }
     }
-    const bool ok = bfs_sync(c, timeout, [&] {
+    const bool ok = grid_sync(&c->bar, timeout, [&] {
       c->q[cur] = 0;
       c->level = step;
     });
@@ -316,7 +277,7 @@ int bfs_reach(tkc_ctx *ctx, const u32 *off, const u32 *col, const u32 *roff, con
   note_launches(1);
   TKC_TRY(cudaLaunchCooperativeKernel((const void *)k_bfs_reach, dim3(blocks), dim3(kBfsThreads), args, 0, st));
   int err = 0;
-  TKC_TRY(read_back(&err, &c->err, sizeof(int), st));
+  TKC_TRY(read_back(&err, &c->bar.err, sizeof(int), st));
   TKC_TRY(cudaFreeAsync(q, st));
   TKC_TRY(cudaFreeAsync(qo, st));
   TKC_TRY(cudaFreeAsync(c, st));
@@ -396,74 +357,79 @@ __global__ void k_fwbw_mark_many(const u32 *fw, const u32 *bw, const u32 *gid, c
 
 // ---------------------------------------------------------------- colouring
 
-__global__ void k_color_init(const uint8_t *active, u32 n, u32 *color, u32 *found, u32 *cnt) {
-  u32 c = 0;
-  for (u32 v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+// One colouring round over the active vertices, one cooperative launch: the
+// colours (the largest id that reaches a vertex) propagate along arcs until
+// nothing changes, then `found` spreads backwards from the roots among
+// vertices of one colour, and what was found is assigned.
+// changed: two zero words, used in turn.
+__global__ void __launch_bounds__(kLoopTPB) k_color_round(const u32 *off, const u32 *col, const u32 *ioff,
+                                                          const u32 *icol, u32 n, uint8_t *active, u32 *color,
+                                                          u32 *found, u32 *comp, u32 *changed, GridBar *bar,
+                                                          u64 timeout) {
+  const int lane = threadIdx.x & 31;
+  const u32 first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+  for (u32 v = first; v < n; v += step) {
     color[v] = active[v] ? v : INF;
     found[v] = 0;
-    c += active[v];
   }
-  c = __reduce_add_sync(FULL, c);
-  if ((threadIdx.x & 31) == 0 && c) atomicAdd(cnt, c);
-}
-
-// colour[w] = max(colour[w], colour[v]) over active arcs v -> w
-__global__ void k_color_prop(const u32 *off, const u32 *col, u32 n, const uint8_t *active, u32 *color,
-                             u32 *changed) {
-  const int lane = threadIdx.x & 31;
-  for (u32 base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; base < n; base += gridDim.x * blockDim.x) {
-    u32 v = base + lane;
-    u32 mask = __ballot_sync(FULL, v < n && active[v]);
-    u32 ch = 0;
-    while (mask) {
-      int src = __ffs(mask) - 1;
-      mask &= mask - 1;
-      u32 x = base + src;
-      u32 cx = color[x];
-      for (u32 i = off[x] + lane; i < off[x + 1]; i += 32) {
-        u32 w = col[i];
-        if (active[w] && color[w] < cx) {
-          atomicMax(&color[w], cx);
-          ch = 1;
+  if (!grid_sync(bar, timeout, [] {})) return;
+  u32 round = 0;
+  // colour[w] = max(colour[w], colour[v]) over active arcs v -> w
+  for (;; ++round) {
+    u32 *chg = changed + (round & 1);
+    for (u32 base = first & ~31u; base < n; base += step) {
+      const u32 v = base + lane;
+      u32 mask = __ballot_sync(FULL, v < n && active[v]);
+      u32 ch = 0;
+      while (mask) {
+        const int src = __ffs(mask) - 1;
+        mask &= mask - 1;
+        const u32 x = base + src;
+        const u32 cx = color[x];
+        for (u32 i = off[x] + lane; i < off[x + 1]; i += 32) {
+          const u32 w = col[i];
+          if (active[w] && color[w] < cx) {
+            atomicMax(&color[w], cx);
+            ch = 1;
+          }
         }
       }
+      if (__any_sync(FULL, ch) && lane == 0) *chg = 1;
     }
-    if (__any_sync(FULL, ch) && lane == 0) *changed = 1;
+    if (!grid_sync(bar, timeout, [&] { changed[(round & 1) ^ 1] = 0; })) return;
+    if (*(volatile u32 *)chg == 0) break;
   }
-}
-
-__global__ void k_roots(const uint8_t *active, const u32 *color, u32 n, u32 *found) {
-  for (u32 v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
+  ++round;
+  // the roots
+  for (u32 v = first; v < n; v += step)
     if (active[v] && color[v] == v) found[v] = 1;
-}
-
-// found spreads backwards (along in-arcs) among vertices of the same colour
-__global__ void k_back_prop(const u32 *ioff, const u32 *icol, u32 n, const uint8_t *active, const u32 *color,
-                            u32 *found, u32 *changed) {
-  const int lane = threadIdx.x & 31;
-  for (u32 base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; base < n; base += gridDim.x * blockDim.x) {
-    u32 v = base + lane;
-    u32 mask = __ballot_sync(FULL, v < n && active[v] && found[v]);
-    u32 ch = 0;
-    while (mask) {
-      int src = __ffs(mask) - 1;
-      mask &= mask - 1;
-      u32 x = base + src;
-      u32 cx = color[x];
-      for (u32 i = ioff[x] + lane; i < ioff[x + 1]; i += 32) {
-        u32 u = icol[i];
-        if (active[u] && color[u] == cx && !found[u]) {
-          found[u] = 1;
-          ch = 1;
+  if (!grid_sync(bar, timeout, [] {})) return;
+  // found spreads along in-arcs among vertices of the same colour
+  for (;; ++round) {
+    u32 *chg = changed + (round & 1);
+    for (u32 base = first & ~31u; base < n; base += step) {
+      const u32 v = base + lane;
+      u32 mask = __ballot_sync(FULL, v < n && active[v] && found[v]);
+      u32 ch = 0;
+      while (mask) {
+        const int src = __ffs(mask) - 1;
+        mask &= mask - 1;
+        const u32 x = base + src;
+        const u32 cx = color[x];
+        for (u32 i = ioff[x] + lane; i < ioff[x + 1]; i += 32) {
+          const u32 u = icol[i];
+          if (active[u] && color[u] == cx && !found[u]) {
+            found[u] = 1;
+            ch = 1;
+          }
         }
       }
+      if (__any_sync(FULL, ch) && lane == 0) *chg = 1;
     }
-    if (__any_sync(FULL, ch) && lane == 0) *changed = 1;
+    if (!grid_sync(bar, timeout, [&] { changed[(round & 1) ^ 1] = 0; })) return;
+    if (*(volatile u32 *)chg == 0) break;
   }
-}
-
-__global__ void k_color_assign(u32 n, uint8_t *active, const u32 *color, const u32 *found, u32 *comp) {
-  for (u32 v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
+  for (u32 v = first; v < n; v += step)
     if (active[v] && found[v]) {
       comp[v] = color[v];
       active[v] = 0;
@@ -612,7 +578,7 @@ __global__ void k_sinks(const u32 *wgt, const u32 *soff, u32 n, u32 *rem, u32 *l
 // Evaluates alpha/omega of the ready SCCs (all successors done).  A lane
 // reduces over the successors of its own SCC when there are at most 32; the
 // whole warp over longer successor lists.
-__global__ void k_dp_eval(const u32 *list, u32 cnt, const u32 *soff, const u32 *succ, const u32 *wgt,
+__device__ __forceinline__ void dp_eval(const u32 *list, u32 cnt, const u32 *soff, const u32 *succ, const u32 *wgt,
                           const u32 *dist_from_big, const u32 *dist_to_big, u32 big, u64 reach_big, u32 n, u64 *A,
                           u64 *O) {
   const int lane = threadIdx.x & 31;
@@ -686,8 +652,8 @@ __device__ __forceinline__ void ready_append(bool rel, u32 p, u32 *next, u32 *ne
 // Releases the predecessors of the SCCs just evaluated: an SCC whose last
 // unevaluated successor this was joins the next ready list.  A lane walks
 // lists of at most 32, the warp longer ones; lists above kDpHuge are left to
-// k_dp_release_huge (listed in huge[]).
-__global__ void k_dp_release(const u32 *list, u32 cnt, const u32 *poff, const u32 *pred, u32 *rem, u32 *next,
+// dp_release_huge (listed in huge[]).
+__device__ __forceinline__ void dp_release(const u32 *list, u32 cnt, const u32 *poff, const u32 *pred, u32 *rem, u32 *next,
                              u32 *next_cnt, u32 *huge, u32 *nhuge) {
   const int lane = threadIdx.x & 31;
   for (u32 base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; base < cnt; base += gridDim.x * blockDim.x) {
@@ -732,10 +698,9 @@ __global__ void k_dp_release(const u32 *list, u32 cnt, const u32 *poff, const u3
 }
 
 // The listed SCCs with more than kDpHuge predecessors, each by the whole grid.
-__global__ void k_dp_release_huge(const u32 *huge, const u32 *nhuge, const u32 *poff, const u32 *pred, u32 *rem,
+__device__ __forceinline__ void dp_release_huge(const u32 *huge, u32 nh, const u32 *poff, const u32 *pred, u32 *rem,
                                   u32 *next, u32 *next_cnt) {
   const int lane = threadIdx.x & 31;
-  const u32 nh = *nhuge;
   for (u32 h = 0; h < nh; ++h) {
     const u32 c = huge[h];
     const u32 b = poff[c], e = poff[c + 1];
@@ -748,6 +713,36 @@ __global__ void k_dp_release_huge(const u32 *huge, const u32 *nhuge, const u32 *
         rel = atomicSub(&rem[p], 1u) == 1u;
       }
       ready_append(rel, p, next, next_cnt, lane);
+    }
+  }
+}
+
+// Sinks first until every SCC is evaluated, one cooperative launch: a round
+// evaluates the ready list and releases the predecessors into the next one
+// (and, when there are any, the long predecessor lists by the whole grid).
+// cnt[3]: list lengths, round r's in cnt[r % 2], and unused; nhuge[3]: in turn.
+__global__ void __launch_bounds__(kLoopTPB) k_dp(u32 *listA, u32 *listB, u32 *cnt, const u32 *soff, const u32 *succ,
+                                                 const u32 *poff, const u32 *pred, const u32 *wgt,
+                                                 const u32 *dist_from_big, const u32 *dist_to_big, u32 big,
+                                                 u64 reach_big, u32 n, u64 *A, u64 *O, u32 *rem, u32 *huge, u32 *nhuge,
+                                                 GridBar *bar, u64 timeout) {
+  for (u32 r = 0;; ++r) {
+    const u32 c = *(volatile u32 *)&cnt[r & 1];
+    if (c == 0) return;
+    const u32 *cur = r & 1 ? listB : listA;
+    u32 *next = r & 1 ? listA : listB, *next_cnt = &cnt[(r & 1) ^ 1], *nh = &nhuge[r % 3];
+    dp_eval(cur, c, soff, succ, wgt, dist_from_big, dist_to_big, big, reach_big, n, A, O);
+    dp_release(cur, c, poff, pred, rem, next, next_cnt, huge, nh);
+    // every block has read cnt[r % 2] and, a round ago, nhuge[(r + 2) % 3]
+    if (!grid_sync(bar, timeout, [&] {
+          cnt[r & 1] = 0;
+          nhuge[(r + 2) % 3] = 0;
+        }))
+      return;
+    const u32 m = *(volatile u32 *)nh;
+    if (m) {
+      dp_release_huge(huge, m, poff, pred, rem, next, next_cnt);
+      if (!grid_sync(bar, timeout, [] {})) return;
     }
   }
 }
@@ -809,18 +804,36 @@ int reach_directed_gpu(tkc_graph *g, const u32 *gid, u32 ng) {
   TKC_TRY(b.get(&best, 1));
   int rc = TKC_OK;
   u32 pivot0 = INF;  // the first pivot, whose full forward and backward reach fw/bw keep
+  GridBar *bar = nullptr;
+  TKC_TRY(b.get(&bar, 1));
+  TKC_TRY(cudaMemsetAsync(bar, 0, sizeof(GridBar), st));
+  const u64 timeout = grid_timeout(g->ctx);
+  // launches that loop over rounds: the device barrier's error word is read
+  // with the next host read
+  auto loop_launch = [&](const void *kernel, int blocks, void **args) {
+    if (blocks <= 0) return cudaErrorCooperativeLaunchTooLarge;
+    note_launches(1);
+    return cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(kLoopTPB), args, 0, st);
+  };
+  auto loop_error = [&]() {
+    int e = 0;
+    cudaError_t ce = read_back(&e, &bar->err, sizeof(int), st);
+    if (ce != cudaSuccess) {
+      tkc_set_last_cuda_error(ce, "readback", __FILE__, __LINE__);
+      return (int)TKC_ECUDA;
+    }
+    return e;
+  };
   TKC_LAUNCH(k_trim_init<<<grid_of(n), 256, 0, st>>>(g->off, g->ioff, n, outd, ind, active));
   for (int round = 0;; ++round) {
     // trim until stable
-    for (int it = 0;; ++it) {
-      if (it > (int)n + 1) return TKC_ETIMEOUT;
-      TKC_TRY(cudaMemsetAsync(flag, 0, sizeof(u32), st));
-      TKC_LAUNCH(k_trim_round<<<grid_of(n), 256, 0, st>>>(g->off, g->col, g->ioff, g->icol, n, outd, ind, active,
-                                                          comp, flag));
-      if (!read_u32(flag, st, &rc)) break;
-      TKC_RC(rc);
+    {
+      TKC_TRY(cudaMemsetAsync(flag, 0, 2 * sizeof(u32), st));
+      u64 to = timeout;
+      void *args[] = {(void *)&g->off, (void *)&g->col, (void *)&g->ioff, (void *)&g->icol, (void *)&n, (void *)&outd,
+                      (void *)&ind, (void *)&active, (void *)&comp, (void *)&flag, (void *)&bar, (void *)&to};
+      TKC_TRY(loop_launch((const void *)k_trim, grid_blocks(g->ctx, k_trim, kLoopTPB, n), args));
     }
-    TKC_RC(rc);
     // pivot of the largest remaining SCC candidate
     TKC_TRY(cudaMemsetAsync(best, 0, sizeof(u64), st));
     TKC_LAUNCH(k_pivot<<<grid_of(n), 256, 0, st>>>(outd, ind, active, n, best));
@@ -861,27 +874,17 @@ int reach_directed_gpu(tkc_graph *g, const u32 *gid, u32 ng) {
       continue;  // trim again, then colour
     }
     // colouring round over the remaining vertices
-    TKC_TRY(cudaMemsetAsync(flag + 1, 0, sizeof(u32), st));
-    TKC_LAUNCH(k_color_init<<<grid_of(n), 256, 0, st>>>(active, n, color, found, flag + 1));
-    for (int it = 0;; ++it) {
-      if (it > (int)n + 1) return TKC_ETIMEOUT;
-      TKC_TRY(cudaMemsetAsync(flag, 0, sizeof(u32), st));
-      TKC_LAUNCH(k_color_prop<<<grid_of(n), 256, 0, st>>>(g->off, g->col, n, active, color, flag));
-      if (!read_u32(flag, st, &rc)) break;
-      TKC_RC(rc);
+    {
+      TKC_TRY(cudaMemsetAsync(flag, 0, 2 * sizeof(u32), st));
+      u64 to = timeout;
+      void *args[] = {(void *)&g->off, (void *)&g->col, (void *)&g->ioff, (void *)&g->icol, (void *)&n,
+                      (void *)&active, (void *)&color, (void *)&found, (void *)&comp, (void *)&flag, (void *)&bar,
+                      (void *)&to};
+      TKC_TRY(loop_launch((const void *)k_color_round, grid_blocks(g->ctx, k_color_round, kLoopTPB, n), args));
+      TKC_RC(loop_error());  // a round that ran out of its budget would repeat for ever
     }
-    TKC_RC(rc);
-    TKC_LAUNCH(k_roots<<<grid_of(n), 256, 0, st>>>(active, color, n, found));
-    for (int it = 0;; ++it) {
-      if (it > (int)n + 1) return TKC_ETIMEOUT;
-      TKC_TRY(cudaMemsetAsync(flag, 0, sizeof(u32), st));
-      TKC_LAUNCH(k_back_prop<<<grid_of(n), 256, 0, st>>>(g->ioff, g->icol, n, active, color, found, flag));
-      if (!read_u32(flag, st, &rc)) break;
-      TKC_RC(rc);
-    }
-    TKC_RC(rc);
-    TKC_LAUNCH(k_color_assign<<<grid_of(n), 256, 0, st>>>(n, active, color, found, comp));
   }
+  TKC_RC(loop_error());
   TKC_TRY(cudaMemcpyAsync(g->comp, comp, (size_t)n * sizeof(u32), cudaMemcpyDeviceToDevice, st));
   // component sizes and the biggest SCC
   TKC_TRY(b.get(&wgt, n));
@@ -905,7 +908,7 @@ int reach_directed_gpu(tkc_graph *g, const u32 *gid, u32 ng) {
   }
   TKC_TRY(cudaMemsetAsync(flag, 0, sizeof(u32), st));
   TKC_LAUNCH(k_count_reached<<<grid_of(n), 256, 0, st>>>(fw, n, flag));
-  const u64 reach_big = read_u32(flag, st, &rc);
+  u64 reach_big = read_u32(flag, st, &rc);
   TKC_RC(rc);
   // condensation arcs, sorted by (cu, cv) and deduplicated
   const unsigned cross_grid = grid_of(arc_threads(g->arcs));
@@ -952,30 +955,23 @@ int reach_directed_gpu(tkc_graph *g, const u32 *gid, u32 ng) {
   TKC_TRY(b.get(&listB, n));
   TKC_TRY(b.get(&A, n));
   TKC_TRY(b.get(&O, n));
-  TKC_TRY(cudaMemsetAsync(flag, 0, 2 * sizeof(u32), st));
-  TKC_LAUNCH(k_sinks<<<grid_of(n), 256, 0, st>>>(wgt, soff, n, rem, listA, flag));
-  u32 cnt = read_u32(flag, st, &rc);
-  TKC_RC(rc);
-  u32 *cur_list = listA, *nxt_list = listB, *huge = nullptr;
+  u32 *huge = nullptr, *cnt = nullptr;
   TKC_TRY(b.get(&huge, (size_t)mu / kDpHuge + 1));
-  for (u32 round = 0; cnt > 0; ++round) {
-    if (round > n) return TKC_ETIMEOUT;
-    TKC_TRY(cudaMemsetAsync(flag + 1, 0, 2 * sizeof(u32), st));
-    TKC_LAUNCH(k_dp_eval<<<grid_of(cnt), 256, 0, st>>>(cur_list, cnt, soff, sv, wgt, fw, bw, big, reach_big, n, A,
-                                                         O));
-    TKC_LAUNCH(k_dp_release<<<grid_of(cnt), 256, 0, st>>>(cur_list, cnt, poff, pred, rem, nxt_list, flag + 1, huge,
-                                                            flag + 2));
-    TKC_LAUNCH(k_dp_release_huge<<<grid_of((u64)mu / 4 + 1), 256, 0, st>>>(huge, flag + 2, poff, pred, rem,
-                                                                             nxt_list, flag + 1));
-    TKC_TRY(cudaGetLastError());
-    cnt = read_u32(flag + 1, st, &rc);
-    TKC_RC(rc);
-    std::swap(cur_list, nxt_list);
+  TKC_TRY(b.get(&cnt, 6));
+  TKC_TRY(cudaMemsetAsync(cnt, 0, 6 * sizeof(u32), st));
+  TKC_LAUNCH(k_sinks<<<grid_of(n), 256, 0, st>>>(wgt, soff, n, rem, listA, cnt));
+  {
+    u32 *nhuge = cnt + 3;
+    u64 to = timeout;
+    void *args[] = {(void *)&listA, (void *)&listB, (void *)&cnt, (void *)&soff, (void *)&sv, (void *)&poff,
+                    (void *)&pred, (void *)&wgt, (void *)&fw, (void *)&bw, (void *)&big, (void *)&reach_big,
+                    (void *)&n, (void *)&A, (void *)&O, (void *)&rem, (void *)&huge, (void *)&nhuge, (void *)&bar,
+                    (void *)&to};
+    TKC_TRY(loop_launch((const void *)k_dp, grid_blocks(g->ctx, k_dp, kLoopTPB, n), args));
   }
   TKC_LAUNCH(k_write_bounds<<<grid_of(n), 256, 0, st>>>(comp, n, A, O, wgt, g->alpha, g->omega, g->scc_size));
   TKC_TRY(cudaGetLastError());
-  TKC_TRY(cudaStreamSynchronize(st));
-  return TKC_OK;
+  return loop_error();
 }
 
 }  // namespace tkc
