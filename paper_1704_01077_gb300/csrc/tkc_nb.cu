@@ -18,7 +18,7 @@
 // to ~16M vertices) once per arc.
 //
 // Gather layout, balanced for skewed degrees: one warp per 32 consecutive
-// vertices; a vertex of degree <= 8 is summed by its own lane, one of degree
+// vertices; a vertex of degree <= kLight is summed by its own lane, one of degree
 // <= kHeavy by the whole warp (coalesced column reads), and a heavier one by
 // one warp per kSeg-arc segment from a segment list built once per call, with
 // an atomic add of each segment's capped partial sum.
@@ -42,9 +42,14 @@ static constexpr unsigned FULL = 0xffffffffu;
 
 constexpr u64 kCap = 1ull << 32;      // counts at or above this are stored as this
 constexpr int kKeyFrac = 46;          // order key = floor(S * 2^46 / (r-1)^2)
-constexpr u32 kHeavy = 1024;          // degrees above this go to the segment list
+// Degrees above this go to the segment list.  (Neighbouring vertices of a
+// Barabasi-Albert graph are hubs together: with the line at 1 024 one warp had
+// 32 rows of hundreds of arcs to itself, 170 us a sweep of 10 M arcs.)
+constexpr u32 kHeavy = 256;
 constexpr u32 kSeg = 1024;            // arcs per segment
-constexpr u32 kLight = 8;             // degrees up to this are summed by one lane
+// Degrees up to this are summed by one lane, four loads in flight (a warp on a
+// row of about ten arcs leaves two thirds of its lanes idle).
+constexpr u32 kLight = 32;
 
 int radix_sort_u32_pairs(u32 *key, u32 *val, u32 n, int bits, cudaStream_t st);
 int scan_exclusive_u32(const u32 *in, u32 *out, u64 len, u32 *tmp, cudaStream_t st);
@@ -88,7 +93,12 @@ __device__ __forceinline__ void nb_gather(u32 n, const u32 *off, const u32 *col,
     const u32 deg = e - b;
     u64 s = 0;
     if (deg <= kLight) {
-      for (u32 a = b; a < e; ++a) s += prev[col[a]];
+      u32 a = b;
+      for (; e - a >= 4; a += 4) {
+        const u32 c0 = col[a], c1 = col[a + 1], c2 = col[a + 2], c3 = col[a + 3];
+        s += prev[c0] + prev[c1] + prev[c2] + prev[c3];
+      }
+      for (; a < e; ++a) s += prev[col[a]];
     }
     // medium rows: the whole warp, one row at a time
     unsigned mid = __ballot_sync(FULL, deg > kLight && deg <= kHeavy);
