@@ -544,6 +544,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   int blocks = o.blocks ? (int)o.blocks : (int)std::min<u64>(maxb, (u64)T * std::max<u64>(8, ((u64)g->n + 511) / 512));
   blocks = std::min(blocks, maxb);
   blocks = std::max<int>(T, blocks / (int)T * (int)T);  // a multiple of the team count
+  p.team_blocks = std::max<u32>((u32)blocks / T, (u32)std::min<u64>(maxb, std::max<u64>(8, ((u64)g->n + 511) / 512)));
   // optional per-step trace for profiling: TKC_TRACE=<csv path>
   const char *trace_path = getenv("TKC_TRACE");
   const uint32_t trace_cap = 1u << 20;

@@ -1164,11 +1164,21 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
   __shared__ Smem<W> sm;
   // this block's team: its own control block, slots, rows, lists and stamps
   __shared__ RunParams p;
-  const uint32_t bpt = gridDim.x / p0.teams;  // blocks per team
+  // teams: no more than batches left by the filter, each then of more blocks (at
+  // most p0.team_blocks, a warp per 32 vertices); spare blocks leave at once
+  uint32_t teams = p0.teams;
+  if (p0.norder_dev && p0.ng == 1) {
+    const uint32_t batches = (p0.sh->norder + p0.B - 1) / p0.B;
+    teams = batches < teams ? (batches ? batches : 1u) : teams;
+  }
+  uint32_t bpt = gridDim.x / teams;  // blocks per team
+  if (teams != p0.teams && bpt > p0.team_blocks) bpt = p0.team_blocks;
   const uint32_t team = blockIdx.x / bpt;
   const uint32_t tb = blockIdx.x % bpt;
+  if (team >= teams) return;
   if (threadIdx.x == 0) {
     p = p0;
+    p.teams = teams;
     p.team = team;
     p.ctl = p0.ctl + team;
     p.slots = p0.slots + (size_t)team * 64 * kMaxWords;

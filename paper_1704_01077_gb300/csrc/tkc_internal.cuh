@@ -168,6 +168,7 @@ struct RunParams {
   // own batches; per-team buffers sit at team * stride from the base pointers
   uint32_t teams;
   uint32_t team;         // this block's team (set by the kernel)
+  uint32_t team_blocks;  // most blocks of a team when there are fewer teams than planned
   uint64_t row_stride;   // 64-bit words between the teams' seen/F0/F1/N rows
   uint64_t vtx_stride;   // 32-bit words between the teams' lists and stamps
   uint64_t fb_stride;    // 32-bit words between the teams' frontier bitmaps
