@@ -303,7 +303,7 @@ struct MlpState {
   unsigned short *wb = nullptr;   // bf16 copy used by the forward passes
   float *m = nullptr, *v = nullptr;  // Adam moments
   float *grad = nullptr;          // gradient scratch
-  float *loss = nullptr;          // loss accumulator
+  double *loss = nullptr;         // loss accumulator
   uint64_t step = 0;
   uint64_t version = 0;           // bumped whenever the weights change
   bool ready = false;

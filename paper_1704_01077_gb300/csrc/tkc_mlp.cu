@@ -217,128 +217,219 @@ __global__ void k_features_standardize(float *x, u32 n, const double *sums) {
 
 // ---------------------------------------------------------------- MLP kernels
 
-__device__ __forceinline__ void load_weights(const unsigned short *wb, float *ws) {
-  for (int i = threadIdx.x; i < P; i += blockDim.x) ws[i] = __bfloat162float(__ushort_as_bfloat16(wb[i]));
-  __syncthreads();
+__device__ __forceinline__ float weight(const unsigned short *wb, int i) {
+  return __bfloat162float(__ushort_as_bfloat16(wb[i]));
 }
 
-constexpr int FT = 64;  // samples per forward block
+constexpr int FT = 128;  // samples per forward block
 
-// y[i] for m samples, one thread per sample; the first hidden layer of the
-// block's samples is kept in shared memory, unit-major so that the threads
-// of a warp read consecutive words.
+// y[i] for m samples, one thread per sample with its first hidden layer in
+// registers: the 64 products of a second-layer unit then read only the unit's
+// weights, four to a (broadcast) shared-memory load, so the pass is bound by
+// its 4 096 multiply-adds per sample (with the layer in shared memory each of
+// them loaded two words).
 __global__ void __launch_bounds__(FT) k_mlp_forward(const float *x, u32 m, const unsigned short *wb, float *y) {
-  __shared__ float ws[P];
-  __shared__ float h1[H][FT];
-  load_weights(wb, ws);
-  const int t = threadIdx.x;
+  __shared__ __align__(16) float ws[P + 3];
+  for (int i = threadIdx.x; i < P; i += FT) ws[i] = weight(wb, i);
+  __syncthreads();
+  static_assert(oW2 % 4 == 0 && H % 4 == 0, "the second layer's rows are read four words at a time");
   for (u32 i0 = blockIdx.x * FT; i0 < m; i0 += gridDim.x * FT) {
-    const u32 i = i0 + t;
+    const u32 i = i0 + threadIdx.x;
     const bool valid = i < m;
     float xi[F];
 #pragma unroll
     for (int f = 0; f < F; ++f) xi[f] = valid ? x[(size_t)i * F + f] : 0.f;
+    float h1[H];
+#pragma unroll
     for (int o = 0; o < H; ++o) {
       float a = ws[oB1 + o];
 #pragma unroll
       for (int f = 0; f < F; ++f) a = fmaf(ws[oW1 + o * F + f], xi[f], a);
-      h1[o][t] = a > 0.f ? a : 0.f;
+      h1[o] = a > 0.f ? a : 0.f;
     }
     float out = ws[oB3];
+#pragma unroll 2
     for (int o = 0; o < H; ++o) {
       float a = ws[oB2 + o];
-#pragma unroll 16
-      for (int j = 0; j < H; ++j) a = fmaf(ws[oW2 + o * H + j], h1[j][t], a);
+      const float4 *w = reinterpret_cast<const float4 *>(ws + oW2 + o * H);
+#pragma unroll
+      for (int j = 0; j < H / 4; ++j) {
+        const float4 q = w[j];
+        a = fmaf(q.x, h1[4 * j], a);
+        a = fmaf(q.y, h1[4 * j + 1], a);
+        a = fmaf(q.z, h1[4 * j + 2], a);
+        a = fmaf(q.w, h1[4 * j + 3], a);
+      }
       out = fmaf(ws[oW3 + o], a > 0.f ? a : 0.f, out);
     }
     if (valid) y[i] = out;
   }
 }
 
-constexpr int TS = 64;  // samples per gradient tile
+constexpr int TS = 16;        // samples per gradient tile
+constexpr int kGradTPB = 256;
+constexpr int W2S = H + 1;    // row stride of W2 in shared memory: rows and columns both without conflicts
+constexpr int TH = H + 4;     // row stride of the tiles (16-byte aligned rows)
+
+__global__ void k_mlp_zero(float *grad, double *loss) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P; i += gridDim.x * blockDim.x) grad[i] = 0.f;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *loss = 0.0;
+}
 
 // Gradient of the mean squared error L = (1/m) sum (y_i - t_i)^2 with
-// respect to the parameters, the forward pass using the bf16 weights.  One
-// block per tile of 64 samples; dense tile products in shared memory; block
-// sums added to grad with atomics.
-__global__ void k_mlp_grad(const float *x, const float *t, u32 m, const unsigned short *wb, float *grad,
-                           float *loss) {
-  extern __shared__ float sm[];
-  float *ws = sm;                 // P
-  float *X = ws + P + 3;          // TS x F   (+3 keeps the tiles 16-byte apart)
-  float *H1 = X + TS * F;         // TS x H   post-activation
-  float *H2 = H1 + TS * H;        // TS x H   post-activation
-  float *D2 = H2 + TS * H;        // TS x H   dL/d(pre-activation 2)
-  float *D1 = D2 + TS * H;        // TS x H   dL/d(pre-activation 1)
-  float *dy = D1 + TS * H;        // TS
-  load_weights(wb, ws);
-  const u32 base = blockIdx.x * TS;
-  for (int i = threadIdx.x; i < TS * F; i += blockDim.x) {
-    u32 s = base + i / F;
-    X[i] = s < m ? x[(size_t)s * F + i % F] : 0.f;
+// respect to the parameters, the forward pass using the bf16 weights.  A block
+// takes tiles of 16 samples, keeps its share of the parameter sums in registers over its tiles, and
+// adds them to grad at the end.  Thread t = 16 y + x computes, of the 16 x 64
+// tile products, sample y and units x, x + 16, x + 32, x + 48, and of the 64 x
+// 64 sums of the second layer rows 4 y .. 4 y + 3 and those four columns.
+// (Bound by latency: 27 million multiply-adds.  With W2's rows 64 words apart
+// every read of a column hit one bank 32 times: 56 us for 2 048 samples.)
+__global__ void __launch_bounds__(kGradTPB) k_mlp_grad(const float *x, const float *t, u32 m, const unsigned short *wb,
+                                                       float *grad, double *loss) {
+  __shared__ float w2[H * W2S], w1[H * F], b1[H], b2[H], w3[H];
+  __shared__ __align__(16) float X[TS * F], H1[TS * TH], H2[TS * TH], D2[TS * TH];  // H2 holds D1 later
+  __shared__ float dy[TS], s_b3;
+  for (int i = threadIdx.x; i < P; i += kGradTPB) {
+    const float w = weight(wb, i);
+    if (i < oB1) w1[i - oW1] = w;
+    else if (i < oW2) b1[i - oB1] = w;
+    else if (i < oB2) w2[(i - oW2) / H * W2S + (i - oW2) % H] = w;
+    else if (i < oW3) b2[i - oB2] = w;
+    else if (i < oB3) w3[i - oW3] = w;
+    else s_b3 = w;
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < TS * H; i += blockDim.x) {
-    int s = i / H, o = i % H;
-    float a = ws[oB1 + o];
-    for (int f = 0; f < F; ++f) a = fmaf(ws[oW1 + o * F + f], X[s * F + f], a);
-    H1[i] = a > 0.f ? a : 0.f;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < TS * H; i += blockDim.x) {
-    int s = i / H, o = i % H;
-    float a = ws[oB2 + o];
-    for (int j = 0; j < H; ++j) a = fmaf(ws[oW2 + o * H + j], H1[s * H + j], a);
-    H2[i] = a > 0.f ? a : 0.f;
-  }
-  __syncthreads();
-  if (threadIdx.x < TS) {
-    int s = threadIdx.x;
-    float yv = ws[oB3];
-    for (int o = 0; o < H; ++o) yv = fmaf(ws[oW3 + o], H2[s * H + o], yv);
-    bool valid = base + s < m;
-    float e = valid ? yv - t[base + s] : 0.f;
-    dy[s] = 2.f * e / (float)m;
-    float l = e * e / (float)m;
-    for (int o = 16; o; o >>= 1) l += __shfl_down_sync(FULL, l, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, l);
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < TS * H; i += blockDim.x) {
-    int s = i / H, o = i % H;
-    D2[i] = H2[i] > 0.f ? dy[s] * ws[oW3 + o] : 0.f;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < TS * H; i += blockDim.x) {
-    int s = i / H, j = i % H;
-    float a = 0.f;
-    for (int o = 0; o < H; ++o) a = fmaf(D2[s * H + o], ws[oW2 + o * H + j], a);
-    D1[i] = H1[i] > 0.f ? a : 0.f;
-  }
-  __syncthreads();
-  // parameter gradients: sums over the tile's samples
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    float g = 0.f;
-    if (p < oB1) {
-      int o = p / F, f = p % F;
-      for (int s = 0; s < TS; ++s) g = fmaf(D1[s * H + o], X[s * F + f], g);
-    } else if (p < oW2) {
-      int o = p - oB1;
-      for (int s = 0; s < TS; ++s) g += D1[s * H + o];
-    } else if (p < oB2) {
-      int o = (p - oW2) / H, j = (p - oW2) % H;
-      for (int s = 0; s < TS; ++s) g = fmaf(D2[s * H + o], H1[s * H + j], g);
-    } else if (p < oW3) {
-      int o = p - oB2;
-      for (int s = 0; s < TS; ++s) g += D2[s * H + o];
-    } else if (p < oB3) {
-      int o = p - oW3;
-      for (int s = 0; s < TS; ++s) g = fmaf(dy[s], H2[s * H + o], g);
-    } else {
-      for (int s = 0; s < TS; ++s) g += dy[s];
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  float g2[4][4] = {}, g1[2] = {0.f, 0.f}, gb = 0.f;  // this thread's sums
+  double l = 0.0;  // of many small terms from every block: added up in 64 bits
+  for (u32 base = blockIdx.x * TS; base < m; base += gridDim.x * TS) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < TS * F; i += kGradTPB) {
+      const u32 s = base + i / F;
+      X[i] = s < m ? x[(size_t)s * F + i % F] : 0.f;
     }
-    if (g != 0.f) atomicAdd(&grad[p], g);
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int o = tx + 16 * q;
+      float a = b1[o];
+#pragma unroll
+      for (int f = 0; f < F; ++f) a = fmaf(w1[o * F + f], X[ty * F + f], a);
+      H1[ty * TH + o] = a > 0.f ? a : 0.f;
+    }
+    __syncthreads();
+    {
+      float a[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) a[q] = b2[tx + 16 * q];
+#pragma unroll 4
+      for (int j = 0; j < H; j += 4) {
+        const float4 h = *reinterpret_cast<const float4 *>(H1 + ty * TH + j);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float *w = w2 + (tx + 16 * q) * W2S + j;
+          a[q] = fmaf(w[0], h.x, a[q]);
+          a[q] = fmaf(w[1], h.y, a[q]);
+          a[q] = fmaf(w[2], h.z, a[q]);
+          a[q] = fmaf(w[3], h.w, a[q]);
+        }
+      }
+      float part = 0.f;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int o = tx + 16 * q;
+        a[q] = a[q] > 0.f ? a[q] : 0.f;
+        H2[ty * TH + o] = a[q];
+        part = fmaf(w3[o], a[q], part);
+      }
+      // y: the 16 threads of a sample are half a warp
+#pragma unroll
+      for (int d = 8; d; d >>= 1) part += __shfl_xor_sync(FULL, part, d);
+      if (tx == 0) {
+        const bool valid = base + ty < m;
+        const float e = valid ? part + s_b3 - t[base + ty] : 0.f;
+        dy[ty] = 2.f * e / (float)m;
+        l += (double)e * (double)e / (double)m;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int o = tx + 16 * q;
+      D2[ty * TH + o] = H2[ty * TH + o] > 0.f ? dy[ty] * w3[o] : 0.f;
+    }
+    __syncthreads();
+    // sums of the second layer, of the biases' and of the output's weights
+#pragma unroll 4
+    for (int s = 0; s < TS; ++s) {
+      const float4 d = *reinterpret_cast<const float4 *>(D2 + s * TH + 4 * ty);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float h = H1[s * TH + tx + 16 * q];
+        g2[0][q] = fmaf(d.x, h, g2[0][q]);
+        g2[1][q] = fmaf(d.y, h, g2[1][q]);
+        g2[2][q] = fmaf(d.z, h, g2[2][q]);
+        g2[3][q] = fmaf(d.w, h, g2[3][q]);
+      }
+    }
+    if (threadIdx.x >= 64 && threadIdx.x < 128) {
+      const int o = threadIdx.x - 64;
+      for (int s = 0; s < TS; ++s) gb += D2[s * TH + o];
+    } else if (threadIdx.x >= 128 && threadIdx.x < 192) {
+      const int o = threadIdx.x - 128;
+      for (int s = 0; s < TS; ++s) gb = fmaf(dy[s], H2[s * TH + o], gb);
+    } else if (threadIdx.x == 192) {
+      for (int s = 0; s < TS; ++s) gb += dy[s];
+    }
+    __syncthreads();
+    // D1 = dL/d(pre-activation 1), over H2
+    {
+      float a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+      for (int o = 0; o < H; o += 4) {
+        const float4 d = *reinterpret_cast<const float4 *>(D2 + ty * TH + o);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float *w = w2 + o * W2S + tx + 16 * q;
+          a[q] = fmaf(d.x, w[0], a[q]);
+          a[q] = fmaf(d.y, w[W2S], a[q]);
+          a[q] = fmaf(d.z, w[2 * W2S], a[q]);
+          a[q] = fmaf(d.w, w[3 * W2S], a[q]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int j = tx + 16 * q;
+        H2[ty * TH + j] = H1[ty * TH + j] > 0.f ? a[q] : 0.f;
+      }
+    }
+    __syncthreads();
+    const float *D1 = H2;
+    for (int r = 0; r < 2; ++r) {
+      const int p = threadIdx.x + r * kGradTPB;
+      if (p < H * F)
+        for (int s = 0; s < TS; ++s) g1[r] = fmaf(D1[s * TH + p / F], X[s * F + p % F], g1[r]);
+    }
+    if (threadIdx.x < 64)
+      for (int s = 0; s < TS; ++s) gb += D1[s * TH + threadIdx.x];
   }
+  // the block's sums
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (g2[r][q] != 0.f) atomicAdd(&grad[oW2 + (4 * ty + r) * H + tx + 16 * q], g2[r][q]);
+  for (int r = 0; r < 2; ++r) {
+    const int p = threadIdx.x + r * kGradTPB;
+    if (p < H * F && g1[r] != 0.f) atomicAdd(&grad[oW1 + p], g1[r]);
+  }
+  const int pb = threadIdx.x < 64 ? oB1 + threadIdx.x
+                 : threadIdx.x < 128 ? oB2 + threadIdx.x - 64
+                 : threadIdx.x < 192 ? oW3 + threadIdx.x - 128
+                                     : oB3;
+  if (threadIdx.x <= 192 && gb != 0.f) atomicAdd(&grad[pb], gb);
+  // the losses of tx == 0, two samples per warp
+  l += __shfl_xor_sync(FULL, l, 16);
+  if ((threadIdx.x & 31) == 0 && l != 0.0) atomicAdd(loss, l);
 }
 
 // Adam (Kingma & Ba 2015) on the fp32 master weights; refreshes the bf16 copy.
@@ -396,7 +487,7 @@ static int ensure_mlp(tkc_ctx *ctx) {
   TKC_TRY(cudaMalloc(&s.m, P * sizeof(float)));
   TKC_TRY(cudaMalloc(&s.v, P * sizeof(float)));
   TKC_TRY(cudaMalloc(&s.grad, P * sizeof(float)));
-  TKC_TRY(cudaMalloc(&s.loss, sizeof(float)));
+  TKC_TRY(cudaMalloc(&s.loss, sizeof(double)));
   return TKC_OK;
 }
 
@@ -620,33 +711,42 @@ int tkc_mlp_forward(tkc_ctx *ctx, const float *x, uint32_t m, float *y) {
   return TKC_OK;
 }
 
-static int gradient(tkc_ctx *ctx, const float *x, const float *t, u32 m, float *loss) {
+// The gradient into `grad` (device); the loss stays in the model's loss word.
+static int gradient(tkc_ctx *ctx, const float *x, const float *t, u32 m, float *grad) {
   cudaStream_t st = ctx->stream;
   MlpState &s = ctx->mlp;
-  TKC_TRY(cudaMemsetAsync(s.grad, 0, P * sizeof(float), st));
-  TKC_TRY(cudaMemsetAsync(s.loss, 0, sizeof(float), st));
-  size_t smem = (P + 3 + TS * F + 4 * TS * H + TS) * sizeof(float);
-  TKC_TRY(cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  TKC_LAUNCH(k_mlp_grad<<<(m + TS - 1) / TS, 256, smem, st>>>(x, t, m, s.wb, s.grad, s.loss));
+  TKC_LAUNCH(k_mlp_zero<<<(P + 255) / 256, 256, 0, st>>>(grad, s.loss));
+  // a tile per block, at most a block per SM
+  const unsigned blocks = (unsigned)std::min<u64>(((u64)m + TS - 1) / TS, (u64)ctx->num_sms);
+  TKC_LAUNCH(k_mlp_grad<<<blocks, kGradTPB, 0, st>>>(x, t, m, s.wb, grad, s.loss));
   TKC_TRY(cudaGetLastError());
-  if (loss) TKC_TRY(cudaMemcpyAsync(loss, s.loss, sizeof(float), cudaMemcpyDeviceToHost, st));
+  return TKC_OK;
+}
+
+// Waits for the stream; the loss into *loss (may be null).
+static int finish_step(tkc_ctx *ctx, float *loss) {
+  double l = 0.0;
+  if (!loss) {
+    TKC_TRY(cudaStreamSynchronize(ctx->stream));
+    return TKC_OK;
+  }
+  TKC_TRY(read_back(&l, ctx->mlp.loss, sizeof(double), ctx->stream));
+  *loss = (float)l;
   return TKC_OK;
 }
 
 int tkc_mlp_gradient(tkc_ctx *ctx, const float *x, const float *t, uint32_t m, float *grad, float *loss) {
   if (!ctx || !x || !t || !grad || m == 0 || !ctx->mlp.ready) return TKC_EINVAL;
   TKC_RC(enter(ctx));
-  TKC_RC(gradient(ctx, x, t, m, loss));
-  TKC_TRY(cudaMemcpyAsync(grad, ctx->mlp.grad, P * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
-  TKC_TRY(cudaStreamSynchronize(ctx->stream));
-  return TKC_OK;
+  TKC_RC(gradient(ctx, x, t, m, grad));
+  return finish_step(ctx, loss);
 }
 
 int tkc_mlp_train_step(tkc_ctx *ctx, const float *x, const float *t, uint32_t m, float lr, float *loss) {
   if (!ctx || !x || !t || m == 0 || !ctx->mlp.ready || !(lr > 0.f)) return TKC_EINVAL;
   TKC_RC(enter(ctx));
   MlpState &s = ctx->mlp;
-  TKC_RC(gradient(ctx, x, t, m, loss));
+  TKC_RC(gradient(ctx, x, t, m, s.grad));
   s.step++;
   const double b1 = 0.9, b2 = 0.999;
   float c1 = (float)(1.0 - pow(b1, (double)s.step)), c2 = (float)(1.0 - pow(b2, (double)s.step));
@@ -654,8 +754,7 @@ int tkc_mlp_train_step(tkc_ctx *ctx, const float *x, const float *t, uint32_t m,
                                                          c2, 1e-8f));
   TKC_TRY(cudaGetLastError());
   s.version++;
-  TKC_TRY(cudaStreamSynchronize(ctx->stream));
-  return TKC_OK;
+  return finish_step(ctx, loss);
 }
 
 }  // extern "C"
