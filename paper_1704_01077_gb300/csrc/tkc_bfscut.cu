@@ -388,6 +388,33 @@ __device__ __forceinline__ void clear_frontier(u64 *F, uint32_t *FB, const uint3
   }
 }
 
+// Zeroes the rows of vertices [v0, v1).
+template <int W>
+__device__ __forceinline__ void clear_rows(u64 *F, uint32_t v0, uint32_t v1, uint64_t gthread, uint64_t nthreads) {
+  if constexpr (W == 1) {
+    for (uint64_t i = v0 + gthread; i < v1; i += nthreads) F[i] = 0;
+  } else {
+    ulonglong2 *q = reinterpret_cast<ulonglong2 *>(F);
+    for (uint64_t i = (uint64_t)v0 * (W / 2) + gthread; i < (uint64_t)v1 * (W / 2); i += nthreads)
+      q[i] = make_ulonglong2(0, 0);
+  }
+}
+
+// Zeroes the frontier's rows and bits: by its list, or, when a bottom-up level
+// left it without one, all of [v0, v1).
+template <int W>
+__device__ __forceinline__ void clear_old_frontier(bool has_list, u64 *F, uint32_t *FB, const uint32_t *list,
+                                                   uint32_t count, uint32_t v0, uint32_t v1, uint64_t gthread,
+                                                   uint64_t nthreads) {
+  if (count == 0) return;
+  if (has_list) {
+    clear_frontier<W>(F, FB, list, count, v0, v1, gthread, nthreads);
+  } else {
+    clear_rows<W>(F, v0, v1, gthread, nthreads);
+    for (uint64_t i = v0 / 32 + gthread; i < v1 / 32 + 1; i += nthreads) FB[i] = 0;
+  }
+}
+
 // updateBoundsLB: the slots whose bits are new in this vertex's row found it at
 // this depth.
 template <int W>
@@ -423,6 +450,7 @@ struct Smem {
   u64 scan64[kMaxThreads / 32 + 1];
   u64 acc[4];
   unsigned bu_next;  // bottom-up level: next of this block's vertex chunks
+  u64 bu_new;        // and its new vertices, packed like nl_packed
   alignas(8) uint32_t cmd[kCmdWords];  // the step's control words (Ctl from `step` on)
 };
 static_assert(offsetof(Ctl, step) % 8 == 0 && kCmdWords <= 64, "the control words are copied as they lie");
@@ -812,6 +840,8 @@ __device__ __noinline__ void epilogue_level(const RunParams &p, Smem<W> &sm) {
     c->bdepth += 1;
     c->fl_count = (uint32_t)nl;
     c->fl_arcs = nla;
+    c->fl_list = dir == 0;
+    if (dir != 0) c->clear_all = 1;
     c->level_id += 1;
 #pragma unroll
     for (int j = 0; j < W; ++j) c->active[j] = sm.active[j];
@@ -825,8 +855,13 @@ __device__ __noinline__ void epilogue_level(const RunParams &p, Smem<W> &sm) {
       // (bottom-up) matches against rows of abandoned searches
       c->step = 2;
     } else {
-      c->step = 0;
-      c->dir = choose_dir(p, nla);
+      const int next = choose_dir(p, nla);
+      if (next == 0 && dir != 0) {
+        c->step = 2;  // the bottom-up level left no list: build it from the bitmap
+      } else {
+        c->step = 0;
+        c->dir = next;
+      }
     }
     // cost model of the level just run (bytes that must move):
     //  top-down : per frontier vertex list+offsets (16) + F row read and clear;
@@ -835,9 +870,8 @@ __device__ __noinline__ void epilogue_level(const RunParams &p, Smem<W> &sm) {
     //  bottom-up: per swept list entry (vertices with an in-arc) the entry (4)
     //             and its seen row; per scanned vertex in-offsets (8); per
     //             scanned in-arc its column (4) and frontier-bitmap word (4);
-    //             per frontier in-neighbour found its F row; per new vertex
-    //             seen/F writes + list (8); per old frontier vertex list (4) +
-    //             F row clear
+    //             per F row loaded the row; per new vertex seen/F writes; per
+    //             old frontier vertex F row clear
     const u64 rb = 8ull * W;
     u64 bytes;
     if (dir == 0) {
@@ -848,7 +882,7 @@ __device__ __noinline__ void epilogue_level(const RunParams &p, Smem<W> &sm) {
       atomicAdd(&c->st_td_new, nl);
     } else {
       const u64 swept = p.g_bu ? p.g_bu[2 * (size_t)c->bgraph] : p.bu_list ? p.n_bu : p.n;
-      bytes = swept * (4 + rb) + lsv * 8 + lsa * 8 + lsr * rb + nl * (8 + 2 * rb) + fl * (4 + rb);
+      bytes = swept * (4 + rb) + lsv * 8 + lsa * 8 + lsr * rb + nl * 2 * rb + fl * rb;
       atomicAdd(&c->st_bu_levels, 1ull);
       atomicAdd(&c->st_bu_swept, swept);
       atomicAdd(&c->st_bu_rows, lsr);
@@ -886,7 +920,7 @@ __device__ __noinline__ void epilogue_level(const RunParams &p, Smem<W> &sm) {
 }
 
 // Epilogue after a compaction step: the compacted list (built in the next-list
-// buffer) becomes the frontier list, and the level's direction is chosen from
+// buffer, from the old list or from the frontier's bitmap) becomes the frontier list, and the level's direction is chosen from
 // its arcs.
 template <int W>
 __device__ __noinline__ void epilogue_compact(const RunParams &p, Smem<W> &sm) {
@@ -898,6 +932,7 @@ __device__ __noinline__ void epilogue_compact(const RunParams &p, Smem<W> &sm) {
     c->lcur ^= 1;
     c->fl_count = (uint32_t)after;
     c->fl_arcs = packed & kArcMask;
+    c->fl_list = 1;
     c->st_compactions += 1;
     c->st_compact_dropped += before - after;
     // list entry and row read per old entry, row cleared per dropped one, list written per kept one
@@ -987,6 +1022,7 @@ __device__ __noinline__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
       c->fl_count = 0;
       c->fl_arcs = 0;
       c->vl_count = 0;
+      c->clear_all = 0;
       c->nl_packed = 0;
       c->level_id += 1;
       for (int j = 0; j < W; ++j) c->active[j] = 0;
@@ -1112,8 +1148,9 @@ __device__ __noinline__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
   __syncthreads();
   if (threadIdx.x == 0) {
     // the clear step just zeroed these rows
-    c->alg_bytes += (u64)(c->vl_count + c->fl_count) * (4 + 8ull * W);
-    c->st_cleared += (u64)c->vl_count + c->fl_count;
+    const u64 seen_rows = !c->clear_all ? c->vl_count : c->bgraph >= 0 && p.g_bu ? p.g_base[c->bgraph + 1] - p.g_base[c->bgraph] : p.n;
+    c->alg_bytes += (seen_rows + c->fl_count) * 8ull * W + (c->clear_all ? 0ull : 4ull * c->vl_count);
+    c->st_cleared += seen_rows + c->fl_count;
     c->st_seeded += assigned;
     c->cursor = last_base;
     c->bfs_started += started;
@@ -1121,6 +1158,8 @@ __device__ __noinline__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
     c->edges_visited += arcs_total;
     c->fl_count = assigned;
     c->fl_arcs = arcs_total;
+    c->fl_list = 1;
+    c->clear_all = 0;
     c->vl_count = assigned;
     c->bdepth = 0;
     c->nl_packed = 0;
@@ -1234,30 +1273,31 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
     if (step == 1) {
       if (tb == 0) trace_stamp(p, 8);
       // ---- clear step: zero the rows touched by the finished batch
-      const uint32_t vl = vc->vl_count;
-      for (uint64_t i = gthread; i < (uint64_t)vl * W; i += nthreads) {
-        uint32_t v = p.VL[i / W];
-        p.seen[(size_t)v * W + (i % W)] = 0;
+      if (vc->clear_all) {
+        clear_rows<W>(p.seen, v0, v1, gthread, nthreads);
+      } else {
+        const uint32_t vl = vc->vl_count;
+        for (uint64_t i = gthread; i < (uint64_t)vl * W; i += nthreads) {
+          uint32_t v = p.VL[i / W];
+          p.seen[(size_t)v * W + (i % W)] = 0;
+        }
       }
-      clear_frontier<W>(Fcur, FBcur, FL, fl_count, v0, v1, gthread, nthreads);
+      clear_old_frontier<W>(vc->fl_list, Fcur, FBcur, FL, fl_count, v0, v1, gthread, nthreads);
       if (tb == 0) trace_stamp(p, 12);
       if (!team_sync(c, p.sh, bpt, p.timeout, [&] { epilogue_seed<W>(p, sm); })) break;
       continue;
     }
     if (step == 2) {
-      // ---- compaction: keep the frontier entries with a bit of a search
+      // ---- compaction: list the frontier vertices with a bit of a search
       // still active (rows masked to those bits); zero the rows and frontier
       // bits of the others, which only abandoned or finished searches used
       u64 act[W];
 #pragma unroll
       for (int q = 0; q < W; ++q) act[q] = vc->active[q];
-      for (uint32_t base = gwarp * 32; base < fl_count; base += nwarps * 32) {
-        const uint32_t i = base + lane;
-        const bool valid = i < fl_count;
-        uint32_t u = 0, od = 0;
+      auto keep_active = [&](uint32_t u, bool valid) {
+        uint32_t od = 0;
         bool keep = false;
         if (valid) {
-          u = FL[i];
           u64 row[W], f[W];
           load_row<W>(Fcur, u, row);
           bool same = true;
@@ -1272,6 +1312,23 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
           if (keep) od = p.off[u + 1] - p.off[u];
         }
         warp_append(keep, u, od, &c->nl_packed, NL, NLoff, lane);
+      };
+      if (vc->fl_list) {
+        for (uint32_t base = gwarp * 32; base < fl_count; base += nwarps * 32) {
+          const bool valid = base + lane < fl_count;
+          keep_active(valid ? FL[base + lane] : 0u, valid);
+        }
+      } else {
+        // no list: the frontier's bitmap, 32 words a warp, a word's vertices at a time
+        const uint32_t w1 = v1 / 32 + 1;
+        for (uint32_t base = v0 / 32 + gwarp * 32; base < w1; base += nwarps * 32) {
+          const uint32_t word = base + lane < w1 ? FBcur[base + lane] : 0u;
+          for (unsigned m = __ballot_sync(FULL, word != 0); m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
+            const uint32_t bits = __shfl_sync(FULL, word, src);
+            keep_active((base + src) * 32 + lane, (bits >> lane) & 1u);
+          }
+        }
       }
       if (!team_sync(c, p.sh, bpt, p.timeout, [&] { epilogue_compact<W>(p, sm); })) break;
       continue;
@@ -1290,10 +1347,11 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
       sm.acc[2] = 0;
       sm.acc[3] = 0;
       sm.bu_next = 0;
+      sm.bu_new = 0;
     }
     __syncthreads();
-    u64 scanned = 0, scanned_v = 0;
-    uint32_t rows_read = 0;
+    u64 scanned = 0;
+    uint32_t scanned_v = 0, rows_read = 0;
     if (dir == 0) {
       // ---- phase A, top-down: OR each frontier row into its out-neighbours' N rows
       constexpr uint32_t APS = 32 / W;  // arcs per warp step
@@ -1395,9 +1453,9 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
           if (p.lvl) record_levels<W>(p, w, nw, depth);
         }
         warp_count_slots<W>(nw, od, sm.cnt, sm.wsum, lane);
-        warp_append_plain(valid && was_empty, w, &c->vl_count, p.VL, lane);
+        if (!vc->clear_all) warp_append_plain(valid && was_empty, w, &c->vl_count, p.VL, lane);
       }
-      clear_frontier<W>(Fcur, FBcur, FL, fl_count, v0, v1, gthread, nthreads);
+      clear_old_frontier<W>(vc->fl_list, Fcur, FBcur, FL, fl_count, v0, v1, gthread, nthreads);
     } else {
       // ---- phase A, bottom-up: each vertex ORs its in-neighbours' frontier rows
       u64 act[W];
@@ -1413,6 +1471,11 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
       const uint32_t nheavy = bg >= 0 ? p.g_bu[2 * bg + 1] : list ? p.n_bu_heavy : 0u;
       const uint32_t nlight = bg >= 0 ? p.g_bu[2 * bg] - nheavy : list ? p.n_bu - nheavy : p.n;
       const uint32_t hg = (nheavy + 31) / 32;
+      // a frontier of more than half the swept vertices: its bits are not worth
+      // testing (a row that is not on it is zero)
+      const bool dense = (u64)fl_count * 2 > (u64)nheavy + nlight;
+      u64 new_arcs = 0;
+      uint32_t new_count = 0;
       // chunks of kBuChunkVerts entries, of 32 when that leaves warps with fewer
       // than four chunks: a level then waits for a warp's 32 entries, not 128
       const uint32_t bch = nlight >= 4 * kBuChunkVerts * nwarps ? kBuChunkVerts : 32u;
@@ -1440,7 +1503,7 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
           }
           u64 nw[W], sr[W], miss[W];
           uint32_t od = 0, e0 = 0, ee = 0;
-          bool was_empty = false, any = false, heavy = false;
+          bool any = false, heavy = false;
 #pragma unroll
           for (int q = 0; q < W; ++q) {
             nw[q] = 0;
@@ -1448,7 +1511,6 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
           }
           if (valid) {
             load_row<W>(p.seen, w, sr);
-            was_empty = !row_nonzero<W>(sr);
 #pragma unroll
             for (int q = 0; q < W; ++q) {
               miss[q] = act[q] & ~sr[q];
@@ -1474,14 +1536,14 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
               }
 #pragma unroll
               for (int j = 0; j < U; ++j)
-                f0[j] = c0[j] != 0xffffffffu ? (FBcur[c0[j] >> 5] >> (c0[j] & 31)) & 1u : 0u;
+                f0[j] = c0[j] != 0xffffffffu && (dense || ((FBcur[c0[j] >> 5] >> (c0[j] & 31)) & 1u));
               for (; e < ee; e += U) {
                 uint32_t c2[U], f1[U];
 #pragma unroll
                 for (int j = 0; j < U; ++j) c2[j] = e + 2 * U + j < ee ? p.icol[e + 2 * U + j] : 0xffffffffu;
 #pragma unroll
                 for (int j = 0; j < U; ++j)
-                  f1[j] = c1[j] != 0xffffffffu ? (FBcur[c1[j] >> 5] >> (c1[j] & 31)) & 1u : 0u;
+                  f1[j] = c1[j] != 0xffffffffu && (dense || ((FBcur[c1[j] >> 5] >> (c1[j] & 31)) & 1u));
 #pragma unroll
                 for (int j = 0; j < U; ++j) {
                   if (f0[j]) {
@@ -1543,7 +1605,7 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
               }
 #pragma unroll
               for (int j = 0; j < HU; ++j)
-                fb[j] = uu[j] != 0xffffffffu ? (FBcur[uu[j] >> 5] >> (uu[j] & 31)) & 1u : 0u;
+                fb[j] = uu[j] != 0xffffffffu && (dense || ((FBcur[uu[j] >> 5] >> (uu[j] & 31)) & 1u));
 #pragma unroll
               for (int j = 0; j < HU; ++j) {
                 if (fb[j]) {
@@ -1599,27 +1661,31 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
             }
           }
           warp_count_slots<W>(nw, od, sm.cnt, sm.wsum, lane);
-          warp_append(isnew, w, od, &c->nl_packed, NL, NLoff, lane);
-          warp_append_plain(isnew && was_empty, w, &c->vl_count, p.VL, lane);
+          // counted, not listed: a list costs two more round trips of atomics
+          // per 32 vertices, and the next bottom-up level needs none
+          new_arcs += od;
+          new_count += isnew;
         }
       }
+      for (int o = 16; o > 0; o >>= 1) new_arcs += __shfl_down_sync(FULL, new_arcs, o);
+      new_count = __reduce_add_sync(FULL, new_count);
+      if (lane == 0 && new_count) atomicAdd(&sm.bu_new, ((u64)new_count << kPackShift) | new_arcs);
       if (tb == 0) trace_stamp(p, 9);
       if (!team_sync(c, p.sh, bpt, p.timeout, [] {})) break;
       if (tb == 0) trace_stamp(p, 10);
       // ---- phase B: only the old frontier rows need clearing
-      clear_frontier<W>(Fcur, FBcur, FL, fl_count, v0, v1, gthread, nthreads);
+      clear_old_frontier<W>(vc->fl_list, Fcur, FBcur, FL, fl_count, v0, v1, gthread, nthreads);
     }
     if (tb == 0) trace_stamp(p, 11);
     // flush the block's per-slot counters
-    u64 rows64 = rows_read;
+    // (a lane's counts are below 2^32: half-words add up in one reduction each)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      scanned += __shfl_down_sync(FULL, scanned, o);
-      scanned_v += __shfl_down_sync(FULL, scanned_v, o);
-      rows64 += __shfl_down_sync(FULL, rows64, o);
-    }
+    for (int o = 16; o > 0; o >>= 1) scanned += __shfl_down_sync(FULL, scanned, o);
+    scanned_v = __reduce_add_sync(FULL, scanned_v);
+    const u64 rows64 = (u64)__reduce_add_sync(FULL, rows_read & 0xffffu) +
+                       ((u64)__reduce_add_sync(FULL, rows_read >> 16) << 16);
     if (lane == 0 && scanned) atomicAdd(&sm.acc[3], scanned);
-    if (lane == 0 && scanned_v) atomicAdd(&sm.acc[2], scanned_v);
+    if (lane == 0 && scanned_v) atomicAdd(&sm.acc[2], (u64)scanned_v);
     if (lane == 0 && rows64) atomicAdd(&c->lvl_scan_r, rows64);
     __syncthreads();
     for (int i = threadIdx.x; i < 64 * W; i += TPB) {
@@ -1633,6 +1699,7 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
       atomicAdd(&c->lvl_scan_a, sm.acc[3]);
     }
     if (threadIdx.x == 0 && sm.acc[2]) atomicAdd(&c->lvl_scan_v, sm.acc[2]);
+    if (threadIdx.x == 0 && sm.bu_new) atomicAdd(&c->nl_packed, sm.bu_new);
     if (tb == 0) trace_stamp(p, 12);
     if (!team_sync(c, p.sh, bpt, p.timeout, [&] { epilogue_level<W>(p, sm); })) break;
   }

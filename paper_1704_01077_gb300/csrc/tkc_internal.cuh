@@ -72,10 +72,12 @@ struct Ctl {
   int cur;           // which frontier buffer / list is current
   int lcur;          // which list buffer holds the current frontier list (compaction swaps it alone)
   int bgraph;        // several graphs: the graph of every search of the batch, -1 when they differ
+  int fl_list;       // the current frontier has a list (a bottom-up level leaves only rows and bitmap)
+  int clear_all;     // the batch ran a bottom-up level: its rows are cleared by range, not by list
   unsigned int bdepth;    // depth reached by the current batch (0 after seeding)
   unsigned int level_id;  // global level stamp
   unsigned int fl_count;  // current frontier list size
-  unsigned int vl_count;  // visited-list size (vertices with a non-zero seen row)
+  unsigned int vl_count;  // visited-list size (vertices with a non-zero seen row; clear_all = 0)
   unsigned long long fl_arcs;    // arcs out of the current frontier list
   unsigned long long active[kMaxWords];
   unsigned long long nl_packed;  // next list: count << 38 | arcs
