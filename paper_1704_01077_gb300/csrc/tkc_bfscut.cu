@@ -323,6 +323,42 @@ __device__ __forceinline__ void warp_append(bool pred, uint32_t v, uint32_t od, 
   }
 }
 
+// warp_append for T entries per lane, one atomic for all of them (in lane order).
+template <int T>
+__device__ __forceinline__ void warp_append_steps(const bool (&pred)[T], const uint32_t (&v)[T],
+                                                  const uint32_t (&od)[T], u64 *packed, uint32_t *list,
+                                                  uint32_t *loff, int lane) {
+  uint32_t cnt = 0, arcs = 0;
+#pragma unroll
+  for (int t = 0; t < T; ++t) {
+    cnt += pred[t];
+    arcs += pred[t] ? od[t] : 0u;
+  }
+  if (__ballot_sync(FULL, cnt != 0) == 0) return;
+  uint32_t ci = cnt, ai = arcs;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t tc = __shfl_up_sync(FULL, ci, o), ta = __shfl_up_sync(FULL, ai, o);
+    if (lane >= o) {
+      ci += tc;
+      ai += ta;
+    }
+  }
+  u64 base = 0;
+  if (lane == 31) base = atomicAdd(packed, ((u64)ci << kPackShift) | (u64)ai);
+  base = __shfl_sync(FULL, base, 31);
+  uint32_t pos = (uint32_t)(base >> kPackShift) + ci - cnt;
+  uint32_t at = (uint32_t)(base & kArcMask) + ai - arcs;
+#pragma unroll
+  for (int t = 0; t < T; ++t) {
+    if (!pred[t]) continue;
+    list[pos] = v[t];
+    loff[pos] = at;
+    ++pos;
+    at += od[t];
+  }
+}
+
 __device__ __forceinline__ void warp_append_plain(bool pred, uint32_t v, unsigned *counter, uint32_t *list,
                                                   int lane) {
   uint32_t mask = __ballot_sync(FULL, pred);
@@ -1403,19 +1439,28 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
 #pragma unroll
           for (int t = 0; t < TU; ++t) ww[t] = fw[t] ? p.col[p.off[uw[t]] + (uint32_t)(ew[t] - FLoff[iw[t]])] : 0;
 #pragma unroll
-          for (int t = 0; t < TU; ++t) bw[t] = fw[t] ? fw[t] & ~p.seen[(size_t)ww[t] * W + j] : 0;
-#pragma unroll
-          for (int t = 0; t < TU; ++t) cw[t] = bw[t] ? *(volatile u64 *)(p.N + (size_t)ww[t] * W + j) : 0;
+          for (int t = 0; t < TU; ++t) {
+            bw[t] = fw[t] ? fw[t] & ~p.seen[(size_t)ww[t] * W + j] : 0;
+            cw[t] = fw[t] ? *(volatile u64 *)(p.N + (size_t)ww[t] * W + j) : 0;
+          }
+          // The word's first contributor saw it zero, so only those may be the
+          // vertex's first: of one word the one whose OR met zero, of several
+          // the one whose stamp is new.  Their degrees are loaded beside the
+          // atomics, and the TU steps append together (one returning atomic).
+          bool app[TU];
+          uint32_t od[TU];
 #pragma unroll
           for (int t = 0; t < TU; ++t) {
-            bool app = false;
-            if (bw[t] & ~cw[t]) {
-              u64 old = atomicOr(p.N + (size_t)ww[t] * W + j, bw[t]);
-              if (old == 0) app = atomicExch(&p.stamp[ww[t]], level_id) != level_id;
+            const bool go = (bw[t] & ~cw[t]) != 0, first = go && cw[t] == 0;
+            od[t] = first ? p.off[ww[t] + 1] - p.off[ww[t]] : 0;
+            if constexpr (W == 1) {
+              app[t] = go && atomicOr(p.N + ww[t], bw[t]) == 0;
+            } else {
+              if (go) atomicOr(p.N + (size_t)ww[t] * W + j, bw[t]);
+              app[t] = first && atomicExch(&p.stamp[ww[t]], level_id) != level_id;
             }
-            uint32_t od = app ? p.off[ww[t] + 1] - p.off[ww[t]] : 0;
-            warp_append(app, ww[t], od, &c->nl_packed, NL, NLoff, lane);
           }
+          warp_append_steps<TU>(app, ww, od, &c->nl_packed, NL, NLoff, lane);
           ent = __reduce_max_sync(FULL, ii);
         }
       }
