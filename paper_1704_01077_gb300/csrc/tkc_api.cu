@@ -45,9 +45,9 @@ cudaError_t tkc::dev_malloc_bytes(void **p, size_t bytes, cudaStream_t st) {
   return cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
 }
 
-cudaError_t tkc::read_back(void *dst, const void *src, size_t bytes, cudaStream_t st) {
-  tkc_ctx *ctx = t_ctx;
-  if (bytes > ctx->stage_bytes && bytes <= kStageMost) {
+// Whether the page-locked buffer holds `bytes` (grown up to kStageMost).
+static bool stage_room(tkc_ctx *ctx, size_t bytes) {
+  if (bytes > ctx->stage_bytes && bytes <= tkc::kStageMost) {
     if (ctx->stage) cudaFreeHost(ctx->stage);
     ctx->stage = nullptr;
     ctx->stage_bytes = 0;
@@ -55,11 +55,35 @@ cudaError_t tkc::read_back(void *dst, const void *src, size_t bytes, cudaStream_
     if (cudaMallocHost(&ctx->stage, want) == cudaSuccess) ctx->stage_bytes = want;
     else cudaGetLastError();  // no page-locked memory left: straight into the caller's
   }
-  const bool staged = bytes <= ctx->stage_bytes;
+  return bytes <= ctx->stage_bytes;
+}
+
+cudaError_t tkc::read_back(void *dst, const void *src, size_t bytes, cudaStream_t st) {
+  tkc_ctx *ctx = t_ctx;
+  const bool staged = stage_room(ctx, bytes);
   cudaError_t e = cudaMemcpyAsync(staged ? ctx->stage : dst, src, bytes, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e == cudaSuccess && staged) memcpy(dst, ctx->stage, bytes);
   return e;
+}
+
+cudaError_t tkc::read_back2(void *dst, const void *src, size_t bytes, void *dst2, const void *src2, size_t bytes2,
+                            cudaStream_t st) {
+  if (bytes2 == 0) return read_back(dst, src, bytes, st);
+  tkc_ctx *ctx = t_ctx;
+  const size_t at = (bytes + 15) / 16 * 16;
+  if (!stage_room(ctx, at + bytes2)) {
+    cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, st);
+    return e == cudaSuccess ? read_back(dst2, src2, bytes2, st) : e;
+  }
+  unsigned char *h = static_cast<unsigned char *>(ctx->stage);
+  cudaError_t e = cudaMemcpyAsync(h, src, bytes, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(h + at, src2, bytes2, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return e;
+  memcpy(dst, h, bytes);
+  memcpy(dst2, h + at, bytes2);
+  return cudaSuccess;
 }
 
 void tkc::note_launches(unsigned count) { g_launches.fetch_add(count, std::memory_order_relaxed); }
@@ -75,6 +99,8 @@ typedef unsigned long long u64;
 
 static constexpr uint64_t kDefaultTimeout = 1ull << 34;
 
+constexpr size_t kShBytes = 128;  // the shared block's place before the control blocks
+
 template <typename T>
 static int dalloc(T **p, size_t count, cudaStream_t st) {
   if (*p) {
@@ -88,11 +114,13 @@ static int dalloc(T **p, size_t count, cudaStream_t st) {
 int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u32 teams) {
   Workspace &w = ctx->ws;
   cudaStream_t st = ctx->stream;
-  if (!w.sh) {
-    TKC_RC(dalloc(&w.sh, 1, st));
-  }
   if (teams > w.teams_cap) {
-    TKC_RC(dalloc(&w.ctl, 2 * (size_t)teams, st));
+    // the shared block, then the control blocks: read back together
+    static_assert(sizeof(Shared) <= kShBytes, "the shared block fits its place");
+    unsigned char *base = reinterpret_cast<unsigned char *>(w.sh);
+    TKC_RC(dalloc(&base, kShBytes + 2 * (size_t)teams * sizeof(Ctl), st));
+    w.sh = reinterpret_cast<Shared *>(base);
+    w.ctl = reinterpret_cast<Ctl *>(base + kShBytes);
     TKC_RC(dalloc(&w.slots, (size_t)teams * 64 * kMaxWords, st));
     TKC_RC(dalloc(&w.cnt, (size_t)teams * 64 * kMaxWords, st));
     TKC_RC(dalloc(&w.wsum, (size_t)teams * 64 * kMaxWords, st));
@@ -181,7 +209,7 @@ static int ensure_filter(tkc_ctx *ctx, u32 count, u32 nopen) {
 static void free_workspace(tkc_ctx *ctx) {
   Workspace &w = ctx->ws;
   void *ptrs[] = {w.seen, w.F0, w.F1, w.N, w.FB0, w.FB1, w.L0, w.L1, w.Loff0, w.Loff1, w.VL, w.stamp, w.res_S, w.res_r,
-                  w.slots, w.cnt, w.wsum, w.top_S, w.top_r, w.top_id, w.ctl, w.out, w.tied, w.g_ntop, w.g_lock, w.g_stop, w.g_ctr, w.sh, w.x,
+                  w.slots, w.cnt, w.wsum, w.top_S, w.top_r, w.top_id, w.out, w.tied, w.g_ntop, w.g_lock, w.g_stop, w.g_ctr, w.sh, w.x,
                   w.f_order, w.f_keep, w.f_count, w.f_end, w.lvl2,
                   w.o_order, w.o_key, w.o_taken};
   for (void *p : ptrs)
@@ -215,6 +243,7 @@ struct GraphOut {
   u32 base;       // first id of the graph in the run's (union) numbering
   u32 kk;         // min(k, n)
   u32 nzero;      // vertices of out-degree 0 (closeness 0)
+  const u32 *nzero_dev;  // or the device word that holds their number
   const u32 *zero_ids;  // those vertices in increasing id order (graph-local ids)
 };
 
@@ -255,7 +284,8 @@ struct OutPack {
   __host__ __device__ size_t id() const { return r() + 4 * (size_t)m; }
   __host__ __device__ size_t tied() const { return id() + 4 * (size_t)m; }
   __host__ __device__ size_t ntop() const { return tied() + 4 * (size_t)ng; }
-  __host__ __device__ size_t bytes() const { return ntop() + 4 * (size_t)ng; }
+  __host__ __device__ size_t nzero() const { return ntop() + 4 * (size_t)ng; }
+  __host__ __device__ size_t bytes() const { return nzero() + 4 * (size_t)ng; }
 };
 
 // Final list of graph blockIdx.x: its top entries, then (if fewer than k of
@@ -275,6 +305,7 @@ __global__ void k_output(const u64 *top_S, const u32 *top_r, const u32 *top_id, 
   if (threadIdx.x == 0) {
     ((u32 *)(out + pk.tied()))[g] = tied[g];
     ((u32 *)(out + pk.ntop()))[g] = ntop;
+    ((u32 *)(out + pk.nzero()))[g] = G.nzero_dev ? *G.nzero_dev : G.nzero;
   }
   for (u32 i = threadIdx.x; i < G.kk; i += blockDim.x) {
     size_t src = (size_t)g * kk + i;
@@ -359,6 +390,10 @@ struct RunSetup {
   const u32 *g_end;
   u32 g_rest;
   const u32 *g_base;        // first vertex of each graph (ng + 1 words)
+  // what the output step needs: given, it is enqueued right after the search
+  // and `out` receives the packed results with the search's own wait
+  const std::vector<GraphOut> *go;
+  std::vector<unsigned char> *out;
 };
 
 // Teams used when the options leave it to the library, so that the latency of
@@ -400,6 +435,67 @@ static bool labelled_by_size(const tkc_options &o, u32 B, u32 size_n) {
 // many batches: on R-MAT 22 it costs 3.4 to 5 ms of device work and saved 0.2 ms
 // per 128-source batch (51 -> 35 ms over 81 batches); the filter leaves one.
 constexpr u32 kLabelBatches = 24;
+
+// Enqueues the output step of a run: ties and the final lists, packed into the
+// workspace's out buffer.
+static int enqueue_output(tkc_ctx *ctx, const RunSetup &rs, const std::vector<GraphOut> &go_h) {
+  Workspace &w = ctx->ws;
+  cudaStream_t st = ctx->stream;
+  const u32 ng = rs.ng;
+  GraphOut *go = nullptr;
+  TKC_TRY(dev_malloc(&go, ng * sizeof(GraphOut), st));
+  TKC_TRY(cudaMemcpyAsync(go, go_h.data(), ng * sizeof(GraphOut), cudaMemcpyHostToDevice, st));
+  TKC_TRY(cudaMemsetAsync(w.tied, 0, ng * sizeof(unsigned), st));
+  unsigned blocks = (unsigned)std::max<u64>(1, std::min<u64>((rs.g->n + 255) / 256, (u64)ctx->num_sms * 8));
+  TKC_LAUNCH(k_count_ties<<<blocks, 256, 0, st>>>(w.res_S, w.res_r, rs.gid, rs.g->n, w.top_S, w.top_r, w.g_ntop,
+                                                  rs.kk, go, rs.harmonic, w.tied));
+  const OutPack pk{rs.kk * ng, ng};
+  if (pk.bytes() > w.out_cap) {
+    w.out_cap = 0;
+    TKC_RC(dalloc(&w.out, std::max<size_t>(pk.bytes(), 65536), st));
+    w.out_cap = std::max<size_t>(pk.bytes(), 65536);
+  }
+  TKC_LAUNCH(k_output<<<ng, 256, 0, st>>>(w.top_S, w.top_r, w.top_id, w.g_ntop, rs.kk, go, rs.harmonic, w.tied,
+                                          w.g_ctr, pk, w.out));
+  TKC_TRY(cudaGetLastError());
+  TKC_TRY(cudaFreeAsync(go, st));
+  return TKC_OK;
+}
+
+// Output step of a run: ties, final lists, copies into the callers' results.
+// outs[i] receives graph i.  Returns per-graph tie counts and counters in the
+// host vectors.  (The search's own wait has brought the packed results when
+// the run was set up with rs.go; else they are made and read here.)
+static int finish_run(tkc_ctx *ctx, const RunSetup &rs, const std::vector<GraphOut> &go_h, tkc_result *outs,
+                      std::vector<unsigned> &tied, std::vector<u64> &gctr) {
+  const u32 ng = rs.ng;
+  const OutPack pk{rs.kk * ng, ng};
+  std::vector<unsigned char> own;
+  if (!rs.out) {
+    TKC_RC(enqueue_output(ctx, rs, go_h));
+    own.resize(pk.bytes());
+    TKC_TRY(read_back(own.data(), ctx->ws.out, pk.bytes(), ctx->stream));
+  }
+  const unsigned char *h = rs.out ? rs.out->data() : own.data();
+  const u32 *h_tied = (const u32 *)(h + pk.tied()), *h_ntop = (const u32 *)(h + pk.ntop());
+  const u32 *h_nzero = (const u32 *)(h + pk.nzero());
+  const u64 *h_ctr = (const u64 *)(h + pk.ctr());
+  tied.assign(h_tied, h_tied + ng);
+  gctr.assign(h_ctr, h_ctr + 4 * (size_t)ng);
+  for (u32 i = 0; i < ng; ++i) {
+    tkc_result *out = &outs[i];
+    const u32 kg = go_h[i].kk;
+    const size_t src = (size_t)i * rs.kk;
+    if (h_ntop[i] < kg) tied[i] = h_nzero[i];  // the k-th is a closeness-0 vertex
+    if (!kg) continue;
+    if (out->ids) memcpy(out->ids, h + pk.id() + 4 * src, kg * sizeof(u32));
+    if (out->dist_sum) memcpy(out->dist_sum, h + pk.S() + 8 * src, kg * sizeof(u64));
+    if (out->reach) memcpy(out->reach, h + pk.r() + 4 * src, kg * sizeof(u32));
+    if (out->farness) memcpy(out->farness, h + pk.f() + 8 * src, kg * sizeof(double));
+    if (out->closeness) memcpy(out->closeness, h + pk.c() + 8 * src, kg * sizeof(double));
+  }
+  return TKC_OK;
+}
 
 static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   const tkc_graph *g = rs.g;
@@ -475,8 +571,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     p.lab = lab ? g->s_lab : nullptr;
     p.unlab = lab ? g->s_unlab : nullptr;
     p.bu_list = g->bu_list;
-    p.n_bu = g->n_bu;
-    p.n_bu_heavy = g->n_bu_heavy;
+    p.bu_cnt = g->s_cnt;
     p.g_bu = lab ? nullptr : g->g_bu;
     p.g_base = p.g_bu ? rs.g_base : nullptr;
     p.heavy_in = g->heavy_in ? g->heavy_in : kHeavyIn;
@@ -595,8 +690,17 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   }
   TKC_RC(launch_phase(T, w.ctl + open_teams));
   TKC_TRY(cudaEventRecord(ctx->ev[5], st));
-  TKC_TRY(read_back(cs.data(), w.ctl, cs.size() * sizeof(Ctl), st));
-  TKC_TRY(read_back(&hsh, w.sh, sizeof(Shared), st));
+  size_t out_bytes = 0;
+  if (rs.go) {
+    TKC_RC(enqueue_output(ctx, rs, *rs.go));
+    out_bytes = OutPack{rs.kk * rs.ng, rs.ng}.bytes();
+    rs.out->resize(out_bytes);
+  }
+  TKC_TRY(cudaEventRecord(ctx->ev[2], st));
+  std::vector<unsigned char> back(kShBytes + cs.size() * sizeof(Ctl));
+  TKC_TRY(read_back2(back.data(), w.sh, back.size(), rs.go ? rs.out->data() : nullptr, w.out, out_bytes, st));
+  memcpy(&hsh, back.data(), sizeof(Shared));
+  memcpy(cs.data(), back.data() + kShBytes, cs.size() * sizeof(Ctl));
   // the teams' counters add up; levels and batches too (they ran side by side)
   for (const Ctl &x : cs) {
     hctl->edges_visited += x.edges_visited;
@@ -683,54 +787,6 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     TKC_TRY(cudaStreamSynchronize(st));
     return hctl->err;
   }
-  return TKC_OK;
-}
-
-// Output step of a run: ties, final lists, copies into the callers' results.
-// outs[i] receives graph i.  Returns per-graph g_ntop and counters in the
-// host vectors.
-static int finish_run(tkc_ctx *ctx, const RunSetup &rs, const std::vector<GraphOut> &go_h, tkc_result *outs,
-                      std::vector<unsigned> &ntop, std::vector<unsigned> &tied, std::vector<u64> &gctr) {
-  Workspace &w = ctx->ws;
-  cudaStream_t st = ctx->stream;
-  const u32 ng = rs.ng;
-  GraphOut *go = nullptr;
-  TKC_TRY(dev_malloc(&go, ng * sizeof(GraphOut), st));
-  TKC_TRY(cudaMemcpyAsync(go, go_h.data(), ng * sizeof(GraphOut), cudaMemcpyHostToDevice, st));
-  TKC_TRY(cudaMemsetAsync(w.tied, 0, ng * sizeof(unsigned), st));
-  unsigned blocks = (unsigned)std::max<u64>(1, std::min<u64>((rs.g->n + 255) / 256, (u64)ctx->num_sms * 8));
-  TKC_LAUNCH(k_count_ties<<<blocks, 256, 0, st>>>(w.res_S, w.res_r, rs.gid, rs.g->n, w.top_S, w.top_r, w.g_ntop,
-                                                  rs.kk, go, rs.harmonic, w.tied));
-  const OutPack pk{rs.kk * ng, ng};
-  if (pk.bytes() > w.out_cap) {
-    w.out_cap = 0;
-    TKC_RC(dalloc(&w.out, std::max<size_t>(pk.bytes(), 65536), st));
-    w.out_cap = std::max<size_t>(pk.bytes(), 65536);
-  }
-  TKC_LAUNCH(k_output<<<ng, 256, 0, st>>>(w.top_S, w.top_r, w.top_id, w.g_ntop, rs.kk, go, rs.harmonic, w.tied,
-                                          w.g_ctr, pk, w.out));
-  TKC_TRY(cudaGetLastError());
-  TKC_TRY(cudaFreeAsync(go, st));
-  std::vector<unsigned char> h(pk.bytes());
-  TKC_TRY(read_back(h.data(), w.out, pk.bytes(), st));
-  const u32 *h_tied = (const u32 *)(h.data() + pk.tied()), *h_ntop = (const u32 *)(h.data() + pk.ntop());
-  const u64 *h_ctr = (const u64 *)(h.data() + pk.ctr());
-  ntop.assign(h_ntop, h_ntop + ng);
-  tied.assign(h_tied, h_tied + ng);
-  gctr.assign(h_ctr, h_ctr + 4 * (size_t)ng);
-  for (u32 i = 0; i < ng; ++i) {
-    tkc_result *out = &outs[i];
-    const u32 kg = go_h[i].kk;
-    const size_t src = (size_t)i * rs.kk;
-    if (!kg) continue;
-    if (out->ids) memcpy(out->ids, h.data() + pk.id() + 4 * src, kg * sizeof(u32));
-    if (out->dist_sum) memcpy(out->dist_sum, h.data() + pk.S() + 8 * src, kg * sizeof(u64));
-    if (out->reach) memcpy(out->reach, h.data() + pk.r() + 4 * src, kg * sizeof(u32));
-    if (out->farness) memcpy(out->farness, h.data() + pk.f() + 8 * src, kg * sizeof(double));
-    if (out->closeness) memcpy(out->closeness, h.data() + pk.c() + 8 * src, kg * sizeof(double));
-  }
-  for (u32 i = 0; i < ng; ++i)
-    if (ntop[i] < go_h[i].kk) tied[i] = go_h[i].nzero;  // the k-th is a closeness-0 vertex
   return TKC_OK;
 }
 
@@ -1053,7 +1109,7 @@ void tkc_free_graph(tkc_graph *g) {
   if (g->icol && g->icol != g->col) cudaFreeAsync(g->icol, st);
   void *ptrs[] = {g->off, g->col, g->deg_order, g->given_order, g->alpha, g->omega, g->scc_size, g->features,
                   g->learned_order, g->seeded_order, g->nb_order, g->nb_S, g->nb_r, g->nb_key, g->nb_hkey,
-                  g->nb_horder, g->comp, g->zero_ids, g->cls, g->n_cls};
+                  g->nb_horder, g->comp, g->zero_ids, g->n_zero, g->cls, g->n_cls};
   for (void *p : ptrs)
     if (p) cudaFreeAsync(p, st);
   g->ctx->graphs_alive--;
@@ -1280,22 +1336,24 @@ static int topk_one(tkc_graph *g, uint32_t k, tkc_result *out, int harmonic) {
   rs.nocut_prefix = (u32)std::min<u64>((u64)o.seed_factor * kk, 0xffffffffull);
   rs.kk = kk;
   rs.ng = 1;
+  std::vector<GraphOut> go(1);
+  go[0].n = g->n;
+  go[0].base = 0;
+  go[0].kk = kk;
+  go[0].nzero = 0;
+  go[0].nzero_dev = g->n_zero;
+  go[0].zero_ids = g->zero_ids;
+  std::vector<unsigned char> packed;
+  rs.go = &go;
+  rs.out = &packed;
   r.batch_bits = bits;
   Ctl hc;
   int rc_run = run_search(ctx, rs, &hc);
   ctx->opt = saved;
   TKC_RC(rc_run);
-  std::vector<GraphOut> go(1);
-  go[0].n = g->n;
-  go[0].base = 0;
-  go[0].kk = kk;
-  go[0].nzero = g->n_zero;
-  go[0].zero_ids = g->zero_ids;
-  std::vector<unsigned> ntop, tied;
+  std::vector<unsigned> tied;
   std::vector<u64> gctr;
-  TKC_RC(finish_run(ctx, rs, go, &r, ntop, tied, gctr));
-  TKC_TRY(cudaEventRecord(ctx->ev[2], st));
-  TKC_TRY(cudaStreamSynchronize(st));
+  TKC_RC(finish_run(ctx, rs, go, &r, tied, gctr));
   r.n_tied_at_kth = tied[0];
   r.edges_visited = hc.edges_visited;
   r.edges_scanned = hc.edges_scanned;
@@ -1406,10 +1464,11 @@ static int topk_shard(tkc_graph *g, uint32_t k, uint32_t first, uint32_t shard, 
   go[0].base = 0;
   go[0].kk = kk;
   go[0].nzero = g->n - g->n_src_deg;
+  go[0].nzero_dev = nullptr;
   go[0].zero_ids = g->deg_order + g->n_src_deg;
-  std::vector<unsigned> ntop, tied;
+  std::vector<unsigned> tied;
   std::vector<u64> gctr;
-  TKC_RC(finish_run(ctx, rs, go, &r, ntop, tied, gctr));
+  TKC_RC(finish_run(ctx, rs, go, &r, tied, gctr));
   TKC_TRY(cudaEventRecord(ctx->ev[2], st));
   TKC_TRY(cudaStreamSynchronize(st));
   r.n_tied_at_kth = tied[0];
@@ -1733,10 +1792,11 @@ static int topk_bound(tkc_graph *g, uint32_t k, tkc_result *out) {
   go[0].base = 0;
   go[0].kk = kk;
   go[0].nzero = n - g->n_src_deg;
+  go[0].nzero_dev = nullptr;
   go[0].zero_ids = g->deg_order + g->n_src_deg;
-  std::vector<unsigned> ntop, tied;
+  std::vector<unsigned> tied;
   std::vector<u64> gctr;
-  LB_RC(finish_run(ctx, rs, go, &r, ntop, tied, gctr));
+  LB_RC(finish_run(ctx, rs, go, &r, tied, gctr));
   LB_TRY(cudaEventRecord(ctx->ev[2], st));
   LB_TRY(cudaStreamSynchronize(st));
   cleanup();
@@ -1942,21 +2002,23 @@ static int topk_many(tkc_ctx *ctx, tkc_graph *const *gs, uint32_t ng, uint32_t k
     rs.order = gorder;
     rs.g_end = gend + ng;  // ends of the graphs' runs after their openings
   }
-  Ctl hc;
-  MULTI_RC(run_search(ctx, rs, &hc));
   std::vector<GraphOut> go(ng);
   for (u32 i = 0; i < ng; ++i) {
     go[i].n = gs[i]->n;
     go[i].base = vbase[i];
     go[i].kk = std::min<u32>(k, gs[i]->n);
     go[i].nzero = zpos[i + 1] - zpos[i];
+    go[i].nzero_dev = nullptr;
     go[i].zero_ids = zlist + zpos[i];
   }
-  std::vector<unsigned> ntop, tied;
+  std::vector<unsigned char> packed;
+  rs.go = &go;
+  rs.out = &packed;
+  Ctl hc;
+  MULTI_RC(run_search(ctx, rs, &hc));
+  std::vector<unsigned> tied;
   std::vector<u64> gctr;
-  MULTI_RC(finish_run(ctx, rs, go, outs, ntop, tied, gctr));
-  MULTI_TRY(cudaEventRecord(ctx->ev[2], st));
-  MULTI_TRY(cudaStreamSynchronize(st));
+  MULTI_RC(finish_run(ctx, rs, go, outs, tied, gctr));
   float ms0 = 0, ms1 = 0, ms2 = 0;
   cudaEventElapsedTime(&ms0, ctx->ev[0], ctx->ev[1]);
   cudaEventElapsedTime(&ms1, ctx->ev[1], ctx->ev[2]);

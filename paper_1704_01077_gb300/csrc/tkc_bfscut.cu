@@ -1272,6 +1272,10 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
     p.VL = p0.VL + team * p0.vtx_stride;
     p.stamp = p0.stamp + team * p0.vtx_stride;
     if (p0.norder_dev) p.norder = p0.sh->norder;
+    if (p0.bu_cnt) {
+      p.n_bu = p0.bu_cnt[0];
+      p.n_bu_heavy = p0.bu_cnt[1];
+    }
     if (p0.trace) {
       p.trace_cap = p0.trace_cap / p0.teams;
       p.trace = p0.trace + (size_t)team * p.trace_cap * 16;

@@ -147,6 +147,7 @@ struct RunParams {
   // others by label (nullptr: every vertex, by label)
   const uint32_t *bu_list;
   uint32_t n_bu, n_bu_heavy;
+  const uint32_t *bu_cnt;  // device words the kernel reads those two from (nullptr: as given)
   // several graphs in their own ids: graph g's vertices with an in-arc are
   // bu_list[g_base[g], g_base[g] + g_bu[2 g]), the g_bu[2 g + 1] long rows
   // first; a batch of one graph's searches runs bottom-up over that part
@@ -246,7 +247,7 @@ struct Workspace {
   unsigned long long *wsum = nullptr;
   unsigned long long *top_S = nullptr;
   uint32_t *top_r = nullptr, *top_id = nullptr;
-  Ctl *ctl = nullptr;               // two per team: the opening's and the main launch's
+  Ctl *ctl = nullptr;               // two per team: the opening's and the main launch's (after *sh, same allocation)
   uint32_t *f_order = nullptr;      // source order kept by the filter
   uint8_t *f_keep = nullptr;        // its keep flags
   uint32_t *f_count = nullptr;      // kept positions per tile
@@ -294,6 +295,9 @@ cudaError_t dev_malloc(T **p, size_t bytes, cudaStream_t st) {
 // Short reads go through the context's page-locked buffer: a copy into
 // pageable memory is staged by the driver and costs about 4 us more.
 cudaError_t read_back(void *dst, const void *src, size_t bytes, cudaStream_t st);
+// Two reads, one wait (bytes2 may be 0).
+cudaError_t read_back2(void *dst, const void *src, size_t bytes, void *dst2, const void *src2, size_t bytes2,
+                       cudaStream_t st);
 constexpr size_t kPoolKeepShare = 32;
 constexpr size_t kStageMost = 1u << 20;
 }  // namespace tkc
@@ -349,7 +353,7 @@ struct tkc_graph {
   uint32_t *deg_order = nullptr;              // computeBoundsDeg order (all n vertices)
   uint32_t n_src_deg = 0;                     // vertices with out-degree >= 1 (prefix of deg_order)
   mutable uint32_t *zero_ids = nullptr;       // vertices of out-degree 0, id order (ensure_zero_list)
-  mutable uint32_t n_zero = 0;
+  mutable uint32_t *n_zero = nullptr;         // device: how many
   mutable bool have_zero = false;
   uint32_t *given_order = nullptr;            // filtered caller order
   uint32_t n_src_given = 0;
@@ -389,7 +393,6 @@ struct tkc_graph {
   mutable uint32_t *s_cnt = nullptr;          // device: the bottom-up list's counts (n_bu, n_bu_heavy)
   mutable cudaEvent_t s_ready = nullptr;      // the copy is being built on the context's helper stream
   mutable uint32_t *bu_list = nullptr;        // bottom-up sweep order of that CSR: vertices with an in-arc, hubs first
-  mutable uint32_t n_bu = 0, n_bu_heavy = 0;
   mutable uint32_t *g_bu = nullptr;           // a union in its own ids: per graph n_bu and n_bu_heavy (device)
   mutable uint32_t heavy_in = 0;              // the list's long-row threshold (kHeavyIn or kHeavyInLabelled)
 };

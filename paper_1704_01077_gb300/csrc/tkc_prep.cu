@@ -575,7 +575,8 @@ __global__ void k_zero_flag(const u32 *off, u32 n, u32 *flag) {
     flag[v] = v < n && off[v + 1] == off[v];
 }
 
-__global__ void k_zero_out(const u32 *off, const u32 *pos, u32 n, u32 *out) {
+__global__ void k_zero_out(const u32 *off, const u32 *pos, u32 n, u32 *out, u32 *cnt) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *cnt = pos[n];
   for (u32 v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
     if (off[v + 1] == off[v]) out[pos[v]] = v;
 }
@@ -597,14 +598,11 @@ int ensure_zero_list(const tkc_graph *g) {
   if (!g->zero_ids) TKC_TRY(dev_malloc(&g->zero_ids, (size_t)n * sizeof(u32), st));
   TKC_LAUNCH(k_zero_flag<<<grid_for((u64)n + 1, 256), 256, 0, st>>>(g->off, n, flag));
   TKC_RC(scan_exclusive(flag, flag, (u64)n + 1, tmp, st));
-  TKC_LAUNCH(k_zero_out<<<grid_for(n, 256), 256, 0, st>>>(g->off, flag, n, g->zero_ids));
+  if (!g->n_zero) TKC_TRY(dev_malloc(&g->n_zero, sizeof(u32), st));
+  TKC_LAUNCH(k_zero_out<<<grid_for(n, 256), 256, 0, st>>>(g->off, flag, n, g->zero_ids, g->n_zero));
   TKC_TRY(cudaGetLastError());
-  u32 cnt = 0;
-  TKC_TRY(cudaMemcpyAsync(&cnt, flag + n, sizeof(u32), cudaMemcpyDeviceToHost, st));
   TKC_TRY(cudaFreeAsync(flag, st));
   TKC_TRY(cudaFreeAsync(tmp, st));
-  TKC_TRY(cudaStreamSynchronize(st));
-  g->n_zero = cnt;
   g->have_zero = true;
   return TKC_OK;
 }
@@ -803,7 +801,6 @@ void free_search_csr(const tkc_graph *g) {
   g->g_bu = nullptr;
   g->s_off = g->s_col = g->s_ioff = g->s_icol = g->s_lab = g->s_unlab = g->s_cnt = nullptr;
   g->bu_list = nullptr;
-  g->n_bu = g->n_bu_heavy = 0;
   g->s_mode = -1;
 }
 
@@ -820,7 +817,7 @@ void free_search_csr(const tkc_graph *g) {
 // slots, ties and outputs keep the graph's own ids; only the search's rows
 // are indexed by labels.
 // The labelled copy and its bottom-up list, enqueued on `st` without a host
-// wait (the list's counts land in g->s_cnt).  The graph's in-arc CSR exists.
+// wait (the list's counts stay in g->s_cnt, where the search reads them).  The graph's in-arc CSR exists.
 static int build_labelled_copy(const tkc_graph *g, cudaStream_t st) {
   const u32 n = g->n;
   u32 *keys = nullptr, *gcol = nullptr, *tmp = nullptr;
@@ -869,23 +866,13 @@ static int build_labelled_copy(const tkc_graph *g, cudaStream_t st) {
   return build_bu_list(g->s_ioff, n, g->heavy_in, st, &g->bu_list, g->s_cnt);
 }
 
-// Reads the bottom-up list's counts once the work that writes them is done.
-static int read_bu_counts(const tkc_graph *g) {
-  cudaStream_t st = g->ctx->stream;
-  u32 c[2] = {0, 0};
-  TKC_TRY(read_back(c, g->s_cnt, sizeof(c), st));
-  g->n_bu = c[0];
-  g->n_bu_heavy = c[1];
-  return TKC_OK;
-}
-
 // A copy started on the helper stream: the context's stream waits for it.
 static int finish_started_copy(const tkc_graph *g) {
   if (!g->s_ready) return TKC_OK;
   TKC_TRY(cudaStreamWaitEvent(g->ctx->stream, g->s_ready, 0));
   TKC_TRY(cudaEventDestroy(g->s_ready));
   g->s_ready = nullptr;
-  return read_bu_counts(g);
+  return TKC_OK;
 }
 
 int ensure_search_csr(const tkc_graph *g, bool relabel, const u32 *gid, u32 ng) {
@@ -905,7 +892,6 @@ int ensure_search_csr(const tkc_graph *g, bool relabel, const u32 *gid, u32 ng) 
   } else {
     TKC_RC(build_labelled_copy(g, st));
   }
-  TKC_RC(read_bu_counts(g));
   g->s_mode = want;
   return TKC_OK;
 }
