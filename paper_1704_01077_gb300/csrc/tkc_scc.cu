@@ -49,11 +49,14 @@ unsigned grid_of(u64 work, unsigned tpb = 256, unsigned cap = 152 * 16) {
 
 // ---------------------------------------------------------------- trimming
 
-__global__ void k_trim_init(const u32 *off, const u32 *ioff, u32 n, u32 *outd, u32 *ind, uint8_t *active) {
+// (comp: every vertex its own until its SCC is found, so that later passes may
+// run before the host knows that all are)
+__global__ void k_trim_init(const u32 *off, const u32 *ioff, u32 n, u32 *outd, u32 *ind, uint8_t *active, u32 *comp) {
   for (u32 v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
     outd[v] = off[v + 1] - off[v];
     ind[v] = ioff[v + 1] - ioff[v];
     active[v] = 1;
+    comp[v] = v;
   }
 }
 
@@ -223,65 +226,88 @@ __global__ void __launch_bounds__(kBfsThreads) k_bfs_reach(const u32 *off, const
   }
 }
 
-__global__ void k_bfs_start(const u32 *off, u32 *mark, u32 *q0, u64 *qo0, BfsCtl *c, u32 src) {
+// The vertex a packed maximum names (k_pivot, k_biggest), INF for none.
+__device__ __forceinline__ u32 named_vertex(u64 best) { return best ? 0xffffffffu - (u32)(best & 0xffffffffu) : INF; }
+
+// From vertex src, or with src = INF from the pivot named by *best (none: the
+// search ends at once).
+__global__ void k_bfs_start(const u32 *off, u32 *mark, u32 *q0, u64 *qo0, BfsCtl *c, u32 src, const u64 *best) {
+  if (src == INF) src = named_vertex(*best);
+  if (src == INF) return;
   mark[src] = 0;
   q0[0] = src;
   qo0[0] = 0;
   c->q[0] = (1ull << kQShift) | (unsigned long long)(off[src + 1] - off[src]);
 }
 
-// Several sources at once (nsrc distinct vertices, device array): all at step 0.
-__global__ void k_bfs_start_many(const u32 *off, const u32 *src, u32 nsrc, u32 *mark, u32 *q0, u64 *qo0,
+// Several sources at once (*nsrc distinct vertices): all at step 0.  One block.
+__global__ void k_bfs_start_many(const u32 *off, const u32 *src, const u32 *nsrc, u32 *mark, u32 *q0, u64 *qo0,
                                  BfsCtl *c) {
-  u64 arcs = 0;
-  for (u32 i = 0; i < nsrc; ++i) {
-    const u32 v = src[i];
-    mark[v] = 0;
-    q0[i] = v;
-    qo0[i] = arcs;
-    arcs += off[v + 1] - off[v];
+  __shared__ u64 s_warp[32], s_run;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const u32 n = *nsrc;
+  if (threadIdx.x == 0) s_run = 0;
+  __syncthreads();
+  for (u32 base = 0; base < n; base += blockDim.x) {
+    const u32 i = base + threadIdx.x;
+    u32 v = 0;
+    u64 d = 0;
+    if (i < n) {
+      v = src[i];
+      d = off[v + 1] - off[v];
+    }
+    u64 incl = d;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const u64 t = __shfl_up_sync(FULL, incl, o);
+      if (lane >= o) incl += t;
+    }
+    if (lane == 31) s_warp[wid] = incl;
+    __syncthreads();
+    u64 before = s_run;
+    for (int w = 0; w < wid; ++w) before += s_warp[w];
+    if (i < n) {
+      mark[v] = 0;
+      q0[i] = v;
+      qo0[i] = before + incl - d;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int w = 0; w < nw; ++w) s_run += s_warp[w];
+    __syncthreads();
   }
-  c->q[0] = ((unsigned long long)nsrc << kQShift) | arcs;
+  if (threadIdx.x == 0) c->q[0] = ((unsigned long long)n << kQShift) | s_run;
 }
 
-// Reachability from src (or, with srcs, from the nsrc vertices of the device
-// array srcs) along (off, col) into mark (see k_bfs_reach); one cooperative
-// launch.
+// Reachability along (off, col) into mark (see k_bfs_reach) from vertex src;
+// from the pivot that *best names (src = INF); or from the *nsrc vertices of
+// srcs.  One cooperative launch, no host wait: *c (zero) holds its error word
+// for the caller.
 int bfs_reach(tkc_ctx *ctx, const u32 *off, const u32 *col, const u32 *roff, const u32 *rcol, u32 n, u64 arcs,
-              u32 *mark, u32 src, cudaStream_t st, const u32 *srcs = nullptr, u32 nsrc = 0) {
-  static int per_sm = 0;
-  if (!per_sm) {
-    TKC_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bfs_reach, kBfsThreads, 0));
-    if (per_sm <= 0) return TKC_ECUDA;
-  }
+              u32 *mark, u32 src, const u64 *best, const u32 *srcs, const u32 *nsrc, BfsCtl *c, cudaStream_t st) {
   u32 *q = nullptr;
   u64 *qo = nullptr;
-  BfsCtl *c = nullptr;
   TKC_TRY(dev_malloc(&q, (size_t)2 * n * sizeof(u32), st));
   TKC_TRY(dev_malloc(&qo, (size_t)2 * n * sizeof(u64), st));
-  TKC_TRY(dev_malloc(&c, sizeof(BfsCtl), st));
-  TKC_TRY(cudaMemsetAsync(c, 0, sizeof(BfsCtl), st));
   TKC_TRY(cudaMemsetAsync(mark, 0xff, (size_t)n * sizeof(u32), st));
   u32 *q0 = q, *q1 = q + n;
   u64 *qo0 = qo, *qo1 = qo + n;
   if (srcs) {
-    TKC_LAUNCH(k_bfs_start_many<<<1, 1, 0, st>>>(off, srcs, nsrc, mark, q0, qo0, c));
+    TKC_LAUNCH(k_bfs_start_many<<<1, 1024, 0, st>>>(off, srcs, nsrc, mark, q0, qo0, c));
   } else {
-    TKC_LAUNCH(k_bfs_start<<<1, 1, 0, st>>>(off, mark, q0, qo0, c, src));
+    TKC_LAUNCH(k_bfs_start<<<1, 1, 0, st>>>(off, mark, q0, qo0, c, src, best));
   }
-  u64 timeout = ctx->opt.timeout_cycles ? ctx->opt.timeout_cycles : (1ull << 34);
+  u64 timeout = grid_timeout(ctx);
   void *args[] = {(void *)&off,  (void *)&col, (void *)&roff, (void *)&rcol, (void *)&n,
                   (void *)&arcs, (void *)&mark, (void *)&q0,  (void *)&q1,   (void *)&qo0,
                   (void *)&qo1,  (void *)&c,    (void *)&timeout};
-  const int blocks = std::max(1, std::min(per_sm * ctx->num_sms, (int)((n + kBfsThreads - 1) / kBfsThreads)));
+  const int blocks = grid_blocks(ctx, k_bfs_reach, kBfsThreads, n);
+  if (blocks <= 0) return TKC_ECUDA;
   note_launches(1);
   TKC_TRY(cudaLaunchCooperativeKernel((const void *)k_bfs_reach, dim3(blocks), dim3(kBfsThreads), args, 0, st));
-  int err = 0;
-  TKC_TRY(read_back(&err, &c->bar.err, sizeof(int), st));
   TKC_TRY(cudaFreeAsync(q, st));
   TKC_TRY(cudaFreeAsync(qo, st));
-  TKC_TRY(cudaFreeAsync(c, st));
-  return err ? err : TKC_OK;
+  return TKC_OK;
 }
 
 // ---------------------------------------------------------------- pivot and FW-BW
@@ -302,7 +328,8 @@ __global__ void k_pivot(const u32 *outd, const u32 *ind, const uint8_t *active, 
   if ((threadIdx.x & 31) == 0 && b) atomicMax(best, b);
 }
 
-__global__ void k_fwbw_mark(const u32 *fw, const u32 *bw, u32 n, uint8_t *active, u32 *comp, u32 pivot) {
+__global__ void k_fwbw_mark(const u32 *fw, const u32 *bw, u32 n, uint8_t *active, u32 *comp, const u64 *best) {
+  const u32 pivot = named_vertex(*best);  // none: nothing is reached both ways
   for (u32 v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
     if (active[v] && fw[v] != INF && bw[v] != INF) {
       comp[v] = pivot;
@@ -469,6 +496,9 @@ __global__ void k_biggest(const u32 *wgt, const u32 *minid, u32 n, u64 *best) {
   if ((threadIdx.x & 31) == 0 && b) atomicMax(best, b);
 }
 
+// The biggest SCC: that of the vertex *best names.
+__global__ void k_big(const u32 *comp, const u64 *best, u32 *big) { *big = comp[named_vertex(*best)]; }
+
 __global__ void k_count_reached(const u32 *dist, u32 n, u32 *cnt) {
   u32 c = 0;
   for (u32 v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) c += dist[v] != INF;
@@ -550,7 +580,8 @@ __global__ void k_unique_compact(const u32 *cu, const u32 *cv, const u32 *pos, u
 
 // Predecessor lists: each pair's source into its target's list (positions
 // claimed once per warp and target SCC).
-__global__ void k_pred_scatter(const u32 *ou, const u32 *ov, u32 m, const u32 *poff, u32 *pcur, u32 *pred) {
+__global__ void k_pred_scatter(const u32 *ou, const u32 *ov, const u32 *pairs, const u32 *poff, u32 *pcur, u32 *pred) {
+  const u32 m = *pairs;
   const int lane = threadIdx.x & 31;
   for (u32 base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; base < m; base += gridDim.x * blockDim.x) {
     const u32 i = base + lane;
@@ -771,155 +802,156 @@ struct DevBufs {
   }
 };
 
-u32 read_u32(const u32 *d, cudaStream_t st, int *rc) {
-  u32 h = 0;
-  cudaError_t e = cudaMemcpyAsync(&h, d, sizeof(u32), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) {
-    tkc_set_last_cuda_error(e, "readback", __FILE__, __LINE__);
-    *rc = TKC_ECUDA;
-  }
-  return h;
-}
-
 }  // namespace
 
+// Device words of one call, read together.
+struct SccWords {
+  GridBar bar;       // of the launches that loop over rounds
+  BfsCtl bfs[4];     // of the reach searches
+  u64 best0, best;   // the first pivot; the latest one, later the biggest SCC's vertex
+  u64 left;          // the pivot of what neither trimming nor the first pivot took (0: nothing)
+  u32 flag[2];       // round flags
+  u32 big, reach;    // the biggest SCC, vertices reached from the first pivot (or from big)
+};
+
 int reach_directed_gpu(tkc_graph *g, const u32 *gid, u32 ng) {
-  cudaStream_t st = g->ctx->stream;
+  tkc_ctx *ctx = g->ctx;
+  cudaStream_t st = ctx->stream;
   const u32 n = g->n;
+  const bool many = gid && ng > 1;
   DevBufs b;
   b.st = st;
-  u32 *outd, *ind, *comp, *fw, *bw, *color, *found, *flag, *wgt, *minid;
+  u32 *outd, *ind, *comp, *fw, *bw, *color, *found, *wgt, *minid;
   uint8_t *active;
-  u64 *best;
+  SccWords *wd;
   TKC_TRY(b.get(&outd, n));
   TKC_TRY(b.get(&ind, n));
   TKC_TRY(b.get(&comp, n));
   TKC_TRY(b.get(&fw, n));
   TKC_TRY(b.get(&bw, n));
-  TKC_TRY(b.get(&color, n));
-  TKC_TRY(b.get(&found, n));
-  TKC_TRY(b.get(&flag, 4));
+  TKC_TRY(b.get(&wgt, n));
+  TKC_TRY(b.get(&minid, n));
   TKC_TRY(b.get(&active, n));
-  TKC_TRY(b.get(&best, 1));
-  int rc = TKC_OK;
-  u32 pivot0 = INF;  // the first pivot, whose full forward and backward reach fw/bw keep
-  GridBar *bar = nullptr;
-  TKC_TRY(b.get(&bar, 1));
-  TKC_TRY(cudaMemsetAsync(bar, 0, sizeof(GridBar), st));
-  const u64 timeout = grid_timeout(g->ctx);
-  // launches that loop over rounds: the device barrier's error word is read
-  // with the next host read
+  TKC_TRY(b.get(&wd, 1));
+  TKC_TRY(cudaMemsetAsync(wd, 0, sizeof(SccWords), st));
+  u64 timeout = grid_timeout(ctx);
+  GridBar *bar = &wd->bar;
+  u32 *flag = wd->flag;
   auto loop_launch = [&](const void *kernel, int blocks, void **args) {
     if (blocks <= 0) return cudaErrorCooperativeLaunchTooLarge;
     note_launches(1);
     return cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(kLoopTPB), args, 0, st);
   };
-  auto loop_error = [&]() {
-    int e = 0;
-    cudaError_t ce = read_back(&e, &bar->err, sizeof(int), st);
-    if (ce != cudaSuccess) {
-      tkc_set_last_cuda_error(ce, "readback", __FILE__, __LINE__);
-      return (int)TKC_ECUDA;
-    }
+  SccWords h = {};
+  auto error_of = [&]() {
+    int e = h.bar.err;
+    for (const BfsCtl &c : h.bfs)
+      if (!e) e = c.bar.err;
     return e;
   };
-  TKC_LAUNCH(k_trim_init<<<grid_of(n), 256, 0, st>>>(g->off, g->ioff, n, outd, ind, active));
-  for (int round = 0;; ++round) {
-    // trim until stable
-    {
-      TKC_TRY(cudaMemsetAsync(flag, 0, 2 * sizeof(u32), st));
-      u64 to = timeout;
-      void *args[] = {(void *)&g->off, (void *)&g->col, (void *)&g->ioff, (void *)&g->icol, (void *)&n, (void *)&outd,
-                      (void *)&ind, (void *)&active, (void *)&comp, (void *)&flag, (void *)&bar, (void *)&to};
-      TKC_TRY(loop_launch((const void *)k_trim, grid_blocks(g->ctx, k_trim, kLoopTPB, n), args));
-    }
-    // pivot of the largest remaining SCC candidate
+  // trims until stable, then finds the pivot of what is left
+  auto trim_and_pivot = [&](u64 *best) -> int {
+    TKC_TRY(cudaMemsetAsync(flag, 0, 2 * sizeof(u32), st));
     TKC_TRY(cudaMemsetAsync(best, 0, sizeof(u64), st));
+    void *args[] = {(void *)&g->off, (void *)&g->col, (void *)&g->ioff, (void *)&g->icol, (void *)&n, (void *)&outd,
+                    (void *)&ind, (void *)&active, (void *)&comp, (void *)&flag, (void *)&bar, (void *)&timeout};
+    TKC_TRY(loop_launch((const void *)k_trim, grid_blocks(ctx, k_trim, kLoopTPB, n), args));
     TKC_LAUNCH(k_pivot<<<grid_of(n), 256, 0, st>>>(outd, ind, active, n, best));
-    u64 hb = 0;
-    TKC_TRY(read_back(&hb, best, sizeof(u64), st));
-    if (hb == 0) break;  // nothing left
-    if (round == 0 && gid && ng > 1) {
-      // Several graphs: one pivot per graph and one forward and one backward
-      // search from all of them, so that every graph's largest SCC is found in
-      // this round (with a single pivot, only one graph's would be, and the
-      // colouring rounds would take the rest).
-      u64 *gbest;
-      u32 *piv, *plist, *pcnt;
-      TKC_TRY(b.get(&gbest, ng));
-      TKC_TRY(b.get(&piv, ng));
-      TKC_TRY(b.get(&plist, ng));
-      TKC_TRY(b.get(&pcnt, 1));
-      TKC_TRY(cudaMemsetAsync(gbest, 0, (size_t)ng * sizeof(u64), st));
-      TKC_TRY(cudaMemsetAsync(pcnt, 0, sizeof(u32), st));
-      TKC_LAUNCH(k_pivot_many<<<grid_of(n), 256, 0, st>>>(outd, ind, active, gid, n, gbest));
-      TKC_LAUNCH(k_pivot_list<<<grid_of(ng), 256, 0, st>>>(gbest, ng, piv, plist, pcnt));
-      const u32 np = read_u32(pcnt, st, &rc);
-      TKC_RC(rc);
-      TKC_RC(bfs_reach(g->ctx, g->off, g->col, g->ioff, g->icol, n, g->arcs, fw, 0, st, plist, np));
-      TKC_RC(bfs_reach(g->ctx, g->ioff, g->icol, g->off, g->col, n, g->arcs, bw, 0, st, plist, np));
-      TKC_LAUNCH(k_fwbw_mark_many<<<grid_of(n), 256, 0, st>>>(fw, bw, gid, piv, n, active, comp));
-      continue;  // trim again, then colour; pivot0 stays INF (fw/bw hold no single vertex's reach)
-    }
-    if (round == 0) {
-      // The BFS run over the whole graph, not only the untrimmed vertices: a
-      // trimmed vertex is its own SCC, so the intersection is the same, and
-      // the full reach sets serve again below when this SCC is the biggest.
-      u32 pivot = 0xffffffffu - (u32)(hb & 0xffffffffu);
-      TKC_RC(bfs_reach(g->ctx, g->off, g->col, g->ioff, g->icol, n, g->arcs, fw, pivot, st));
-      TKC_RC(bfs_reach(g->ctx, g->ioff, g->icol, g->off, g->col, n, g->arcs, bw, pivot, st));
-      TKC_LAUNCH(k_fwbw_mark<<<grid_of(n), 256, 0, st>>>(fw, bw, n, active, comp, pivot));
-      pivot0 = pivot;
-      continue;  // trim again, then colour
-    }
-    // colouring round over the remaining vertices
-    {
-      TKC_TRY(cudaMemsetAsync(flag, 0, 2 * sizeof(u32), st));
-      u64 to = timeout;
-      void *args[] = {(void *)&g->off, (void *)&g->col, (void *)&g->ioff, (void *)&g->icol, (void *)&n,
-                      (void *)&active, (void *)&color, (void *)&found, (void *)&comp, (void *)&flag, (void *)&bar,
-                      (void *)&to};
-      TKC_TRY(loop_launch((const void *)k_color_round, grid_blocks(g->ctx, k_color_round, kLoopTPB, n), args));
-      TKC_RC(loop_error());  // a round that ran out of its budget would repeat for ever
-    }
-  }
-  TKC_RC(loop_error());
-  TKC_TRY(cudaMemcpyAsync(g->comp, comp, (size_t)n * sizeof(u32), cudaMemcpyDeviceToDevice, st));
-  // component sizes and the biggest SCC
-  TKC_TRY(b.get(&wgt, n));
-  TKC_TRY(b.get(&minid, n));
-  TKC_TRY(cudaMemsetAsync(wgt, 0, (size_t)n * sizeof(u32), st));
-  TKC_TRY(cudaMemsetAsync(minid, 0xff, (size_t)n * sizeof(u32), st));
-  TKC_LAUNCH(k_comp_stats<<<grid_of(n), 256, 0, st>>>(comp, n, wgt, minid));
-  TKC_TRY(cudaMemsetAsync(best, 0, sizeof(u64), st));
-  TKC_LAUNCH(k_biggest<<<grid_of(n), 256, 0, st>>>(wgt, minid, n, best));
-  u64 hb = 0;
-  TKC_TRY(read_back(&hb, best, sizeof(u64), st));
-  const u32 big_min = 0xffffffffu - (u32)(hb & 0xffffffffu);
-  u32 big = 0;
-  TKC_TRY(read_back(&big, comp + big_min, sizeof(u32), st));
-  // exact reach of the biggest SCC (forward), and the SCCs that reach it
-  // (backward); only reachability is used, the same from every vertex of the
-  // SCC, so the first pivot's sweeps serve when it lies in the biggest SCC
-  if (big != pivot0) {
-    TKC_RC(bfs_reach(g->ctx, g->off, g->col, g->ioff, g->icol, n, g->arcs, fw, big, st));
-    TKC_RC(bfs_reach(g->ctx, g->ioff, g->icol, g->off, g->col, n, g->arcs, bw, big, st));
-  }
-  TKC_TRY(cudaMemsetAsync(flag, 0, sizeof(u32), st));
-  TKC_LAUNCH(k_count_reached<<<grid_of(n), 256, 0, st>>>(fw, n, flag));
-  u64 reach_big = read_u32(flag, st, &rc);
-  TKC_RC(rc);
-  // condensation arcs, sorted by (cu, cv) and deduplicated
+    TKC_TRY(cudaGetLastError());
+    return TKC_OK;
+  };
+  // sizes of the SCCs, the biggest one, what the first pivot reaches, and the
+  // arcs between SCCs (counted per block; their number is blk[cross_grid])
   const unsigned cross_grid = grid_of(arc_threads(g->arcs));
   u32 *blk = nullptr, *blk_tmp = nullptr;
   TKC_TRY(b.get(&blk, (size_t)cross_grid + 1));
   TKC_TRY(b.get(&blk_tmp, ((size_t)cross_grid + 1) / 4096 + 2));
-  TKC_TRY(cudaMemsetAsync(blk + cross_grid, 0, sizeof(u32), st));
-  TKC_LAUNCH(k_cross<false><<<cross_grid, 256, 0, st>>>(g->off, g->col, comp, n, g->arcs, blk, nullptr, nullptr));
-  TKC_RC(scan_exclusive_u32(blk, blk, (u64)cross_grid + 1, blk_tmp, st));
-  const u32 m = read_u32(blk + cross_grid, st, &rc);
-  TKC_RC(rc);
+  auto statistics = [&]() -> int {
+    TKC_TRY(cudaMemsetAsync(wgt, 0, (size_t)n * sizeof(u32), st));
+    TKC_TRY(cudaMemsetAsync(minid, 0xff, (size_t)n * sizeof(u32), st));
+    TKC_TRY(cudaMemsetAsync(&wd->best, 0, sizeof(u64), st));
+    TKC_TRY(cudaMemsetAsync(&wd->reach, 0, sizeof(u32), st));
+    TKC_LAUNCH(k_comp_stats<<<grid_of(n), 256, 0, st>>>(comp, n, wgt, minid));
+    TKC_LAUNCH(k_biggest<<<grid_of(n), 256, 0, st>>>(wgt, minid, n, &wd->best));
+    TKC_LAUNCH(k_big<<<1, 1, 0, st>>>(comp, &wd->best, &wd->big));
+    TKC_LAUNCH(k_count_reached<<<grid_of(n), 256, 0, st>>>(fw, n, &wd->reach));
+    TKC_TRY(cudaMemsetAsync(blk + cross_grid, 0, sizeof(u32), st));
+    TKC_LAUNCH(k_cross<false><<<cross_grid, 256, 0, st>>>(g->off, g->col, comp, n, g->arcs, blk, nullptr, nullptr));
+    return scan_exclusive_u32(blk, blk, (u64)cross_grid + 1, blk_tmp, st);
+  };
+  TKC_LAUNCH(k_trim_init<<<grid_of(n), 256, 0, st>>>(g->off, g->ioff, n, outd, ind, active, comp));
+  TKC_RC(trim_and_pivot(&wd->best0));
+  // Forward and backward reach of the pivot.  The searches run over the whole
+  // graph, not only the untrimmed vertices: a trimmed vertex is its own SCC, so
+  // the intersection is the same, and the full reach sets serve again below
+  // when this SCC is the biggest.
+  if (many) {
+    // Several graphs: one pivot per graph and one forward and one backward
+    // search from all of them, so that every graph's largest SCC is found in
+    // this round (with a single pivot, only one graph's would be, and the
+    // colouring rounds would take the rest).
+    u64 *gbest;
+    u32 *piv, *plist, *pcnt;
+    TKC_TRY(b.get(&gbest, ng));
+    TKC_TRY(b.get(&piv, ng));
+    TKC_TRY(b.get(&plist, ng));
+    TKC_TRY(b.get(&pcnt, 1));
+    TKC_TRY(cudaMemsetAsync(gbest, 0, (size_t)ng * sizeof(u64), st));
+    TKC_TRY(cudaMemsetAsync(pcnt, 0, sizeof(u32), st));
+    TKC_LAUNCH(k_pivot_many<<<grid_of(n), 256, 0, st>>>(outd, ind, active, gid, n, gbest));
+    TKC_LAUNCH(k_pivot_list<<<grid_of(ng), 256, 0, st>>>(gbest, ng, piv, plist, pcnt));
+    TKC_RC(bfs_reach(ctx, g->off, g->col, g->ioff, g->icol, n, g->arcs, fw, 0, nullptr, plist, pcnt, &wd->bfs[0], st));
+    TKC_RC(bfs_reach(ctx, g->ioff, g->icol, g->off, g->col, n, g->arcs, bw, 0, nullptr, plist, pcnt, &wd->bfs[1], st));
+    TKC_LAUNCH(k_fwbw_mark_many<<<grid_of(n), 256, 0, st>>>(fw, bw, gid, piv, n, active, comp));
+  } else {
+    TKC_RC(bfs_reach(ctx, g->off, g->col, g->ioff, g->icol, n, g->arcs, fw, INF, &wd->best0, nullptr, nullptr,
+                     &wd->bfs[0], st));
+    TKC_RC(bfs_reach(ctx, g->ioff, g->icol, g->off, g->col, n, g->arcs, bw, INF, &wd->best0, nullptr, nullptr,
+                     &wd->bfs[1], st));
+    TKC_LAUNCH(k_fwbw_mark<<<grid_of(n), 256, 0, st>>>(fw, bw, n, active, comp, &wd->best0));
+  }
+  TKC_RC(trim_and_pivot(&wd->left));
+  // Usually nothing is left, so what follows is enqueued before the host knows
+  // (one wait for all of it; every vertex has a valid SCC name throughout).
+  TKC_RC(statistics());
+  u32 m = 0;
+  TKC_TRY(read_back2(&h, wd, sizeof(SccWords), &m, blk + cross_grid, sizeof(u32), st));
+  TKC_RC(error_of());
+  if (h.left) {
+    TKC_TRY(b.get(&color, n));
+    TKC_TRY(b.get(&found, n));
+    while (h.left) {
+      // colouring round over the remaining vertices
+      TKC_TRY(cudaMemsetAsync(flag, 0, 2 * sizeof(u32), st));
+      void *args[] = {(void *)&g->off, (void *)&g->col, (void *)&g->ioff, (void *)&g->icol, (void *)&n,
+                      (void *)&active, (void *)&color, (void *)&found, (void *)&comp, (void *)&flag, (void *)&bar,
+                      (void *)&timeout};
+      TKC_TRY(loop_launch((const void *)k_color_round, grid_blocks(ctx, k_color_round, kLoopTPB, n), args));
+      TKC_RC(trim_and_pivot(&wd->left));
+      TKC_TRY(read_back(&h, wd, sizeof(SccWords), st));
+      TKC_RC(error_of());  // (a round that ran out of its budget would repeat for ever)
+    }
+    TKC_RC(statistics());
+    TKC_TRY(read_back2(&h, wd, sizeof(SccWords), &m, blk + cross_grid, sizeof(u32), st));
+  }
+  TKC_TRY(cudaMemcpyAsync(g->comp, comp, (size_t)n * sizeof(u32), cudaMemcpyDeviceToDevice, st));
+  // exact reach of the biggest SCC (forward), and the SCCs that reach it
+  // (backward); only reachability is used, the same from every vertex of the
+  // SCC, so the first pivot's sweeps serve when it names the biggest SCC
+  const u32 pivot0 = many || !h.best0 ? INF : 0xffffffffu - (u32)(h.best0 & 0xffffffffu);
+  u32 big = h.big;
+  if (big != pivot0) {
+    TKC_RC(bfs_reach(ctx, g->off, g->col, g->ioff, g->icol, n, g->arcs, fw, big, nullptr, nullptr, nullptr, &wd->bfs[2],
+                     st));
+    TKC_RC(bfs_reach(ctx, g->ioff, g->icol, g->off, g->col, n, g->arcs, bw, big, nullptr, nullptr, nullptr, &wd->bfs[3],
+                     st));
+    TKC_TRY(cudaMemsetAsync(&wd->reach, 0, sizeof(u32), st));
+    TKC_LAUNCH(k_count_reached<<<grid_of(n), 256, 0, st>>>(fw, n, &wd->reach));
+    TKC_TRY(read_back(&h, wd, sizeof(SccWords), st));
+    TKC_RC(error_of());
+  }
+  u64 reach_big = h.reach;
+  // condensation arcs, sorted by (cu, cv) and deduplicated
   u32 *cu, *cv, *pos, *tmp, *su, *sv, *soff, *poff, *pcur, *pred, *rem, *listA, *listB;
   u64 *A, *O;
   TKC_TRY(b.get(&cu, m));
@@ -941,13 +973,11 @@ int reach_directed_gpu(tkc_graph *g, const u32 *gid, u32 ng) {
   TKC_TRY(cudaMemsetAsync(soff, 0, ((size_t)n + 1) * sizeof(u32), st));
   TKC_TRY(cudaMemsetAsync(poff, 0, ((size_t)n + 1) * sizeof(u32), st));
   TKC_LAUNCH(k_unique_compact<<<grid_of(m), 256, 0, st>>>(cu, cv, pos, m, su, sv, soff, poff));
-  const u32 mu = read_u32(pos + m, st, &rc);
-  TKC_RC(rc);
   TKC_RC(scan_exclusive_u32(soff, soff, (u64)n + 1, tmp, st));
   TKC_RC(scan_exclusive_u32(poff, poff, (u64)n + 1, tmp, st));
-  TKC_TRY(b.get(&pred, mu));
+  TKC_TRY(b.get(&pred, m));
   TKC_TRY(cudaMemsetAsync(pcur, 0, (size_t)n * sizeof(u32), st));
-  TKC_LAUNCH(k_pred_scatter<<<grid_of(mu), 256, 0, st>>>(su, sv, mu, poff, pcur, pred));
+  TKC_LAUNCH(k_pred_scatter<<<grid_of(m), 256, 0, st>>>(su, sv, pos + m, poff, pcur, pred));
   // su is sorted by source with unique pairs, so sv is the successor list
   // indexed by soff; Algorithm 6 sinks first
   TKC_TRY(b.get(&rem, n));
@@ -956,22 +986,22 @@ int reach_directed_gpu(tkc_graph *g, const u32 *gid, u32 ng) {
   TKC_TRY(b.get(&A, n));
   TKC_TRY(b.get(&O, n));
   u32 *huge = nullptr, *cnt = nullptr;
-  TKC_TRY(b.get(&huge, (size_t)mu / kDpHuge + 1));
+  TKC_TRY(b.get(&huge, (size_t)m / kDpHuge + 1));
   TKC_TRY(b.get(&cnt, 6));
   TKC_TRY(cudaMemsetAsync(cnt, 0, 6 * sizeof(u32), st));
   TKC_LAUNCH(k_sinks<<<grid_of(n), 256, 0, st>>>(wgt, soff, n, rem, listA, cnt));
   {
     u32 *nhuge = cnt + 3;
-    u64 to = timeout;
     void *args[] = {(void *)&listA, (void *)&listB, (void *)&cnt, (void *)&soff, (void *)&sv, (void *)&poff,
                     (void *)&pred, (void *)&wgt, (void *)&fw, (void *)&bw, (void *)&big, (void *)&reach_big,
                     (void *)&n, (void *)&A, (void *)&O, (void *)&rem, (void *)&huge, (void *)&nhuge, (void *)&bar,
-                    (void *)&to};
-    TKC_TRY(loop_launch((const void *)k_dp, grid_blocks(g->ctx, k_dp, kLoopTPB, n), args));
+                    (void *)&timeout};
+    TKC_TRY(loop_launch((const void *)k_dp, grid_blocks(ctx, k_dp, kLoopTPB, n), args));
   }
   TKC_LAUNCH(k_write_bounds<<<grid_of(n), 256, 0, st>>>(comp, n, A, O, wgt, g->alpha, g->omega, g->scc_size));
   TKC_TRY(cudaGetLastError());
-  return loop_error();
+  TKC_TRY(read_back(&h, wd, sizeof(SccWords), st));
+  return error_of();
 }
 
 }  // namespace tkc
