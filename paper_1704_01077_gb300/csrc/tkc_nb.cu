@@ -47,6 +47,7 @@ constexpr int kKeyFrac = 46;          // order key = floor(S * 2^46 / (r-1)^2)
 // 32 rows of hundreds of arcs to itself, 170 us a sweep of 10 M arcs.)
 constexpr u32 kHeavy = 256;
 constexpr u32 kSeg = 1024;            // arcs per segment
+static_assert(kSeg >= kHeavy, "a heavy row of d arcs has at most d / kHeavy segments");
 // Degrees up to this are summed by one lane, four loads in flight (a warp on a
 // row of about ten arcs leaves two thirds of its lanes idle).
 constexpr u32 kLight = 32;
@@ -288,17 +289,26 @@ __global__ void k_nb_level(u32 n, u32 k, u32 K, int directed, const u32 *__restr
   nb_level<false>(n, k, K, directed, gid, gdir, off, alpha, omega, prev2, cur, st, left, err);
 }
 
+// Device words of one computation of the bound, read together.
+struct NbWords {
+  GridBar bar;   // of k_nb_sweeps
+  u32 left[2];   // unfinished vertices, used in turn
+  u32 levels;    // sweeps run
+  int err;       // what no input can cause
+};
+
 // All sweeps of a small graph in one cooperative launch: two barriers a sweep
 // instead of three launches, a copy and a host wait (about 20 us, and up to
 // 256 sweeps on a street network).  N0, N1, N2: the count arrays, N~_i in
-// N[i % 3]; left[2]: unfinished vertices, two zero words used in turn; *levels
-// = sweeps run.
+// N[i % 3]; *segs heavy-row segments; wd: zero.
 constexpr int kNbTPB = 256;
 __global__ void __launch_bounds__(kNbTPB) k_nb_sweeps(u32 n, u32 K, int directed, const u32 *gid, const uint8_t *gdir,
                                                       const u32 *off, const u32 *col, const u32 *alpha,
                                                       const u32 *omega, u64 *N0, u64 *N1, u64 *N2, NbState st,
-                                                      u32 nseg, const u32 *seg_row, const u32 *seg_begin, u32 *left,
-                                                      u32 *levels, int *err, GridBar *bar, u64 timeout) {
+                                                      const u32 *segs, const u32 *seg_row, const u32 *seg_begin,
+                                                      NbWords *wd, u64 timeout) {
+  GridBar *bar = &wd->bar;
+  const u32 nseg = *segs;
   for (u32 k = 1; k <= K; ++k) {
     u64 *cur = k % 3 == 0 ? N0 : k % 3 == 1 ? N1 : N2;
     u64 *prev1 = k % 3 == 0 ? N2 : k % 3 == 1 ? N0 : N1;
@@ -308,11 +318,11 @@ __global__ void __launch_bounds__(kNbTPB) k_nb_sweeps(u32 n, u32 K, int directed
       if (nseg) nb_gather_heavy(nseg, seg_row, seg_begin, off, col, prev1, cur);
       if (!grid_sync(bar, timeout, [] {})) return;
     }
-    u32 *l = left + (k & 1);
-    nb_level<true>(n, k, K, directed, gid, gdir, off, alpha, omega, prev2, cur, st, l, err);
+    u32 *l = wd->left + (k & 1);
+    nb_level<true>(n, k, K, directed, gid, gdir, off, alpha, omega, prev2, cur, st, l, &wd->err);
     if (!grid_sync(bar, timeout, [&] {
-          left[(k & 1) ^ 1] = 0;
-          *levels = k;
+          wd->left[(k & 1) ^ 1] = 0;
+          wd->levels = k;
         }))
       return;
     if (*(volatile u32 *)l == 0) return;
@@ -348,18 +358,24 @@ __global__ void k_nb_keys(u32 n, NbState st, u64 *S_out, u32 *r_out, u64 *key, u
   }
 }
 
-__global__ void k_iota(u32 n, u32 *a) {
-  for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) a[i] = i;
+__global__ void k_src_flag(u32 n, const u32 *off, u32 *flag) {
+  for (u32 v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
+    flag[v] = off[v + 1] > off[v];
+  if (blockIdx.x == 0 && threadIdx.x == 0) flag[n] = 0;
 }
 
-// split keys of the listed sources, and the largest key
-__global__ void k_key_parts(u32 ns, const u32 *src, const u64 *key, u32 *lo, u64 *maxkey) {
+// the sources ascending, their low key words, and the largest key
+__global__ void k_src_emit(u32 n, const u32 *pos, const u64 *key, u32 *src, u32 *lo, u64 *maxkey) {
   u64 m = 0;
-  for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i < ns; i += gridDim.x * blockDim.x) {
-    const u64 kv = key[src[i]];
-    lo[i] = (u32)kv;
+  for (u32 v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+    const u32 p = pos[v];
+    if (pos[v + 1] == p) continue;
+    const u64 kv = key[v];
+    src[p] = v;
+    lo[p] = (u32)kv;
     m = max(m, kv);
   }
+  __syncwarp();
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, (u64)__shfl_xor_sync(FULL, m, o));
   if ((threadIdx.x & 31) == 0 && m) atomicMax(maxkey, m);
@@ -374,25 +390,28 @@ __global__ void k_key_hi(u32 ns, const u32 *val, const u64 *key, u32 *hi) {
 
 // The vertices of g with out-degree >= 1, sorted by (key, id): stable LSD radix
 // passes over the low and then the high 32 key bits, ids starting ascending.
-// Writes *count of them to order (device); synchronises the stream.
+// Writes *count of them to order (device).  One host wait, for their number
+// and the key bits in use.
 int nb_sort_sources(tkc_graph *g, const u64 *key, u32 *order, u32 *count) {
   cudaStream_t st = g->ctx->stream;
   const u32 n = g->n;
   *count = 0;
   if (n == 0) return TKC_OK;
-  u32 *ids = nullptr, *lo = nullptr;
+  u32 *pos = nullptr, *tmp = nullptr, *lo = nullptr;
   u64 *maxkey = nullptr;
-  TKC_TRY(dev_malloc(&ids, (size_t)n * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&pos, ((size_t)n + 1) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&tmp, (((size_t)n + 1) / 4096 + 16) * sizeof(u32), st));
   TKC_TRY(dev_malloc(&lo, (size_t)n * sizeof(u32), st));
   TKC_TRY(dev_malloc(&maxkey, sizeof(u64), st));
   TKC_TRY(cudaMemsetAsync(maxkey, 0, sizeof(u64), st));
-  TKC_LAUNCH(k_iota<<<grid_of(n), 256, 0, st>>>(n, ids));
-  TKC_RC(filter_order(g, ids, order, count));  // synchronises
-  const u32 ns = *count;
+  TKC_LAUNCH(k_src_flag<<<grid_of(n), 256, 0, st>>>(n, g->off, pos));
+  TKC_RC(scan_exclusive_u32(pos, pos, (u64)n + 1, tmp, st));
+  TKC_LAUNCH(k_src_emit<<<grid_of(n), 256, 0, st>>>(n, pos, key, order, lo, maxkey));
+  u32 ns = 0;
+  u64 mk = 0;
+  TKC_TRY(read_back2(&ns, pos + n, sizeof(u32), &mk, maxkey, sizeof(u64), st));
+  *count = ns;
   if (ns) {
-    TKC_LAUNCH(k_key_parts<<<grid_of(ns), 256, 0, st>>>(ns, order, key, lo, maxkey));
-    u64 mk = 0;
-    TKC_TRY(read_back(&mk, maxkey, sizeof(u64), st));
     int bits = 0;
     while (bits < 64 && (mk >> bits) != 0) ++bits;
     if (bits <= 32) {
@@ -403,10 +422,10 @@ int nb_sort_sources(tkc_graph *g, const u64 *key, u32 *order, u32 *count) {
       TKC_RC(radix_sort_u32_pairs(lo, order, ns, bits - 32, st));
     }
   }
-  TKC_TRY(cudaFreeAsync(ids, st));
+  TKC_TRY(cudaFreeAsync(pos, st));
+  TKC_TRY(cudaFreeAsync(tmp, st));
   TKC_TRY(cudaFreeAsync(lo, st));
   TKC_TRY(cudaFreeAsync(maxkey, st));
-  TKC_TRY(cudaStreamSynchronize(st));
   return TKC_OK;
 }
 
@@ -449,8 +468,7 @@ int ensure_nb_bounds(tkc_graph *g, u32 K, const u32 *gid, const uint8_t *gdir) {
   u64 *N[3] = {nullptr, nullptr, nullptr};
   NbState s{};
   u32 *segpos = nullptr, *seg_row = nullptr, *seg_begin = nullptr, *tmp = nullptr;
-  u32 *left = nullptr;
-  int *err = nullptr;
+  NbWords *wd = nullptr;
   for (int i = 0; i < 3; ++i) TKC_TRY(dev_malloc(&N[i], n1 * sizeof(u64), st));
   TKC_TRY(dev_malloc(&s.c, n1 * sizeof(u64), st));
   TKC_TRY(dev_malloc(&s.P, n1 * sizeof(u64), st));
@@ -460,48 +478,31 @@ int ensure_nb_bounds(tkc_graph *g, u32 K, const u32 *gid, const uint8_t *gdir) {
   TKC_TRY(dev_malloc(&s.hU, n1 * sizeof(double), st));
   TKC_TRY(dev_malloc(&segpos, (n1 + 1) * sizeof(u32), st));
   TKC_TRY(dev_malloc(&tmp, ((n1 + 1) / 4096 + 16) * sizeof(u32), st));
-  TKC_TRY(dev_malloc(&left, 2 * sizeof(u32), st));
-  TKC_TRY(dev_malloc(&err, sizeof(int), st));
-  TKC_TRY(cudaMemsetAsync(err, 0, sizeof(int), st));
+  TKC_TRY(dev_malloc(&seg_row, ((size_t)g->arcs / kHeavy + 1) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&seg_begin, ((size_t)g->arcs / kHeavy + 1) * sizeof(u32), st));
+  TKC_TRY(dev_malloc(&wd, sizeof(NbWords), st));
+  TKC_TRY(cudaMemsetAsync(wd, 0, sizeof(NbWords), st));
   // heavy-row segments
   TKC_LAUNCH(k_seg_count<<<grid_of(n), 256, 0, st>>>(n, g->off, segpos));
   TKC_RC(scan_exclusive_u32(segpos, segpos, (u64)n + 1, tmp, st));
-  u32 nseg = 0;
-  TKC_TRY(read_back(&nseg, segpos + n, sizeof(u32), st));
-  if (nseg) {
-    TKC_TRY(dev_malloc(&seg_row, (size_t)nseg * sizeof(u32), st));
-    TKC_TRY(dev_malloc(&seg_begin, (size_t)nseg * sizeof(u32), st));
-    TKC_LAUNCH(k_seg_emit<<<grid_of(n), 256, 0, st>>>(n, g->off, segpos, seg_row, seg_begin));
-  }
+  TKC_LAUNCH(k_seg_emit<<<grid_of(n), 256, 0, st>>>(n, g->off, segpos, seg_row, seg_begin));
   // sweeps: N[i % 3] holds N~_i
   TKC_LAUNCH(k_nb_init<<<grid_of(n), 256, 0, st>>>(n, s, N[0], N[2]));
-  u32 levels = 0;
-  int loop_err = 0;
+  NbWords h = {};
   if (n <= kNbLoop) {
     // (the sums of heavy rows at level 2 start from N[2], zeroed by k_nb_init)
-    GridBar *bar = nullptr;
-    TKC_TRY(dev_malloc(&bar, sizeof(GridBar) + 4 * sizeof(u32), st));
-    TKC_TRY(cudaMemsetAsync(bar, 0, sizeof(GridBar) + 4 * sizeof(u32), st));
-    u32 *words = reinterpret_cast<u32 *>(bar + 1), *d_levels = words + 2;
+    const u32 *segs = segpos + n;
     u64 timeout = grid_timeout(ctx);
     void *args[] = {(void *)&n,       (void *)&K,    (void *)&g->directed, (void *)&gid,     (void *)&gdir,
                     (void *)&g->off,  (void *)&g->col, (void *)&g->alpha,  (void *)&g->omega, (void *)&N[0],
-                    (void *)&N[1],    (void *)&N[2], (void *)&s,           (void *)&nseg,    (void *)&seg_row,
-                    (void *)&seg_begin, (void *)&words, (void *)&d_levels, (void *)&err,     (void *)&bar,
-                    (void *)&timeout};
+                    (void *)&N[1],    (void *)&N[2], (void *)&s,           (void *)&segs,    (void *)&seg_row,
+                    (void *)&seg_begin, (void *)&wd, (void *)&timeout};
     const int blocks = grid_blocks(ctx, k_nb_sweeps, kNbTPB, n);
     if (blocks <= 0) return TKC_ECUDA;
     note_launches(1);
     TKC_TRY(cudaLaunchCooperativeKernel((const void *)k_nb_sweeps, dim3(blocks), dim3(kNbTPB), args, 0, st));
-    struct {
-      GridBar bar;
-      u32 left[2], levels;
-    } h;
-    TKC_TRY(read_back(&h, bar, sizeof(GridBar) + 3 * sizeof(u32), st));
-    TKC_TRY(cudaFreeAsync(bar, st));
-    loop_err = h.bar.err;
-    levels = h.levels;
   } else {
+    u32 nseg = 0, levels = 0;
     const unsigned gwarps = grid_of((u64)((n + 31) / 32) * 32, 256);
     for (u32 k = 1; k <= K; ++k) {
       u64 *cur = N[k % 3], *prev1 = N[(k + 2) % 3], *prev2 = N[(k + 1) % 3];
@@ -510,26 +511,30 @@ int ensure_nb_bounds(tkc_graph *g, u32 K, const u32 *gid, const uint8_t *gdir) {
         if (nseg) TKC_LAUNCH(k_nb_gather_heavy<<<grid_of((u64)nseg * 32, 256), 256, 0, st>>>(
                       nseg, seg_row, seg_begin, g->off, g->col, prev1, cur));
       }
-      TKC_TRY(cudaMemsetAsync(left, 0, sizeof(u32), st));
+      TKC_TRY(cudaMemsetAsync(wd->left, 0, sizeof(u32), st));
       TKC_LAUNCH(k_nb_level<<<grid_of(n), 256, 0, st>>>(n, k, K, g->directed, gid, gdir, g->off, g->alpha, g->omega,
-                                                        prev2, cur, s, left, err));
+                                                        prev2, cur, s, wd->left, &wd->err));
       TKC_TRY(cudaGetLastError());
       u32 h_left = 0;
-      TKC_TRY(read_back(&h_left, left, sizeof(u32), st));
+      if (k == 1) {
+        TKC_TRY(read_back2(&h_left, wd->left, sizeof(u32), &nseg, segpos + n, sizeof(u32), st));
+      } else {
+        TKC_TRY(read_back(&h_left, wd->left, sizeof(u32), st));
+      }
       levels = k;
       if (h_left == 0) break;
     }
+    g->nb_levels = levels;
   }
-  TKC_LAUNCH(k_nb_keys<<<grid_of(n), 256, 0, st>>>(n, s, g->nb_S, g->nb_r, g->nb_key, g->nb_hkey, err));
-  int h_err = 0;
-  TKC_TRY(read_back(&h_err, err, sizeof(int), st));
+  TKC_LAUNCH(k_nb_keys<<<grid_of(n), 256, 0, st>>>(n, s, g->nb_S, g->nb_r, g->nb_key, g->nb_hkey, &wd->err));
+  TKC_TRY(read_back(&h, wd, sizeof(NbWords), st));
   for (int i = 0; i < 3; ++i) TKC_TRY(cudaFreeAsync(N[i], st));
-  void *frees[] = {s.c, s.P, s.bS, s.bR, s.flag, s.hU, segpos, seg_row, seg_begin, tmp, left, err};
+  void *frees[] = {s.c, s.P, s.bS, s.bR, s.flag, s.hU, segpos, seg_row, seg_begin, tmp, wd};
   for (void *p : frees)
     if (p) TKC_TRY(cudaFreeAsync(p, st));
-  if (loop_err) return loop_err;
-  if (h_err) return TKC_EGRAPH;
-  g->nb_levels = levels;
+  if (h.bar.err) return h.bar.err;
+  if (h.err) return TKC_EGRAPH;
+  if (n <= kNbLoop) g->nb_levels = h.levels;
   g->nb_cap = K;
   return TKC_OK;
 }
