@@ -309,7 +309,8 @@ struct MlpState {
   unsigned short *wb = nullptr;   // bf16 copy used by the forward passes
   float *m = nullptr, *v = nullptr;  // Adam moments
   float *grad = nullptr;          // gradient scratch
-  double *loss = nullptr;         // loss accumulator
+  double *loss = nullptr;         // loss of the latest gradient
+  float *part = nullptr;          // the gradient blocks' parameter sums and losses
   uint64_t step = 0;
   uint64_t version = 0;           // bumped whenever the weights change
   bool ready = false;

@@ -266,29 +266,28 @@ __global__ void __launch_bounds__(FT) k_mlp_forward(const float *x, u32 m, const
   }
 }
 
+constexpr int PS = (P + 31) / 32 * 32;  // a block's row of parameter sums
 constexpr int TS = 16;        // samples per gradient tile
 constexpr int kGradTPB = 256;
 constexpr int W2S = H + 1;    // row stride of W2 in shared memory: rows and columns both without conflicts
 constexpr int TH = H + 4;     // row stride of the tiles (16-byte aligned rows)
 
-__global__ void k_mlp_zero(float *grad, double *loss) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P; i += gridDim.x * blockDim.x) grad[i] = 0.f;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *loss = 0.0;
-}
-
 // Gradient of the mean squared error L = (1/m) sum (y_i - t_i)^2 with
 // respect to the parameters, the forward pass using the bf16 weights.  A block
-// takes tiles of 16 samples, keeps its share of the parameter sums in registers over its tiles, and
-// adds them to grad at the end.  Thread t = 16 y + x computes, of the 16 x 64
+// takes tiles of 16 samples, keeps its share of the parameter sums in
+// registers over its tiles, and writes them to its row of `part` (and its loss
+// to lossp) at the end.  Thread t = 16 y + x computes, of the 16 x 64
 // tile products, sample y and units x, x + 16, x + 32, x + 48, and of the 64 x
 // 64 sums of the second layer rows 4 y .. 4 y + 3 and those four columns.
 // (Bound by latency: 27 million multiply-adds.  With W2's rows 64 words apart
 // every read of a column hit one bank 32 times: 56 us for 2 048 samples.)
 __global__ void __launch_bounds__(kGradTPB) k_mlp_grad(const float *x, const float *t, u32 m, const unsigned short *wb,
-                                                       float *grad, double *loss) {
+                                                       float *part, double *lossp) {
   __shared__ float w2[H * W2S], w1[H * F], b1[H], b2[H], w3[H];
   __shared__ __align__(16) float X[TS * F], H1[TS * TH], H2[TS * TH], D2[TS * TH];  // H2 holds D1 later
   __shared__ float dy[TS], s_b3;
+  __shared__ double s_loss[kGradTPB / 32];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // k_mlp_sum may be launched
   for (int i = threadIdx.x; i < P; i += kGradTPB) {
     const float w = weight(wb, i);
     if (i < oB1) w1[i - oW1] = w;
@@ -413,23 +412,72 @@ __global__ void __launch_bounds__(kGradTPB) k_mlp_grad(const float *x, const flo
       for (int s = 0; s < TS; ++s) gb += D1[s * TH + threadIdx.x];
   }
   // the block's sums
+  float *row = part + (size_t)blockIdx.x * PS;
 #pragma unroll
   for (int r = 0; r < 4; ++r)
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if (g2[r][q] != 0.f) atomicAdd(&grad[oW2 + (4 * ty + r) * H + tx + 16 * q], g2[r][q]);
+    for (int q = 0; q < 4; ++q) row[oW2 + (4 * ty + r) * H + tx + 16 * q] = g2[r][q];
   for (int r = 0; r < 2; ++r) {
     const int p = threadIdx.x + r * kGradTPB;
-    if (p < H * F && g1[r] != 0.f) atomicAdd(&grad[oW1 + p], g1[r]);
+    if (p < H * F) row[oW1 + p] = g1[r];
   }
   const int pb = threadIdx.x < 64 ? oB1 + threadIdx.x
                  : threadIdx.x < 128 ? oB2 + threadIdx.x - 64
                  : threadIdx.x < 192 ? oW3 + threadIdx.x - 128
                                      : oB3;
-  if (threadIdx.x <= 192 && gb != 0.f) atomicAdd(&grad[pb], gb);
+  if (threadIdx.x <= 192) row[pb] = gb;
   // the losses of tx == 0, two samples per warp
   l += __shfl_xor_sync(FULL, l, 16);
-  if ((threadIdx.x & 31) == 0 && l != 0.0) atomicAdd(loss, l);
+  if ((threadIdx.x & 31) == 0) s_loss[threadIdx.x >> 5] = l;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int w = 0; w < kGradTPB / 32; ++w) t += s_loss[w];
+    lossp[blockIdx.x] = t;
+  }
+}
+
+// The gradient and the loss from the blocks' sums: 32 parameters a block, the
+// rows split over its 8 warps, added up four at a time and then by warps, in a
+// fixed order.  (Block sums added to grad by atomics, 128 to a word, made the
+// error against 64 bits 2.5e-7 for 2 048 samples, this 0.3e-7 to 0.8e-7; a
+// 64-bit sum here is no nearer and 4 us slower.)  It is launched early and
+// waits for the sums on the device, so that its launch overlaps them.
+constexpr int kSumWarps = 8;
+__global__ void __launch_bounds__(32 * kSumWarps) k_mlp_sum(const float *part, const double *lossp, u32 rows,
+                                                            float *grad, double *loss) {
+  __shared__ float s[kSumWarps][32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int p = blockIdx.x * 32 + lane;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  float a = 0.f;
+  if (p < P) {
+    u32 r = wid;
+#pragma unroll 4
+    for (; r + 3 * kSumWarps < rows; r += 4 * kSumWarps) {
+      const float *q = part + (size_t)r * PS + p;
+      a += (q[0] + q[kSumWarps * PS]) + (q[2 * kSumWarps * PS] + q[3 * kSumWarps * PS]);
+    }
+    for (; r < rows; r += kSumWarps) a += part[(size_t)r * PS + p];
+  }
+  s[wid][lane] = a;
+  __syncthreads();
+  if (wid == 0 && p < P) {
+    float t[kSumWarps];
+#pragma unroll
+    for (int w = 0; w < kSumWarps; ++w) t[w] = s[w][lane];
+#pragma unroll
+    for (int d = 1; d < kSumWarps; d *= 2)
+#pragma unroll
+      for (int w = 0; w < kSumWarps; w += 2 * d) t[w] += t[w + d];
+    grad[p] = t[0];
+  } else if (wid == 1 && blockIdx.x == 0) {
+    double l = 0.0;
+    for (u32 r = lane; r < rows; r += 32) l += lossp[r];
+#pragma unroll
+    for (int d = 16; d; d >>= 1) l += __shfl_xor_sync(FULL, l, d);
+    if (lane == 0) *loss = l;
+  }
 }
 
 // Adam (Kingma & Ba 2015) on the fp32 master weights; refreshes the bf16 copy.
@@ -493,7 +541,7 @@ static int ensure_mlp(tkc_ctx *ctx) {
 
 void free_mlp(tkc_ctx *ctx) {
   MlpState &s = ctx->mlp;
-  void *ptrs[] = {s.w, s.wb, s.m, s.v, s.grad, s.loss};
+  void *ptrs[] = {s.w, s.wb, s.m, s.v, s.grad, s.loss, s.part};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   s = MlpState();
@@ -715,10 +763,22 @@ int tkc_mlp_forward(tkc_ctx *ctx, const float *x, uint32_t m, float *y) {
 static int gradient(tkc_ctx *ctx, const float *x, const float *t, u32 m, float *grad) {
   cudaStream_t st = ctx->stream;
   MlpState &s = ctx->mlp;
-  TKC_LAUNCH(k_mlp_zero<<<(P + 255) / 256, 256, 0, st>>>(grad, s.loss));
+  if (!s.part) TKC_TRY(cudaMalloc(&s.part, (size_t)ctx->num_sms * (PS * sizeof(float) + sizeof(double))));
+  double *lossp = reinterpret_cast<double *>(s.part + (size_t)ctx->num_sms * PS);
   // a tile per block, at most a block per SM
   const unsigned blocks = (unsigned)std::min<u64>(((u64)m + TS - 1) / TS, (u64)ctx->num_sms);
-  TKC_LAUNCH(k_mlp_grad<<<blocks, kGradTPB, 0, st>>>(x, t, m, s.wb, grad, s.loss));
+  TKC_LAUNCH(k_mlp_grad<<<blocks, kGradTPB, 0, st>>>(x, t, m, s.wb, s.part, lossp));
+  cudaLaunchAttribute early = {};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((P + 31) / 32);
+  cfg.blockDim = dim3(32 * kSumWarps);
+  cfg.stream = st;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  note_launches(1);
+  TKC_TRY(cudaLaunchKernelEx(&cfg, k_mlp_sum, (const float *)s.part, (const double *)lossp, (u32)blocks, grad, s.loss));
   TKC_TRY(cudaGetLastError());
   return TKC_OK;
 }
