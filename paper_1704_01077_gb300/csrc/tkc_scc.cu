@@ -496,14 +496,30 @@ __global__ void k_biggest(const u32 *wgt, const u32 *minid, u32 n, u64 *best) {
   if ((threadIdx.x & 31) == 0 && b) atomicMax(best, b);
 }
 
-// The biggest SCC: that of the vertex *best names.
-__global__ void k_big(const u32 *comp, const u64 *best, u32 *big) { *big = comp[named_vertex(*best)]; }
+// The biggest SCC: that of the vertex *best names; the graph it lies in (gid
+// may be null: 0) and that graph's pivot.
+__global__ void k_big(const u32 *comp, const u64 *best, const u32 *gid, const u32 *piv, const u64 *best0, u32 *big,
+                      u32 *big_graph, u32 *big_pivot) {
+  const u32 v = named_vertex(*best);
+  *big = comp[v];
+  *big_graph = gid ? gid[v] : 0;
+  *big_pivot = gid ? piv[gid[v]] : named_vertex(*best0);
+}
 
-__global__ void k_count_reached(const u32 *dist, u32 n, u32 *cnt) {
+// Vertices reached, of graph *only (gid may be null: all).
+__global__ void k_count_reached(const u32 *dist, u32 n, const u32 *gid, const u32 *only, u32 *cnt) {
   u32 c = 0;
-  for (u32 v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) c += dist[v] != INF;
+  const u32 g = gid ? *only : 0;
+  for (u32 v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
+    c += dist[v] != INF && (!gid || gid[v] == g);
   c = __reduce_add_sync(FULL, c);
   if ((threadIdx.x & 31) == 0 && c) atomicAdd(cnt, c);
+}
+
+// Forgets what the searches reached in the other graphs.
+__global__ void k_keep_graph(const u32 *gid, u32 g, u32 n, u32 *fw, u32 *bw) {
+  for (u32 v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
+    if (gid[v] != g) fw[v] = bw[v] = INF;
 }
 
 // ---------------------------------------------------------------- condensation
@@ -808,10 +824,11 @@ struct DevBufs {
 struct SccWords {
   GridBar bar;       // of the launches that loop over rounds
   BfsCtl bfs[4];     // of the reach searches
-  u64 best0, best;   // the first pivot; the latest one, later the biggest SCC's vertex
+  u64 best0, best;   // the first pivot; the biggest SCC's vertex
   u64 left;          // the pivot of what neither trimming nor the first pivot took (0: nothing)
   u32 flag[2];       // round flags
-  u32 big, reach;    // the biggest SCC, vertices reached from the first pivot (or from big)
+  u32 big, big_graph, big_pivot;  // the biggest SCC, its graph and that graph's pivot
+  u32 reach;                      // vertices reached from that pivot (or from big)
 };
 
 int reach_directed_gpu(tkc_graph *g, const u32 *gid, u32 ng) {
@@ -863,7 +880,7 @@ int reach_directed_gpu(tkc_graph *g, const u32 *gid, u32 ng) {
   // sizes of the SCCs, the biggest one, what the first pivot reaches, and the
   // arcs between SCCs (counted per block; their number is blk[cross_grid])
   const unsigned cross_grid = grid_of(arc_threads(g->arcs));
-  u32 *blk = nullptr, *blk_tmp = nullptr;
+  u32 *blk = nullptr, *blk_tmp = nullptr, *piv = nullptr;
   TKC_TRY(b.get(&blk, (size_t)cross_grid + 1));
   TKC_TRY(b.get(&blk_tmp, ((size_t)cross_grid + 1) / 4096 + 2));
   auto statistics = [&]() -> int {
@@ -873,8 +890,9 @@ int reach_directed_gpu(tkc_graph *g, const u32 *gid, u32 ng) {
     TKC_TRY(cudaMemsetAsync(&wd->reach, 0, sizeof(u32), st));
     TKC_LAUNCH(k_comp_stats<<<grid_of(n), 256, 0, st>>>(comp, n, wgt, minid));
     TKC_LAUNCH(k_biggest<<<grid_of(n), 256, 0, st>>>(wgt, minid, n, &wd->best));
-    TKC_LAUNCH(k_big<<<1, 1, 0, st>>>(comp, &wd->best, &wd->big));
-    TKC_LAUNCH(k_count_reached<<<grid_of(n), 256, 0, st>>>(fw, n, &wd->reach));
+    TKC_LAUNCH(k_big<<<1, 1, 0, st>>>(comp, &wd->best, many ? gid : nullptr, piv, &wd->best0, &wd->big, &wd->big_graph,
+                                 &wd->big_pivot));
+    TKC_LAUNCH(k_count_reached<<<grid_of(n), 256, 0, st>>>(fw, n, many ? gid : nullptr, &wd->big_graph, &wd->reach));
     TKC_TRY(cudaMemsetAsync(blk + cross_grid, 0, sizeof(u32), st));
     TKC_LAUNCH(k_cross<false><<<cross_grid, 256, 0, st>>>(g->off, g->col, comp, n, g->arcs, blk, nullptr, nullptr));
     return scan_exclusive_u32(blk, blk, (u64)cross_grid + 1, blk_tmp, st);
@@ -891,7 +909,7 @@ int reach_directed_gpu(tkc_graph *g, const u32 *gid, u32 ng) {
     // this round (with a single pivot, only one graph's would be, and the
     // colouring rounds would take the rest).
     u64 *gbest;
-    u32 *piv, *plist, *pcnt;
+    u32 *plist, *pcnt;
     TKC_TRY(b.get(&gbest, ng));
     TKC_TRY(b.get(&piv, ng));
     TKC_TRY(b.get(&plist, ng));
@@ -937,16 +955,18 @@ int reach_directed_gpu(tkc_graph *g, const u32 *gid, u32 ng) {
   TKC_TRY(cudaMemcpyAsync(g->comp, comp, (size_t)n * sizeof(u32), cudaMemcpyDeviceToDevice, st));
   // exact reach of the biggest SCC (forward), and the SCCs that reach it
   // (backward); only reachability is used, the same from every vertex of the
-  // SCC, so the first pivot's sweeps serve when it names the biggest SCC
-  const u32 pivot0 = many || !h.best0 ? INF : 0xffffffffu - (u32)(h.best0 & 0xffffffffu);
+  // SCC, so the sweeps from its graph's pivot serve when that names the biggest
+  // SCC (several graphs: without what the other graphs' pivots reached)
   u32 big = h.big;
-  if (big != pivot0) {
+  if (big == h.big_pivot) {
+    if (many) TKC_LAUNCH(k_keep_graph<<<grid_of(n), 256, 0, st>>>(gid, h.big_graph, n, fw, bw));
+  } else {
     TKC_RC(bfs_reach(ctx, g->off, g->col, g->ioff, g->icol, n, g->arcs, fw, big, nullptr, nullptr, nullptr, &wd->bfs[2],
                      st));
     TKC_RC(bfs_reach(ctx, g->ioff, g->icol, g->off, g->col, n, g->arcs, bw, big, nullptr, nullptr, nullptr, &wd->bfs[3],
                      st));
     TKC_TRY(cudaMemsetAsync(&wd->reach, 0, sizeof(u32), st));
-    TKC_LAUNCH(k_count_reached<<<grid_of(n), 256, 0, st>>>(fw, n, &wd->reach));
+    TKC_LAUNCH(k_count_reached<<<grid_of(n), 256, 0, st>>>(fw, n, nullptr, nullptr, &wd->reach));
     TKC_TRY(read_back(&h, wd, sizeof(SccWords), st));
     TKC_RC(error_of());
   }
