@@ -1056,38 +1056,37 @@ int tkc_load_csr_many(tkc_ctx *ctx, uint32_t ng, const uint32_t *n, const uint64
   // every graph's checks, then one host read of all their flags; the symmetry
   // checks of the undirected ones follow (they need checked rows)
   u32 *flags = nullptr;
+  CsrCheck *table = nullptr;
+  std::vector<CsrCheck> ht(ng);
+  u32 blocks[2] = {0, 0};
+  for (u32 i = 0; i < ng; ++i) check_entry(out[i], blocks, &ht[i]);
   std::vector<u32> hf(ng, 0);
   cudaError_t e = dev_malloc(&flags, (size_t)ng * sizeof(u32), st);
+  if (e == cudaSuccess) e = dev_malloc(&table, (size_t)ng * sizeof(CsrCheck), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, (size_t)ng * sizeof(u32), st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(table, ht.data(), (size_t)ng * sizeof(CsrCheck), cudaMemcpyHostToDevice, st);
+  int rc = TKC_OK;
+  u32 bad = ng;
+  for (int pass = 0; pass < 2 && e == cudaSuccess && rc == TKC_OK; ++pass) {
+    if (blocks[pass] == 0) continue;
+    rc = enqueue_check_many(ctx, table, ng, pass, blocks[pass], flags);
+    if (rc != TKC_OK) break;
+    e = read_back(hf.data(), flags, (size_t)ng * sizeof(u32), st);
+    if (e != cudaSuccess) break;
+    for (u32 i = 0; i < ng && rc == TKC_OK; ++i)
+      if (hf[i]) {
+        rc = TKC_EGRAPH;
+        bad = i;
+      }
+  }
+  if (table) cudaFreeAsync(table, st);
+  if (flags) cudaFreeAsync(flags, st);
   if (e != cudaSuccess) {
     tkc_set_last_cuda_error(e, "tkc_load_csr_many", __FILE__, __LINE__);
     return fail(e == cudaErrorMemoryAllocation ? TKC_ENOMEM : TKC_ECUDA, ng);
   }
-  for (int pass = 0; pass < 2; ++pass) {
-    bool any = false;
-    for (u32 i = 0; i < ng; ++i) {
-      const int rc = pass == 0 ? enqueue_validate(out[i], flags + i) : enqueue_symmetric(out[i], flags + i);
-      if (rc != TKC_OK) {
-        cudaFreeAsync(flags, st);
-        return fail(rc, i);
-      }
-      any |= pass == 0 || !out[i]->directed;
-    }
-    if (!any) break;
-    e = cudaMemcpyAsync(hf.data(), flags, (size_t)ng * sizeof(u32), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) {
-      tkc_set_last_cuda_error(e, "tkc_load_csr_many", __FILE__, __LINE__);
-      cudaFreeAsync(flags, st);
-      return fail(TKC_ECUDA, ng);
-    }
-    for (u32 i = 0; i < ng; ++i)
-      if (hf[i]) {
-        cudaFreeAsync(flags, st);
-        return fail(TKC_EGRAPH, i);
-      }
-  }
-  cudaFreeAsync(flags, st);
+  if (rc != TKC_OK) return fail(rc, bad);
   for (u32 i = 0; i < ng; ++i)
     if (!out[i]->directed) {
       out[i]->ioff = out[i]->off;

@@ -90,16 +90,24 @@ inline uint64_t arc_threads(uint64_t arcs) { return (arcs + arc_chunk(arcs) - 1)
 // grid's warps in tasks of arc_chunk(arcs) consecutive indices (task c to warp
 // c mod warps: a kernel launched twice with the same grid gives each block
 // the same arcs).
+// Block `block` of `nblocks`: of the grid, or of the part of it that a launch
+// over several graphs gives this one.
 template <bool kRowStart = false, typename F>
-__device__ __forceinline__ void grid_walk_arcs(const uint32_t *off, uint32_t n, uint64_t arcs, F &&f) {
+__device__ __forceinline__ void blocks_walk_arcs(const uint32_t *off, uint32_t n, uint64_t arcs, uint32_t block,
+                                                 uint32_t nblocks, F &&f) {
   const int lane = threadIdx.x & 31;
-  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  const uint64_t warp = ((uint64_t)block * blockDim.x + threadIdx.x) >> 5;
+  const uint64_t nwarps = ((uint64_t)nblocks * blockDim.x) >> 5;
   const uint32_t chunk = arc_chunk(arcs);
   for (uint64_t a0 = warp * chunk; a0 < arcs; a0 += nwarps * chunk) {
     const uint64_t a1 = a0 + chunk < arcs ? a0 + chunk : arcs;
     warp_walk_arcs<kRowStart>(off, n, a0, a1, lane, f);
   }
+}
+
+template <bool kRowStart = false, typename F>
+__device__ __forceinline__ void grid_walk_arcs(const uint32_t *off, uint32_t n, uint64_t arcs, F &&f) {
+  blocks_walk_arcs<kRowStart>(off, n, arcs, blockIdx.x, gridDim.x, f);
 }
 
 }  // namespace tkc

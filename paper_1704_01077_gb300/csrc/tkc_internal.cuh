@@ -401,8 +401,15 @@ struct tkc_graph {
 namespace tkc {
 // tkc_prep.cu
 int validate_graph(tkc_graph *g);
-int enqueue_validate(const tkc_graph *g, uint32_t *flag);   // no host wait
-int enqueue_symmetric(const tkc_graph *g, uint32_t *flag);  // after enqueue_validate passed
+// One graph of a launch that checks many: its blocks in the launch of each
+// check (structure, symmetry).
+struct CsrCheck {
+  const uint32_t *off, *col;
+  uint64_t arcs;
+  uint32_t n, blk0[2], nblk[2];
+};
+void check_entry(const tkc_graph *g, uint32_t blk0[2], CsrCheck *c);
+int enqueue_check_many(tkc_ctx *ctx, const CsrCheck *t, uint32_t ng, int sym, uint32_t blocks, uint32_t *flags);
 int build_in_csr(const tkc_graph *g);
 int ensure_in_csr(const tkc_graph *g);
 int ensure_degree_order(tkc_graph *g);
