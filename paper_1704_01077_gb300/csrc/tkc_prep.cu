@@ -404,20 +404,28 @@ int ensure_in_csr(const tkc_graph *g) {
 
 static constexpr int kRsTPB = 256;
 static constexpr int kRsWarps = kRsTPB / 32;
-static constexpr int kRsRounds = 16;  // elements per lane
-static constexpr int kRsTile = kRsTPB * kRsRounds;
+// Elements per lane.  A pass is a chain of as many digit ranks per warp, so up
+// to kRsFew tiles of 4 the tiles are that short (65 536 pairs with tiles of 16
+// kept 16 blocks busy: 18 us a pass with its scan, 9 us now).  Up to kRsFew tiles of either length
+// every block adds up the tiles' digit counts itself (k_rs_scatter, kOwnScan)
+// and the scan between the two launches of a pass is left out.
+static constexpr int kRsShort = 4, kRsLong = 16;
+static constexpr u32 kRsFew = 128;
 
+// Digit counts of the tiles: hist[digit * ntiles + tile], with kOwnScan
+// hist[tile * 256 + digit].
+template <int kRounds, bool kOwnScan>
 __global__ void k_rs_count(const u32 *__restrict__ key, u32 n, int shift, u32 *__restrict__ hist, u32 ntiles) {
   __shared__ u32 cnt[256];
   cnt[threadIdx.x] = 0;
   __syncthreads();
 #pragma unroll 4
-  for (int r = 0; r < kRsRounds; ++r) {
-    const u64 i = (u64)blockIdx.x * kRsTile + r * kRsTPB + threadIdx.x;
+  for (int r = 0; r < kRounds; ++r) {
+    const u64 i = (u64)blockIdx.x * (kRsTPB * kRounds) + r * kRsTPB + threadIdx.x;
     if (i < n) atomicAdd(&cnt[(key[i] >> shift) & 255u], 1u);
   }
   __syncthreads();
-  hist[threadIdx.x * ntiles + blockIdx.x] = cnt[threadIdx.x];
+  hist[kOwnScan ? blockIdx.x * 256 + threadIdx.x : threadIdx.x * ntiles + blockIdx.x] = cnt[threadIdx.x];
 }
 
 // Rank of this lane's element among its warp's so far with the same digit d
@@ -436,22 +444,46 @@ __device__ __forceinline__ u32 warp_rank(u32 d, u32 *counts, int lane) {
 // warps' counts per digit are summed in warp order, and hist (scanned) holds
 // where each tile's elements of a digit start.  Eight bits a pass: half the
 // passes, and so half the traffic and launches, of four bits.
+template <int kRounds, bool kOwnScan>
 __global__ void __launch_bounds__(kRsTPB) k_rs_scatter(const u32 *__restrict__ key, const u32 *__restrict__ val,
                                                        u32 *__restrict__ key_out, u32 *__restrict__ val_out, u32 n,
                                                        int shift, const u32 *__restrict__ hist, u32 ntiles) {
   __shared__ u32 cnt[kRsWarps][256];
+  __shared__ u32 s_digits[kRsWarps];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (int i = threadIdx.x; i < kRsWarps * 256; i += kRsTPB) (&cnt[0][0])[i] = 0;
   __syncthreads();
-  const u64 base = (u64)blockIdx.x * kRsTile + wid * (32 * kRsRounds) + lane;
-  u32 k[kRsRounds], rank[kRsRounds];
+  const u64 base = (u64)blockIdx.x * (kRsTPB * kRounds) + wid * (32 * kRounds) + lane;
+  u32 k[kRounds], rank[kRounds];
 #pragma unroll
-  for (int r = 0; r < kRsRounds; ++r) k[r] = base + 32 * r < n ? key[base + 32 * r] : 0u;
+  for (int r = 0; r < kRounds; ++r) k[r] = base + 32 * r < n ? key[base + 32 * r] : 0u;
 #pragma unroll
-  for (int r = 0; r < kRsRounds; ++r)
+  for (int r = 0; r < kRounds; ++r)
     rank[r] = warp_rank(base + 32 * r < n ? (k[r] >> shift) & 255u : 256u, cnt[wid], lane);
   __syncthreads();
-  u32 at = hist[threadIdx.x * ntiles + blockIdx.x];
+  u32 at;  // where this tile's elements of digit threadIdx.x start
+  if (kOwnScan) {
+    static_assert(kRsTPB == 256, "a thread per digit");
+    u32 before = 0, total = 0;
+#pragma unroll 8
+    for (u32 t = 0; t < ntiles; ++t) {
+      const u32 c = hist[t * 256 + threadIdx.x];
+      if (t < blockIdx.x) before += c;
+      total += c;
+    }
+    u32 incl = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const u32 t = __shfl_up_sync(FULL, incl, o);
+      if (lane >= o) incl += t;
+    }
+    if (lane == 31) s_digits[wid] = incl;
+    __syncthreads();
+    at = incl - total + before;
+    for (int w = 0; w < wid; ++w) at += s_digits[w];
+  } else {
+    at = hist[threadIdx.x * ntiles + blockIdx.x];
+  }
 #pragma unroll
   for (int w = 0; w < kRsWarps; ++w) {
     const u32 t = cnt[w][threadIdx.x];
@@ -460,7 +492,7 @@ __global__ void __launch_bounds__(kRsTPB) k_rs_scatter(const u32 *__restrict__ k
   }
   __syncthreads();
 #pragma unroll
-  for (int r = 0; r < kRsRounds; ++r) {
+  for (int r = 0; r < kRounds; ++r) {
     if (base + 32 * r >= n) break;
     const u32 pos = cnt[wid][(k[r] >> shift) & 255u] + rank[r];
     key_out[pos] = k[r];
@@ -538,7 +570,9 @@ static int radix_sort_pairs(u32 *key, u32 *val, u32 n, int bits, cudaStream_t st
     TKC_TRY(cudaGetLastError());
     return TKC_OK;
   }
-  u32 ntiles = (n + kRsTile - 1) / kRsTile;
+  const int rounds = n <= kRsFew * kRsTPB * kRsShort ? kRsShort : kRsLong;
+  const u32 ntiles = (n + kRsTPB * rounds - 1) / (kRsTPB * rounds);
+  const bool own = ntiles <= kRsFew;
   u32 *k2 = nullptr, *v2 = nullptr, *hist = nullptr, *tmp = nullptr;
   size_t hlen = (size_t)256 * ntiles;
   TKC_TRY(dev_malloc(&k2, (size_t)n * sizeof(u32), st));
@@ -547,9 +581,17 @@ static int radix_sort_pairs(u32 *key, u32 *val, u32 n, int bits, cudaStream_t st
   TKC_TRY(dev_malloc(&tmp, (hlen / kScanTile + 2) * sizeof(u32), st));
   u32 *ka = key, *va = val, *kb = k2, *vb = v2;
   for (int ps = 0; ps < passes; ++ps) {
-    TKC_LAUNCH(k_rs_count<<<ntiles, kRsTPB, 0, st>>>(ka, n, 8 * ps, hist, ntiles));
-    TKC_RC(scan_exclusive(hist, hist, hlen, tmp, st));
-    TKC_LAUNCH(k_rs_scatter<<<ntiles, kRsTPB, 0, st>>>(ka, va, kb, vb, n, 8 * ps, hist, ntiles));
+    if (rounds == kRsShort) {
+      TKC_LAUNCH(k_rs_count<kRsShort, true><<<ntiles, kRsTPB, 0, st>>>(ka, n, 8 * ps, hist, ntiles));
+      TKC_LAUNCH(k_rs_scatter<kRsShort, true><<<ntiles, kRsTPB, 0, st>>>(ka, va, kb, vb, n, 8 * ps, hist, ntiles));
+    } else if (own) {
+      TKC_LAUNCH(k_rs_count<kRsLong, true><<<ntiles, kRsTPB, 0, st>>>(ka, n, 8 * ps, hist, ntiles));
+      TKC_LAUNCH(k_rs_scatter<kRsLong, true><<<ntiles, kRsTPB, 0, st>>>(ka, va, kb, vb, n, 8 * ps, hist, ntiles));
+    } else {
+      TKC_LAUNCH(k_rs_count<kRsLong, false><<<ntiles, kRsTPB, 0, st>>>(ka, n, 8 * ps, hist, ntiles));
+      TKC_RC(scan_exclusive(hist, hist, hlen, tmp, st));
+      TKC_LAUNCH(k_rs_scatter<kRsLong, false><<<ntiles, kRsTPB, 0, st>>>(ka, va, kb, vb, n, 8 * ps, hist, ntiles));
+    }
     TKC_TRY(cudaGetLastError());
     std::swap(ka, kb);
     std::swap(va, vb);
