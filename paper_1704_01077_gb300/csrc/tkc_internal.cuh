@@ -305,12 +305,13 @@ constexpr size_t kStageMost = 1u << 20;
 // Source-order model: 5 -> 64 -> 64 -> 1 MLP, fp32 master weights with a
 // bf16 copy for the forward passes, Adam moments.
 struct MlpState {
-  float *w = nullptr;             // TKC_MLP_PARAMS fp32 master weights
+  float *w = nullptr;             // TKC_MLP_PARAMS fp32 master weights (and the allocation of them all)
   unsigned short *wb = nullptr;   // bf16 copy used by the forward passes
   float *m = nullptr, *v = nullptr;  // Adam moments
   float *grad = nullptr;          // gradient scratch
   double *loss = nullptr;         // loss of the latest gradient
-  float *part = nullptr;          // the gradient blocks' parameter sums and losses
+  float *part = nullptr;          // the gradient blocks' parameter sums
+  double *lossp = nullptr;        // and their losses
   uint64_t step = 0;
   uint64_t version = 0;           // bumped whenever the weights change
   bool ready = false;

@@ -280,7 +280,8 @@ constexpr int TH = H + 4;     // row stride of the tiles (16-byte aligned rows)
 // tile products, sample y and units x, x + 16, x + 32, x + 48, and of the 64 x
 // 64 sums of the second layer rows 4 y .. 4 y + 3 and those four columns.
 // (Bound by latency: 27 million multiply-adds.  With W2's rows 64 words apart
-// every read of a column hit one bank 32 times: 56 us for 2 048 samples.)
+// every read of a column hit one bank 32 times and 2 048 samples took 56 us,
+// now 11.)
 __global__ void __launch_bounds__(kGradTPB) k_mlp_grad(const float *x, const float *t, u32 m, const unsigned short *wb,
                                                        float *part, double *lossp) {
   __shared__ float w2[H * W2S], w1[H * F], b1[H], b2[H], w3[H];
@@ -527,23 +528,36 @@ __global__ void k_score_keys(const float *y, u32 n, u32 *key, u32 *val) {
 
 int filter_order(tkc_graph *g, const u32 *d_order_all, u32 *d_out, u32 *count);
 
+// The model's buffers, one allocation (an allocation takes about 40 us).
 static int ensure_mlp(tkc_ctx *ctx) {
   MlpState &s = ctx->mlp;
   if (s.w) return TKC_OK;
-  TKC_TRY(cudaMalloc(&s.w, P * sizeof(float)));
-  TKC_TRY(cudaMalloc(&s.wb, P * sizeof(unsigned short)));
-  TKC_TRY(cudaMalloc(&s.m, P * sizeof(float)));
-  TKC_TRY(cudaMalloc(&s.v, P * sizeof(float)));
-  TKC_TRY(cudaMalloc(&s.grad, P * sizeof(float)));
-  TKC_TRY(cudaMalloc(&s.loss, sizeof(double)));
+  unsigned char *base = nullptr;
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    unsigned char *p = base + at;
+    at += (bytes + 255) / 256 * 256;
+    return p;
+  };
+  for (int pass = 0; pass < 2; ++pass) {
+    if (pass) TKC_TRY(cudaMalloc(&base, at));
+    at = 0;
+    float *w = (float *)take(P * sizeof(float));
+    s.wb = (unsigned short *)take(P * sizeof(unsigned short));
+    s.m = (float *)take(P * sizeof(float));
+    s.v = (float *)take(P * sizeof(float));
+    s.grad = (float *)take(P * sizeof(float));
+    s.loss = (double *)take(sizeof(double));
+    s.lossp = (double *)take((size_t)ctx->num_sms * sizeof(double));
+    s.part = (float *)take((size_t)ctx->num_sms * PS * sizeof(float));
+    if (pass) s.w = w;  // (set last: it says that the buffers are there)
+  }
   return TKC_OK;
 }
 
 void free_mlp(tkc_ctx *ctx) {
   MlpState &s = ctx->mlp;
-  void *ptrs[] = {s.w, s.wb, s.m, s.v, s.grad, s.loss, s.part};
-  for (void *p : ptrs)
-    if (p) cudaFree(p);
+  if (s.w) cudaFree(s.w);
   s = MlpState();
 }
 
@@ -763,11 +777,9 @@ int tkc_mlp_forward(tkc_ctx *ctx, const float *x, uint32_t m, float *y) {
 static int gradient(tkc_ctx *ctx, const float *x, const float *t, u32 m, float *grad) {
   cudaStream_t st = ctx->stream;
   MlpState &s = ctx->mlp;
-  if (!s.part) TKC_TRY(cudaMalloc(&s.part, (size_t)ctx->num_sms * (PS * sizeof(float) + sizeof(double))));
-  double *lossp = reinterpret_cast<double *>(s.part + (size_t)ctx->num_sms * PS);
   // a tile per block, at most a block per SM
   const unsigned blocks = (unsigned)std::min<u64>(((u64)m + TS - 1) / TS, (u64)ctx->num_sms);
-  TKC_LAUNCH(k_mlp_grad<<<blocks, kGradTPB, 0, st>>>(x, t, m, s.wb, s.part, lossp));
+  TKC_LAUNCH(k_mlp_grad<<<blocks, kGradTPB, 0, st>>>(x, t, m, s.wb, s.part, s.lossp));
   cudaLaunchAttribute early = {};
   early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   early.val.programmaticStreamSerializationAllowed = 1;
@@ -778,7 +790,7 @@ static int gradient(tkc_ctx *ctx, const float *x, const float *t, u32 m, float *
   cfg.attrs = &early;
   cfg.numAttrs = 1;
   note_launches(1);
-  TKC_TRY(cudaLaunchKernelEx(&cfg, k_mlp_sum, (const float *)s.part, (const double *)lossp, (u32)blocks, grad, s.loss));
+  TKC_TRY(cudaLaunchKernelEx(&cfg, k_mlp_sum, (const float *)s.part, (const double *)s.lossp, (u32)blocks, grad, s.loss));
   TKC_TRY(cudaGetLastError());
   return TKC_OK;
 }
