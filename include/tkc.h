@@ -103,7 +103,8 @@ typedef struct {
                               vary from run to run (results never do). */
   uint32_t relabel;        /* vertex labels of the search's rows: 0 = library choice (batched searches on graphs
                               of 2^20 vertices or more -- for several graphs in one launch, when the largest has
-                              -- walk a copy of the graph whose vertices are numbered by
+                              -- that have at least 24 batches left once the opening batch's threshold has
+                              dropped what it abandons walk a copy of the graph whose vertices are numbered by
                               in-degree, largest first, so that the rows levels touch most share L2; else the
                               graph itself), 1 = always that copy, 2 = never.  Sources, ties and every id in
                               the results are the graph's own ids whatever the choice; results never depend
@@ -200,8 +201,9 @@ int tkc_topk_closeness(tkc_graph *g, uint32_t k, tkc_result *out);
  * reach bounds are computed once on the union, and the threshold evolves
  * differently); ms_* are shared.  options.order: TKC_ORDER_DEG or
  * TKC_ORDER_NB (each graph stops on its own).  The union's sources run as
- * every graph's first batch, then the rest graph by graph, each graph's in its
- * own order, so a batch shares one graph's rows and arcs.  Errors: TKC_EINVAL (null ctx,
+ * every graph's first batch, then what their thresholds leave of the rest, graph
+ * by graph, each graph's in its own order, so a batch shares one graph's rows
+ * and arcs.  Errors: TKC_EINVAL (null ctx,
  * null gs or outs with ng > 0, k > TKC_MAX_K, another order, a capacity too
  * small), TKC_ENOMEM, TKC_ECUDA, TKC_ETIMEOUT. */
 int tkc_topk_closeness_multi(tkc_ctx *ctx, tkc_graph *const *gs, uint32_t ng, uint32_t k, tkc_result *outs);

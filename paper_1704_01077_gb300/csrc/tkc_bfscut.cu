@@ -6,17 +6,31 @@
 // slot b, top-down only).  One loop iteration advances every active slot by one
 // BFS level:
 //   phase A  expand: top-down over the frontier list (atomic OR into N) or
-//            bottom-up over all vertices (OR of in-neighbours' F rows, stopping
-//            once every missing bit is found), direction chosen per level;
+//            bottom-up over the vertices with an in-arc (OR of in-neighbours' F
+//            rows, stopping once every missing bit is found), direction chosen
+//            per level;
 //   phase B  finalize: new = N, seen |= new, F' = new, per-slot level sizes and
-//            out-degree sums by warp bit-transpose + popcount; old F rows cleared;
-//   epilogue (last block to reach the grid barrier): per-slot S, n_d, gamma,
+//            out-degree sums by warp bit-transpose + popcount; old F rows cleared
+//            (after a bottom-up level, which appends to no list, by the bits of
+//            the old frontier's bitmap);
+//   epilogue (last block to reach the team's barrier): per-slot S, n_d, gamma,
 //            merge of finished searches into the top-k, x = k-th farness, the
 //            BFSCut test of the Section 6 lemma at r in [alpha', omega] (Section 8.2), and
 //            the next step's direction.
 // When every slot of a batch is done, a clear step zeroes the rows the batch
 // touched and the epilogue seeds the next batch from the source order,
 // abandoning sources already at level 0 when their bound exceeds x.
+//
+// A call is an opening launch over a batch of promising sources (k_open_keys,
+// k_open_pick), a filter that drops the sources which the threshold it leaves
+// abandons after levels 0, 1 and 2 (k_filter_test, k_filter_compact), and the
+// main launch over the rest by teams of SMs; one-source searches and the
+// deterministic schedule are a single launch over the order as it stands.
+//
+// What bounds it: on small graphs the chain of dependent memory accesses of a
+// level (two barriers, an epilogue, an L2 load 150 ns, a returning atomic 440
+// ns); on large ones the gathers of bottom-up levels, by latency and
+// instructions issued rather than by bandwidth (DRAM at a tenth to a quarter).
 //
 // Every grid-wide wait is bounded by a clock64 budget; on expiry the kernel
 // records TKC_ETIMEOUT and every block returns.

@@ -8,8 +8,8 @@
 // backtracking walks on undirected graphs, Eq. 3 does not).  A sweep is one
 // gather over the CSR plus one per-vertex pass that turns the sum into N~_k,
 // evaluates the reach candidates of Eq. 6 that fall on level k's linear piece
-// and counts the vertices still unfinished.  The host loop stops when none is
-// left or after max_levels sweeps.
+// and counts the vertices still unfinished, until none is left or after
+// max_levels sweeps (in one launch up to kNbLoop vertices, by a host loop above).
 //
 // Counts are exact below 2^32 and stored as 2^32 from there on (any count >= n
 // bounds a level; a count computed from a capped one is capped).  Per-vertex

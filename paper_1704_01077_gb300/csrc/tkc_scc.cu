@@ -12,7 +12,8 @@
 //            reach it (backward propagation); repeat on what is left.
 //     Each SCC is named by one of its vertices.
 //  2. The biggest SCC (ties: the one holding the smallest vertex id) gets its
-//     exact reach from one BFS; a backward BFS marks the SCCs that reach it.
+//     exact reach from one BFS; a backward BFS marks the SCCs that reach it (the
+//     pivot's, when that SCC is its own).
 //  3. Condensation arcs (SCC pairs) are sorted and deduplicated, so the DAG's
 //     arc set has no repeats, and Algorithm 6's recurrences are evaluated
 //     sinks-first by peeling: an SCC is ready once all its successors are.
