@@ -269,8 +269,9 @@ int tkc_topk_harmonic_multi(tkc_ctx *ctx, tkc_graph *const *gs, uint32_t ng, uin
  * directed) gets the bound S(w) >= L(d(s,w)) - outdeg(w), L(i) = 2 x (vertices
  * within one level of i; directed: at most one level deeper) + the level
  * distance of all other vertices - 2, over R(s) including s.  The search runs
- * in rounds of options.teams batches of options.batch_bits sources (defaults: 4 x 128 from 2^16 vertices up,
- * else 1 x 256; batch_bits 1 = one source per round):
+ * in rounds of options.teams batches of options.batch_bits sources (defaults: 4 x 128, in the first round
+ * of a graph below 2^16 vertices 2 x 128; batch_bits given and teams 0: one batch below 2^16 vertices, 512 sources
+ * from there up; batch_bits 1 = one source per round):
  * the unsearched vertices of smallest bound key floor(2^46 S_lb/(r-1)^2), ties
  * by their position in the initial order, and stops when that key exceeds the
  * k-th farness strictly.  Results as tkc_topk_closeness (bfs_cut = 0).  Errors:

@@ -1664,16 +1664,23 @@ static int topk_bound(tkc_graph *g, uint32_t k, tkc_result *out) {
   }
   const u32 *order0 = nb ? g->nb_order : g->deg_order;
   const u32 n0 = nb ? g->n_src_nb : g->n_src_deg;
-  // defaults measured with NBBound on a 301 x 299 grid: 64 sources x 8 teams 122 ms, 128 x 4 111 ms,
-  // 256 x 2 110 ms, 64 x 16 131 ms (more sources per round refresh the bounds less often)
-  const bool large = n >= (1u << 16);
-  const u32 B = o.batch_bits ? o.batch_bits : (large ? 128u : 256u);
+  // defaults (512 sources a round) measured with NBBound on grids: 301 x 299, 64 sources x 8 teams 109 ms,
+  // 128 x 4 101 ms, 256 x 2 103 ms, 256 x 1 and 128 x 2 130 ms and more; 200 x 200, 256 x 1 63 ms, 256 x 2 49 ms,
+  // 128 x 4 47 ms; 60 x 60, 7.6, 5.6 and 5.1 ms (1 024 sources a round: 0 to 25% faster on grids of these
+  // sizes, but every round is searched to its end)
+  const u32 B = o.batch_bits ? o.batch_bits : 128u;
   const u32 cap = std::min<u32>(n + 1, 65535u);  // levels per search (depth < n)
-  // teams run one batch each per round (0: one team below 2^16 vertices, else as many as make 512 sources)
+  // teams run one batch each per round (0: as many as make 512 sources, or hold them all; one for a batch width
+  // asked for on a graph below 2^16 vertices)
+  const bool rounds_of_512 = !o.batch_bits || n >= (1u << 16);
   int maxb = max_coresident_blocks(ctx, words_for(B));
   if (maxb <= 0) return TKC_ECUDA;
-  const u32 T = std::max<u32>(1, std::min<u32>(B <= 1 ? 1u : (o.teams ? o.teams : (large ? 512u / B : 1u)), (u32)maxb));
+  const u32 lib_T = rounds_of_512 ? std::min<u32>(512u / B, (n0 + B - 1) / B) : 1u;
+  const u32 T = std::max<u32>(1, std::min<u32>(B <= 1 ? 1u : (o.teams ? o.teams : lib_T), (u32)maxb));
   const u32 TB = T * B;  // sources per round
+  // by default the first round of a graph below 2^16 vertices has 256: often all it takes with the NB order (a
+  // Barabasi-Albert graph of 50 000, NBBound: 2.0 ms, with 512 sources 2.4 ms)
+  const u32 first_round = !o.batch_bits && !o.teams && n < (1u << 16) ? std::min<u32>(TB, 256u) : TB;
   TKC_RC(ensure_workspace(ctx, n, words_for(B), kk, 1, T));
   u64 *bS = nullptr, *key = nullptr, *Ltab = nullptr, *smax = nullptr, *bkeys = nullptr;
   u32 *bR = nullptr, *cand = nullptr, *pos = nullptr, *tmp = nullptr, *lo = nullptr, *hist = nullptr, *depth = nullptr;
@@ -1732,7 +1739,7 @@ static int topk_bound(tkc_graph *g, uint32_t k, tkc_result *out) {
     u32 m = 0;
     LB_RC(lb_sorted_candidates(g, order0, n0, done, key, cand, &m, pos, tmp, lo, smax));
     if (m == 0) break;
-    const u32 take = std::min<u32>(TB, m);
+    const u32 take = std::min<u32>(nround ? TB : first_round, m);
     // the batch's keys and the current k-th entry decide the stop
     LB_RC(lb_gather_keys(g, take, cand, key, bkeys));
     LB_TRY(cudaMemcpyAsync(h_key.data(), bkeys, take * sizeof(u64), cudaMemcpyDeviceToHost, st));
@@ -1776,7 +1783,7 @@ static int topk_bound(tkc_graph *g, uint32_t k, tkc_result *out) {
     rs.hist_cap = cap;
     rs.lvl_stride = TB;
     rs.keep_lists = nround > 0;
-    rs.force_teams = T;
+    rs.force_teams = std::min<u32>(T, (cnt + B - 1) / B);
     Ctl hc;
     LB_RC(run_search(ctx, rs, &hc));
     float ms = 0;
