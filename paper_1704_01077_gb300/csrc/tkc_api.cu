@@ -1683,13 +1683,13 @@ static int topk_bound(tkc_graph *g, uint32_t k, tkc_result *out) {
   const u32 first_round = !o.batch_bits && !o.teams && n < (1u << 16) ? std::min<u32>(TB, 256u) : TB;
   TKC_RC(ensure_workspace(ctx, n, words_for(B), kk, 1, T));
   u64 *bS = nullptr, *key = nullptr, *Ltab = nullptr, *smax = nullptr, *bkeys = nullptr;
-  u32 *bR = nullptr, *cand = nullptr, *pos = nullptr, *tmp = nullptr, *lo = nullptr, *hist = nullptr, *depth = nullptr;
+  u32 *bR = nullptr, *cand = nullptr, *pos = nullptr, *tmp = nullptr, *lo = nullptr, *hist = nullptr;
   u32 *srcs = nullptr;
   uint8_t *done = nullptr;
   uint16_t *lvl = nullptr;
   int rc = TKC_OK;
   auto cleanup = [&]() {
-    void *ptrs[] = {bS, key, Ltab, smax, bkeys, bR, cand, pos, tmp, lo, hist, depth, done, lvl, srcs};
+    void *ptrs[] = {bS, key, Ltab, smax, bkeys, bR, cand, pos, tmp, lo, hist, done, lvl, srcs};
     for (void *q : ptrs)
       if (q) cudaFreeAsync(q, st);
     cudaStreamSynchronize(st);
@@ -1723,7 +1723,7 @@ static int topk_bound(tkc_graph *g, uint32_t k, tkc_result *out) {
   LB_TRY(dev_malloc(&smax, sizeof(u64), st));
   LB_TRY(dev_malloc(&hist, (size_t)TB * cap * sizeof(u32), st));
   LB_TRY(dev_malloc(&Ltab, (size_t)TB * cap * sizeof(u64), st));
-  LB_TRY(dev_malloc(&depth, (size_t)TB * sizeof(u32), st));
+  LB_TRY(cudaMemsetAsync(hist, 0, (size_t)TB * cap * sizeof(u32), st));  // (each round leaves it so: lb_update)
   LB_TRY(dev_malloc(&bkeys, (size_t)TB * sizeof(u64), st));
   LB_TRY(dev_malloc(&srcs, (size_t)TB * sizeof(u32), st));
   LB_TRY(dev_malloc(&lvl, n1 * TB * sizeof(uint16_t), st));
@@ -1765,7 +1765,6 @@ static int topk_bound(tkc_graph *g, uint32_t k, tkc_result *out) {
       }
     }
     if (cnt == 0) break;
-    LB_TRY(cudaMemsetAsync(hist, 0, (size_t)TB * cap * sizeof(u32), st));
     LB_TRY(cudaMemsetAsync(srcs, 0xff, (size_t)TB * sizeof(u32), st));
     RunSetup rs;
     memset(&rs, 0, sizeof(rs));
@@ -1796,7 +1795,7 @@ static int topk_bound(tkc_graph *g, uint32_t k, tkc_result *out) {
     total.bfs_finished += hc.bfs_finished;
     total.levels += hc.levels;
     total.alg_bytes += hc.alg_bytes;
-    LB_RC(lb_update(g, TB, TB, srcs, lvl, hist, cap, depth, Ltab, w.res_r, bS, bR, key, done));
+    LB_RC(lb_update(g, TB, TB, srcs, lvl, hist, cap, Ltab, w.res_r, bS, bR, key, done));
     ++nround;
   }
   RunSetup rs;

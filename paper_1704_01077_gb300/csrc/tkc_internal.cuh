@@ -442,7 +442,7 @@ int lb_sorted_candidates(tkc_graph *g, const uint32_t *order0, uint32_t n0, cons
 int lb_gather_keys(tkc_graph *g, uint32_t cnt, const uint32_t *cand, const unsigned long long *key,
                    unsigned long long *out);
 int lb_update(tkc_graph *g, uint32_t B, uint32_t nsrc, const uint32_t *srcs, uint16_t *lvl, uint32_t *hist,
-              uint32_t cap, uint32_t *depth, unsigned long long *Ltab, const uint32_t *res_r, unsigned long long *bS,
+              uint32_t cap, unsigned long long *Ltab, const uint32_t *res_r, unsigned long long *bS,
               uint32_t *bR, unsigned long long *key, uint8_t *done);
 // tkc_mlp.cu
 int ensure_features(tkc_graph *g);

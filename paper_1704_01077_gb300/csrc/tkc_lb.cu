@@ -68,99 +68,166 @@ __global__ void k_lb_key_hi(u32 m, const u32 *cand, const u64 *key, u32 *hi) {
   for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) hi[i] = (u32)(key[cand[i]] >> 32);
 }
 
-// One thread per source: L(i) for every level i of its BFS, from the level
-// sizes with running prefix sums G(j) = sum_{t<=j} g_t, M(j) = sum_{t<=j} t g_t:
+// One warp per source: L(i) for every level i of its BFS, from the level sizes
+// g_j (non-zero up to the depth D, zero beyond; g_0 = 1) with prefix sums
+// G(j) = sum_{t<=j} g_t, M(j) = sum_{t<=j} t g_t:
 //   sum_{j <= i-2} g_j (i-j)  = i G(i-2) - M(i-2)
 //   sum_{j >= i+2} g_j (j-i)  = (M_all - M(i+1)) - i (G_all - G(i+1))
-__global__ void k_lb_table(u32 nsrc, u32 *hist, u32 cap, const u32 *depth, int directed, u64 *Ltab) {
-  const u32 s = blockIdx.x * blockDim.x + threadIdx.x;
+// 32 levels a step; the level sizes are zeroed again behind it, so that the
+// next round finds them so.  (A thread per source behind a pass over all
+// levels a search could have, and a memset of them: 0.27 ms a round on a
+// 301 x 299 grid.)
+__global__ void k_lb_table(u32 nsrc, u32 *hist, u32 cap, int directed, u64 *Ltab) {
+  const int lane = threadIdx.x & 31;
+  const u32 s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (s >= nsrc) return;
   u32 *g = hist + (size_t)s * cap;
   u64 *L = Ltab + (size_t)s * cap;
-  const u32 D = depth[s];
-  g[0] = 1;  // the source
+  // the depth and the totals
+  u32 D = 0;
   u64 Gall = 0, Mall = 0;
-  for (u32 j = 0; j <= D; ++j) {
-    Gall += g[j];
-    Mall += (u64)j * g[j];
-  }
-  // G(i-2), M(i-2) and G(i+1), M(i+1) advance with i
-  u64 Glo = 0, Mlo = 0;         // up to i-2
-  u64 Ghi = g[0], Mhi = 0;      // up to i+1, start at i = 0: levels 0 and 1
-  if (D >= 1) {
-    Ghi += g[1];
-    Mhi += g[1];
-  }
-  for (u32 i = 0; i <= D; ++i) {
-    if (i >= 2) {
-      Glo += g[i - 2];
-      Mlo += (u64)(i - 2) * g[i - 2];
+  for (u32 base = 0;; base += 32) {
+    const u32 j = base + lane;
+    const u32 c = j == 0 ? 1u : j < cap ? g[j] : 0u;
+    const unsigned empty = __ballot_sync(FULL, c == 0);
+    const int used = empty ? __ffs(empty) - 1 : 32;
+    if (lane < used) {
+      Gall += c;
+      Mall += (u64)j * c;
     }
-    const u64 above = (Mall - Mhi) - (u64)i * (Gall - Ghi);
-    u64 v;
-    if (directed) {
-      v = 2 * Ghi + above - 2;
-    } else {
-      const u64 near = (i >= 1 ? g[i - 1] : 0) + g[i] + (i + 1 <= D ? g[i + 1] : 0);
-      const u64 below = (u64)i * Glo - Mlo;
-      v = 2 * near + below + above - 2;
-    }
-    L[i] = v;
-    if (i + 2 <= D) {
-      Ghi += g[i + 2];
-      Mhi += (u64)(i + 2) * g[i + 2];
-    }
+    if (used) D = base + used - 1;
+    if (empty) break;
   }
-}
-
-// Depth of each slot's BFS: its deepest non-empty level.
-__global__ void k_lb_depth(u32 nsrc, const u32 *hist, u32 cap, u32 *depth) {
-  const u32 s = blockIdx.x;
-  if (s >= nsrc) return;
-  u32 best = 0;
-  for (u32 j = 1 + threadIdx.x; j < cap; j += blockDim.x)
-    if (hist[(size_t)s * cap + j]) best = max(best, j);
-  best = __reduce_max_sync(FULL, best);
-  __shared__ u32 wbest[32];
-  if ((threadIdx.x & 31) == 0) wbest[threadIdx.x >> 5] = best;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    u32 b = 0;
-    for (u32 i = 0; i < blockDim.x / 32; ++i) b = max(b, wbest[i]);
-    depth[s] = b;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    Gall += __shfl_xor_sync(FULL, Gall, o);
+    Mall += __shfl_xor_sync(FULL, Mall, o);
   }
-}
-
-// One thread per vertex: raise its bound with every slot that found it, then
-// reset its level row for the next round.
-__global__ void k_lb_update(u32 n, u32 B, u32 nsrc, uint16_t *lvl, const u32 *srcs, const u32 *comp, const u32 *off,
-                            const u64 *Ltab, u32 cap, const u32 *res_r, u64 *bS, u32 *bR, u64 *key) {
-  for (u32 w = blockIdx.x * blockDim.x + threadIdx.x; w < n; w += gridDim.x * blockDim.x) {
-    uint16_t *row = lvl + (size_t)w * B;
-    const u64 od = off[w + 1] - off[w];
-    const u32 cw = comp[w];
-    u64 S = bS[w], r = bR[w];
-    bool changed = false;
-    for (u32 s = 0; s < nsrc; ++s) {
-      const uint16_t l = row[s];
-      if (l == 0xffffu) continue;
-      row[s] = 0xffffu;
-      const u32 src = srcs[s];
-      if (src == 0xffffffffu || src == w || comp[src] != cw || od == 0) continue;
-      const u64 cS = Ltab[(size_t)s * cap + l] - od;
-      const u64 cr = res_r[src];
-      // keep the larger of cS/(cr-1)^2 and S/(r-1)^2 (r <= 1: no bound yet)
-      if (cr <= 1) continue;
-      if (r <= 1 || (u128)cS * (u128)((r - 1) * (r - 1)) > (u128)S * (u128)((cr - 1) * (cr - 1))) {
-        S = cS;
-        r = cr;
-        changed = true;
+  auto size_of = [&](u32 j) { return j == 0 ? 1u : j <= D ? g[j] : 0u; };
+  u64 Gbase = 0, Mbase = 0;  // up to the levels before this step's
+  for (u32 base = 0; base <= D; base += 32) {
+    const u32 i = base + lane;
+    const u64 c = size_of(i), prev = i ? size_of(i - 1) : 0u, next = size_of(i + 1);
+    u64 G = c, M = i * c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const u64 tg = __shfl_up_sync(FULL, G, o), tm = __shfl_up_sync(FULL, M, o);
+      if (lane >= o) {
+        G += tg;
+        M += tm;
       }
     }
-    if (changed) {
-      bS[w] = S;
-      bR[w] = (u32)r;
-      key[w] = (u64)(((u128)S << kKeyFrac) / (u128)((r - 1) * (r - 1)));
+    G += Gbase;
+    M += Mbase;
+    Gbase = __shfl_sync(FULL, G, 31);
+    Mbase = __shfl_sync(FULL, M, 31);
+    if (i <= D) {
+      const u64 Ghi = G + next, Mhi = M + (u64)(i + 1) * next;  // up to i+1
+      const u64 above = (Mall - Mhi) - (u64)i * (Gall - Ghi);
+      u64 v;
+      if (directed) {
+        v = 2 * Ghi + above - 2;
+      } else {
+        const u64 Glo = G - c - prev, Mlo = M - i * c - (i ? (u64)(i - 1) * prev : 0u);  // up to i-2
+        v = 2 * (prev + c + next) + ((u64)i * Glo - Mlo) + above - 2;
+      }
+      L[i] = v;
+    }
+  }
+  __syncwarp();
+  for (u32 j = lane; j <= D; j += 32) g[j] = 0;
+}
+
+// Raises every vertex's bound with every slot that found it, then resets its
+// level row for the next round.  kLanes lanes a vertex, each taking every
+// kLanes-th group of 8 slots (a 16-byte load of the row); the sources' graph
+// data are staged per block, kStage slots at a time.  Bounds of one reach are
+// compared by their sums: (cS / (r-1)^2 > S / (r-1)^2 as cS > S), only others
+// by 128-bit products.  (A thread per vertex, a slot at a time: 0.75 ms a round
+// of 512 slots on a 301 x 299 grid.)  `vec`: rows of a multiple of 8 slots.
+constexpr int kLanes = 4;
+constexpr u32 kStage = 512;
+__device__ __forceinline__ bool lb_higher(u64 cS, u64 cr, u64 S, u64 r) {
+  if (r <= 1) return true;  // no bound yet
+  if (cr == r) return cS > S;
+  return (u128)cS * (u128)((r - 1) * (r - 1)) > (u128)S * (u128)((cr - 1) * (cr - 1));
+}
+template <bool kVec>
+__global__ void __launch_bounds__(256) k_lb_update(u32 n, u32 B, u32 nsrc, uint16_t *lvl, const u32 *srcs,
+                                                   const u32 *comp, const u32 *off, const u64 *Ltab, u32 cap,
+                                                   const u32 *res_r, u64 *bS, u32 *bR, u64 *key) {
+  constexpr u32 kGroup = kVec ? 8 : 1;
+  __shared__ u32 s_src[kStage], s_comp[kStage], s_r[kStage];
+  const u32 q = threadIdx.x % kLanes;
+  const u32 per_grid = gridDim.x * (blockDim.x / kLanes);
+  for (u32 s0 = 0; s0 < nsrc; s0 += kStage) {
+    const u32 ns = nsrc - s0 < kStage ? nsrc - s0 : kStage;
+    __syncthreads();
+    for (u32 i = threadIdx.x; i < ns; i += blockDim.x) {
+      const u32 src = srcs[s0 + i];
+      s_src[i] = src;
+      s_comp[i] = src == 0xffffffffu ? 0u : comp[src];
+      s_r[i] = src == 0xffffffffu ? 0u : res_r[src];  // 0: gives no bound
+    }
+    __syncthreads();
+    // (every lane of a warp takes part in every step: the exchange below)
+    for (u32 w0 = blockIdx.x * (blockDim.x / kLanes); w0 < n; w0 += per_grid) {
+      const u32 w = w0 + threadIdx.x / kLanes;
+      const bool valid = w < n;
+      u64 S = 0, r = 0;
+      bool changed = false;
+      if (valid) {
+        uint16_t *row = lvl + (size_t)w * B + s0;
+        const u64 od = off[w + 1] - off[w];
+        const u32 cw = comp[w];
+        S = bS[w];
+        r = bR[w];
+        auto slot = [&](u32 i, u32 l) {
+          if (l == 0xffffu) return;
+          const u64 cr = s_r[i];
+          if (s_src[i] == w || s_comp[i] != cw || od == 0 || cr <= 1) return;
+          const u64 cS = Ltab[(size_t)(s0 + i) * cap + l] - od;
+          if (lb_higher(cS, cr, S, r)) {
+            S = cS;
+            r = cr;
+            changed = true;
+          }
+        };
+        for (u32 i = q * kGroup; i < ns; i += kLanes * kGroup) {
+          if constexpr (kVec) {
+            uint4 *p = reinterpret_cast<uint4 *>(row + i);
+            const uint4 x = *p;
+            if ((x.x & x.y & x.z & x.w) == 0xffffffffu) continue;
+            *p = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+            const u32 h[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+            for (u32 j = 0; j < 4; ++j) {
+              slot(i + 2 * j, h[j] & 0xffffu);
+              slot(i + 2 * j + 1, h[j] >> 16);
+            }
+          } else {
+            const u32 l = row[i];
+            if (l == 0xffffu) continue;
+            row[i] = 0xffffu;
+            slot(i, l);
+          }
+        }
+      }
+#pragma unroll
+      for (int o = 1; o < kLanes; o <<= 1) {
+        const u64 oS = __shfl_xor_sync(FULL, S, o), orr = __shfl_xor_sync(FULL, r, o);
+        const bool oc = __shfl_xor_sync(FULL, (int)changed, o) != 0;
+        if (oc && (!changed || lb_higher(oS, orr, S, r))) {
+          S = oS;
+          r = orr;
+          changed = true;
+        }
+      }
+      if (valid && changed && q == 0) {
+        bS[w] = S;
+        bR[w] = (u32)r;
+        key[w] = (u64)(((u128)S << kKeyFrac) / (u128)((r - 1) * (r - 1)));
+      }
     }
   }
 }
@@ -238,14 +305,19 @@ int lb_gather_keys(tkc_graph *g, u32 cnt, const u32 *cand, const u64 *key, u64 *
 
 // After a round of complete searches from srcs[0..nsrc) (0xffffffff: slot
 // unused): level bounds per source, then every vertex's bound.  lvl rows (B =
-// row length) are reset to 0xffff.
-int lb_update(tkc_graph *g, u32 B, u32 nsrc, const u32 *srcs, uint16_t *lvl, u32 *hist, u32 cap, u32 *depth,
+// row length) are reset to 0xffff, the level sizes (hist) to 0.
+int lb_update(tkc_graph *g, u32 B, u32 nsrc, const u32 *srcs, uint16_t *lvl, u32 *hist, u32 cap,
               u64 *Ltab, const u32 *res_r, u64 *bS, u32 *bR, u64 *key, uint8_t *done) {
   cudaStream_t st = g->ctx->stream;
-  TKC_LAUNCH(k_lb_depth<<<nsrc, 256, 0, st>>>(nsrc, hist, cap, depth));
-  TKC_LAUNCH(k_lb_table<<<(nsrc + 63) / 64, 64, 0, st>>>(nsrc, hist, cap, depth, g->directed, Ltab));
-  TKC_LAUNCH(k_lb_update<<<grid_of(g->n), 256, 0, st>>>(g->n, B, nsrc, lvl, srcs, g->comp, g->off, Ltab, cap, res_r,
-                                                         bS, bR, key));
+  TKC_LAUNCH(k_lb_table<<<(nsrc + 7) / 8, 256, 0, st>>>(nsrc, hist, cap, g->directed, Ltab));
+  const unsigned blocks = grid_of((u64)g->n * kLanes);
+  if (B % 8 == 0) {
+    TKC_LAUNCH(k_lb_update<true><<<blocks, 256, 0, st>>>(g->n, B, nsrc, lvl, srcs, g->comp, g->off, Ltab, cap, res_r, bS,
+                                                         bR, key));
+  } else {
+    TKC_LAUNCH(k_lb_update<false><<<blocks, 256, 0, st>>>(g->n, B, nsrc, lvl, srcs, g->comp, g->off, Ltab, cap, res_r,
+                                                          bS, bR, key));
+  }
   TKC_LAUNCH(k_lb_done<<<(nsrc + 255) / 256, 256, 0, st>>>(nsrc, srcs, done));
   TKC_TRY(cudaGetLastError());
   return TKC_OK;
