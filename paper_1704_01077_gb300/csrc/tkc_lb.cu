@@ -9,9 +9,9 @@
 // Algorithm 1 runs in rounds: the B unsearched vertices of smallest bound key
 // (ties by their position in the initial order) are searched completely by the
 // persistent kernel, which records for every vertex the level at which each
-// slot found it and each slot's level sizes; then one thread per source turns
-// its level sizes into L(i) (O(depth), prefix sums), and one thread per vertex
-// raises the vertex's bound with every slot that found it.  The host loop ends
+// slot found it and each slot's level sizes; then a warp per source turns its
+// level sizes into L(i) (O(depth), prefix sums), and four lanes per vertex
+// raise the vertex's bound with every slot that found it.  The host loop ends
 // when the head of the order has a key above the k-th farness.
 #include <cuda_runtime.h>
 #include <stdint.h>
