@@ -16,13 +16,16 @@ namespace tkc {
 // Largest u in [0, n) with off[u] <= a, for a < off[n] (so that u's row holds
 // arc a).  32-way search: each round every lane probes one of 32 evenly
 // spaced offsets and the range shrinks to one gap.  Called by all 32 lanes
-// with the same arguments; every lane returns the same u.
+// with the same arguments; every lane returns the same u.  Lane 0's probe holds
+// by the invariant and is not asked: the check of a CSR walks offsets that may
+// not start at 0, and a round in which no lane answered would have no gap to
+// shrink to.  So u < n and the search ends whatever the offsets hold.
 __device__ __forceinline__ uint32_t warp_arc_source(const uint32_t *off, uint32_t n, uint64_t a, int lane) {
   uint32_t lo = 0, hi = n;  // off[lo] <= a; the answer lies in [lo, hi)
   while (hi - lo > 1) {
     const uint32_t step = (hi - lo + 31) / 32;
     const uint32_t p = lo + step * (uint32_t)lane;
-    const bool ok = p < hi && off[p] <= a;  // true on a prefix of the lanes, lane 0 included
+    const bool ok = lane == 0 || (p < hi && off[p] <= a);  // true on a prefix of the lanes
     const unsigned m = __ballot_sync(0xffffffffu, ok);
     const uint32_t l = 31u - (uint32_t)__clz(m);
     lo += step * l;
