@@ -28,6 +28,8 @@ int tkc::enter(tkc_ctx *ctx) {
 
 cudaError_t tkc::dev_malloc_bytes(void **p, size_t bytes, cudaStream_t st) {
   tkc_ctx *ctx = t_ctx;
+  *p = nullptr;
+  if (ctx->fail_alloc && --ctx->fail_alloc == 0) return cudaErrorMemoryAllocation;
   if (!ctx->pool) {
     cudaMemPoolProps props;
     memset(&props, 0, sizeof(props));
@@ -89,6 +91,7 @@ cudaError_t tkc::read_back2(void *dst, const void *src, size_t bytes, void *dst2
 void tkc::note_launches(unsigned count) { g_launches.fetch_add(count, std::memory_order_relaxed); }
 
 void tkc_set_last_cuda_error(cudaError_t e, const char *what, const char *file, int line) {
+  cudaGetLastError();  // reported here: the next launch check must not meet it again
   snprintf(g_last_err, sizeof(g_last_err), "%s: %s (%s:%d)", cudaGetErrorString(e), what, file, line);
 }
 
@@ -111,13 +114,19 @@ static int dalloc(T **p, size_t count, cudaStream_t st) {
   return TKC_OK;
 }
 
+// Every block of buffers is without capacity while it is being replaced: after
+// a failed allocation the next call makes the whole block again.
 int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u32 teams) {
   Workspace &w = ctx->ws;
   cudaStream_t st = ctx->stream;
+  ctx->last_shard = nullptr;  // what follows replaces the finished searches' (S, r)
   if (teams > w.teams_cap) {
+    w.teams_cap = w.n_cap = 0;  // (per-team vertex buffers are reallocated for the new team count)
     // the shared block, then the control blocks: read back together
     static_assert(sizeof(Shared) <= kShBytes, "the shared block fits its place");
     unsigned char *base = reinterpret_cast<unsigned char *>(w.sh);
+    w.sh = nullptr;
+    w.ctl = nullptr;
     TKC_RC(dalloc(&base, kShBytes + 2 * (size_t)teams * sizeof(Ctl), st));
     w.sh = reinterpret_cast<Shared *>(base);
     w.ctl = reinterpret_cast<Ctl *>(base + kShBytes);
@@ -127,10 +136,10 @@ int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u3
     TKC_TRY(cudaMemsetAsync(w.cnt, 0, (size_t)teams * 64 * kMaxWords * sizeof(unsigned), st));
     TKC_TRY(cudaMemsetAsync(w.wsum, 0, (size_t)teams * 64 * kMaxWords * sizeof(u64), st));
     w.teams_cap = teams;
-    w.n_cap = 0;  // per-team vertex buffers are reallocated for the new team count
   }
   if (top_entries > w.top_cap) {
     u32 cap = std::max<u32>(top_entries, TKC_MAX_K);
+    w.top_cap = 0;
     TKC_RC(dalloc(&w.top_S, cap, st));
     TKC_RC(dalloc(&w.top_r, cap, st));
     TKC_RC(dalloc(&w.top_id, cap, st));
@@ -138,6 +147,7 @@ int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u3
   }
   if (ng > w.ng_cap) {
     u32 cap = std::max<u32>(ng, 16);
+    w.ng_cap = 0;
     TKC_RC(dalloc(&w.tied, cap, st));
     TKC_RC(dalloc(&w.g_ntop, cap, st));
     TKC_RC(dalloc(&w.g_lock, cap, st));
@@ -151,6 +161,7 @@ int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u3
   if (n > w.n_cap) {
     u32 cap = std::max<u32>(n, 1024);
     size_t tv = (size_t)T * cap, tfb = (size_t)T * (cap / 32 + 1);
+    w.n_cap = w.words_cap = 0;  // (rows are reallocated for the new n)
     TKC_RC(dalloc(&w.L0, tv, st));
     TKC_RC(dalloc(&w.L1, tv, st));
     TKC_RC(dalloc(&w.Loff0, tv, st));
@@ -167,10 +178,10 @@ int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u3
     TKC_TRY(cudaMemsetAsync(w.stamp, 0xff, tv * sizeof(u32), st));
     w.level_base = 0;
     w.n_cap = cap;
-    w.words_cap = 0;  // rows must be reallocated for the new n
   }
   if (words > w.words_cap) {
     size_t rows = (size_t)T * w.n_cap * words;
+    w.words_cap = 0;
     TKC_RC(dalloc(&w.seen, rows, st));
     TKC_RC(dalloc(&w.F0, rows, st));
     TKC_RC(dalloc(&w.F1, rows, st));
@@ -217,8 +228,10 @@ static void free_workspace(tkc_ctx *ctx) {
   w = Workspace();
 }
 
-// Row buffers hold only the current run's bits; the kernel leaves them zero
-// when it ends normally.  After an error they are cleared here.
+// Row buffers hold only the current run's bits, and level stamps only grow from
+// run to run; the kernel leaves both so when it ends normally.  After an error
+// -- the kernel's own, or one of the host's between a run's launches and the
+// read of their outcome -- they are set right here.
 static int reset_rows(tkc_ctx *ctx) {
   Workspace &w = ctx->ws;
   const size_t T = w.teams_cap;
@@ -232,6 +245,9 @@ static int reset_rows(tkc_ctx *ctx) {
   TKC_TRY(cudaMemsetAsync(w.FB1, 0, T * ((size_t)w.n_cap / 32 + 1) * sizeof(u32), st));
   TKC_TRY(cudaMemsetAsync(w.cnt, 0, T * 64 * kMaxWords * sizeof(unsigned), st));
   TKC_TRY(cudaMemsetAsync(w.wsum, 0, T * 64 * kMaxWords * sizeof(u64), st));
+  TKC_TRY(cudaMemsetAsync(w.stamp, 0xff, T * w.n_cap * sizeof(u32), st));
+  w.level_base = 0;
+  w.dirty = false;
   return TKC_OK;
 }
 
@@ -538,11 +554,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   if (o.deterministic && !rs.force_teams) T = 1;
   T = std::max<u32>(1, std::min<u32>(T, (u32)maxb));
   TKC_RC(ensure_workspace(ctx, g->n, rs.W, rs.kk * rs.ng, rs.ng, T));
-  if (w.level_base > 0xF0000000u) {
-    TKC_TRY(cudaMemsetAsync(w.stamp, 0xff, (size_t)w.teams_cap * w.n_cap * sizeof(u32), st));
-    w.level_base = 0;
-  }
-  ctx->last_shard = nullptr;  // this run replaces the finished searches' (S, r)
+  if (w.dirty || w.level_base > 0xF0000000u) TKC_RC(reset_rows(ctx));
   // Opening: a batch of promising sources (k_open_keys) -- or as many batches
   // as it takes for a full k-list -- runs alone (one graph: on the whole grid;
   // several: every graph's opening batch, on the teams), so that thresholds
@@ -677,6 +689,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     const int most = teams > 1 || o.blocks ? blocks : std::min<int>(blocks, std::max<int>(8, (int)((g->n + 511) / 512)));
     return run_bfscut(ctx, p, rs.W, std::max<int>((int)teams, most / (int)teams * (int)teams));
   };
+  w.dirty = true;  // until the launches' outcome has been read
   if (opening) {
     if (pick) {
       // the opening's sources keep their order, the uncut prefix first
@@ -748,6 +761,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   }
   if (!hctl->err) hctl->err = hsh.err;
   w.level_base = hctl->level_id + 1;
+  w.dirty = hctl->err != 0;
   if (p.trace) {
     u64 *tbase = opening ? p.trace - (size_t)p.trace_cap * 16 : p.trace;
     std::vector<u64> tr((size_t)trace_cap * 16);
@@ -897,6 +911,14 @@ using namespace tkc;
 extern "C" {
 
 uint64_t tkc_kernel_launches(void) { return g_launches.load(std::memory_order_relaxed); }
+
+// For tests: the nth next device allocation of the context fails as one without
+// memory does (0: none).  Returns what was left of an earlier count.
+uint64_t tkc_internal_fail_allocation(tkc_ctx *ctx, uint64_t nth) {
+  const uint64_t left = ctx->fail_alloc;
+  ctx->fail_alloc = nth;
+  return left;
+}
 
 int tkc_last_run_stats(const tkc_ctx *ctx, tkc_run_stats *out) {
   if (!ctx || !out) return TKC_EINVAL;

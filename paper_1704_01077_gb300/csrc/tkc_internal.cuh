@@ -271,6 +271,7 @@ struct Workspace {
   uint32_t ng_cap = 0;    // graphs of tied / g_ntop / g_ctr / x_*
   uint32_t teams_cap = 0; // teams the per-team buffers are sized for
   unsigned int level_base = 0;  // stamp epoch carried across runs
+  bool dirty = false;     // a run ended with an error: rows and stamps are not as a run expects them
 };
 
 }  // namespace tkc
@@ -337,6 +338,7 @@ struct tkc_ctx {
   cudaMemPool_t pool = nullptr;  // device memory of the context and its graphs
   void *stage = nullptr;         // page-locked host buffer of short reads (read_back)
   size_t stage_bytes = 0;
+  uint64_t fail_alloc = 0;       // the fail_alloc-th next device allocation fails (0: none; tests)
   tkc::Workspace ws;
   cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   cudaStream_t aux = nullptr;    // helper stream: the labelled copy, built while `stream` preprocesses
