@@ -1173,12 +1173,22 @@ int tkc_set_source_order(tkc_graph *g, const uint32_t *order) {
   TKC_RC(enter(g->ctx));
   cudaStream_t st = g->ctx->stream;
   if (g->n == 0) return TKC_OK;
-  u32 *tmp = nullptr;
-  if (!g->given_order) TKC_TRY(dev_malloc(&g->given_order, (size_t)g->n * sizeof(u32), st));
+  // (the handle's order is replaced when the new one is complete)
+  u32 *tmp = nullptr, *out = nullptr, count = 0;
   TKC_TRY(dev_malloc(&tmp, (size_t)g->n * sizeof(u32), st));
-  TKC_TRY(cudaMemcpyAsync(tmp, order, g->n * sizeof(u32), cudaMemcpyHostToDevice, st));
-  TKC_RC(filter_order(g, tmp, g->given_order, &g->n_src_given));
-  TKC_TRY(cudaFreeAsync(tmp, st));
+  cudaError_t e = cudaMemcpyAsync(tmp, order, g->n * sizeof(u32), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = dev_malloc(&out, (size_t)g->n * sizeof(u32), st);
+  const int rc = e == cudaSuccess ? filter_order(g, tmp, out, &count) : TKC_OK;
+  cudaFreeAsync(tmp, st);
+  if (e != cudaSuccess || rc != TKC_OK) {
+    if (out) cudaFreeAsync(out, st);
+    cudaStreamSynchronize(st);  // the copy reads the caller's memory
+    TKC_TRY(e);
+    return rc;
+  }
+  if (g->given_order) TKC_TRY(cudaFreeAsync(g->given_order, st));
+  g->given_order = out;
+  g->n_src_given = count;
   TKC_TRY(cudaStreamSynchronize(st));
   return TKC_OK;
 }

@@ -571,6 +571,8 @@ static int reset_adam(tkc_ctx *ctx) {
   return TKC_OK;
 }
 
+static int make_features(tkc_graph *g, float *x);
+
 int ensure_features(tkc_graph *g) {
   if (g->features) return TKC_OK;
   TKC_RC(ensure_reach_bounds(g));  // provides the SCC sizes
@@ -578,10 +580,23 @@ int ensure_features(tkc_graph *g) {
   cudaStream_t st = g->ctx->stream;
   const u32 n = g->n;
   if (n == 0) return TKC_OK;
+  float *x = nullptr;
+  TKC_TRY(dev_malloc(&x, (size_t)n * F * sizeof(float), st));
+  const int rc = make_features(g, x);
+  if (rc != TKC_OK) {  // the handle stays without: its pointer says that they are complete
+    cudaFreeAsync(x, st);
+    return rc;
+  }
+  g->features = x;
+  return TKC_OK;
+}
+
+static int make_features(tkc_graph *g, float *x) {
+  cudaStream_t st = g->ctx->stream;
+  const u32 n = g->n;
   float *w2 = nullptr;
   u32 *c0 = nullptr, *c1 = nullptr;
   double *sums = nullptr;
-  TKC_TRY(dev_malloc(&g->features, (size_t)n * F * sizeof(float), st));
   TKC_TRY(dev_malloc(&w2, (size_t)n * sizeof(float), st));
   TKC_TRY(dev_malloc(&c0, (size_t)n * sizeof(u32), st));
   TKC_TRY(dev_malloc(&c1, (size_t)n * sizeof(u32), st));
@@ -612,8 +627,8 @@ int ensure_features(tkc_graph *g) {
   TKC_TRY(cudaFreeAsync(d0, st));
   TKC_TRY(cudaFreeAsync(d1, st));
   TKC_TRY(cudaMemsetAsync(sums, 0, 2 * F * sizeof(double), st));
-  TKC_LAUNCH(k_features_raw<<<grid_of(n), 256, 0, st>>>(g->off, g->ioff, w2, c0, g->scc_size, n, g->features, sums));
-  TKC_LAUNCH(k_features_standardize<<<grid_of((u64)n * F), 256, 0, st>>>(g->features, n, sums));
+  TKC_LAUNCH(k_features_raw<<<grid_of(n), 256, 0, st>>>(g->off, g->ioff, w2, c0, g->scc_size, n, x, sums));
+  TKC_LAUNCH(k_features_standardize<<<grid_of((u64)n * F), 256, 0, st>>>(x, n, sums));
   TKC_TRY(cudaGetLastError());
   TKC_TRY(cudaFreeAsync(w2, st));
   TKC_TRY(cudaFreeAsync(c0, st));

@@ -452,12 +452,10 @@ int ensure_nb_bounds(tkc_graph *g, u32 K, const u32 *gid, const uint8_t *gdir) {
   cudaStream_t st = ctx->stream;
   const u32 n = g->n;
   const size_t n1 = std::max<size_t>(n, 1);
-  if (!g->nb_hkey) {
-    TKC_TRY(dev_malloc(&g->nb_S, n1 * sizeof(u64), st));
-    TKC_TRY(dev_malloc(&g->nb_r, n1 * sizeof(u32), st));
-    TKC_TRY(dev_malloc(&g->nb_key, n1 * sizeof(u64), st));
-    TKC_TRY(dev_malloc(&g->nb_hkey, n1 * sizeof(u64), st));
-  }
+  if (!g->nb_S) TKC_TRY(dev_malloc(&g->nb_S, n1 * sizeof(u64), st));
+  if (!g->nb_r) TKC_TRY(dev_malloc(&g->nb_r, n1 * sizeof(u32), st));
+  if (!g->nb_key) TKC_TRY(dev_malloc(&g->nb_key, n1 * sizeof(u64), st));
+  if (!g->nb_hkey) TKC_TRY(dev_malloc(&g->nb_hkey, n1 * sizeof(u64), st));
   if (n == 0) {
     g->n_src_nb = 0;
     g->nb_levels = 0;

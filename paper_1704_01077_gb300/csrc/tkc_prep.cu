@@ -369,10 +369,11 @@ static int fill_in_arcs(const u32 *off, const u32 *col, u32 n, u64 arcs, const u
 }
 
 // Transpose of the CSR (off, col) with n vertices: the in-arc CSR.  *ioff and
-// *icol are allocated here.
+// *icol are allocated here (on failure: null or an allocation, without content).
 static int transpose_csr(const u32 *off, const u32 *col, u32 n, u64 arcs, u32 **ioff, u32 **icol,
                          cudaStream_t st) {
   u32 *tmp = nullptr;
+  *ioff = *icol = nullptr;
   TKC_TRY(dev_malloc(ioff, ((size_t)n + 1) * sizeof(u32), st));
   TKC_TRY(dev_malloc(icol, std::max<size_t>(arcs, 1) * sizeof(u32), st));
   TKC_TRY(dev_malloc(&tmp, (((size_t)n + 1) / kScanTile + 2) * sizeof(u32), st));
@@ -390,7 +391,17 @@ static int transpose_csr(const u32 *off, const u32 *col, u32 n, u64 arcs, u32 **
 // In-arc CSR of g.
 int build_in_csr(const tkc_graph *g) {
   if (g->n == 0) return TKC_OK;
-  return transpose_csr(g->off, g->col, g->n, g->arcs, &g->ioff, &g->icol, g->ctx->stream);
+  cudaStream_t st = g->ctx->stream;
+  u32 *ioff, *icol;
+  const int rc = transpose_csr(g->off, g->col, g->n, g->arcs, &ioff, &icol, st);
+  if (rc != TKC_OK) {  // the handle stays without one: its pointer says that it is complete
+    if (ioff) cudaFreeAsync(ioff, st);
+    if (icol) cudaFreeAsync(icol, st);
+    return rc;
+  }
+  g->ioff = ioff;
+  g->icol = icol;
+  return TKC_OK;
 }
 
 // The in-arc CSR, built the first time a step needs it (a graph loaded only
@@ -1011,10 +1022,16 @@ int start_search_csr(const tkc_graph *g) {
   }
   TKC_TRY(cudaEventRecord(ctx->aux_in, ctx->stream));
   TKC_TRY(cudaStreamWaitEvent(ctx->aux, ctx->aux_in, 0));
-  TKC_RC(build_labelled_copy(g, ctx->aux));
   cudaEvent_t ready = nullptr;
   TKC_TRY(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
-  TKC_TRY(cudaEventRecord(ready, ctx->aux));
+  const int rc = build_labelled_copy(g, ctx->aux);
+  cudaError_t e = rc == TKC_OK ? cudaEventRecord(ready, ctx->aux) : cudaSuccess;
+  if (rc != TKC_OK || e != cudaSuccess) {
+    cudaEventDestroy(ready);
+    cudaStreamSynchronize(ctx->aux);  // what was begun is freed on the other stream
+    TKC_TRY(e);
+    return rc;
+  }
   g->s_ready = ready;
   g->s_mode = 1;
   return TKC_OK;
