@@ -121,7 +121,7 @@ int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u3
   cudaStream_t st = ctx->stream;
   ctx->last_shard = nullptr;  // what follows replaces the finished searches' (S, r)
   if (teams > w.teams_cap) {
-    w.teams_cap = w.n_cap = 0;  // (per-team vertex buffers are reallocated for the new team count)
+    w.teams_cap = 0;
     // the shared block, then the control blocks: read back together
     static_assert(sizeof(Shared) <= kShBytes, "the shared block fits its place");
     unsigned char *base = reinterpret_cast<unsigned char *>(w.sh);
@@ -157,31 +157,44 @@ int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u3
     TKC_RC(dalloc(&w.f_end, cap, st));
     w.ng_cap = cap;
   }
-  const u32 T = w.teams_cap;
   if (n > w.n_cap) {
-    u32 cap = std::max<u32>(n, 1024);
-    size_t tv = (size_t)T * cap, tfb = (size_t)T * (cap / 32 + 1);
-    w.n_cap = w.words_cap = 0;  // (rows are reallocated for the new n)
+    const u32 cap = std::max<u32>(n, 1024);
+    w.n_cap = 0;
+    TKC_RC(dalloc(&w.res_S, cap, st));
+    TKC_RC(dalloc(&w.res_r, cap, st));
+    TKC_RC(dalloc(&w.lvl2, cap, st));
+    w.n_cap = cap;
+  }
+  // The teams' rows, lists and bitmaps lie as this run needs them, each team's
+  // from a 256-byte boundary: a context that ran 128 teams on 16 384 vertices
+  // needs no 128 sets of rows for 4 teams on 4 million.  Rows and bitmaps are
+  // zero between runs and stamps older than any level to come, under any layout.
+  w.vtx_stride = std::max<size_t>(((size_t)n + 63) / 64 * 64, 1024);
+  w.fb_stride = ((size_t)n / 32 + 64) / 64 * 64;
+  w.row_stride = w.vtx_stride * words;
+  const size_t tv = teams * w.vtx_stride, tfb = teams * w.fb_stride, rows = teams * w.row_stride;
+  if (tv > w.vtx_cap) {
+    w.vtx_cap = 0;
     TKC_RC(dalloc(&w.L0, tv, st));
     TKC_RC(dalloc(&w.L1, tv, st));
     TKC_RC(dalloc(&w.Loff0, tv, st));
     TKC_RC(dalloc(&w.Loff1, tv, st));
     TKC_RC(dalloc(&w.VL, tv, st));
     TKC_RC(dalloc(&w.stamp, tv, st));
-    TKC_RC(dalloc(&w.res_S, cap, st));
-    TKC_RC(dalloc(&w.res_r, cap, st));
-    TKC_RC(dalloc(&w.lvl2, cap, st));
+    TKC_TRY(cudaMemsetAsync(w.stamp, 0xff, tv * sizeof(u32), st));
+    w.level_base = 0;
+    w.vtx_cap = tv;
+  }
+  if (tfb > w.fb_cap) {
+    w.fb_cap = 0;
     TKC_RC(dalloc(&w.FB0, tfb, st));
     TKC_RC(dalloc(&w.FB1, tfb, st));
     TKC_TRY(cudaMemsetAsync(w.FB0, 0, tfb * sizeof(u32), st));
     TKC_TRY(cudaMemsetAsync(w.FB1, 0, tfb * sizeof(u32), st));
-    TKC_TRY(cudaMemsetAsync(w.stamp, 0xff, tv * sizeof(u32), st));
-    w.level_base = 0;
-    w.n_cap = cap;
+    w.fb_cap = tfb;
   }
-  if (words > w.words_cap) {
-    size_t rows = (size_t)T * w.n_cap * words;
-    w.words_cap = 0;
+  if (rows > w.rows_cap) {
+    w.rows_cap = 0;
     TKC_RC(dalloc(&w.seen, rows, st));
     TKC_RC(dalloc(&w.F0, rows, st));
     TKC_RC(dalloc(&w.F1, rows, st));
@@ -190,7 +203,7 @@ int ensure_workspace(tkc_ctx *ctx, u32 n, int words, u32 top_entries, u32 ng, u3
     TKC_TRY(cudaMemsetAsync(w.F0, 0, rows * sizeof(u64), st));
     TKC_TRY(cudaMemsetAsync(w.F1, 0, rows * sizeof(u64), st));
     TKC_TRY(cudaMemsetAsync(w.N, 0, rows * sizeof(u64), st));
-    w.words_cap = words;
+    w.rows_cap = rows;
   }
   return TKC_OK;
 }
@@ -234,18 +247,17 @@ static void free_workspace(tkc_ctx *ctx) {
 // read of their outcome -- they are set right here.
 static int reset_rows(tkc_ctx *ctx) {
   Workspace &w = ctx->ws;
-  const size_t T = w.teams_cap;
-  size_t rows = T * w.n_cap * w.words_cap;
+  const size_t T = w.teams_cap, rows = w.rows_cap;
   cudaStream_t st = ctx->stream;
   TKC_TRY(cudaMemsetAsync(w.seen, 0, rows * sizeof(u64), st));
   TKC_TRY(cudaMemsetAsync(w.F0, 0, rows * sizeof(u64), st));
   TKC_TRY(cudaMemsetAsync(w.F1, 0, rows * sizeof(u64), st));
   TKC_TRY(cudaMemsetAsync(w.N, 0, rows * sizeof(u64), st));
-  TKC_TRY(cudaMemsetAsync(w.FB0, 0, T * ((size_t)w.n_cap / 32 + 1) * sizeof(u32), st));
-  TKC_TRY(cudaMemsetAsync(w.FB1, 0, T * ((size_t)w.n_cap / 32 + 1) * sizeof(u32), st));
+  TKC_TRY(cudaMemsetAsync(w.FB0, 0, w.fb_cap * sizeof(u32), st));
+  TKC_TRY(cudaMemsetAsync(w.FB1, 0, w.fb_cap * sizeof(u32), st));
   TKC_TRY(cudaMemsetAsync(w.cnt, 0, T * 64 * kMaxWords * sizeof(unsigned), st));
   TKC_TRY(cudaMemsetAsync(w.wsum, 0, T * 64 * kMaxWords * sizeof(u64), st));
-  TKC_TRY(cudaMemsetAsync(w.stamp, 0xff, T * w.n_cap * sizeof(u32), st));
+  TKC_TRY(cudaMemsetAsync(w.stamp, 0xff, w.vtx_cap * sizeof(u32), st));
   w.level_base = 0;
   w.dirty = false;
   return TKC_OK;
@@ -634,9 +646,9 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   p.hist_cap = rs.hist_cap;
   p.lvl_stride = rs.lvl_stride;
   p.teams = T;
-  p.row_stride = (u64)w.n_cap * w.words_cap;
-  p.vtx_stride = w.n_cap;
-  p.fb_stride = w.n_cap / 32 + 1;
+  p.row_stride = w.row_stride;
+  p.vtx_stride = w.vtx_stride;
+  p.fb_stride = w.fb_stride;
   p.sh = w.sh;
   p.x = w.x;
   // default: a level runs bottom-up when its frontier's arcs exceed 1/8 of all arcs

@@ -235,8 +235,9 @@ struct RunParams {
 };
 
 struct Workspace {
-  uint32_t n_cap = 0;
-  int words_cap = 0;
+  uint32_t n_cap = 0;     // vertices of res_* and lvl2
+  size_t rows_cap = 0, vtx_cap = 0, fb_cap = 0;           // words of a row, list (or stamp) and bitmap buffer, all teams'
+  size_t row_stride = 0, vtx_stride = 0, fb_stride = 0;   // from one team's to the next, in the present run
   unsigned long long *seen = nullptr, *F0 = nullptr, *F1 = nullptr, *N = nullptr;
   uint32_t *FB0 = nullptr, *FB1 = nullptr;
   uint32_t *L0 = nullptr, *L1 = nullptr, *Loff0 = nullptr, *Loff1 = nullptr, *VL = nullptr, *stamp = nullptr;
@@ -269,7 +270,7 @@ struct Workspace {
   uint32_t top_cap = 0;   // entries of top_* (graphs x k)
   size_t out_cap = 0;     // bytes of out
   uint32_t ng_cap = 0;    // graphs of tied / g_ntop / g_ctr / x_*
-  uint32_t teams_cap = 0; // teams the per-team buffers are sized for
+  uint32_t teams_cap = 0; // teams of ctl, slots, cnt and wsum
   unsigned int level_base = 0;  // stamp epoch carried across runs
   bool dirty = false;     // a run ended with an error: rows and stamps are not as a run expects them
 };
