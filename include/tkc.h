@@ -138,8 +138,12 @@ typedef struct {
 } tkc_result;
 
 /* Creates a context on opt->device (NULL opt = defaults).  No paper
- * counterpart: owns the stream, options and device workspace; the caller owns
- * *out until tkc_destroy.  Errors: TKC_EINVAL (null out, an option out of
+ * counterpart: owns the stream, options, device workspace and a memory pool
+ * that everything on the device comes from; the caller owns *out until
+ * tkc_destroy.  The pool keeps up to 1/32 of the device's memory (9 GB of 280)
+ * that nothing uses, so that calls need not map their scratch anew; tkc_destroy
+ * gives it back, and so does any context on the device that finds no memory.
+ * A program that needs it for other allocations destroys idle contexts.  Errors: TKC_EINVAL (null out, an option out of
  * range: batch_bits, order, nb_levels, large_blocks, deterministic, relabel), TKC_ENOMEM, TKC_ECUDA
  * (no such device, no cooperative launch); *out is NULL on error. */
 int tkc_create(tkc_ctx **out, const tkc_options *opt);

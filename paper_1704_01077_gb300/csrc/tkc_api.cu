@@ -26,6 +26,18 @@ int tkc::enter(tkc_ctx *ctx) {
   return TKC_OK;
 }
 
+// The pools of the live contexts.  What one keeps idle is given back to the
+// driver when another (or it itself) finds no memory.  (Never destructed: a
+// context may be destroyed while the process ends.)
+static std::mutex g_pools_lock;
+static std::vector<tkc_ctx *> &g_pools = *new std::vector<tkc_ctx *>();
+
+static void trim_pools(int device) {
+  std::lock_guard<std::mutex> hold(g_pools_lock);
+  for (tkc_ctx *c : g_pools)
+    if (c->device == device) cudaMemPoolTrimTo(c->pool, 0);
+}
+
 cudaError_t tkc::dev_malloc_bytes(void **p, size_t bytes, cudaStream_t st) {
   tkc_ctx *ctx = t_ctx;
   *p = nullptr;
@@ -43,8 +55,18 @@ cudaError_t tkc::dev_malloc_bytes(void **p, size_t bytes, cudaStream_t st) {
     }
     uint64_t keep = ctx->total_mem / kPoolKeepShare;
     cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    std::lock_guard<std::mutex> hold(g_pools_lock);
+    g_pools.push_back(ctx);
   }
-  return cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
+  cudaError_t e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    cudaStreamSynchronize(st);  // (memory freed in stream order counts as used until then)
+    trim_pools(ctx->device);
+    e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
+    if (e != cudaSuccess) *p = nullptr;
+  }
+  return e;
 }
 
 // Whether the page-locked buffer holds `bytes` (grown up to kStageMost).
@@ -1020,7 +1042,13 @@ void tkc_destroy(tkc_ctx *ctx) {
   }
   if (ctx->aux_in) cudaEventDestroy(ctx->aux_in);
   if (ctx->stage) cudaFreeHost(ctx->stage);
-  if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+  if (ctx->pool) {
+    {
+      std::lock_guard<std::mutex> hold(g_pools_lock);
+      g_pools.erase(std::find(g_pools.begin(), g_pools.end(), ctx));
+    }
+    cudaMemPoolDestroy(ctx->pool);
+  }
   delete ctx;
 }
 
