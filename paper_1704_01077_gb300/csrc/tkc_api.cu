@@ -41,7 +41,11 @@ static void trim_pools(int device) {
 cudaError_t tkc::dev_malloc_bytes(void **p, size_t bytes, cudaStream_t st) {
   tkc_ctx *ctx = t_ctx;
   *p = nullptr;
-  if (ctx->fail_alloc && --ctx->fail_alloc == 0) return cudaErrorMemoryAllocation;
+  if (ctx->fail_alloc && --ctx->fail_alloc == 0) {
+    ctx->no_memory = !ctx->fail_once;
+    return cudaErrorMemoryAllocation;
+  }
+  if (ctx->no_memory) return cudaErrorMemoryAllocation;
   if (!ctx->pool) {
     cudaMemPoolProps props;
     memset(&props, 0, sizeof(props));
@@ -250,6 +254,20 @@ static int ensure_filter(tkc_ctx *ctx, u32 count, u32 nopen) {
   if (!w.f_count) TKC_RC(dalloc(&w.f_count, kFilterTiles, ctx->stream));
   w.f_cap = cap;
   return TKC_OK;
+}
+
+// Frees the per-team rows, lists and bitmaps.
+static void free_team_buffers(tkc_ctx *ctx) {
+  Workspace &w = ctx->ws;
+  for (u64 **p : {&w.seen, &w.F0, &w.F1, &w.N}) {
+    if (*p) cudaFreeAsync(*p, ctx->stream);
+    *p = nullptr;
+  }
+  for (u32 **p : {&w.FB0, &w.FB1, &w.L0, &w.L1, &w.Loff0, &w.Loff1, &w.VL, &w.stamp}) {
+    if (*p) cudaFreeAsync(*p, ctx->stream);
+    *p = nullptr;
+  }
+  w.rows_cap = w.vtx_cap = w.fb_cap = 0;
 }
 
 static void free_workspace(tkc_ctx *ctx) {
@@ -564,6 +582,24 @@ static int finish_run(tkc_ctx *ctx, const RunSetup &rs, const std::vector<GraphO
   return TKC_OK;
 }
 
+// Bytes for the per-team buffers of several graphs' union, which want `want`:
+// a quarter of the device's memory and half of what a call can still get.  (The
+// driver is asked only before the buffers grow by more than 1/64 of the device.)
+static u64 memory_for_teams(const tkc_ctx *ctx, u64 want) {
+  const Workspace &w = ctx->ws;
+  const u64 held = 32 * (u64)w.rows_cap + 24 * (u64)w.vtx_cap;
+  u64 budget = ctx->total_mem / 4;
+  if (want > held && want > ctx->total_mem / 64) {
+    size_t free_now = 0, total = 0;
+    uint64_t reserved = 0, used = 0;
+    if (cudaMemGetInfo(&free_now, &total) == cudaSuccess && ctx->pool &&
+        cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
+        cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess)
+      budget = std::min<u64>(budget, (free_now + (reserved - std::min(used, reserved)) + held) / 2);
+  }
+  return budget;
+}
+
 static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   const tkc_graph *g = rs.g;
   Workspace &w = ctx->ws;
@@ -577,17 +613,24 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
           : rs.nocut && rs.ng == 1 ? nocut_teams(g->n, rs.B, (u32)rs.W, (u32)maxb, rs.norder)
                                    : default_teams(g->n, rs.B, (u32)maxb, nb_one, rs.ng);
   // several graphs: every team's rows and lists cover the union, so as many
-  // teams as a quarter of the device's memory holds
+  // teams as a quarter of the device's memory holds, and half of what is free
   if (rs.ng > 1 && !o.teams) {
     const u64 per_team = (u64)g->n * (32 * rs.W + 24) + 1;
-    T = (u32)std::max<u64>(1, std::min<u64>(T, ctx->total_mem / 4 / per_team));
+    T = (u32)std::max<u64>(1, std::min<u64>(T, memory_for_teams(ctx, T * per_team) / per_team));
   }
   if (rs.force_teams) T = rs.force_teams;
   // deterministic schedule: one team, so x moves only at its level barriers
   // (updateBoundsLB rounds fix their own team count: no cuts, already exact)
   if (o.deterministic && !rs.force_teams) T = 1;
   T = std::max<u32>(1, std::min<u32>(T, (u32)maxb));
-  TKC_RC(ensure_workspace(ctx, g->n, rs.W, rs.kk * rs.ng, rs.ng, T));
+  // a team count of the library's choice: fewer when memory does not hold them
+  int rc_ws = ensure_workspace(ctx, g->n, rs.W, rs.kk * rs.ng, rs.ng, T);
+  while (rc_ws == TKC_ENOMEM && T > 1 && !o.teams && !rs.force_teams) {
+    free_team_buffers(ctx);
+    T /= 2;
+    rc_ws = ensure_workspace(ctx, g->n, rs.W, rs.kk * rs.ng, rs.ng, T);
+  }
+  TKC_RC(rc_ws);
   if (w.dirty || w.level_base > 0xF0000000u) TKC_RC(reset_rows(ctx));
   // Opening: a batch of promising sources (k_open_keys) -- or as many batches
   // as it takes for a full k-list -- runs alone (one graph: on the whole grid;
@@ -946,11 +989,20 @@ extern "C" {
 
 uint64_t tkc_kernel_launches(void) { return g_launches.load(std::memory_order_relaxed); }
 
-// For tests: the nth next device allocation of the context fails as one without
-// memory does (0: none).  Returns what was left of an earlier count.
+// For tests: the nth next device allocation of the context and all after it
+// fail as ones without memory do (0: none).  Returns what was left of an earlier
+// count, 0 when it had run out.
 uint64_t tkc_internal_fail_allocation(tkc_ctx *ctx, uint64_t nth) {
   const uint64_t left = ctx->fail_alloc;
   ctx->fail_alloc = nth;
+  ctx->no_memory = ctx->fail_once = false;
+  return left;
+}
+
+// The same for the nth one alone.
+uint64_t tkc_internal_fail_allocation_once(tkc_ctx *ctx, uint64_t nth) {
+  const uint64_t left = tkc_internal_fail_allocation(ctx, nth);
+  ctx->fail_once = true;
   return left;
 }
 

@@ -339,7 +339,9 @@ struct tkc_ctx {
   cudaMemPool_t pool = nullptr;  // device memory of the context and its graphs
   void *stage = nullptr;         // page-locked host buffer of short reads (read_back)
   size_t stage_bytes = 0;
-  uint64_t fail_alloc = 0;       // the fail_alloc-th next device allocation fails (0: none; tests)
+  uint64_t fail_alloc = 0;       // device allocations until one fails (0: none will; tests)
+  bool fail_once = false;        // that one alone, or
+  bool no_memory = false;        // all from there on
   tkc::Workspace ws;
   cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   cudaStream_t aux = nullptr;    // helper stream: the labelled copy, built while `stream` preprocesses
