@@ -1642,6 +1642,11 @@ int tkc_autotune(tkc_graph *g, uint32_t k, tkc_options *best) {
   if (kk == 0) return TKC_OK;
   TKC_RC(ensure_degree_order(g));
   TKC_RC(ensure_reach_bounds(g));
+  // Every configuration walks the same labelling: the copy that a batched search
+  // of this size may build is built before the first is timed.  (Built by the
+  // first one that leaves enough batches, it took 3.4 to 5 ms of that one's time
+  // on R-MAT 22 and nothing of the others'.)
+  if (labelled_by_size(ctx->opt, 64u, g->n)) TKC_RC(ensure_search_csr(g, true));
   cudaStream_t st = ctx->stream;
   const u32 ns = g->n_src_deg;
   const u32 head = std::min<u32>(ns, 1024);
