@@ -774,7 +774,9 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
       p.order = w.o_order;
     }
     p.norder = nopen;
+    TKC_TRY(cudaEventRecord(ctx->ev[6], st));
     TKC_RC(launch_phase(open_teams, w.ctl));
+    TKC_TRY(cudaEventRecord(ctx->ev[7], st));
     // the whole order but the picked ones, or what follows the opening
     const u32 first = pick ? 0u : nopen;
     p.order = rs.order + first;
@@ -795,6 +797,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     p.g_rest = 0;
     if (p.trace) p.trace += (size_t)p.trace_cap * 16;
   }
+  if (opening) TKC_TRY(cudaEventRecord(ctx->ev[3], st));
   TKC_RC(launch_phase(T, w.ctl + open_teams));
   TKC_TRY(cudaEventRecord(ctx->ev[5], st));
   size_t out_bytes = 0;
@@ -885,10 +888,12 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     rs_out.compactions = hctl->st_compactions;
     rs_out.compacted_away = hctl->st_compact_dropped;
     rs_out.alg_bytes = hctl->alg_bytes;
-    float kms = 0;
+    // the search kernel's launches, without what lies between them (the filter, a host wait, the copy's construction)
+    float kms = 0, oms = 0;
     TKC_TRY(cudaEventSynchronize(ctx->ev[5]));
-    cudaEventElapsedTime(&kms, ctx->ev[4], ctx->ev[5]);
-    rs_out.ms_kernel = kms;
+    cudaEventElapsedTime(&kms, ctx->ev[opening ? 3 : 4], ctx->ev[5]);
+    if (opening) cudaEventElapsedTime(&oms, ctx->ev[6], ctx->ev[7]);
+    rs_out.ms_kernel = kms + oms;
   }
   if (hctl->err) {
     TKC_RC(reset_rows(ctx));
@@ -1502,13 +1507,12 @@ static int topk_one(tkc_graph *g, uint32_t k, tkc_result *out, int harmonic) {
   r.bfs_finished = hc.bfs_finished;
   r.levels = hc.levels;
   r.alg_bytes = hc.alg_bytes;
-  float ms0 = 0, ms1 = 0, ms2 = 0;
+  float ms0 = 0, ms1 = 0;
   cudaEventElapsedTime(&ms0, ctx->ev[0], ctx->ev[1]);
   cudaEventElapsedTime(&ms1, ctx->ev[1], ctx->ev[2]);
-  cudaEventElapsedTime(&ms2, ctx->ev[4], ctx->ev[5]);
   r.ms_pre = ms0;
   r.ms_bfs = ms1;
-  r.ms_kernel = ms2;
+  r.ms_kernel = ctx->last_stats.ms_kernel;
   *out = r;
   return TKC_OK;
 }
@@ -1624,9 +1628,7 @@ static int topk_shard(tkc_graph *g, uint32_t k, uint32_t first, uint32_t shard, 
   cudaEventElapsedTime(&ms1, ctx->ev[1], ctx->ev[2]);
   r.ms_pre = ms0;
   r.ms_bfs = ms1;
-  float ms2 = 0;
-  cudaEventElapsedTime(&ms2, ctx->ev[4], ctx->ev[5]);
-  r.ms_kernel = ms2;
+  r.ms_kernel = ctx->last_stats.ms_kernel;
   ctx->last_shard = g;
   *out = r;
   return TKC_OK;
@@ -1914,10 +1916,7 @@ static int topk_bound(tkc_graph *g, uint32_t k, tkc_result *out) {
     rs.force_teams = std::min<u32>(T, (cnt + B - 1) / B);
     Ctl hc;
     LB_RC(run_search(ctx, rs, &hc));
-    float ms = 0;
-    LB_TRY(cudaEventSynchronize(ctx->ev[5]));
-    LB_TRY(cudaEventElapsedTime(&ms, ctx->ev[4], ctx->ev[5]));
-    ms_kernel += ms;
+    ms_kernel += ctx->last_stats.ms_kernel;
     total.edges_visited += hc.edges_visited;
     total.edges_scanned += hc.edges_scanned;
     total.bfs_started += hc.bfs_started;
@@ -2170,10 +2169,9 @@ static int topk_many(tkc_ctx *ctx, tkc_graph *const *gs, uint32_t ng, uint32_t k
   std::vector<unsigned> tied;
   std::vector<u64> gctr;
   MULTI_RC(finish_run(ctx, rs, go, outs, tied, gctr));
-  float ms0 = 0, ms1 = 0, ms2 = 0;
+  float ms0 = 0, ms1 = 0;
   cudaEventElapsedTime(&ms0, ctx->ev[0], ctx->ev[1]);
   cudaEventElapsedTime(&ms1, ctx->ev[1], ctx->ev[2]);
-  cudaEventElapsedTime(&ms2, ctx->ev[4], ctx->ev[5]);
   for (u32 i = 0; i < ng; ++i) {
     tkc_result &r = outs[i];
     r.n_tied_at_kth = tied[i];
@@ -2187,7 +2185,7 @@ static int topk_many(tkc_ctx *ctx, tkc_graph *const *gs, uint32_t ng, uint32_t k
     r.batch_bits = bits;
     r.ms_pre = ms0;
     r.ms_bfs = ms1;
-    r.ms_kernel = ms2;
+    r.ms_kernel = ctx->last_stats.ms_kernel;
   }
 #undef MULTI_TRY
 #undef MULTI_RC

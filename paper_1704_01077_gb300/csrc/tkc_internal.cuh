@@ -343,7 +343,9 @@ struct tkc_ctx {
   bool fail_once = false;        // that one alone, or
   bool no_memory = false;        // all from there on
   tkc::Workspace ws;
-  cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+  // a call's start, the end of its preprocessing, its end; the start of the main
+  // launch after an opening; a search's start and end; the opening's start and end
+  cudaEvent_t ev[8] = {};
   cudaStream_t aux = nullptr;    // helper stream: the labelled copy, built while `stream` preprocesses
   cudaEvent_t aux_in = nullptr;  // orders the helper stream after `stream`'s work so far
   int graphs_alive = 0;
