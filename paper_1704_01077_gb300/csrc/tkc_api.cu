@@ -38,6 +38,20 @@ static void trim_pools(int device) {
     if (c->device == device) cudaMemPoolTrimTo(c->pool, 0);
 }
 
+// Bytes of memory of a device, asked for once per process (16 us).
+static size_t device_bytes(int device) {
+  static std::atomic<size_t> known[64];
+  std::atomic<size_t> *k = device >= 0 && device < 64 ? &known[device] : nullptr;
+  size_t total = k ? k->load(std::memory_order_relaxed) : 0, free_now = 0;
+  if (total) return total;
+  if (cudaMemGetInfo(&free_now, &total) != cudaSuccess) {  // (of the current device: every caller has entered its context)
+    cudaGetLastError();
+    return 0;
+  }
+  if (k) k->store(total, std::memory_order_relaxed);
+  return total;
+}
+
 cudaError_t tkc::dev_malloc_bytes(void **p, size_t bytes, cudaStream_t st) {
   tkc_ctx *ctx = t_ctx;
   *p = nullptr;
@@ -57,7 +71,7 @@ cudaError_t tkc::dev_malloc_bytes(void **p, size_t bytes, cudaStream_t st) {
       ctx->pool = nullptr;
       return e;
     }
-    uint64_t keep = ctx->total_mem / kPoolKeepShare;
+    uint64_t keep = device_bytes(ctx->device) / kPoolKeepShare;
     cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
     std::lock_guard<std::mutex> hold(g_pools_lock);
     g_pools.push_back(ctx);
@@ -588,9 +602,9 @@ static int finish_run(tkc_ctx *ctx, const RunSetup &rs, const std::vector<GraphO
 static u64 memory_for_teams(const tkc_ctx *ctx, u64 want) {
   const Workspace &w = ctx->ws;
   const u64 held = 32 * (u64)w.rows_cap + 24 * (u64)w.vtx_cap;
-  u64 budget = ctx->total_mem / 4;
-  if (want > held && want > ctx->total_mem / 64) {
-    size_t free_now = 0, total = 0;
+  size_t free_now = 0, total = device_bytes(ctx->device);
+  u64 budget = total / 4;
+  if (want > held && want > total / 64) {
     uint64_t reserved = 0, used = 0;
     if (cudaMemGetInfo(&free_now, &total) == cudaSuccess && ctx->pool &&
         cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
@@ -1057,8 +1071,6 @@ int tkc_create(tkc_ctx **out, const tkc_options *opt) {
   int coop = 0;
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device);
   cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device);
-  size_t mem_free = 0;
-  cudaMemGetInfo(&mem_free, &ctx->total_mem);
   if (!coop || ctx->num_sms <= 0) {
     delete ctx;
     return TKC_ECUDA;

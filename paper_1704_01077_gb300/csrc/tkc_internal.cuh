@@ -335,7 +335,6 @@ struct tkc_ctx {
   cudaStream_t stream = nullptr;
   tkc_options opt{};
   int num_sms = 0;
-  size_t total_mem = 0;  // bytes of device memory
   cudaMemPool_t pool = nullptr;  // device memory of the context and its graphs
   void *stage = nullptr;         // page-locked host buffer of short reads (read_back)
   size_t stage_bytes = 0;
