@@ -319,7 +319,7 @@ int tkc_set_source_order(tkc_graph *g, const uint32_t *order);
 /* Reach bounds alpha(v) <= r(v) <= omega(v) (Section 8.4, Algorithm 6; exact
  * component size for undirected graphs) into host arrays alpha[n], omega[n].
  * Errors: TKC_EINVAL (null g, or a null array with n > 0), TKC_ENOMEM,
- * TKC_ECUDA, TKC_ETIMEOUT (an SCC iteration exceeded n + 1 rounds). */
+ * TKC_ECUDA, TKC_ETIMEOUT (a device-side wait exceeded its budget). */
 int tkc_reach_bounds(tkc_graph *g, uint32_t *alpha, uint32_t *omega);
 
 /* computeBoundsNB (Section 5, Algorithm 3; Eq. 3 for directed graphs; Eq. 6

@@ -480,11 +480,14 @@ struct RunSetup {
 
 // Teams used when the options leave it to the library, so that the latency of
 // one team's level steps overlaps with the others'.  NBCut on one graph
-// examines few sources, each batch deeper: fewer, larger teams (measured on
-// R-MAT 22: 4 teams 357 ms, 9 teams 372 ms, 19 teams 411 ms).  Several graphs:
+// examines few sources, each batch deeper: fewer, larger teams (search kernel
+// with 1, 2, 4, 9 and 19 teams: directed Erdos-Renyi, 1.2 million vertices 18.2,
+// 14.6, 14.4, 17.9 and 21.8 ms, 200 000 vertices 2.32, 1.62, 1.26, 1.33 and 1.46;
+// Barabasi-Albert 10^6, k = 100 1.04, 1.03, 1.23, 1.25 and 1.22; on R-MAT 17 to 22
+// the filter leaves one batch and the count makes no difference).  Several graphs:
 // four blocks per team, since a level of one of the graphs is short (512
-// graphs of 1 000 to 200 000 vertices, 128-bit batches: 19 teams 203 ms a
-// call, 38 teams 184 ms).  Small graphs: teams of as many blocks as give every
+// graphs of 1 000 to 200 000 vertices, 128-bit batches: 19 teams 130 ms a
+// call, 38 teams 114, 76 teams 113).  Small graphs: teams of as many blocks as give every
 // warp of a sweep one group of 32 vertices, at most eight, since batches of
 // side-by-side teams cut against an older threshold.
 static u32 default_teams(u32 n, u32 B, u32 maxb, bool nb, u32 ng) {
@@ -501,9 +504,14 @@ static u32 default_teams(u32 n, u32 B, u32 maxb, bool nb, u32 ng) {
 // then has no barrier to wait at -- while their rows and lists together fit
 // L2.  A batch takes about 1 + 9/b on a team of b blocks (R-MAT 14, 64-bit
 // batches: 0.73, 0.40, 0.31, 0.26, 0.22 ms for 1 to 5 blocks), and the teams
-// take ceil(batches / teams) of them; the least product decides.  (128 batches
-// on 109 teams of one block took 1.21 ms, on 76 teams of two 0.80, on 128
-// teams 0.73.)
+// take ceil(batches / teams) of them; the least product decides.  (Search kernel
+// at the count this chooses, and at the best of 1, 4, 9, 19, 25, 38, 50, 76, 100,
+// 128 and 152 teams: R-MAT 14, 8 192 sources 128: 0.87 ms, 76: 0.84; R-MAT 12, 2 048
+// sources 32: 0.27, 38: 0.26; Barabasi-Albert 20 000, 10 000 sources 50: 1.24, 76:
+// 1.21; 100 000, 4 000 sources 21: 1.78, 38: 1.90; 300 000, 2 048 sources 16: 2.82, 19: 3.07;
+// Erdos-Renyi 50 000, 10 000 sources 44: 3.24, 38: 3.11; 60 x 60 grid, 1 800
+// sources 29: 1.87, 38: 1.92; farthest off on Erdos-Renyi 5 000, 2 500 sources 40: 0.56,
+// 25: 0.39.)  120 MB: the chip's 129 MB of L2 less what the graph itself takes of it.
 static u32 nocut_teams(u32 n, u32 B, u32 W, u32 maxb, u32 norder) {
   const u64 fit = (120ull << 20) / ((u64)n * (32 * W + 24) + 1);
   const u32 batches = std::max<u32>(1, (norder + B - 1) / B);
@@ -532,7 +540,8 @@ static bool labelled_by_size(const tkc_options &o, u32 B, u32 size_n) {
 
 // With an opening the copy is built only when the filter leaves at least this
 // many batches: on R-MAT 22 it costs 3.4 to 5 ms of device work and saved 0.2 ms
-// per 128-source batch (51 -> 35 ms over 81 batches); the filter leaves one.
+// per 128-source batch (51 -> 35 ms over the 81 batches that a search without the
+// filter took there; the filter leaves one).
 constexpr u32 kLabelBatches = 24;
 
 // Enqueues the output step of a run: ties and the final lists, packed into the

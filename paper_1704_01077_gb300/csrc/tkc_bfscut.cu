@@ -195,8 +195,10 @@ constexpr double kHMargin = 1.0 + 1.0 / 1048576.0;
 
 // Bottom-up walks, batches of at most 256 bits: in-arcs a lane takes per step
 // when it walks a short in-row alone (U), and per lane per step when the warp
-// walks a long one (HU).  Measured on R-MAT 22, NBCut: 4 and 4 beat 2 and 8
-// either way (2 to 5% slower).
+// walks a long one (HU).  Search kernel, distance sums of 4 096 sources of
+// R-MAT 20 and NBCut on a directed Erdos-Renyi graph of 1.2 million vertices and
+// 9.6 million arcs (both on the labelled copy): 4 and 4 10.7 and 14.4 ms; U 2
+// 10.6 and 14.3, U 8 11.1 and 14.8; HU 2 11.0 and 14.2, HU 8 11.1 and 14.4.
 #ifndef TKC_BU_U
 #define TKC_BU_U 4
 #endif
@@ -207,8 +209,8 @@ constexpr double kHMargin = 1.0 + 1.0 / 1048576.0;
 // Threads per block of the search kernel (one block per SM).  The level loops
 // wait on dependent row gathers, so more resident warps hide more latency:
 // the 64- and 128-bit kernels run 32 warps per SM, at the price of a few
-// spilled registers (measured on R-MAT 22, NBCut: 1024 threads beat 768 by 5%
-// for 128-bit batches; DegCut and NBCut, 64-bit: 1024 beat 512 by 30%).
+// spilled registers (the two searches above, 64- and 128-bit: 1024 threads 10.7
+// and 14.4 ms, 512 threads 15.3 and 17.0; 768 threads for 128-bit batches 15.1).
 #ifndef TKC_THREADS_W2
 #define TKC_THREADS_W2 1024
 #endif
@@ -2229,9 +2231,11 @@ int run_filter(tkc_ctx *ctx, const RunParams &p, const tkc_graph *g, uint32_t op
   return TKC_OK;
 }
 
-// The larger blocks pay off on batched searches of large graphs (R-MAT 20 and
-// 22); one-source searches and graphs below 2^20 vertices (BA 10^6: 1.75 ms of
-// kernel time at 512 threads, 1.98 ms at 768) run 512 threads per block.
+// The larger blocks pay off on batched searches of large graphs (NBCut on
+// R-MAT 22 1.36 -> 1.07 ms of kernel time); one-source searches and graphs below
+// 2^20 vertices run 512 threads per block.  Near the line it depends on the graph
+// (NBCut, 512 and 1024 threads: R-MAT 16 0.25 and 0.28 ms, R-MAT 18 0.28 and 0.31,
+// R-MAT 19 0.37 and 0.39, Barabasi-Albert 131 072 0.27 and 0.31, 10^6 1.23 and 1.02).
 static bool wide_blocks(const RunParams &p) {
   if (p.large_blocks) return p.large_blocks == 1;
   return p.B > 1 && p.n >= (1u << 20);

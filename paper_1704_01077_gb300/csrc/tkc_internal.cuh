@@ -45,8 +45,8 @@ constexpr uint32_t kBuChunkVerts = 128;  // bottom-up levels: list entries per c
 // In id order a warp's 32 lanes hold rows of unrelated lengths, so rows
 // beyond a few steps of a lane go to the warp (kHeavyIn); in the in-degree
 // labelling neighbouring rows have similar lengths and a lane may keep longer
-// ones (kHeavyInLabelled; R-MAT 22, NBCut, search kernel: 24 -> 34.5 ms,
-// 48 -> 33.1, 96 -> 32.4, 192 to 384 -> 32.5).
+// ones (kHeavyInLabelled; distance sums of 4 096 sources of R-MAT 20, search
+// kernel: 24 -> 11.8 ms, 48 -> 11.3, 96 -> 10.7, 192 -> 10.7).
 #ifndef TKC_HEAVY_IN
 #define TKC_HEAVY_IN 24
 #endif
