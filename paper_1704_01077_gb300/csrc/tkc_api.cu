@@ -623,6 +623,17 @@ static u64 memory_for_teams(const tkc_ctx *ctx, u64 want) {
   return budget;
 }
 
+// Time of one launch of the search kernel, first team's start to last team's end.
+static double launch_ms(const Ctl *c, u32 teams) {
+  u64 first = ~0ull, last = 0;
+  for (u32 t = 0; t < teams; ++t) {
+    if (!c[t].t_end) continue;  // (a team that the filter left nothing for)
+    first = std::min<u64>(first, c[t].t_start);
+    last = std::max<u64>(last, c[t].t_end);
+  }
+  return last > first ? 1e-6 * (double)(last - first) : 0.0;
+}
+
 static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   const tkc_graph *g = rs.g;
   Workspace &w = ctx->ws;
@@ -780,7 +791,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
   memset(hctl, 0, sizeof(Ctl));
   std::vector<Ctl> cs(open_teams + T);
   Shared hsh;
-  TKC_TRY(cudaEventRecord(ctx->ev[4], st));
+  TKC_TRY(cudaEventRecord(ctx->ev[3], st));
   p.trace_cap = p.trace ? trace_cap / 2 : 0;  // half for each launch
   auto launch_phase = [&](u32 teams, Ctl *ctl) {
     p.teams = teams;
@@ -797,9 +808,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
       p.order = w.o_order;
     }
     p.norder = nopen;
-    TKC_TRY(cudaEventRecord(ctx->ev[6], st));
     TKC_RC(launch_phase(open_teams, w.ctl));
-    TKC_TRY(cudaEventRecord(ctx->ev[7], st));
     // the whole order but the picked ones, or what follows the opening
     const u32 first = pick ? 0u : nopen;
     p.order = rs.order + first;
@@ -820,9 +829,8 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     p.g_rest = 0;
     if (p.trace) p.trace += (size_t)p.trace_cap * 16;
   }
-  if (opening) TKC_TRY(cudaEventRecord(ctx->ev[3], st));
   TKC_RC(launch_phase(T, w.ctl + open_teams));
-  TKC_TRY(cudaEventRecord(ctx->ev[5], st));
+  TKC_TRY(cudaEventRecord(ctx->ev[4], st));
   size_t out_bytes = 0;
   if (rs.go) {
     TKC_RC(enqueue_output(ctx, rs, *rs.go));
@@ -912,11 +920,7 @@ static int run_search(tkc_ctx *ctx, const RunSetup &rs, Ctl *hctl) {
     rs_out.compacted_away = hctl->st_compact_dropped;
     rs_out.alg_bytes = hctl->alg_bytes;
     // the search kernel's launches, without what lies between them (the filter, a host wait, the copy's construction)
-    float kms = 0, oms = 0;
-    TKC_TRY(cudaEventSynchronize(ctx->ev[5]));
-    cudaEventElapsedTime(&kms, ctx->ev[opening ? 3 : 4], ctx->ev[5]);
-    if (opening) cudaEventElapsedTime(&oms, ctx->ev[6], ctx->ev[7]);
-    rs_out.ms_kernel = kms + oms;
+    rs_out.ms_kernel = launch_ms(cs.data(), open_teams) + launch_ms(cs.data() + open_teams, T);
   }
   if (hctl->err) {
     TKC_RC(reset_rows(ctx));
@@ -1448,7 +1452,7 @@ static int time_config(tkc_graph *g, const u32 *order, u32 norder, u32 kk, u32 b
   ctx->opt = saved;
   if (rc != TKC_OK) return rc;
   float t = 0;
-  cudaEventElapsedTime(&t, ctx->ev[4], ctx->ev[5]);
+  cudaEventElapsedTime(&t, ctx->ev[3], ctx->ev[4]);
   *ms = t;
   return TKC_OK;
 }

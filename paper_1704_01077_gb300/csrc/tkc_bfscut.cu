@@ -62,6 +62,11 @@ __device__ __forceinline__ void st_release_u32(unsigned *p, unsigned v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 __device__ __forceinline__ int ld_volatile_i32(const int *p) { return *(volatile const int *)p; }
+__device__ __forceinline__ unsigned long long now_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
 // One 128-bit word, read and written whole.
 __device__ __forceinline__ ulonglong2 ld_relaxed_128(const ulonglong2 *p) {
   ulonglong2 v;
@@ -751,8 +756,7 @@ __device__ __forceinline__ void trace_stamp(const RunParams &p, int slot) {
   if (p.trace && threadIdx.x == 0) {
     u64 idx = ((volatile Ctl *)p.ctl)->trace_n;
     if (idx < p.trace_cap) {
-      u64 t;
-      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+      const u64 t = now_ns();
       p.trace[idx * 16 + slot] = t;
     }
   }
@@ -954,8 +958,7 @@ __device__ __noinline__ void epilogue_level(const RunParams &p, Smem<W> &sm) {
     if (p.trace) {
       u64 idx = c->trace_n++;
       if (idx < p.trace_cap) {
-        u64 t;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+        const u64 t = now_ns();
         u64 *rec = p.trace + idx * 16;
         rec[0] = t;
         rec[1] = (u64)dir;
@@ -1219,8 +1222,7 @@ __device__ __noinline__ void epilogue_seed(const RunParams &p, Smem<W> &sm) {
     if (p.trace) {
       u64 idx = c->trace_n++;
       if (idx < p.trace_cap) {
-        u64 t;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+        const u64 t = now_ns();
         u64 *rec = p.trace + idx * 16;
         rec[0] = t;
         rec[1] = 2;  // seed step
@@ -1296,6 +1298,7 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
       p.trace_cap = p0.trace_cap / p0.teams;
       p.trace = p0.trace + (size_t)team * p.trace_cap * 16;
     }
+    if (tb == 0) p.ctl->t_start = now_ns();
   }
   __syncthreads();
   Ctl *c = p.ctl;
@@ -1768,6 +1771,7 @@ __global__ void __launch_bounds__(TPB, 1) bfscut_kernel(RunParams p0) {
     if (tb == 0) trace_stamp(p, 12);
     if (!team_sync(c, p.sh, bpt, p.timeout, [&] { epilogue_level<W>(p, sm); })) break;
   }
+  if (tb == 0 && threadIdx.x == 0) c->t_end = now_ns();
 }
 
 // ------------------------------------------------------------------ before the launches

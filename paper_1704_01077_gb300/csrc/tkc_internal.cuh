@@ -103,6 +103,7 @@ struct Ctl {
   unsigned long long st_seeded, st_cleared;
   unsigned long long st_compactions, st_compact_dropped;
   unsigned long long st_bu_swept;
+  unsigned long long t_start, t_end;  // the team's first block, ns of the device's global timer
 };
 constexpr int kCmdWords = (offsetof(Ctl, nl_packed) - offsetof(Ctl, step)) / 4;
 
@@ -342,9 +343,8 @@ struct tkc_ctx {
   bool fail_once = false;        // that one alone, or
   bool no_memory = false;        // all from there on
   tkc::Workspace ws;
-  // a call's start, the end of its preprocessing, its end; the start of the main
-  // launch after an opening; a search's start and end; the opening's start and end
-  cudaEvent_t ev[8] = {};
+  // a call's start, the end of its preprocessing, its end; a search's start and end
+  cudaEvent_t ev[5] = {};
   cudaStream_t aux = nullptr;    // helper stream: the labelled copy, built while `stream` preprocesses
   cudaEvent_t aux_in = nullptr;  // orders the helper stream after `stream`'s work so far
   int graphs_alive = 0;
