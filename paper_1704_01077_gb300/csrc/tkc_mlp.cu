@@ -233,13 +233,13 @@ __global__ void __launch_bounds__(FT) k_mlp_forward(const float *x, u32 m, const
   for (int i = threadIdx.x; i < P; i += FT) ws[i] = weight(wb, i);
   __syncthreads();
   static_assert(oW2 % 4 == 0 && H % 4 == 0, "the second layer's rows are read four words at a time");
-  // (64-bit positions: a step past the last of nearly 2^32 samples must not start over)
-  for (u64 i0 = (u64)blockIdx.x * FT; i0 < m; i0 += (u64)gridDim.x * FT) {
-    const u64 i = i0 + threadIdx.x;
+  // (by tiles: a position one step past the last of nearly 2^32 samples would start over)
+  for (u32 tile = blockIdx.x; tile < (m - 1) / FT + 1; tile += gridDim.x) {
+    const u32 i = tile * FT + threadIdx.x;  // tile * FT + FT - 1 is below 2^32
     const bool valid = i < m;
     float xi[F];
 #pragma unroll
-    for (int f = 0; f < F; ++f) xi[f] = valid ? x[i * F + f] : 0.f;
+    for (int f = 0; f < F; ++f) xi[f] = valid ? x[(size_t)i * F + f] : 0.f;
     float h1[H];
 #pragma unroll
     for (int o = 0; o < H; ++o) {
@@ -302,11 +302,12 @@ __global__ void __launch_bounds__(kGradTPB) k_mlp_grad(const float *x, const flo
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   float g2[4][4] = {}, g1[2] = {0.f, 0.f}, gb = 0.f;  // this thread's sums
   double l = 0.0;  // of many small terms from every block: added up in 64 bits
-  for (u64 base = (u64)blockIdx.x * TS; base < m; base += (u64)gridDim.x * TS) {  // (64 bits as in the forward pass)
+  for (u32 tile = blockIdx.x; tile < (m - 1) / TS + 1; tile += gridDim.x) {  // (by tiles as in the forward pass)
+    const u32 base = tile * TS;
     __syncthreads();
     for (int i = threadIdx.x; i < TS * F; i += kGradTPB) {
-      const u64 s = base + i / F;
-      X[i] = s < m ? x[s * F + i % F] : 0.f;
+      const u32 s = base + i / F;
+      X[i] = s < m ? x[(size_t)s * F + i % F] : 0.f;
     }
     __syncthreads();
 #pragma unroll
