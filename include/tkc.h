@@ -380,7 +380,7 @@ int tkc_distance_sums(tkc_graph *g, uint32_t nsrc, const uint32_t *srcs, uint64_
  *    whose GPU work overlaps race on it, so serialise them.
  *  - The call returns after the results are written (it synchronises `stream`).
  * Errors: TKC_EINVAL (n > TKC_NOALLOC_MAX_N, a null pointer, a source out of
- * range or repeated), TKC_EGRAPH (offsets not monotone, offsets[0] != 0,
+ * range or repeated, so nsrc > n too), TKC_EGRAPH (offsets not monotone, offsets[0] != 0,
  * offsets[n] != arcs, a column out of range), TKC_EOVERFLOW, TKC_ECUDA,
  * TKC_ETIMEOUT.  nsrc = 0 returns TKC_OK without touching the device. */
 #define TKC_NOALLOC_MAX_N 65536

@@ -147,6 +147,7 @@ extern "C" int tkc_distance_sums_noalloc(const uint32_t *offsets, const uint32_t
   if (arcs >= (1ull << 32)) return TKC_EOVERFLOW;
   if (nsrc == 0) return TKC_OK;
   if (n == 0 || !offsets || (arcs && !cols) || !srcs || !S || !r) return TKC_EINVAL;
+  if (nsrc > n) return TKC_EINVAL;  // they cannot be distinct (and k_check's 32-bit steps would pass 2^32 near it)
   int dev = 0;
   TKC_TRY(cudaGetDevice(&dev));
   unsigned char *base = nullptr;
